@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <utility>
 
 #include "dev.cuh"
 #include "launch.hpp"
@@ -335,6 +336,12 @@ __global__ void k_efield(DevTree t, const T *V, T *E) {
   T cn = (T)(t.uniform ? t.nc : t.dcnt[v]);
   for (int a = 0; a < t.d; ++a) E[a * t.n_vert + v] = -(acc[a] / cn);
 }
+
+}  // namespace pic
+
+#include "uniform_solve.cuh"
+
+namespace pic {
 
 // ---------------------------------------------------------------------------
 // a1/a2 initial keys and split conversion
@@ -1346,36 +1353,59 @@ void launch_deposit(const DevTree &t, bool split, const int32_t *start, const vo
   launch_vertex_charge(t, split, part, Q, block_sum, total, s);
 }
 
+// One sweep (Vout) or, with r2, the block sums of the squared residual;
+// returns the number of blocks.
+template <typename T>
+static int64_t jacobi_pass(const DevTree &t, const T *b, const T *Vin, T *Vout, T omega, double *r2, cudaStream_t s) {
+  if (t.uniform) {
+    if (t.d == 3)
+      return r2 ? launch_jacobi_uniform<T, 3, true>(t, b, Vin, Vout, omega, r2, s)
+                : launch_jacobi_uniform<T, 3, false>(t, b, Vin, Vout, omega, r2, s);
+    return r2 ? launch_jacobi_uniform<T, 2, true>(t, b, Vin, Vout, omega, r2, s)
+              : launch_jacobi_uniform<T, 2, false>(t, b, Vin, Vout, omega, r2, s);
+  }
+  const unsigned g = grid_for(t.n_vert);
+  COUNT(1);
+  k_jacobi<T><<<g, kBlock, 0, s>>>(t, b, Vin, Vout, omega, r2);
+  return g;
+}
+
+template <typename T>
+static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V, T *Vtmp, int sweeps, T omega,
+                  double *block_sum, double *resid2, cudaStream_t s) {
+  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b); }
+  T *in = V, *out = Vtmp;
+  for (int it = 0; it < sweeps; ++it) {
+    jacobi_pass<T>(t, b, in, out, omega, nullptr, s);
+    std::swap(in, out);
+  }
+  if (in != V) cudaMemcpyAsync(V, in, sizeof(T) * t.n_vert, cudaMemcpyDeviceToDevice, s);
+  const int64_t nb = jacobi_pass<T>(t, b, V, nullptr, omega, block_sum, s);
+  { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
+}
+
 void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,
                   int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s) {
-  unsigned g = grid_for(t.n_vert);
-  if (split) {
-    { COUNT(1); k_rhs<float><<<g, kBlock, 0, s>>>(t, (const float *)Q, total, (float *)b); }
-    float *a = (float *)V, *c = (float *)Vtmp;
-    for (int it = 0; it < sweeps; ++it) {
-      { COUNT(1); k_jacobi<float><<<g, kBlock, 0, s>>>(t, (const float *)b, a, c, (float)omega, nullptr); }
-      float *tmp = a; a = c; c = tmp;
-    }
-    if (a != (float *)V) cudaMemcpyAsync(V, a, sizeof(float) * t.n_vert, cudaMemcpyDeviceToDevice, s);
-    { COUNT(1); k_jacobi<float><<<g, kBlock, 0, s>>>(t, (const float *)b, (const float *)V, nullptr, (float)omega, block_sum); }
-  } else {
-    { COUNT(1); k_rhs<double><<<g, kBlock, 0, s>>>(t, (const double *)Q, total, (double *)b); }
-    double *a = (double *)V, *c = (double *)Vtmp;
-    for (int it = 0; it < sweeps; ++it) {
-      { COUNT(1); k_jacobi<double><<<g, kBlock, 0, s>>>(t, (const double *)b, a, c, omega, nullptr); }
-      double *tmp = a; a = c; c = tmp;
-    }
-    if (a != (double *)V) cudaMemcpyAsync(V, a, sizeof(double) * t.n_vert, cudaMemcpyDeviceToDevice, s);
-    { COUNT(1); k_jacobi<double><<<g, kBlock, 0, s>>>(t, (const double *)b, (const double *)V, nullptr, omega, block_sum); }
-  }
-  { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, g, resid2); }
+  if (split)
+    solve<float>(t, (const float *)Q, total, (float *)b, (float *)V, (float *)Vtmp, sweeps, (float)omega, block_sum,
+                 resid2, s);
+  else
+    solve<double>(t, (const double *)Q, total, (double *)b, (double *)V, (double *)Vtmp, sweeps, omega, block_sum,
+                  resid2, s);
+}
+
+template <typename T>
+static void efield(const DevTree &t, const T *V, T *E, cudaStream_t s) {
+  COUNT(1);
+  const unsigned g = grid_for(t.n_vert);
+  if (!t.uniform) k_efield<T><<<g, kBlock, 0, s>>>(t, V, E);
+  else if (t.d == 3) k_efield_uniform<3><<<g, kBlock, 0, s>>>(t, V, E);
+  else k_efield_uniform<2><<<g, kBlock, 0, s>>>(t, V, E);
 }
 
 void launch_efield(const DevTree &t, bool split, const void *V, void *E, cudaStream_t s) {
-  if (split)
-    { COUNT(1); k_efield<float><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, (const float *)V, (float *)E); }
-  else
-    { COUNT(1); k_efield<double><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, (const double *)V, (double *)E); }
+  if (split) efield<float>(t, (const float *)V, (float *)E, s);
+  else efield<double>(t, (const double *)V, (double *)E, s);
 }
 
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s) {

@@ -364,10 +364,15 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
     I.ion = h->cfg.ion;
     I.ion_load = ht.uniform ? ht.ion_load[0] : 0.0;
     I.diag = ht.uniform ? ht.diag[0] : 0.0;
+    I.h = 1.0 / (double)ht.M;
+    I.rdiag = ht.uniform ? 1.0 / I.diag : 0.0;
+    I.h32 = (float)I.h;
     I.q32 = (float)I.q;
     I.ion32 = (float)I.ion;
     I.ion_load32 = (float)I.ion_load;
     I.diag32 = (float)I.diag;
+    I.rdiag32 = ht.uniform ? 1.0f / I.diag32 : 0.0f;
+    I.rdiag_lo32 = ht.uniform ? (float)(1.0 / (double)I.diag32 - (double)I.rdiag32) : 0.0f;
     nl += ht.n_leaves;
     nv += ht.n_vert;
     npv += ht.n_pv;
