@@ -28,6 +28,8 @@ namespace pic {
 
 __constant__ double c_kref64[8][8];
 __constant__ float c_kref32[8][8];
+__constant__ double c_width64[19];  // 3^-level
+__constant__ float c_width32[19];
 
 constexpr int kBlock = 256;
 constexpr int kScanThreads = 1024;
@@ -132,20 +134,6 @@ __device__ __forceinline__ double diag_val(const DevTree &t, int64_t v, double) 
 }
 __device__ __forceinline__ float diag_val(const DevTree &t, int64_t v, float) {
   return t.uniform ? inst_of_vertex(t, v).diag32 : t.diag32[v];
-}
-
-// Visit the incident leaf corners (lc = leaf * 2^d + corner, ascending) of
-// vertex v with their constraint weights: fn(lc, w).
-template <typename T, typename Fn>
-__device__ __forceinline__ void for_incidences(const DevTree &t, int64_t v, Fn fn) {
-  if (t.uniform) {
-    int32_t lc[8];
-    int m = uniform_incidences(v, t.d, inst_of_vertex(t, v), t.spread, lc);
-    for (int i = 0; i < m; ++i) fn(lc[i], (T)1);
-  } else {
-    const T *ww = inc_weights(t, (T)0);
-    for (int32_t j = t.inc_ptr[v]; j < t.inc_ptr[v + 1]; ++j) fn(t.inc_lc[j], ww[j]);
-  }
 }
 
 // Block partial FP64 sums (fixed reduction tree) for deterministic totals.
@@ -268,78 +256,20 @@ __global__ void k_vertex_charge(DevTree t, const T *__restrict__ part, T *Q, dou
 // a8 solve (auxiliary): b = Q - (sum Q) integral(phi); damped Jacobi
 // ---------------------------------------------------------------------------
 
+// With scale, also omega / diag per vertex.
 template <typename T>
-__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b) {
+__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= t.n_vert) return;
   T tot = (T)(t.n_inst > 1 ? total[1 + t.inst_of_vert[v]] : *total);
   b[v] = Q[v] - tot * ion_load(t, v, (T)0);
-}
-
-// (A V)_v assembled leaf by leaf: sum over incident leaf corners (L, e) of
-// w * sum_f K_ef h^(d-2) V(L, f).
-template <typename T>
-__device__ __forceinline__ T apply_row(const DevTree &t, int64_t v, const T *V) {
-  T y = (T)0;
-  for_incidences<T>(t, v, [&](int32_t lc, T w) {
-    int32_t L = lc / t.nc;
-    int e = lc - L * t.nc;
-    int lev;
-    int32_t c[3] = {0, 0, 0};
-    leaf_info(t, L, &lev, c);
-    T hs = t.d == 2 ? (T)1 : (T)(1.0 / (double)c_pow3[lev]);
-    T yc = (T)0;
-    for (int f = 0; f < t.nc; ++f) yc = yc + (kref_val(e, f, (T)0) * hs) * corner_value(t, L, c, f, V);
-    y = y + w * yc;
-  });
-  return y;
-}
-
-// One sweep V_out = V_in + omega (b - A V_in) / diag; with r2 != NULL also
-// block sums of (b - A V_in)^2 in FP64.
-template <typename T>
-__global__ void k_jacobi(DevTree t, const T *b, const T *Vin, T *Vout, T omega, double *r2) {
-  int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double rr = 0.0;
-  if (v < t.n_vert) {
-    T y = apply_row<T>(t, v, Vin);
-    T r = b[v] - y;
-    if (Vout) Vout[v] = Vin[v] + omega * r / diag_val(t, v, (T)0);
-    rr = (double)r * (double)r;
-  }
-  if (r2) block_sum_store(rr, r2);
-}
-
-// E = -grad V at the vertices: minus the mean over leaves that have v as an
-// unconstrained corner of the leaf's edge difference along each axis.
-template <typename T>
-__global__ void k_efield(DevTree t, const T *V, T *E) {
-  int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= t.n_vert) return;
-  T acc[3] = {(T)0, (T)0, (T)0};
-  for_incidences<T>(t, v, [&](int32_t lc, T) {
-    int32_t L = lc / t.nc;
-    int e = lc - L * t.nc;
-    if (!t.uniform) {
-      if (t.cexp_ptr[lc + 1] - t.cexp_ptr[lc] != 1 || t.cexp_w64[t.cexp_ptr[lc]] != 1.0) return;
-    }
-    int lev;
-    int32_t c[3] = {0, 0, 0};
-    leaf_info(t, L, &lev, c);
-    T h = (T)(1.0 / (double)c_pow3[lev]);
-    for (int a = 0; a < t.d; ++a) {
-      T hi = corner_value(t, L, c, e | (1 << a), V);
-      T lo = corner_value(t, L, c, e & ~(1 << a), V);
-      acc[a] = acc[a] + (hi - lo) / h;
-    }
-  });
-  T cn = (T)(t.uniform ? t.nc : t.dcnt[v]);
-  for (int a = 0; a < t.d; ++a) E[a * t.n_vert + v] = -(acc[a] / cn);
+  if (scale) scale[v] = omega / diag_val(t, v, (T)0);
 }
 
 }  // namespace pic
 
 #include "uniform_solve.cuh"
+#include "adaptive_solve.cuh"
 
 namespace pic {
 
@@ -1189,6 +1119,15 @@ cudaError_t set_constants(cudaStream_t s) {
   uint32_t p3[21];
   p3[0] = 1;
   for (int i = 1; i < 21; ++i) p3[i] = p3[i - 1] * 3u;
+  double w64[19];
+  float w32[19];
+  for (int i = 0; i < 19; ++i) {
+    w64[i] = 1.0 / (double)p3[i];
+    w32[i] = (float)w64[i];
+  }
+  cudaError_t ew = cudaMemcpyToSymbolAsync(c_width64, w64, sizeof(w64), 0, cudaMemcpyHostToDevice, s);
+  if (ew == cudaSuccess) ew = cudaMemcpyToSymbolAsync(c_width32, w32, sizeof(w32), 0, cudaMemcpyHostToDevice, s);
+  if (ew != cudaSuccess) return ew;
   cudaError_t e = cudaFuncSetAttribute(k_sort_large, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(sizeof(int32_t) * kLargeSeg));
   if (e != cudaSuccess) return e;
@@ -1353,59 +1292,77 @@ void launch_deposit(const DevTree &t, bool split, const int32_t *start, const vo
   launch_vertex_charge(t, split, part, Q, block_sum, total, s);
 }
 
-// One sweep (Vout) or, with r2, the block sums of the squared residual;
-// returns the number of blocks.
-template <typename T>
-static int64_t jacobi_pass(const DevTree &t, const T *b, const T *Vin, T *Vout, T omega, double *r2, cudaStream_t s) {
-  if (t.uniform) {
-    if (t.d == 3)
-      return r2 ? launch_jacobi_uniform<T, 3, true>(t, b, Vin, Vout, omega, r2, s)
-                : launch_jacobi_uniform<T, 3, false>(t, b, Vin, Vout, omega, r2, s);
-    return r2 ? launch_jacobi_uniform<T, 2, true>(t, b, Vin, Vout, omega, r2, s)
-              : launch_jacobi_uniform<T, 2, false>(t, b, Vin, Vout, omega, r2, s);
-  }
-  const unsigned g = grid_for(t.n_vert);
-  COUNT(1);
-  k_jacobi<T><<<g, kBlock, 0, s>>>(t, b, Vin, Vout, omega, r2);
-  return g;
-}
-
-template <typename T>
-static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V, T *Vtmp, int sweeps, T omega,
-                  double *block_sum, double *resid2, cudaStream_t s) {
-  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b); }
+// Sweeps on a uniform tree between V and Vtmp, then the residual's block sums;
+// returns their number.
+template <typename T, int D>
+static int64_t sweep_uniform(const DevTree &t, const T *b, T *V, T *Vtmp, int sweeps, T omega, double *r2,
+                             cudaStream_t s) {
   T *in = V, *out = Vtmp;
   for (int it = 0; it < sweeps; ++it) {
-    jacobi_pass<T>(t, b, in, out, omega, nullptr, s);
+    launch_jacobi_uniform<T, D, false>(t, b, in, out, omega, nullptr, s);
     std::swap(in, out);
   }
   if (in != V) cudaMemcpyAsync(V, in, sizeof(T) * t.n_vert, cudaMemcpyDeviceToDevice, s);
-  const int64_t nb = jacobi_pass<T>(t, b, V, nullptr, omega, block_sum, s);
+  return launch_jacobi_uniform<T, D, true>(t, b, V, nullptr, omega, r2, s);
+}
+
+// The same on an adaptive tree, V in place; part: one value per leaf corner.
+template <typename T, int D>
+static int64_t sweep_adaptive(const DevTree &t, const T *b, T *V, T *part, const T *scale, int sweeps, T omega,
+                              double *r2, cudaStream_t s) {
+  const dim3 gc(grid_for(t.n_leaves * t.nc)), gv(grid_for(t.n_vert)), block(kBlock);
+  for (int it = 0; it <= sweeps; ++it) {
+    COUNT(2);
+    launch_pdl(k_corner_pass<T, D, true>, gc, block, s, t, V, part);
+    if (it < sweeps) launch_pdl(k_vertex_pass<T, false>, gv, block, s, t, b, part, scale, V, omega, r2);
+    else launch_pdl(k_vertex_pass<T, true>, gv, block, s, t, b, part, scale, V, omega, r2);
+  }
+  return gv.x;
+}
+
+template <typename T>
+static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V, T *Vtmp, T *part, T *scale, int sweeps,
+                  T omega, double *block_sum, double *resid2, cudaStream_t s) {
+  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale); }
+  int64_t nb;
+  if (t.uniform)
+    nb = t.d == 3 ? sweep_uniform<T, 3>(t, b, V, Vtmp, sweeps, omega, block_sum, s)
+                  : sweep_uniform<T, 2>(t, b, V, Vtmp, sweeps, omega, block_sum, s);
+  else
+    nb = t.d == 3 ? sweep_adaptive<T, 3>(t, b, V, part, scale, sweeps, omega, block_sum, s)
+                  : sweep_adaptive<T, 2>(t, b, V, part, scale, sweeps, omega, block_sum, s);
   { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
 }
 
 void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,
-                  int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s) {
+                  void *part, int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s) {
   if (split)
-    solve<float>(t, (const float *)Q, total, (float *)b, (float *)V, (float *)Vtmp, sweeps, (float)omega, block_sum,
-                 resid2, s);
-  else
-    solve<double>(t, (const double *)Q, total, (double *)b, (double *)V, (double *)Vtmp, sweeps, omega, block_sum,
-                  resid2, s);
+    solve<float>(t, (const float *)Q, total, (float *)b, (float *)V, (float *)Vtmp, (float *)part, nullptr, sweeps,
+                 (float)omega, block_sum, resid2, s);
+  else  // an adaptive solve leaves Vtmp free: it holds omega / diag
+    solve<double>(t, (const double *)Q, total, (double *)b, (double *)V, (double *)Vtmp, (double *)part,
+                  t.uniform ? nullptr : (double *)Vtmp, sweeps, omega, block_sum, resid2, s);
 }
 
 template <typename T>
-static void efield(const DevTree &t, const T *V, T *E, cudaStream_t s) {
-  COUNT(1);
-  const unsigned g = grid_for(t.n_vert);
-  if (!t.uniform) k_efield<T><<<g, kBlock, 0, s>>>(t, V, E);
-  else if (t.d == 3) k_efield_uniform<3><<<g, kBlock, 0, s>>>(t, V, E);
-  else k_efield_uniform<2><<<g, kBlock, 0, s>>>(t, V, E);
+static void efield(const DevTree &t, const T *V, T *E, T *part, cudaStream_t s) {
+  const unsigned g = grid_for(t.n_vert), gc = grid_for(t.n_leaves * t.nc);
+  COUNT(t.uniform ? 1 : 2);
+  if (t.uniform) {
+    if (t.d == 3) k_efield_uniform<3><<<g, kBlock, 0, s>>>(t, V, E);
+    else k_efield_uniform<2><<<g, kBlock, 0, s>>>(t, V, E);
+  } else if (t.d == 3) {
+    k_corner_pass<T, 3, false><<<gc, kBlock, 0, s>>>(t, V, part);
+    k_efield_adaptive<T, 3><<<g, kBlock, 0, s>>>(t, part, E);
+  } else {
+    k_corner_pass<T, 2, false><<<gc, kBlock, 0, s>>>(t, V, part);
+    k_efield_adaptive<T, 2><<<g, kBlock, 0, s>>>(t, part, E);
+  }
 }
 
-void launch_efield(const DevTree &t, bool split, const void *V, void *E, cudaStream_t s) {
-  if (split) efield<float>(t, (const float *)V, (float *)E, s);
-  else efield<double>(t, (const double *)V, (double *)E, s);
+void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s) {
+  if (split) efield<float>(t, (const float *)V, (float *)E, (float *)part, s);
+  else efield<double>(t, (const double *)V, (double *)E, (double *)part, s);
 }
 
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s) {

@@ -187,9 +187,11 @@ void launch_vertex_charge(const DevTree &t, bool split, const void *part, void *
 // total[0] is the FP64 sum over all vertices, total[1 + i] per instance.
 void launch_deposit(const DevTree &t, bool split, const int32_t *start, const void *pos, int64_t n, void *part,
                     void *Q, double *block_sum, double *total, cudaStream_t s);
+// part: scratch of one value per leaf corner (adaptive trees), free after the
+// vertex charges are summed.
 void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,
-                  int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s);
-void launch_efield(const DevTree &t, bool split, const void *V, void *E, cudaStream_t s);
+                  void *part, int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s);
+void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s);
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s);
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s);
 // Field at every leaf corner, the corner expansion applied once per field:

@@ -973,9 +973,9 @@ int field(pic_t h, pic_solve_fn hook, void *user) {
     if (r != 0) return fail(h, PIC_EHOOK, "field-solve hook returned " + std::to_string(r));
     return PIC_OK;
   }
-  launch_solve(h->dt, h->split, h->Q, h->total, h->b, h->V, h->Vtmp, h->cfg.sweeps, h->cfg.omega, h->block_sum,
+  launch_solve(h->dt, h->split, h->Q, h->total, h->b, h->V, h->Vtmp, h->part, h->cfg.sweeps, h->cfg.omega, h->block_sum,
                h->resid2, s);
-  launch_efield(h->dt, h->split, h->V, h->E, s);
+  launch_efield(h->dt, h->split, h->V, h->E, h->part, s);
   CK(cudaGetLastError());
   return PIC_OK;
 }

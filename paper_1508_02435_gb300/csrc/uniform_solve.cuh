@@ -31,7 +31,9 @@ __host__ __device__ constexpr int pop3(int x) { return (x & 1) + ((x >> 1) & 1) 
 
 // Programmatic dependent launch: a sweep's blocks are resident and have done
 // their index arithmetic when the sweep before ends.  The release comes after
-// the wait, so a block that runs sees every sweep but the last complete.
+// the wait, so a block that runs sees every sweep but the last complete.  What
+// the kernel before writes must not be read through the non-coherent path (it
+// changes while the block is resident): those pointers are not __restrict__.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -213,7 +215,7 @@ __device__ __forceinline__ double residual2(const T *y, const T *b) {
 
 // A V at vertex j of an instance (base: its first vertex), and V there.
 template <int D>
-__device__ __forceinline__ float apply_at(const float *__restrict__ base, int32_t M, const int32_t *j,
+__device__ __forceinline__ float apply_at(const float *base, int32_t M, const int32_t *j,
                                           const int32_t *sp, const StencilC<float> &s, float *vc) {
   int32_t o[3][3], w[3] = {0, 0, 0}, stride = 1;
   bool flip[3];
@@ -244,7 +246,7 @@ __device__ __forceinline__ float apply_at(const float *__restrict__ base, int32_
 }
 
 template <int D>
-__device__ __forceinline__ double apply_at(const double *__restrict__ base, int32_t M, const int32_t *j,
+__device__ __forceinline__ double apply_at(const double *base, int32_t M, const int32_t *j,
                                            const int32_t *, const StencilC<double> &s, double *vc) {
   int32_t o[3][3], stride = 1;
 #pragma unroll
@@ -290,7 +292,7 @@ __device__ __forceinline__ void block_sum_store_at(double v, double *out) {
 // One sweep V_out = V_in + omega (b - A V_in) / diag (kRes: block sums of
 // (b - A V_in)^2 to r2 instead).
 template <typename T, int D, bool kRes>
-__global__ void __launch_bounds__(128) k_jacobi_vertex(DevTree t, const T *__restrict__ b, const T *__restrict__ Vin,
+__global__ void __launch_bounds__(128) k_jacobi_vertex(DevTree t, const T *b, const T *Vin,
                                                        T *__restrict__ Vout, T omega, double *r2) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = v < t.n_vert;
@@ -405,7 +407,7 @@ __device__ __forceinline__ void strip_rows(const Slab3<double> &lo, const Slab3<
 
 // The strip's part of one plane: rows y0 - 1 .. y0 + 3, columns x - 1 .. x + 1.
 template <typename T>
-__device__ __forceinline__ void strip_load(const T *__restrict__ p, const int32_t *row, const int32_t *col, T *v) {
+__device__ __forceinline__ void strip_load(const T *p, const int32_t *row, const int32_t *col, T *v) {
 #pragma unroll
   for (int r = 0; r < 5; ++r)
 #pragma unroll
@@ -413,7 +415,7 @@ __device__ __forceinline__ void strip_load(const T *__restrict__ p, const int32_
 }
 
 template <typename T, bool kRes>
-__global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *__restrict__ b, const T *__restrict__ Vin,
+__global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, const T *Vin,
                                                        T *__restrict__ Vout, T omega, double *r2, int len) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M, plane = M * M;
@@ -499,7 +501,7 @@ __device__ __forceinline__ void strip_rows2(const double *v, const StencilC<doub
 }
 
 template <typename T, bool kRes>
-__global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *__restrict__ b, const T *__restrict__ Vin,
+__global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, const T *Vin,
                                                        T *__restrict__ Vout, T omega, double *r2) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M;
@@ -558,10 +560,10 @@ inline int march_length(int64_t M, size_t width) {
 }
 
 template <typename... P, typename... A>
-inline void launch_pdl(void (*k)(P...), dim3 grid, cudaStream_t s, A... args) {
+inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(kJacobiThreads);
+  cfg.blockDim = block;
   cfg.stream = s;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -579,18 +581,18 @@ int64_t launch_jacobi_uniform(const DevTree &t, const T *b, const T *Vin, T *Vou
   COUNT(1);
   if (t.n_inst > 1 || t.n_vert < kStripVertices) {
     const dim3 g(grid_for(t.n_vert, kJacobiThreads));
-    launch_pdl(k_jacobi_vertex<T, D, kRes>, g, s, t, b, Vin, Vout, omega, r2);
+    launch_pdl(k_jacobi_vertex<T, D, kRes>, g, dim3(kJacobiThreads), s, t, b, Vin, Vout, omega, r2);
     return g.x;
   }
   const int64_t M = t.M;
   if (D == 2) {
     const dim3 g(grid_for(M * (M / 3), kJacobiThreads));
-    launch_pdl(k_jacobi_strip2<T, kRes>, g, s, t, b, Vin, Vout, omega, r2);
+    launch_pdl(k_jacobi_strip2<T, kRes>, g, dim3(kJacobiThreads), s, t, b, Vin, Vout, omega, r2);
     return g.x;
   }
   const int len = march_length(M, sizeof(T));
   const dim3 g(grid_for(M * (M / 3), kJacobiThreads), (unsigned)(M / len));
-  launch_pdl(k_jacobi_strip3<T, kRes>, g, s, t, b, Vin, Vout, omega, r2, len);
+  launch_pdl(k_jacobi_strip3<T, kRes>, g, dim3(kJacobiThreads), s, t, b, Vin, Vout, omega, r2, len);
   return (int64_t)g.x * g.y;
 }
 
