@@ -118,7 +118,8 @@ typedef struct {
   int64_t n_buckets;     /* leaves (PIT) or PIDT owner vertices */
   int64_t n_keys;        /* sort keys: leaves (PIT) or owner vertex x 2^d quadrants (PIDT) */
   int32_t uniform;       /* 1 if every leaf is on `depth` */
-  int32_t brick;         /* 1 if steps run the brick path */
+  int32_t brick;         /* 1 if steps run the brick path (the generic passes when
+                            its bricks are crowded: same results) */
   int32_t n_instances;   /* independent plasmas in the handle (1 unless batched) */
   int64_t device_bytes;  /* device memory held by the handle */
 } pic_info_t;

@@ -137,6 +137,7 @@ struct BrickPullArgs {
 
 cudaError_t brick_configure(const BrickGeom &g);
 int32_t brick_stage_cap(int64_t n, int64_t n_units);  // staging slots per destination unit
+bool brick_crowded(int64_t n, int64_t n_units);       // most half bricks hold more than the shared-memory kernels take
 void launch_brick_push(const DevTree &t, const BrickGeom &g, const BrickPushArgs &pa, cudaStream_t s);
 void launch_brick_pull(const DevTree &t, const BrickGeom &g, const BrickPullArgs &qa, int32_t *fcount,
                        int32_t *fcursor, int32_t *tile_sums, int32_t *scratch_total, cudaStream_t s);

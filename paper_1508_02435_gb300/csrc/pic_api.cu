@@ -109,6 +109,7 @@ struct pic_s {
   // brick path (uniform tree, PIT, split precision)
   bool brick = false;
   bool brick_ok = false;    // the brick path applies (its buffers exist)
+  bool brick_crowded = false;  // too many particles per brick: its steps run the generic passes (same bits)
   bool leaf_stale = false;  // leaf[0] not yet expanded from the offsets
   bool q_valid = false;     // Q holds the charges of the current positions
 
@@ -704,6 +705,7 @@ int setup_brick(pic_t h) {
   free_bufs(h, h->brick_bufs);
   h->brick = false;
   h->brick_ok = false;
+  h->brick_crowded = false;
   const auto &t = h->ht0();
   if (h->cfg.path != PIC_PATH_AUTO || !t.uniform || h->scheme != PIC_PIT || !h->split || t.depth < 3 ||
       h->dt.n_inst > 1)
@@ -779,6 +781,7 @@ int setup_brick(pic_t h) {
     return fail(h, PIC_EINVAL, "brick count exceeds scan scratch");
   CK(brick_configure(g));
   h->bg = g;
+  h->brick_crowded = brick_crowded(n, nu);
   h->brick = true;
   h->brick_ok = true;
   return PIC_OK;
@@ -989,7 +992,7 @@ struct MoveKind {
 };
 
 int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
-  if (h->brick && mk.field) return brick_push_and_rebin(h, dt);
+  if (h->brick && !h->brick_crowded && mk.field) return brick_push_and_rebin(h, dt);
   int rc0 = ensure_leaf(h);
   if (rc0) return rc0;
   h->q_valid = false;
@@ -1052,7 +1055,10 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
   }
   delete ps;
   CK(cudaGetLastError());
-  return rebin_and_gather(h, h->start_cur, h->prec != nullptr);
+  int rc = rebin_and_gather(h, h->start_cur, h->prec != nullptr);
+  // a crowded brick handle: the charges follow the step, as the brick pull leaves them
+  if (!rc && h->brick && mk.field) rc = deposit(h);
+  return rc;
 }
 
 int check_handle(pic_t h) { return h ? PIC_OK : PIC_EINVAL; }
