@@ -6,17 +6,17 @@
 //   field     k_efield                                                  (item 3)
 //   push      k_push64 / k_push32: gather E_i = R^T(x_i) E, leapfrog kick
 //             and drift, wrap, re-location (descent / split resolve), new
-//             key, moved flag (warp ballot), bucket counts               (items 3-4)
-//   re-bin    scan(counts) -> k_stayers (stable ranks of stayers) ->
-//             k_compact_movers (ballot words -> mover list in storage
-//             order) -> k_mover_slots -> k_sort_segments -> k_gather_*
-//             (stable: stayers first, then movers in storage order)
+//             key, moved flag (warp ballot), mover ranks                 (items 3-4)
+//   re-bin    rebin.cuh: scans of the ballot words and of the keys -> k_place ->
+//             k_sort_medium/large -> k_gather_* (stable: stayers first, then
+//             movers in storage order)
 //
 // Determinism: no floating-point atomics.  Every sum has a fixed order (bucket
 // order within a leaf, ascending leaf-corner order per vertex); integer atomics
-// only count, and the one order they decide (mover slots) is re-sorted.
+// only count, and the one order they decide (mover ranks) is put right.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <utility>
 
@@ -365,6 +365,21 @@ __global__ void k_rekey32(DevTree t, const int32_t *leaf, const float *o, int64_
 }
 
 // ---------------------------------------------------------------------------
+// a6 stable counting sort
+// ---------------------------------------------------------------------------
+
+constexpr int kMedSeg = 2048;        // longest segment one warp sorts in shared memory
+constexpr int kMedThreads = 256;
+constexpr int kLargeSeg = 16384;     // chunk of a long segment sorted in shared memory
+constexpr int kLargeThreads = 1024;
+
+}  // namespace pic
+
+#include "rebin.cuh"
+
+namespace pic {
+
+// ---------------------------------------------------------------------------
 // a3 + a4 + a1/a2 + a5: fused gather, push, re-location, key, moved flag
 // ---------------------------------------------------------------------------
 
@@ -384,34 +399,6 @@ __device__ __forceinline__ void add_runs(int32_t *count, int32_t key, bool act) 
     const unsigned stop = (heads | ~acts) & after;
     const int end = stop ? __ffs(stop) - 1 : 32;
     atomicAdd(&count[key], end - lane);
-  }
-}
-
-// Bucket counts, mover ballot word and per-block mover count.  kRuns: one
-// atomic per run of equal adjacent keys (3D, where most particles of a warp
-// take distinct new keys); else one per distinct key of the warp (2D, where
-// repeats of a key are often apart; measured faster on each).
-template <bool kRuns>
-__device__ __forceinline__ void count_and_ballot(bool act, int32_t knew, bool moved, int32_t *count,
-                                                 uint32_t *mover_words, int32_t *block_movers) {
-  const unsigned full = 0xffffffffu;
-  int lane = threadIdx.x & 31;
-  if (kRuns) {
-    add_runs(count, knew, act);
-  } else {
-    const unsigned peers = __match_any_sync(full, act ? knew : -1);
-    if (act && lane == __ffs(peers) - 1) atomicAdd(&count[knew], __popc(peers));
-  }
-  unsigned mv = __ballot_sync(full, act && moved);
-  int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (lane == 0) mover_words[gw] = mv;
-  __shared__ int sh[32];
-  if (lane == 0) sh[threadIdx.x >> 5] = __popc(mv);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int s = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-    block_movers[blockIdx.x] = s;
   }
 }
 
@@ -534,7 +521,7 @@ __global__ void k_push64(DevTree t, Push64Args a) {
     }
     if (a.rec || t.scheme != 0) a.keyn[p] = knew;  // PIT rows: the key array is the leaf array
   }
-  count_and_ballot<D == 3>(act, knew, moved, a.count, a.mover_words, a.block_movers);
+  rank_movers<D == 3>(p, moved, knew, a.count, a.words, a.rank);
 }
 
 template <int D>
@@ -659,269 +646,7 @@ __global__ void __launch_bounds__(512, 3) k_push32(DevTree t, Push32Args a) {
     }
     if (a.rec || t.scheme != 0) a.keyn[p] = knew;  // PIT rows: the key array is the leaf array
   }
-  count_and_ballot<D == 3>(act, knew, moved, a.count, a.mover_words, a.block_movers);
-}
-
-// Key counts of freshly converted particles (every particle a mover).
-__global__ void k_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *mover_words,
-                            int32_t *block_movers) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool act = p < n;
-  int32_t k = act ? key[p] : 0;
-  count_and_ballot<false>(act, k, true, count, mover_words, block_movers);
-}
-
-// ---------------------------------------------------------------------------
-// a6 stable counting sort
-// ---------------------------------------------------------------------------
-
-// Exclusive scan of int32 values: tiles of kScanTile elements.
-__device__ __forceinline__ int32_t block_exclusive_scan(int32_t v, int32_t *total) {
-  __shared__ int32_t sh[32];
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int32_t x = v;
-  for (int o = 1; o < 32; o <<= 1) {
-    int32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) sh[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    int32_t s = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0;
-    for (int o = 1; o < 32; o <<= 1) {
-      int32_t y = __shfl_up_sync(0xffffffffu, s, o);
-      if (lane >= o) s += y;
-    }
-    sh[lane] = s;
-  }
-  __syncthreads();
-  int32_t before = w > 0 ? sh[w - 1] : 0;
-  if (total) *total = sh[(blockDim.x >> 5) - 1];
-  int32_t r = before + x - v;
-  __syncthreads();
-  return r;
-}
-
-__global__ void k_scan_reduce(const int32_t *in, int64_t n, int32_t *tile_sums) {
-  int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  int32_t s = 0;
-  for (int i = 0; i < kScanItems; ++i)
-    if (base + i < n) s += in[base + i];
-  int32_t tot;
-  block_exclusive_scan(s, &tot);
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
-}
-
-// Single block: exclusive scan of the tile sums in place, total to *total.
-__global__ void k_scan_tiles(int32_t *tile_sums, int64_t nt, int32_t *total) {
-  int32_t carry = 0;
-  for (int64_t base = 0; base < nt; base += blockDim.x) {
-    int64_t i = base + threadIdx.x;
-    int32_t v = i < nt ? tile_sums[i] : 0;
-    int32_t tot;
-    int32_t ex = block_exclusive_scan(v, &tot);
-    if (i < nt) tile_sums[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) *total = carry;
-}
-
-__global__ void k_scan_apply(const int32_t *in, int64_t n, const int32_t *tile_offsets, int32_t *out,
-                             const int32_t *total) {
-  int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  int32_t vals[kScanItems];
-  int32_t s = 0;
-  for (int i = 0; i < kScanItems; ++i) {
-    vals[i] = base + i < n ? in[base + i] : 0;
-    s += vals[i];
-  }
-  int32_t ex = block_exclusive_scan(s, nullptr) + tile_offsets[blockIdx.x];
-  for (int i = 0; i < kScanItems; ++i) {
-    if (base + i < n) out[base + i] = ex;
-    ex += vals[i];
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = *total;
-}
-
-// Stayers of old bucket k keep their storage order at the head of new bucket k.
-// The largest new bucket goes to *max_bucket with one atomic per block.
-__global__ void k_stayers(const int32_t *old_start, const int32_t *keyn, const int32_t *new_start,
-                          int64_t n_keys, int32_t *perm, int32_t *n_stay, int32_t *max_bucket) {
-  __shared__ int32_t wmax[32];
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int32_t sz = 0;
-  if (k < n_keys) {
-    int32_t r = 0, dst = new_start[k];
-    for (int32_t i = old_start[k]; i < old_start[k + 1]; ++i)
-      if (keyn[i] == (int32_t)k) perm[dst + r++] = i;
-    n_stay[k] = r;
-    sz = new_start[k + 1] - new_start[k];
-  }
-  const int32_t m = __reduce_max_sync(0xffffffffu, sz);
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int32_t b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b = b > wmax[w] ? b : wmax[w];
-    if (b > 0) atomicMax(max_bucket, b);
-  }
-}
-
-// Ballot words -> mover list in storage order.
-__global__ void k_compact_movers(const uint32_t *mover_words, const int32_t *block_offsets, int64_t n,
-                                 int32_t *movers) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int64_t w0 = ((int64_t)blockIdx.x * blockDim.x) >> 5;
-  int32_t off = block_offsets[blockIdx.x];
-  for (int k = 0; k < w; ++k) off += __popc(mover_words[w0 + k]);
-  uint32_t word = mover_words[w0 + w];
-  if (p < n && ((word >> lane) & 1u)) movers[off + __popc(word & ((1u << lane) - 1u))] = (int32_t)p;
-}
-
-__global__ void k_mover_slots(const int32_t *movers, const int32_t *n_movers, const int32_t *keyn,
-                              const int32_t *new_start, const int32_t *n_stay, int32_t *cursor,
-                              int32_t *perm) {
-  int32_t m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= *n_movers) return;
-  int32_t p = movers[m];
-  int32_t k = keyn[p];
-  int32_t slot = atomicAdd(&cursor[k], 1);
-  perm[new_start[k] + n_stay[k] + slot] = p;
-}
-
-// The movers of every bucket in storage order (undoes the atomic slot order).
-// Segments of kSmallSeg movers or fewer are sorted here by one thread; longer
-// ones are listed for k_sort_medium (up to kMedSeg: one warp each) or
-// k_sort_large (one block each).
-constexpr int kSmallSeg = 32;
-constexpr int kMedSeg = 2048;        // longest segment one warp sorts in shared memory
-constexpr int kMedThreads = 256;
-constexpr int kLargeSeg = 16384;     // chunk of a long segment sorted in shared memory
-constexpr int kLargeThreads = 1024;
-__global__ void k_sort_segments(const int32_t *new_start, const int32_t *n_stay, int64_t n_keys, int32_t *perm,
-                                int32_t *large, int32_t *n_large, int32_t *med, int32_t *n_med) {
-  int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_keys) return;
-  int32_t b = new_start[k] + n_stay[k], e = new_start[k + 1];
-  if (e - b > kSmallSeg) {
-    if (e - b <= kMedSeg) med[atomicAdd(n_med, 1)] = (int32_t)k;
-    else large[atomicAdd(n_large, 1)] = (int32_t)k;
-    return;
-  }
-  for (int32_t i = b + 1; i < e; ++i) {
-    int32_t x = perm[i];
-    int32_t j = i - 1;
-    while (j >= b && perm[j] > x) {
-      perm[j + 1] = perm[j];
-      --j;
-    }
-    perm[j + 1] = x;
-  }
-}
-
-// One warp per listed segment of at most kMedSeg movers (grid-stride over the
-// list): the segment is copied into the warp's shared slice, sorted by the
-// bitonic network of segsort.cuh and copied back.
-__global__ void __launch_bounds__(kMedThreads) k_sort_medium(const int32_t *new_start, const int32_t *n_stay,
-                                                             const int32_t *med, const int32_t *n_med,
-                                                             int32_t *perm) {
-  extern __shared__ int32_t sw[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = kMedThreads / 32;
-  int32_t *v = sw + wib * kMedSeg;
-  const int nm = *n_med;
-  for (int li = blockIdx.x * wpb + wib; li < nm; li += gridDim.x * wpb) {
-    const int32_t k = med[li];
-    const int32_t b = new_start[k] + n_stay[k], m = new_start[k + 1] - b;
-    for (int i = lane; i < m; i += 32) v[i] = perm[b + i];
-    __syncwarp();
-    warp_sort_direct<int32_t>(v, m);
-    for (int i = lane; i < m; i += 32) perm[b + i] = v[i];
-    __syncwarp();
-  }
-}
-
-// One block per long segment (grid-stride over the list): the in-place
-// bitonic network of segsort.cuh, chunks of kLargeSeg in shared memory, so a
-// bucket of any size sorts in O(m log^2 m).
-__global__ void __launch_bounds__(kLargeThreads) k_sort_large(const int32_t *new_start, const int32_t *n_stay,
-                                                              const int32_t *large, const int32_t *n_large,
-                                                              int32_t *perm) {
-  extern __shared__ int32_t sv[];
-  const int nl = *n_large;
-  for (int li = blockIdx.x; li < nl; li += gridDim.x) {
-    const int32_t k = large[li];
-    const int32_t b = new_start[k] + n_stay[k], m = new_start[k + 1] - b;
-    block_sort_global<int32_t, int32_t>(perm + b, nullptr, m, sv, nullptr, kLargeSeg);
-    __syncthreads();
-  }
-}
-
-// The whole particle state into bucket order in one pass: positions and
-// velocities ([d][n]), leaves, and keys and ids where given.
-template <typename T>
-__global__ void k_gather_state(const int32_t *perm, int64_t n, int d, const T *x, T *x2, const T *v, T *v2,
-                               const int32_t *leaf, int32_t *leaf2, const int32_t *key, int32_t *key2,
-                               const int32_t *ids, int32_t *ids2) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int32_t i = perm[p];
-  for (int a = 0; a < d; ++a) x2[a * n + p] = x[a * n + i];
-  for (int a = 0; a < d; ++a) v2[a * n + p] = v[a * n + i];
-  leaf2[p] = leaf[i];
-  if (key) key2[p] = key[i];
-  if (ids) ids2[p] = ids[i];
-}
-
-// The pushed-state records in bucket order (two or four 16-byte loads per
-// particle instead of one scattered 4- or 8-byte load per array).
-__global__ void k_gather_rec32(const int32_t *perm, int64_t n, int d, const float4 *rec, float *x2, float *v2,
-                               int32_t *leaf2, int32_t *key2, const int32_t *ids, int32_t *ids2) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int32_t i = perm[p];
-  const float4 r0 = rec[2 * (int64_t)i], r1 = rec[2 * (int64_t)i + 1];
-  x2[p] = r0.x;
-  x2[n + p] = r0.y;
-  if (d == 3) {
-    x2[2 * n + p] = r0.z;
-    v2[p] = r0.w;
-    v2[n + p] = r1.x;
-    v2[2 * n + p] = r1.y;
-  } else {
-    v2[p] = r0.w;
-    v2[n + p] = r1.x;
-  }
-  leaf2[p] = __float_as_int(r1.z);
-  if (key2) key2[p] = __float_as_int(r1.w);
-  if (ids) ids2[p] = ids[i];
-}
-
-__global__ void k_gather_rec64(const int32_t *perm, int64_t n, int d, const double2 *rec, double *x2, double *v2,
-                               int32_t *leaf2, int32_t *key2, const int32_t *ids, int32_t *ids2) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int32_t i = perm[p];
-  const double2 *r = rec + 4 * (int64_t)i;
-  const double2 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
-  x2[p] = r0.x;
-  x2[n + p] = r0.y;
-  if (d == 3) x2[2 * n + p] = r1.x;
-  v2[p] = r1.y;
-  v2[n + p] = r2.x;
-  if (d == 3) v2[2 * n + p] = r2.y;
-  const uint64_t lk = (uint64_t)__double_as_longlong(r3.x);
-  leaf2[p] = (int32_t)(uint32_t)lk;
-  if (key2) key2[p] = (int32_t)(uint32_t)(lk >> 32);
-  if (ids) ids2[p] = ids[i];
-}
-
-template <typename T>
-__global__ void k_gather_vec(const int32_t *perm, int64_t n, int d, const T *src, T *dst) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  int32_t i = perm[p];
-  for (int a = 0; a < d; ++a) dst[a * n + p] = src[a * n + i];
+  rank_movers<D == 3>(p, moved, knew, a.count, a.words, a.rank);
 }
 
 // ---------------------------------------------------------------------------
@@ -1177,12 +902,6 @@ void launch_rekey32(const DevTree &t, const int32_t *leaf, const float *o, int64
   if (n > 0) { COUNT(1); k_rekey32<<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, n, key, err); }
 }
 
-void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *mover_words,
-                      int32_t *block_movers, int block, cudaStream_t s) {
-  const int b = bsz(block);
-  { COUNT(1); k_count_all<<<grid_for(n, b), b, 0, s>>>(key, n, count, mover_words, block_movers); }
-}
-
 // Flag = 1 if keys are not in ascending order.
 __global__ void k_check_sorted(const int32_t *key, int64_t n, int32_t *flag) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1395,79 +1114,6 @@ void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s) {
   COUNT(1);
   if (t.d == 3) k_push32<3><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
   else k_push32<2><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
-}
-
-int64_t scan_tiles_needed(int64_t n) { return (n + kScanTile - 1) / kScanTile; }
-
-void launch_exclusive_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *tile_sums, int32_t *total,
-                           cudaStream_t s) {
-  int64_t nt = scan_tiles_needed(n);
-  if (nt < 1) nt = 1;
-  { COUNT(1); k_scan_reduce<<<(unsigned)nt, kScanThreads, 0, s>>>(in, n, tile_sums); }
-  { COUNT(1); k_scan_tiles<<<1, kScanThreads, 0, s>>>(tile_sums, nt, total); }
-  { COUNT(1); k_scan_apply<<<(unsigned)nt, kScanThreads, 0, s>>>(in, n, tile_sums, out, total); }
-}
-
-void launch_rebin(const RebinArgs &r, cudaStream_t s) {
-  // bucket offsets
-  launch_exclusive_scan(r.count, r.n_keys, r.new_start, r.tile_sums, r.scalars + 0, s);
-  // mover list in storage order
-  const int bp = bsz(r.block);
-  unsigned gp = grid_for(r.n, bp);
-  launch_exclusive_scan(r.block_movers, gp, r.block_offsets, r.tile_sums2, r.scalars + 1, s);
-  if (r.old_start)
-    { COUNT(1); k_stayers<<<grid_for(r.n_keys), kBlock, 0, s>>>(r.old_start, r.keyn, r.new_start, r.n_keys, r.perm, r.n_stay,
-                                                    r.scalars + 2); }
-  else
-    cudaMemsetAsync(r.n_stay, 0, sizeof(int32_t) * r.n_keys, s);
-  { COUNT(1); k_compact_movers<<<gp, bp, 0, s>>>(r.mover_words, r.block_offsets, r.n, r.movers); }
-  cudaMemsetAsync(r.cursor, 0, sizeof(int32_t) * r.n_keys, s);
-  { COUNT(1); k_mover_slots<<<gp, bp, 0, s>>>(r.movers, r.scalars + 1, r.keyn, r.new_start, r.n_stay, r.cursor, r.perm); }
-  cudaMemsetAsync(r.scalars + 5, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(r.scalars + 7, 0, sizeof(int32_t), s);
-  // the mover list is no longer needed: it holds the list of medium segments
-  { COUNT(1); k_sort_segments<<<grid_for(r.n_keys), kBlock, 0, s>>>(r.new_start, r.n_stay, r.n_keys, r.perm, r.cursor,
-                                                                      r.scalars + 5, r.movers, r.scalars + 7); }
-  { COUNT(1); k_sort_medium<<<456, kMedThreads, sizeof(int32_t) * kMedSeg * (kMedThreads / 32), s>>>(
-      r.new_start, r.n_stay, r.movers, r.scalars + 7, r.perm); }
-  { COUNT(1); k_sort_large<<<304, kLargeThreads, sizeof(int32_t) * kLargeSeg, s>>>(r.new_start, r.n_stay, r.cursor,
-                                                                                  r.scalars + 5, r.perm); }
-}
-
-void launch_gather_state(bool split, const int32_t *perm, int64_t n, int d, const void *x, void *x2, const void *v,
-                         void *v2, const int32_t *leaf, int32_t *leaf2, const int32_t *key, int32_t *key2,
-                         const int32_t *ids, int32_t *ids2, cudaStream_t s) {
-  if (n <= 0) return;
-  COUNT(1);
-  if (split)
-    k_gather_state<float><<<grid_for(n), kBlock, 0, s>>>(perm, n, d, (const float *)x, (float *)x2, (const float *)v,
-                                                          (float *)v2, leaf, leaf2, key, key2, ids, ids2);
-  else
-    k_gather_state<double><<<grid_for(n), kBlock, 0, s>>>(perm, n, d, (const double *)x, (double *)x2,
-                                                           (const double *)v, (double *)v2, leaf, leaf2, key, key2,
-                                                           ids, ids2);
-}
-
-void launch_gather_records(bool split, const int32_t *perm, int64_t n, int d, const void *rec, void *x2, void *v2,
-                           int32_t *leaf2, int32_t *key2, const int32_t *ids, int32_t *ids2, cudaStream_t s) {
-  if (n <= 0) return;
-  COUNT(1);
-  if (split)
-    k_gather_rec32<<<grid_for(n), kBlock, 0, s>>>(perm, n, d, (const float4 *)rec, (float *)x2, (float *)v2, leaf2,
-                                                   key2, ids, ids2);
-  else
-    k_gather_rec64<<<grid_for(n), kBlock, 0, s>>>(perm, n, d, (const double2 *)rec, (double *)x2, (double *)v2,
-                                                   leaf2, key2, ids, ids2);
-}
-
-void launch_gather_f64(const int32_t *perm, int64_t n, int d, const double *src, double *dst, cudaStream_t s) {
-  if (n > 0) { COUNT(1); k_gather_vec<double><<<grid_for(n), kBlock, 0, s>>>(perm, n, d, src, dst); }
-}
-void launch_gather_f32(const int32_t *perm, int64_t n, int d, const float *src, float *dst, cudaStream_t s) {
-  if (n > 0) { COUNT(1); k_gather_vec<float><<<grid_for(n), kBlock, 0, s>>>(perm, n, d, src, dst); }
-}
-void launch_gather_i32(const int32_t *perm, int64_t n, const int32_t *src, int32_t *dst, cudaStream_t s) {
-  if (n > 0) { COUNT(1); k_gather_vec<int32_t><<<grid_for(n), kBlock, 0, s>>>(perm, n, 1, src, dst); }
 }
 
 void launch_absolute_split(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, double *x,

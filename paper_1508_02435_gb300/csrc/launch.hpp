@@ -18,9 +18,9 @@ struct Push64Args {
   int32_t *tleaf, *keyn;        // keyn: new key per particle (PIT: the leaf)
   const double *E;              // [d][n_vert]; NULL: no field (the particle-handling move, no kick)
   double qmdt, dt;
-  int32_t *count;               // per key, zeroed before the launch
-  uint32_t *mover_words;        // one ballot word per warp
-  int32_t *block_movers;        // movers per block
+  int32_t *count;               // movers per key, zeroed before the launch
+  uint32_t *words;              // one ballot word of movers per 32 particles
+  int32_t *rank;                // movers: rank among the movers of the new key
   int32_t *err;
   int32_t reflect;              // 1: reflecting walls of the unit box; 0: periodic
   int32_t flops;                // artificial floating-point operations per particle move
@@ -39,8 +39,8 @@ struct Push32Args {
   double dt;
   float sl[19];                 // RN32(dt * 3^level) per level
   int32_t *count;
-  uint32_t *mover_words;
-  int32_t *block_movers;
+  uint32_t *words;
+  int32_t *rank;
   int32_t *err;
   int32_t reflect;              // 1: reflecting walls of the unit box; 0: periodic
   int32_t flops;                // artificial floating-point operations per particle move
@@ -48,17 +48,22 @@ struct Push32Args {
 
 struct RebinArgs {
   int64_t n, n_keys;
-  const int32_t *count;         // per key
+  const int32_t *count;         // movers per new key
   const int32_t *keyn;          // new key per particle (storage order)
-  const int32_t *old_start;     // CSR of the current order, NULL at creation
-  int32_t *new_start;           // n_keys + 1
-  const uint32_t *mover_words;
-  const int32_t *block_movers;
-  int32_t *block_offsets, *movers, *n_stay, *cursor, *perm;
+  const int32_t *old_start;     // CSR of the current order, NULL for fresh particles (all movers)
+  int32_t *new_start;           // [n_keys + 1]
+  const uint32_t *words;        // mover bits
+  int32_t *word_pre;            // [words + 1] movers before each word
+  const int32_t *rank;
+  int32_t *base, *shift;        // [n_keys] first mover slot; stayer slot less stayers before
+  int32_t *perm;
+  int32_t *med, *large;         // keys with long mover segments
   int32_t *tile_sums, *tile_sums2;
-  int32_t *scalars;             // [0] n, [1] movers, [2] max bucket
-  int block;                     // threads per block of the push (ballot words, block counts)
+  int32_t *scalars;             // [0] n, [1] movers, [2] max bucket, [5] long, [7] medium segments (2, 5, 7 zeroed before)
 };
+// Mover segments of up to this many are put in order by the gather; longer
+// ones (at most n / (kRankSegment + 1)) are listed and sorted.
+constexpr int64_t kRankSegment = 64;
 
 // Elements per tile of launch_exclusive_scan: a scan of n elements writes
 // scan_tiles_needed(n) = ceil(n / kScanTileElems) tile sums.
@@ -162,8 +167,7 @@ void launch_init32(const DevTree &t, const double *x, const double *v, int64_t n
 void launch_rekey32(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, int32_t *key, int32_t *err,
                     cudaStream_t s);
 void launch_check_sorted(const int32_t *key, int64_t n, int32_t *flag, cudaStream_t s);
-void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *mover_words,
-                      int32_t *block_movers, int block, cudaStream_t s);
+void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *words, int32_t *rank, cudaStream_t s);
 // Re-refinement: depth-first cell index on level dmax per particle; cells of
 // level m (index key / div) holding more than ppc particles as a bitmap.
 void launch_fine_keys(const DevTree &t, bool split, const void *pos, const int32_t *leaf, int64_t n, int dmax,
@@ -201,18 +205,14 @@ void launch_corner_field32(const DevTree &t, const float *E, float4 *Ec, cudaStr
 void launch_exclusive_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *tile_sums, int32_t *total,
                            cudaStream_t s);
 void launch_rebin(const RebinArgs &r, cudaStream_t s);
-// dst[p] = src[perm[p]] for positions, velocities ([d][n]), leaves and,
-// where not NULL, keys and ids, in one kernel (split: float, else double).
-// Bucket order from the pushed-state records: x2/v2 [d][n] rows, leaf2, and
-// key2 unless NULL (PIT), ids2 from ids unless NULL.
-void launch_gather_records(bool split, const int32_t *perm, int64_t n, int d, const void *rec, void *x2, void *v2,
-                           int32_t *leaf2, int32_t *key2, const int32_t *ids, int32_t *ids2, cudaStream_t s);
-void launch_gather_state(bool split, const int32_t *perm, int64_t n, int d, const void *x, void *x2, const void *v,
-                         void *v2, const int32_t *leaf, int32_t *leaf2, const int32_t *key, int32_t *key2,
-                         const int32_t *ids, int32_t *ids2, cudaStream_t s);
-void launch_gather_f64(const int32_t *perm, int64_t n, int d, const double *src, double *dst, cudaStream_t s);
-void launch_gather_f32(const int32_t *perm, int64_t n, int d, const float *src, float *dst, cudaStream_t s);
-void launch_gather_i32(const int32_t *perm, int64_t n, const int32_t *src, int32_t *dst, cudaStream_t s);
+// The pushed state into bucket order after launch_rebin, in one kernel: from the
+// rows (positions, velocities [d][n], leaves and, where not NULL, keys and ids;
+// split: float, else double) or from the records of the 3D step.  key NULL: PIT.
+void launch_gather_state(bool split, const RebinArgs &r, int d, const void *x, void *x2, const void *v, void *v2,
+                         const int32_t *leaf, int32_t *leaf2, const int32_t *key, int32_t *key2, const int32_t *ids,
+                         int32_t *ids2, cudaStream_t s);
+void launch_gather_records(bool split, const RebinArgs &r, const void *rec, void *x2, void *v2, int32_t *leaf2,
+                           int32_t *key2, const int32_t *ids, int32_t *ids2, cudaStream_t s);
 void launch_absolute_split(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, double *x,
                            cudaStream_t s);
 void launch_widen(const float *in, int64_t n, double *out, cudaStream_t s);

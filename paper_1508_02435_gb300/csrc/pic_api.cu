@@ -78,10 +78,10 @@ struct pic_s {
   int32_t *key[2] = {nullptr, nullptr};  // [1] doubles as the new key
   int32_t *ids[2] = {nullptr, nullptr};
   // re-bin scratch
-  int32_t *start_cur = nullptr, *start_new = nullptr, *count = nullptr, *n_stay = nullptr, *cursor = nullptr;
-  int32_t *perm = nullptr, *movers = nullptr, *block_movers = nullptr, *block_offsets = nullptr;
+  int32_t *start_cur = nullptr, *start_new = nullptr, *count = nullptr, *base = nullptr, *shift = nullptr;
+  int32_t *perm = nullptr, *rank = nullptr, *word_pre = nullptr, *med = nullptr, *large = nullptr;
   int32_t *tile_sums = nullptr, *tile_sums2 = nullptr, *scalars = nullptr, *err = nullptr;
-  uint32_t *mover_words = nullptr;
+  uint32_t *words = nullptr;
   // grid
   void *part = nullptr, *Q = nullptr, *b = nullptr, *V = nullptr, *Vtmp = nullptr, *E = nullptr;
   double *block_sum = nullptr, *total = nullptr, *resid2 = nullptr;
@@ -567,7 +567,7 @@ int alloc_particles(pic_t h) {
   auto &sb = h->state_bufs;
   const int64_t n = h->n, d = h->d;
   const size_t fs = h->split ? sizeof(float) : sizeof(double);
-  const int64_t nblk = (n + 127) / 128 + 1;  // blocks of the smallest tuned block size
+  const int64_t nw = (n + 31) / 32 + 64;  // ballot words, whole blocks of them
   int rc;
   for (int s = 0; s < 2; ++s) {
     char *p;
@@ -591,11 +591,12 @@ int alloc_particles(pic_t h) {
     h->prec = p;
   }
   if ((rc = dalloc(h, sb, &h->perm, n))) return rc;
-  if ((rc = dalloc(h, sb, &h->movers, n))) return rc;
-  if ((rc = dalloc(h, sb, &h->block_movers, nblk))) return rc;
-  if ((rc = dalloc(h, sb, &h->block_offsets, nblk + 1))) return rc;
-  if ((rc = dalloc(h, sb, &h->mover_words, (n + 31) / 32 + 64))) return rc;
-  if ((rc = dalloc(h, sb, &h->tile_sums2, scan_tiles_needed(nblk) + 1))) return rc;
+  if ((rc = dalloc(h, sb, &h->rank, n))) return rc;
+  if ((rc = dalloc(h, sb, &h->words, nw))) return rc;
+  if ((rc = dalloc(h, sb, &h->word_pre, nw))) return rc;
+  if ((rc = dalloc(h, sb, &h->med, n / kRankSegment + 1))) return rc;
+  if ((rc = dalloc(h, sb, &h->large, n / kRankSegment + 1))) return rc;
+  if ((rc = dalloc(h, sb, &h->tile_sums2, scan_tiles_needed(nw) + 1))) return rc;
   if ((rc = dalloc(h, sb, &h->scalars, 8))) return rc;
   if ((rc = dalloc(h, sb, &h->err, 1))) return rc;
   cudaStream_t s = h->stream;
@@ -618,8 +619,8 @@ int alloc_grid(pic_t h) {
   if ((rc = galloc(h, sb, &h->start_cur, nk + 8))) return rc;
   if ((rc = galloc(h, sb, &h->start_new, nk + 8))) return rc;
   if ((rc = galloc(h, sb, &h->count, nk))) return rc;
-  if ((rc = galloc(h, sb, &h->n_stay, nk))) return rc;
-  if ((rc = galloc(h, sb, &h->cursor, nk))) return rc;
+  if ((rc = galloc(h, sb, &h->base, nk))) return rc;
+  if ((rc = galloc(h, sb, &h->shift, nk))) return rc;
   if ((rc = galloc(h, sb, &h->tile_sums, scan_tiles_needed(nk) + 1))) return rc;
   char *p;
   if ((rc = galloc(h, sb, &p, fs * nl * h->dt.nc))) return rc;
@@ -875,51 +876,31 @@ int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
   r.keyn = h->key[1];
   r.old_start = old_start;
   r.new_start = h->start_new;
-  r.mover_words = h->mover_words;
-  r.block_movers = h->block_movers;
-  r.block_offsets = h->block_offsets;
-  r.movers = h->movers;
-  r.n_stay = h->n_stay;
-  r.cursor = h->cursor;
+  r.words = h->words;
+  r.word_pre = h->word_pre;
+  r.rank = h->rank;
+  r.base = h->base;
+  r.shift = h->shift;
+  r.med = h->med;
+  r.large = h->large;
   r.perm = h->perm;
   r.tile_sums = h->tile_sums;
   r.tile_sums2 = h->tile_sums2;
   r.scalars = h->scalars;
-  r.block = h->dt.block_push;
   {
     PhaseScope ps(h, PIC_PHASE_REBIN);
     launch_rebin(r, s);
   }
   PhaseScope ps(h, PIC_PHASE_PERMUTE);
-  const int d = h->d;
-  if (records) {  // the pushed state, one record per particle
-    launch_gather_records(h->split, h->perm, n, d, h->prec, h->pos[0], h->vel[0], h->leaf[0],
-                          h->scheme == PIC_PIT ? nullptr : h->key[0], h->cfg.track_ids ? h->ids[0] : nullptr,
-                          h->cfg.track_ids ? h->ids[1] : nullptr, s);
-    if (h->cfg.track_ids) std::swap(h->ids[0], h->ids[1]);
-  } else if (h->scheme == PIC_PIT) {
-    // one pass over the permutation (measured faster for PIT; PIDT's extra
-    // key array makes the separate passes faster: 6.1 against 6.7 ms on the
-    // 2e8-particle 3D two-stream step)
-    launch_gather_state(h->split, h->perm, n, d, h->pos[1], h->pos[0], h->vel[1], h->vel[0], h->leaf[1],
-                        h->leaf[0], nullptr, nullptr, h->cfg.track_ids ? h->ids[0] : nullptr,
-                        h->cfg.track_ids ? h->ids[1] : nullptr, s);
-    if (h->cfg.track_ids) std::swap(h->ids[0], h->ids[1]);
-  } else if (h->split) {
-    launch_gather_f32(h->perm, n, d, (const float *)h->pos[1], (float *)h->pos[0], s);
-    launch_gather_f32(h->perm, n, d, (const float *)h->vel[1], (float *)h->vel[0], s);
-  } else {
-    launch_gather_f64(h->perm, n, d, (const double *)h->pos[1], (double *)h->pos[0], s);
-    launch_gather_f64(h->perm, n, d, (const double *)h->vel[1], (double *)h->vel[0], s);
-  }
-  if (!records && h->scheme != PIC_PIT) {
-    launch_gather_i32(h->perm, n, h->leaf[1], h->leaf[0], s);
-    launch_gather_i32(h->perm, n, h->key[1], h->key[0], s);
-    if (h->cfg.track_ids) {
-      launch_gather_i32(h->perm, n, h->ids[0], h->ids[1], s);
-      std::swap(h->ids[0], h->ids[1]);
-    }
-  }
+  const bool pidt = h->scheme != PIC_PIT, ids = h->cfg.track_ids != 0;
+  if (records)  // the pushed state, one record per particle
+    launch_gather_records(h->split, r, h->prec, h->pos[0], h->vel[0], h->leaf[0], pidt ? h->key[0] : nullptr,
+                          ids ? h->ids[0] : nullptr, ids ? h->ids[1] : nullptr, s);
+  else
+    launch_gather_state(h->split, r, h->d, h->pos[1], h->pos[0], h->vel[1], h->vel[0], h->leaf[1], h->leaf[0],
+                        pidt ? h->key[1] : nullptr, pidt ? h->key[0] : nullptr, ids ? h->ids[0] : nullptr,
+                        ids ? h->ids[1] : nullptr, s);
+  if (ids) std::swap(h->ids[0], h->ids[1]);
   std::swap(h->start_cur, h->start_new);
   h->leaf_stale = false;
   CK(cudaGetLastError());
@@ -934,8 +915,8 @@ int bin_fresh(pic_t h) {
   h->q_valid = false;
   cudaStream_t s = h->stream;
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
-  launch_count_all(h->key[1], h->n, h->count, h->mover_words, h->block_movers, h->dt.block_push, s);
-  CK(cudaMemsetAsync(h->scalars + 6, 0, sizeof(int32_t), s));
+  launch_count_all(h->key[1], h->n, h->count, h->words, h->rank, s);
+  CK(cudaMemsetAsync(h->scalars + 5, 0, sizeof(int32_t) * 3, s));  // segment lists and the order flag
   launch_check_sorted(h->key[1], h->n, h->scalars + 6, s);
   int32_t unsorted = 1;
   CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -998,7 +979,7 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
   h->q_valid = false;
   cudaStream_t s = h->stream;
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
-  CK(cudaMemsetAsync(h->scalars + 2, 0, sizeof(int32_t), s));
+  CK(cudaMemsetAsync(h->scalars + 2, 0, sizeof(int32_t) * 6, s));  // largest bucket, segment lists
   PhaseScope *ps = new PhaseScope(h, PIC_PHASE_PUSH);
   if (h->split) {
     Push32Args a{};
@@ -1026,8 +1007,8 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
     a.dt = dt;
     for (int l = 0; l <= 18; ++l) a.sl[l] = (float)(dt * (double)pow3(l));
     a.count = h->count;
-    a.mover_words = h->mover_words;
-    a.block_movers = h->block_movers;
+    a.words = h->words;
+    a.rank = h->rank;
     a.err = h->err;
     launch_push32(h->dt, a, s);
   } else {
@@ -1048,8 +1029,8 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
     a.qmdt = h->cfg.qm * dt;
     a.dt = dt;
     a.count = h->count;
-    a.mover_words = h->mover_words;
-    a.block_movers = h->block_movers;
+    a.words = h->words;
+    a.rank = h->rank;
     a.err = h->err;
     launch_push64(h->dt, a, s);
   }
