@@ -38,6 +38,10 @@ struct DevTree {
   int32_t M;  // 3^depth
   const TabEntry *tab;
   int32_t n_tab;
+  // adaptive trees: the table entry of every cell of level jump_level (no leaf
+  // is coarser), row-major; NULL where that level is the root
+  const TabEntry *jump;
+  int32_t jump_level, jump_cells;  // cells per axis: 3^jump_level
   // uniform trees: spread[a * M + c] = base-3 digits of c interleaved on axis a,
   // so the depth-first leaf id of cell c is the sum over the axes
   const int32_t *spread;
@@ -112,71 +116,6 @@ __device__ __forceinline__ int32_t descend_q(const TabEntry *tab, int d, const u
 __device__ __forceinline__ float clamp_off(float f) {
   const float one_minus = 0x1.fffffep-1f;
   return f < 0.0f ? 0.0f : (f > one_minus ? one_minus : f);
-}
-
-// One drop below the integer level: u = RN32(3 f), digit = min(floor u, 2),
-// f = u - digit (the split-precision rule of the design notes).
-__device__ __forceinline__ int drop_digit(float *f, int d) {
-  int dg = 0, mul = 1;
-  for (int a = 0; a < d; ++a) {
-    float u = 3.0f * f[a];
-    int g = (int)floorf(u);
-    g = g > 2 ? 2 : g;
-    f[a] = clamp_off(u - (float)g);
-    dg += g * mul;
-    mul *= 3;
-  }
-  return dg;
-}
-
-// Split-precision re-location: the leaf covering integer cell I on level lev
-// plus fraction f.  Writes the leaf's offsets; returns the leaf id.
-__device__ __forceinline__ int32_t descend_split(const TabEntry *tab, int d, int lev, const int32_t I[3],
-                                                 float f[3], float o_out[3], int *lev_out, int root = 0) {
-  int ent = root, m = 0, nch = d == 3 ? 27 : 9;
-  for (;;) {
-    TabEntry e = tab[ent];
-    if (e.a < 0) {
-      int k = -e.a - 1;
-      int L = m + k;
-      *lev_out = L;
-      if (L <= lev) {  // lift: the covering leaf is on a level <= lev
-        uint32_t sh = c_pow3[lev - L];
-        uint32_t J[3] = {0u, 0u, 0u};
-        for (int a = 0; a < d; ++a) {
-          J[a] = (uint32_t)I[a] / sh;
-          uint32_t r = (uint32_t)I[a] - J[a] * sh;
-          o_out[a] = clamp_off(((float)r + f[a]) / (float)sh);
-        }
-        return e.b + local_index(J[0], J[1], J[2], d, k);
-      }
-      // digits from I down to lev, then drops from the fraction
-      int32_t local = 0;
-      for (int mm = m + 1; mm <= L; ++mm) {
-        int dg;
-        if (mm <= lev) {
-          uint32_t sh = c_pow3[lev - mm];
-          dg = (int)(((uint32_t)I[0] / sh) % 3u) + 3 * (int)(((uint32_t)I[1] / sh) % 3u);
-          if (d == 3) dg += 9 * (int)(((uint32_t)I[2] / sh) % 3u);
-        } else {
-          dg = drop_digit(f, d);
-        }
-        local = local * nch + dg;
-      }
-      for (int a = 0; a < d; ++a) o_out[a] = clamp_off(f[a]);
-      return e.b + local;
-    }
-    int dg;
-    if (m + 1 <= lev) {
-      uint32_t sh = c_pow3[lev - m - 1];
-      dg = (int)(((uint32_t)I[0] / sh) % 3u) + 3 * (int)(((uint32_t)I[1] / sh) % 3u);
-      if (d == 3) dg += 9 * (int)(((uint32_t)I[2] / sh) % 3u);
-    } else {
-      dg = drop_digit(f, d);
-    }
-    ent = e.a + dg;
-    ++m;
-  }
 }
 
 // ---- grid maps ---------------------------------------------------------------

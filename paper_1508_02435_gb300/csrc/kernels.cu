@@ -270,6 +270,7 @@ __global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega,
 
 #include "uniform_solve.cuh"
 #include "adaptive_solve.cuh"
+#include "relocate.cuh"
 
 namespace pic {
 
@@ -277,11 +278,12 @@ namespace pic {
 // a1/a2 initial keys and split conversion
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ int pidt_corner_q(const uint32_t *Q, int lev, int d) {
-  uint32_t s = c_pow3[18 - lev];
+// Upper half of the leaf C of level lev that holds Q, per axis.
+__device__ __forceinline__ int pidt_corner_q(const uint32_t *Q, const uint32_t *C, int lev, int d) {
+  const uint32_t s = c_pow3[18 - lev];
   int a_idx = 0;
   for (int a = 0; a < d; ++a)
-    if (Q[a] % (2u * s) >= s) a_idx |= 1 << a;
+    if (Q[a] - C[a] * (2u * s) >= s) a_idx |= 1 << a;
   return a_idx;
 }
 
@@ -316,9 +318,10 @@ __global__ void k_init64(DevTree t, double *x, int64_t n, int32_t *leaf, int32_t
     Q[a] = quantise(y);
   }
   int lev;
-  int32_t L = descend_q(t.tab, t.d, Q, &lev, root);
+  uint32_t C[3] = {0u, 0u, 0u};
+  const int32_t L = t.d == 3 ? locate_q<3>(t, Q, root, &lev, C) : locate_q<2>(t, Q, root, &lev, C);
   leaf[p] = L;
-  key[p] = key_of(t, L, pidt_corner_q(Q, lev, t.d));
+  key[p] = key_of(t, L, pidt_corner_q(Q, C, lev, t.d));
 }
 
 // Split: leaf by the FP64 owner, o = RN32(clamp(RN64(x 3^l) - c)), v = RN32(v).
@@ -336,7 +339,8 @@ __global__ void k_init32(DevTree t, const double *x, const double *v, int64_t n,
     Q[a] = quantise(y[a]);
   }
   int lev;
-  int32_t L = descend_q(t.tab, t.d, Q, &lev, root);
+  uint32_t C[3] = {0u, 0u, 0u};
+  const int32_t L = t.d == 3 ? locate_q<3>(t, Q, root, &lev, C) : locate_q<2>(t, Q, root, &lev, C);
   leaf[p] = L;
   double s = (double)c_pow3[lev];
   float oo[3] = {0.f, 0.f, 0.f};
@@ -402,252 +406,11 @@ __device__ __forceinline__ void add_runs(int32_t *count, int32_t key, bool act) 
   }
 }
 
-// Artificial work of the paper's experiments (Section 6): `flops` floating
-// point operations per particle move (fused multiply-adds, two each), on a
-// value the move does not use; the never-taken test keeps them.
-template <typename T>
-__device__ __forceinline__ void artificial_flops(T seed, int32_t flops, int32_t *err) {
-  T acc = seed;
-  for (int32_t i = 0; i < flops; i += 2) acc = fma(acc, (T)0.999, (T)1e-3);
-  if (acc == (T)-12345.0) atomicOr(err, 0);
-}
+}  // namespace pic
 
-// Reflection at the walls of the unit box, FP64 (the oracle's reading): the
-// free path y folds into [0, 2); y >= 1 mirrors to 2 - y with the velocity
-// component negated; the far wall itself goes to the largest double below 1.
-__device__ __forceinline__ double fold64(double y, bool *flip) {
-  double m = y - 2.0 * floor(y * 0.5);
-  *flip = false;
-  if (m >= 1.0) {
-    m = 2.0 - m;
-    *flip = true;
-    if (m >= 1.0) m = 0x1.fffffffffffffp-1;
-  }
-  return m;
-}
+#include "push.cuh"
 
-// D = t.d as a compile-time constant: the per-axis loops unroll and the
-// per-particle arrays stay in registers.
-template <int D>
-__global__ void k_push64(DevTree t, Push64Args a) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool act = p < a.n;
-  int32_t knew = 0;
-  bool moved = false;
-  if (act) {
-    constexpr int d = D, nc = 1 << D;
-    const int64_t n = a.n, nv = t.n_vert;
-    int32_t L = a.leaf[p];
-    int lev;
-    int32_t c[3] = {0, 0, 0};
-    leaf_info_d<D>(t, L, &lev, c);
-    double tl[3];
-    local_coords(a.x, n, p, lev, c, d, tl);
-    double E[3] = {0.0, 0.0, 0.0};
-    const InstInfo &I = inst_of_leaf(t, L);
-    if (!a.E) {
-      // the particle-handling move: no field, no kick
-    } else if (t.uniform) {
-      int32_t vid[8];
-      corner_vertices(I, c, d, vid);
-      for (int e = 0; e < nc; ++e) {
-        double w = shape<double>(tl, e, d);
-        for (int ax = 0; ax < d; ++ax) E[ax] = E[ax] + w * a.E[ax * nv + vid[e]];
-      }
-    } else {
-      for (int e = 0; e < nc; ++e) {
-        double w = shape<double>(tl, e, d);
-        for (int ax = 0; ax < d; ++ax) E[ax] = E[ax] + w * corner_value(t, L, c, e, a.E + ax * nv);
-      }
-    }
-    uint32_t Q[3] = {0u, 0u, 0u};
-    double x0n = 0.0, x1n = 0.0, x2n = 0.0, v0n = 0.0, v1n = 0.0, v2n = 0.0;  // record path
-    bool bad = false;
-    for (int ax = 0; ax < d; ++ax) {
-      double vn = a.E ? a.v[ax * n + p] + a.qmdt * E[ax] : a.v[ax * n + p];
-      const double y = a.x[ax * n + p] + vn * a.dt;
-      double xn;
-      if (a.reflect) {
-        bool flip;
-        xn = fold64(y, &flip);
-        if (flip) vn = -vn;
-      } else {
-        xn = wrap01(y);
-      }
-      if (!isfinite(vn) || !isfinite(xn)) { bad = true; xn = 0.0; }
-      if (a.rec) {
-        if (ax == 0) { x0n = xn; v0n = vn; }
-        if (ax == 1) { x1n = xn; v1n = vn; }
-        if (ax == 2) { x2n = xn; v2n = vn; }
-      } else {
-        a.tv[ax * n + p] = vn;
-        a.tx[ax * n + p] = xn;
-      }
-      Q[ax] = quantise(xn);
-    }
-    if (a.flops > 0) artificial_flops<double>(tl[0], a.flops, a.err);
-    if (bad) atomicOr(a.err, 1);
-    int lev2;
-    int32_t L2;
-    if (t.uniform) {
-      uint32_t step = 2u * c_pow3[18 - I.depth];
-      int32_t cc[3] = {(int32_t)(Q[0] / step), (int32_t)(Q[1] / step), d == 3 ? (int32_t)(Q[2] / step) : 0};
-      L2 = I.leaf_off + uniform_leaf_of_cell(t.spread + I.spread_off, I.M, cc, d);
-      lev2 = I.depth;
-    } else {
-      // still inside its leaf (the radius of operation of Section 5.3): the
-      // covering leaf is the old one, no descent
-      const uint32_t step = 2u * c_pow3[18 - lev];
-      bool inside = true;
-      for (int ax = 0; ax < d; ++ax) inside &= Q[ax] / step == (uint32_t)c[ax];
-      if (inside) {
-        L2 = L;
-        lev2 = lev;
-      } else {
-        L2 = descend_q(t.tab, d, Q, &lev2, I.tab_root);
-      }
-    }
-    knew = key_of(t, L2, pidt_corner_q(Q, lev2, d));
-    int32_t kold = t.scheme == 0 ? L : a.key[p];
-    moved = knew != kold;
-    if (a.rec) {  // one 64-byte record per particle: the re-bin gathers it whole
-      double2 *r = a.rec + 4 * p;
-      r[0] = make_double2(x0n, x1n);
-      r[1] = make_double2(x2n, v0n);
-      r[2] = make_double2(v1n, v2n);
-      r[3] = make_double2(__longlong_as_double((long long)(((uint64_t)(uint32_t)knew << 32) | (uint32_t)L2)), 0.0);
-    } else {
-      a.tleaf[p] = L2;
-    }
-    if (a.rec || t.scheme != 0) a.keyn[p] = knew;  // PIT rows: the key array is the leaf array
-  }
-  rank_movers<D == 3>(p, moved, knew, a.count, a.words, a.rank);
-}
-
-template <int D>
-__global__ void __launch_bounds__(512, 3) k_push32(DevTree t, Push32Args a) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  bool act = p < a.n;
-  int32_t knew = 0;
-  bool moved = false;
-  if (act) {
-    constexpr int d = D, nc = 1 << D;
-    const int64_t n = a.n, nv = t.n_vert;
-    int32_t L = a.leaf[p];
-    int lev;
-    int32_t c[3] = {0, 0, 0};
-    leaf_info_d<D>(t, L, &lev, c);
-    float o[3] = {0.f, 0.f, 0.f};
-    for (int ax = 0; ax < d; ++ax) o[ax] = a.o[ax * n + p];
-    float E[3] = {0.f, 0.f, 0.f};
-    const InstInfo &Ins = inst_of_leaf(t, L);
-    if (!a.E && !a.Ec) {
-      // the particle-handling move: no field, no kick
-    } else if (t.uniform) {
-      int32_t vid[8];
-      corner_vertices(Ins, c, d, vid);
-      for (int e = 0; e < nc; ++e) {
-        float w = shape<float>(o, e, d);
-        for (int ax = 0; ax < d; ++ax) E[ax] = E[ax] + w * a.E[ax * nv + vid[e]];
-      }
-    } else if (a.Ec) {  // the corner values, expanded once per field
-      const float4 *ec = a.Ec + (int64_t)L * nc;
-      for (int e = 0; e < nc; ++e) {
-        float w = shape<float>(o, e, d);
-        const float4 q = ec[e];
-        const float qv[3] = {q.x, q.y, q.z};
-        for (int ax = 0; ax < d; ++ax) E[ax] = E[ax] + w * qv[ax];
-      }
-    } else {
-      for (int e = 0; e < nc; ++e) {
-        float w = shape<float>(o, e, d);
-        for (int ax = 0; ax < d; ++ax) E[ax] = E[ax] + w * corner_value(t, L, c, e, a.E + ax * nv);
-      }
-    }
-    const int32_t per = (int32_t)c_pow3[lev];
-    const float sl = a.sl[lev];
-    int32_t I[3] = {0, 0, 0};
-    float f[3] = {0.f, 0.f, 0.f}, vnew[3] = {0.f, 0.f, 0.f};
-    bool bad = false;
-    const bool field = a.E || a.Ec;
-    for (int ax = 0; ax < d; ++ax) {
-      float vn = field ? a.v[ax * n + p] + a.qmdt * E[ax] : a.v[ax * n + p];
-      float tt = o[ax] + vn * sl;
-      if (!isfinite(vn) || !isfinite(tt)) { bad = true; tt = 0.0f; }
-      float fl = floorf(tt);
-      f[ax] = tt - fl;
-      int32_t cc;
-      if (!a.reflect) {
-        if (fabsf(fl) < 1.0e9f) {
-          cc = c[ax] + (int32_t)fl;               // periodic wrap, 32-bit
-          if (cc < 0 || cc >= per) {
-            cc %= per;
-            if (cc < 0) cc += per;
-          }
-        } else {
-          int64_t c64 = ((int64_t)c[ax] + (int64_t)fminf(fmaxf(fl, -1.0e15f), 1.0e15f)) % per;
-          cc = (int32_t)(c64 < 0 ? c64 + per : c64);
-        }
-      } else {
-        // reflecting walls (the oracle's reading): cell index folded modulo
-        // 2 per; the mirrored half maps to (2 per - 1 - Im, 1 - f), or to
-        // (2 per - Im, 0) when f = 0, with the velocity component negated
-        const int64_t p2 = 2 * (int64_t)per;
-        int64_t im = ((int64_t)c[ax] + (int64_t)fminf(fmaxf(fl, -1.0e15f), 1.0e15f)) % p2;
-        if (im < 0) im += p2;
-        if (im < per) {
-          cc = (int32_t)im;
-        } else {
-          vn = -vn;
-          if (f[ax] > 0.0f) {
-            cc = (int32_t)(p2 - 1 - im);
-            f[ax] = clamp_off(1.0f - f[ax]);
-          } else {
-            cc = (int32_t)(p2 - im);
-            if (cc >= per) {
-              cc = per - 1;
-              f[ax] = 0x1.fffffep-1f;
-            }
-          }
-        }
-      }
-      I[ax] = cc;
-      if (a.rec) vnew[ax] = vn;
-      else a.tv[ax * n + p] = vn;
-    }
-    if (a.flops > 0) artificial_flops<float>(o[0], a.flops, a.err);
-    if (bad) atomicOr(a.err, 1);
-    float o2[3] = {0.f, 0.f, 0.f};
-    int lev2;
-    int32_t L2;
-    bool inside = true;  // target cell == the particle's own leaf cell
-    for (int ax = 0; ax < d; ++ax) inside &= I[ax] == c[ax];
-    if (t.uniform) {  // the covering leaf is the target cell itself; o = f
-      L2 = Ins.leaf_off + uniform_leaf_of_cell(t.spread + Ins.spread_off, Ins.M, I, d);
-      for (int ax = 0; ax < d; ++ax) o2[ax] = clamp_off(f[ax]);
-    } else if (inside) {
-      // still inside its leaf (the radius of operation of Section 5.3): no
-      // lift, no drop -- the covering leaf is the old one and o = f
-      L2 = L;
-      lev2 = lev;
-      for (int ax = 0; ax < d; ++ax) o2[ax] = clamp_off(f[ax]);
-    } else {
-      L2 = descend_split(t.tab, d, lev, I, f, o2, &lev2, Ins.tab_root);
-    }
-    knew = key_of(t, L2, pidt_corner_o(o2, d));
-    int32_t kold = t.scheme == 0 ? L : a.key[p];
-    moved = knew != kold;
-    if (a.rec) {  // one 32-byte record per particle: the re-bin gathers it whole
-      a.rec[2 * p] = make_float4(o2[0], o2[1], o2[2], vnew[0]);
-      a.rec[2 * p + 1] = make_float4(vnew[1], vnew[2], __int_as_float(L2), __int_as_float(knew));
-    } else {
-      for (int ax = 0; ax < d; ++ax) a.to[ax * n + p] = o2[ax];
-      a.tleaf[p] = L2;
-    }
-    if (a.rec || t.scheme != 0) a.keyn[p] = knew;  // PIT rows: the key array is the leaf array
-  }
-  rank_movers<D == 3>(p, moved, knew, a.count, a.words, a.rank);
-}
+namespace pic {
 
 // ---------------------------------------------------------------------------
 // misc
@@ -821,15 +584,14 @@ __global__ void k_relocate32(DevTree from, DevTree to, const int32_t *leaf, cons
   if (p >= n) return;
   const int32_t L = leaf[p];
   const int lev = from.leaf_level[L];
-  int32_t I[3] = {0, 0, 0};
+  uint32_t I[3] = {0u, 0u, 0u};
   float f[3] = {0.f, 0.f, 0.f};
   for (int a = 0; a < from.d; ++a) {
-    I[a] = from.leaf_coords[(int64_t)L * from.d + a];
+    I[a] = (uint32_t)from.leaf_coords[(int64_t)L * from.d + a];
     f[a] = o[a * n + p];
   }
   float on[3] = {0.f, 0.f, 0.f};
-  int lev2;
-  leaf2[p] = descend_split(to.tab, to.d, lev, I, f, on, &lev2);
+  leaf2[p] = to.d == 3 ? locate_split<3>(to, lev, I, f, on, 0) : locate_split<2>(to, lev, I, f, on, 0);
   for (int a = 0; a < from.d; ++a) {
     o2[a * n + p] = on[a];
     v2[a * n + p] = v[a * n + p];
@@ -850,6 +612,17 @@ cudaError_t set_constants(cudaStream_t s) {
     w64[i] = 1.0 / (double)p3[i];
     w32[i] = (float)w64[i];
   }
+  uint2 dv[19];
+  double p64[19];
+  for (int i = 0; i < 19; ++i) {
+    uint32_t sh = 0;
+    while ((p3[i] >> (sh + 1)) != 0u) ++sh;
+    dv[i] = make_uint2((uint32_t)(((1ull << (31 + sh)) + p3[i] - 1) / p3[i]), sh);
+    p64[i] = (double)p3[i];
+  }
+  cudaError_t ed = cudaMemcpyToSymbolAsync(c_div3, dv, sizeof(dv), 0, cudaMemcpyHostToDevice, s);
+  if (ed == cudaSuccess) ed = cudaMemcpyToSymbolAsync(c_pow3_64, p64, sizeof(p64), 0, cudaMemcpyHostToDevice, s);
+  if (ed != cudaSuccess) return ed;
   cudaError_t ew = cudaMemcpyToSymbolAsync(c_width64, w64, sizeof(w64), 0, cudaMemcpyHostToDevice, s);
   if (ew == cudaSuccess) ew = cudaMemcpyToSymbolAsync(c_width32, w32, sizeof(w32), 0, cudaMemcpyHostToDevice, s);
   if (ew != cudaSuccess) return ew;
@@ -1084,36 +857,74 @@ void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *p
   else efield<double>(t, (const double *)V, (double *)E, (double *)part, s);
 }
 
-void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s) {
-  COUNT(1);
-  if (t.d == 3) k_push64<3><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
-  else k_push64<2><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
-}
-
-// Field at every leaf corner: the same expansion sums the push would form
-// per particle (corner_value), once per leaf corner.
-__global__ void k_corner_field32(DevTree t, const float *__restrict__ E, float4 *__restrict__ Ec) {
+// Field at every leaf corner, expanded once per field instead of once per
+// particle: kStride values (D of them used) per leaf corner.
+template <typename T, int D, int kStride>
+__global__ void k_corner_field(DevTree t, const T *__restrict__ E, T *__restrict__ Ec) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= t.n_leaves * t.nc) return;
-  const int32_t L = (int32_t)(i / t.nc);
-  const int e = (int)(i - (int64_t)L * t.nc);
-  int lev;
-  int32_t c[3] = {0, 0, 0};
-  leaf_info(t, L, &lev, c);
-  float q[3] = {0.f, 0.f, 0.f};
-  for (int ax = 0; ax < t.d; ++ax) q[ax] = corner_value(t, L, c, e, E + ax * t.n_vert);
-  Ec[i] = make_float4(q[0], q[1], q[2], 0.f);
+  const T *w = corner_weights(t, (T)0);
+  T q[kStride];
+#pragma unroll
+  for (int k = 0; k < kStride; ++k) q[k] = (T)0;
+  for (int32_t j = t.cexp_ptr[i]; j < t.cexp_ptr[i + 1]; ++j) {
+    const T wj = w[j];
+    const T *e = E + t.cexp_vid[j];
+#pragma unroll
+    for (int k = 0; k < D; ++k) q[k] = q[k] + wj * e[k * t.n_vert];
+  }
+  T *out = Ec + i * kStride;
+#pragma unroll
+  for (int k = 0; k < kStride; ++k) out[k] = q[k];
 }
 
-void launch_corner_field32(const DevTree &t, const float *E, float4 *Ec, cudaStream_t s) {
-  const int64_t m = t.n_leaves * t.nc;
-  { COUNT(1); k_corner_field32<<<grid_for(m, 256), 256, 0, s>>>(t, E, Ec); }
+size_t corner_field_bytes(const DevTree &t, bool split) {
+  return (size_t)t.n_leaves * t.nc * (split ? 16 : t.d == 3 ? 32 : 16);
+}
+
+void launch_corner_field(const DevTree &t, bool split, const void *E, void *Ec, cudaStream_t s) {
+  const unsigned g = grid_for(t.n_leaves * t.nc);
+  COUNT(1);
+  if (split) {
+    if (t.d == 3) k_corner_field<float, 3, 4><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
+    else k_corner_field<float, 2, 4><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
+  } else if (t.d == 3) {
+    k_corner_field<double, 3, 4><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
+  } else {
+    k_corner_field<double, 2, 2><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
+  }
 }
 
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s) {
   COUNT(1);
-  if (t.d == 3) k_push32<3><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
-  else k_push32<2><<<grid_for(a.n, bsz(t.block_push)), bsz(t.block_push), 0, s>>>(t, a);
+  const unsigned b = bsz(t.block_push), g = grid_for(a.n, b);
+  if (t.d == 3) {
+    if (t.uniform) k_push32<3, true><<<g, b, 0, s>>>(t, a);
+    else k_push32<3, false><<<g, b, 0, s>>>(t, a);
+  } else {
+    if (t.uniform) k_push32<2, true><<<g, b, 0, s>>>(t, a);
+    else k_push32<2, false><<<g, b, 0, s>>>(t, a);
+  }
+}
+
+void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s) {
+  COUNT(1);
+  const unsigned b = bsz(t.block_push), g = grid_for(a.n, b);
+  if (t.d == 3) {
+    if (t.uniform) k_push64<3, true><<<g, b, 0, s>>>(t, a);
+    else k_push64<3, false><<<g, b, 0, s>>>(t, a);
+  } else {
+    if (t.uniform) k_push64<2, true><<<g, b, 0, s>>>(t, a);
+    else k_push64<2, false><<<g, b, 0, s>>>(t, a);
+  }
+}
+
+void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s) {
+  COUNT(1);
+  int64_t n = 1;
+  for (int a = 0; a < t.d; ++a) n *= t.jump_cells;
+  if (t.d == 3) k_jump_table<3><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
+  else k_jump_table<2><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
 }
 
 void launch_absolute_split(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, double *x,

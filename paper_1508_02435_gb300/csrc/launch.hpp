@@ -8,6 +8,7 @@
 namespace pic {
 
 struct DevTree;
+struct TabEntry;
 
 struct Push64Args {
   int64_t n;
@@ -17,6 +18,7 @@ struct Push64Args {
   double *tx, *tv;              // the pushed state in rows [d][n] and tleaf
   int32_t *tleaf, *keyn;        // keyn: new key per particle (PIT: the leaf)
   const double *E;              // [d][n_vert]; NULL: no field (the particle-handling move, no kick)
+  const double *Ec;             // adaptive trees: field at every leaf corner, 4 (3D) or 2 doubles each
   double qmdt, dt;
   int32_t *count;               // movers per key, zeroed before the launch
   uint32_t *words;              // one ballot word of movers per 32 particles
@@ -199,9 +201,12 @@ void launch_solve(const DevTree &t, bool split, const void *Q, const double *tot
 void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s);
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s);
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s);
-// Field at every leaf corner, the corner expansion applied once per field:
-// Ec[L nc + e] = (E_x, E_y, E_z, 0) at corner e of leaf L (adaptive trees).
-void launch_corner_field32(const DevTree &t, const float *E, float4 *Ec, cudaStream_t s);
+// Field at every leaf corner of an adaptive tree, the corner expansion applied
+// once per field: four floats, or four (3D) or two (2D) doubles per corner.
+size_t corner_field_bytes(const DevTree &t, bool split);
+void launch_corner_field(const DevTree &t, bool split, const void *E, void *Ec, cudaStream_t s);
+// The jump table of t (jump_level and jump_cells set) into `jump`.
+void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s);
 void launch_exclusive_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *tile_sums, int32_t *total,
                            cudaStream_t s);
 void launch_rebin(const RebinArgs &r, cudaStream_t s);

@@ -86,7 +86,7 @@ struct pic_s {
   void *part = nullptr, *Q = nullptr, *b = nullptr, *V = nullptr, *Vtmp = nullptr, *E = nullptr;
   double *block_sum = nullptr, *total = nullptr, *resid2 = nullptr;
   void *Ep = nullptr;  // d * n scratch (gather at the particles, FP64 staging)
-  float4 *ecorner = nullptr;  // split, adaptive: field at every leaf corner
+  char *ecorner = nullptr;    // adaptive: field at every leaf corner
   bool ecorner_valid = false; // ecorner holds the corners of the current E
   float *ebrick = nullptr;    // brick path: the field brick by brick (float4 / float2 per vertex)
   bool ebrick_valid = false;  // ebrick holds the current E
@@ -437,6 +437,25 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
   if ((rc = gupload(h, tb, &dt.tab, tab))) return rc;
   if ((rc = gupload(h, tb, &dt.leaf_level, leaf_level))) return rc;
   if ((rc = gupload(h, tb, &dt.leaf_coords, leaf_coords))) return rc;
+  if (n_inst == 1 && !h0.uniform) {
+    // jump table on the coarsest leaf's level (the first unrefined node in
+    // level order), or as deep as a million cells go
+    int64_t i = 0;
+    while (trees[0].flags[i]) ++i;
+    int64_t cells = 1;
+    for (int l = 0; l < h0.level[i] && cells * h0.nch <= (1 << 20); ++l) {
+      cells *= h0.nch;
+      dt.jump_level = l + 1;
+    }
+    dt.jump_cells = (int32_t)pow3(dt.jump_level);
+    TabEntry *jump = nullptr;
+    if (dt.jump_level > 0) {
+      if ((rc = galloc(h, tb, &jump, cells))) return rc;
+      launch_jump_table(dt, jump, h->stream);
+      CK(cudaGetLastError());
+    }
+    dt.jump = jump;
+  }
   bool device_tables = false;
   if (on_device) {
     // the grid and owner tables of the adaptive tree, built on the GPU
@@ -644,7 +663,7 @@ int alloc_grid(pic_t h) {
   h->ecorner = nullptr;
   h->ecorner_valid = false;
   h->ebrick_valid = false;
-  if (h->split && !h->dt.uniform && (rc = galloc(h, sb, &h->ecorner, nl * h->dt.nc))) return rc;
+  if (!h->dt.uniform && (rc = galloc(h, sb, &h->ecorner, corner_field_bytes(h->dt, h->split)))) return rc;
   return reset_grid_state(h);
 }
 
@@ -981,6 +1000,10 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
   CK(cudaMemsetAsync(h->scalars + 2, 0, sizeof(int32_t) * 6, s));  // largest bucket, segment lists
   PhaseScope *ps = new PhaseScope(h, PIC_PHASE_PUSH);
+  if (h->ecorner && mk.field && !h->ecorner_valid) {
+    launch_corner_field(h->dt, h->split, h->E, h->ecorner, s);
+    h->ecorner_valid = true;
+  }
   if (h->split) {
     Push32Args a{};
     a.n = h->n;
@@ -994,13 +1017,7 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
     a.tleaf = h->leaf[1];
     a.keyn = h->key[1];
     a.E = mk.field ? (const float *)h->E : nullptr;
-    if (h->ecorner && mk.field) {
-      if (!h->ecorner_valid) {
-        launch_corner_field32(h->dt, (const float *)h->E, h->ecorner, s);
-        h->ecorner_valid = true;
-      }
-      a.Ec = h->ecorner;
-    }
+    if (mk.field) a.Ec = (const float4 *)h->ecorner;
     a.reflect = mk.reflect;
     a.flops = mk.flops;
     a.qmdt = (float)(h->cfg.qm * dt);
@@ -1024,6 +1041,7 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
     a.tleaf = h->leaf[1];
     a.keyn = h->key[1];
     a.E = mk.field ? (const double *)h->E : nullptr;
+    if (mk.field) a.Ec = (const double *)h->ecorner;
     a.reflect = mk.reflect;
     a.flops = mk.flops;
     a.qmdt = h->cfg.qm * dt;
