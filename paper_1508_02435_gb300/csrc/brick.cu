@@ -1295,10 +1295,28 @@ __global__ void __launch_bounds__(kPullThreads) k_brick_pull(DevTree t, BrickGeo
   }
 }
 
-__global__ void k_expand_leaves(const int32_t *start, int64_t n_leaves, int32_t *leaf) {
-  int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= n_leaves) return;
-  for (int32_t p = start[l]; p < start[l + 1]; ++p) leaf[p] = (int32_t)l;
+// A warp takes 32 leaves: it spreads their ids over its particle range in
+// shared memory and writes the range out in whole lines (one leaf per thread
+// writing its few particles straight out touches a line per thread and store:
+// 243^3 cells of 8 particles 391 -> 129 us).
+constexpr int kExpandCap = 1024;  // particles of 32 leaves held; fuller warps write straight out
+__global__ void __launch_bounds__(256) k_expand_leaves(const int32_t *__restrict__ start, int64_t n_leaves,
+                                                       int32_t *__restrict__ leaf) {
+  __shared__ int32_t buf[8][kExpandCap];
+  const int lane = threadIdx.x & 31;
+  const int64_t l0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~(int64_t)31, l = l0 + lane;
+  if (l0 >= n_leaves) return;
+  const int32_t b = l < n_leaves ? start[l] : 0, e = l < n_leaves ? start[l + 1] : 0;
+  const int last = (int)(n_leaves - l0 < 32 ? n_leaves - l0 : 32) - 1;
+  const int32_t first = __shfl_sync(0xffffffffu, b, 0), end = __shfl_sync(0xffffffffu, e, last);
+  if (end - first > kExpandCap) {
+    for (int32_t p = b; p < e; ++p) leaf[p] = (int32_t)l;
+    return;
+  }
+  int32_t *mine = buf[threadIdx.x >> 5];
+  for (int32_t p = b; p < e; ++p) mine[p - first] = (int32_t)l;
+  __syncwarp();
+  for (int32_t p = first + lane; p < end; p += 32) leaf[p] = mine[p - first];
 }
 
 // ---------------------------------------------------------------------------

@@ -166,10 +166,6 @@ __global__ void k_sum_blocks(const double *in, int64_t n, double *out) {
   }
 }
 
-// ---------------------------------------------------------------------------
-// a7 deposit
-// ---------------------------------------------------------------------------
-
 __device__ __forceinline__ void local_coords(const double *x, int64_t n, int64_t p, int lev, const int32_t *c,
                                              int d, double *tl) {
   double s = (double)c_pow3[lev];
@@ -177,79 +173,6 @@ __device__ __forceinline__ void local_coords(const double *x, int64_t n, int64_t
     double u = x[a * n + p] * s - (double)c[a];
     tl[a] = u < 0.0 ? 0.0 : (u > 1.0 ? 1.0 : u);
   }
-}
-
-// Per leaf: partial sums of the 2^d shape functions over the leaf's particles
-// in bucket order (PIDT: the leaf's 2^d sub-buckets in corner order).
-template <bool kSplit, int D>
-__global__ void k_leaf_partials(DevTree t, const int32_t *__restrict__ start, const void *pos, int64_t n,
-                                void *part_out) {
-  int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (L >= t.n_leaves) return;
-  int lev;
-  int32_t c[3] = {0, 0, 0};
-  leaf_info_d<D>(t, (int32_t)L, &lev, c);
-  constexpr int nc = 1 << D, d = D;
-  const int na = t.scheme == 0 ? 1 : nc;
-  if (kSplit) {
-    const float *o = (const float *)pos;
-    float acc[nc];
-    for (int e = 0; e < nc; ++e) acc[e] = 0.0f;
-    for (int a = 0; a < na; ++a) {
-      int32_t k = key_of(t, (int32_t)L, a);
-      for (int32_t p = start[k]; p < start[k + 1]; ++p) {
-        float tl[d];
-        for (int b = 0; b < d; ++b) tl[b] = o[b * n + p];
-        for (int e = 0; e < nc; ++e) acc[e] = acc[e] + shape<float>(tl, e, d);
-      }
-    }
-    float *part = (float *)part_out;
-    for (int e = 0; e < nc; ++e) part[L * nc + e] = acc[e];
-  } else {
-    const double *x = (const double *)pos;
-    double acc[nc];
-    for (int e = 0; e < nc; ++e) acc[e] = 0.0;
-    for (int a = 0; a < na; ++a) {
-      int32_t k = key_of(t, (int32_t)L, a);
-      for (int32_t p = start[k]; p < start[k + 1]; ++p) {
-        double tl[d];
-        local_coords(x, n, p, lev, c, d, tl);
-        for (int e = 0; e < nc; ++e) acc[e] = acc[e] + shape<double>(tl, e, d);
-      }
-    }
-    double *part = (double *)part_out;
-    for (int e = 0; e < nc; ++e) part[L * nc + e] = acc[e];
-  }
-}
-
-// Per vertex: S = sum of w * partial over incident leaf corners (ascending),
-// Q = q S + ion * integral(phi_v); block partial sums of Q in FP64.
-__device__ __forceinline__ double inst_q(const InstInfo &I, double) { return I.q; }
-__device__ __forceinline__ float inst_q(const InstInfo &I, float) { return I.q32; }
-__device__ __forceinline__ double inst_ion(const InstInfo &I, double) { return I.ion; }
-__device__ __forceinline__ float inst_ion(const InstInfo &I, float) { return I.ion32; }
-
-template <typename T>
-__global__ void k_vertex_charge(DevTree t, const T *__restrict__ part, T *Q, double *block_sum) {
-  int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double mine = 0.0;
-  if (v < t.n_vert) {
-    const InstInfo &I = inst_of_vertex(t, v);
-    const T q = inst_q(I, (T)0), ion = inst_ion(I, (T)0);
-    T S = (T)0;
-    if (t.uniform) {
-      int32_t lc[8];
-      int m = uniform_incidences(v, t.d, I, t.spread, lc);
-      for (int i = 0; i < m; ++i) S = S + part[lc[i]];
-    } else {
-      const T *w = inc_weights(t, (T)0);
-      for (int32_t j = t.inc_ptr[v]; j < t.inc_ptr[v + 1]; ++j) S = S + w[j] * part[t.inc_lc[j]];
-    }
-    T val = q * S + ion * ion_load(t, v, (T)0);
-    Q[v] = val;
-    mine = (double)val;
-  }
-  block_sum_store(mine, block_sum);
 }
 
 // ---------------------------------------------------------------------------
@@ -409,6 +332,7 @@ __device__ __forceinline__ void add_runs(int32_t *count, int32_t key, bool act) 
 }  // namespace pic
 
 #include "push.cuh"
+#include "deposit.cuh"
 
 namespace pic {
 
@@ -482,49 +406,83 @@ __global__ void k_gather_only32(DevTree t, const float *o, const int32_t *leaf, 
 // a9 re-refinement: depth-first cell index on the finest admissible level
 // ---------------------------------------------------------------------------
 
-// FP64: cell of the quantised position on level dmax.
-__global__ void k_fine_key64(DevTree t, const double *x, int64_t n, int dmax, uint32_t *key) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  uint32_t step = 2u * c_pow3[18 - dmax];
-  uint32_t c[3] = {0u, 0u, 0u};
-  for (int a = 0; a < t.d; ++a) c[a] = quantise(x[a * n + p]) / step;
-  key[p] = (uint32_t)local_index(c[0], c[1], c[2], t.d, dmax);
-}
+// Counts of level m at count + coff[m].
+struct AdaptCheck {
+  int32_t *count;
+  int64_t coff[11];
+  int dmin, dmax;
+  int64_t ppc;
+};
 
-// Split: cell of leaf + offset on level dmax; below the leaf the offset
-// digits follow the drop rule of the split re-location.
-__global__ void k_fine_key32(DevTree t, const int32_t *leaf, const float *o, int64_t n, int dmax, uint32_t *key) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  const int32_t L = leaf[p];
-  const int lev = t.leaf_level[L];
-  uint32_t c[3] = {0u, 0u, 0u};
-  for (int a = 0; a < t.d; ++a) {
-    uint32_t I = (uint32_t)t.leaf_coords[(int64_t)L * t.d + a];
-    if (lev >= dmax) {
-      I /= c_pow3[lev - dmax];
-    } else {
-      float f = o[a * n + p];
-      for (int m = lev; m < dmax; ++m) {
-        float u = 3.0f * f;
-        int dg = (int)floorf(u);
-        dg = dg > 2 ? 2 : dg;
-        f = clamp_off(u - (float)dg);
-        I = 3u * I + (uint32_t)dg;
-      }
-    }
-    c[a] = I;
-  }
-  key[p] = (uint32_t)local_index(c[0], c[1], c[2], t.d, dmax);
-}
-
-// Particles per cell on one level (warp-aggregated).
-__global__ void k_level_count(const uint32_t *key, int64_t n, uint32_t div, int32_t *count) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Particles per cell of level m (depth-first cell index): the cell of the
+// quantised position (FP64), or of leaf + offset, whose digits below the leaf
+// follow the drop rule of the split re-location.
+template <int D>
+__global__ void k_level_count64(const double *x, int64_t n, int m, int32_t *count) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = p < n;
-  const uint32_t c = act ? key[p] / div : 0xffffffffu;
-  add_runs(count, (int32_t)c, act);
+  int32_t cell = -1;
+  if (act) {
+    uint32_t c[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) c[a] = div_pow3(quantise(x[a * n + p]) >> 1, 18 - m);
+    cell = subtree_index<D>(c, m);
+  }
+  add_runs(count, cell, act);
+}
+
+template <int D>
+__global__ void k_level_count32(DevTree t, const int32_t *leaf, const float *o, int64_t n, int m, int32_t *count) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool act = p < n;
+  int32_t cell = -1;
+  if (act) {
+    const int32_t L = leaf[p];
+    const int lev = t.leaf_level[L];
+    uint32_t c[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      uint32_t I = (uint32_t)t.leaf_coords[(int64_t)L * D + a];
+      if (lev >= m) {
+        I = div_pow3(I, lev - m);
+      } else {
+        float f = o[a * n + p];
+        for (int l = lev; l < m; ++l) {
+          const float u = 3.0f * f;
+          int dg = (int)floorf(u);
+          dg = dg > 2 ? 2 : dg;
+          f = clamp_off(u - (float)dg);
+          I = 3u * I + (uint32_t)dg;
+        }
+      }
+      c[a] = I;
+    }
+    cell = subtree_index<D>(c, m);
+  }
+  add_runs(count, cell, act);
+}
+
+// The same from the buckets, for the cells of the installed tree: every leaf's
+// particles go to its cell on level min(its level, top).  (Cells below a leaf
+// stay empty.)
+template <int D>
+__global__ void k_bucket_count(DevTree t, const int32_t *start, AdaptCheck ac, int top) {
+  const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (L >= t.n_leaves) return;
+  int l;
+  int32_t c[3] = {0, 0, 0};
+  leaf_info(t, (int32_t)L, &l, c);
+  const int m = l < top ? l : top;
+  if (m < ac.dmin) return;
+  int32_t cnt = 0;
+  for (int a = 0; a < (t.scheme == 0 ? 1 : t.nc); ++a) {
+    const int32_t k = key_of(t, (int32_t)L, a);
+    cnt += start[k + 1] - start[k];
+  }
+  uint32_t C[D];
+#pragma unroll
+  for (int a = 0; a < D; ++a) C[a] = div_pow3((uint32_t)c[a], l - m);
+  if (cnt) atomicAdd(&ac.count[ac.coff[m] + subtree_index<D>(C, m)], cnt);
 }
 
 __global__ void k_threshold_bits(const int32_t *count, int64_t ncells, int64_t ppc, uint32_t *bits) {
@@ -540,10 +498,11 @@ __global__ void k_threshold_bits(const int32_t *count, int64_t ncells, int64_t p
 
 // Cell counts of one level from those of the level below: the sum over the
 // 3^d children (child ch of cell c is cell c 3^d + ch).
-__global__ void k_count_parent(const int32_t *fine, int64_t ncoarse, int nch, int32_t *coarse) {
+// With `add`, to what the cell holds itself (a leaf on the coarser level).
+__global__ void k_count_parent(const int32_t *fine, int64_t ncoarse, int nch, int32_t *coarse, bool add) {
   int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= ncoarse) return;
-  int32_t t = 0;
+  int32_t t = add ? coarse[c] : 0;
   for (int ch = 0; ch < nch; ++ch) t += fine[c * nch + ch];
   coarse[c] = t;
 }
@@ -551,13 +510,7 @@ __global__ void k_count_parent(const int32_t *fine, int64_t ncoarse, int nch, in
 // Whether the particles-per-cell criterion keeps the installed tree: every
 // leaf on level l needs dmin <= l <= dmax and (l == dmax or its count <= ppc),
 // every ancestor on levels dmin .. l-1 a count > ppc.  Any leaf that fails
-// sets *changed.  Counts of level m at count + coff[m].
-struct AdaptCheck {
-  const int32_t *count;
-  int64_t coff[11];
-  int dmin, dmax;
-  int64_t ppc;
-};
+// sets *changed.
 
 __global__ void k_adapt_check(DevTree t, AdaptCheck ac, int32_t *changed) {
   const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -686,45 +639,65 @@ void launch_check_sorted(const int32_t *key, int64_t n, int32_t *flag, cudaStrea
   if (n > 1) { COUNT(1); k_check_sorted<<<grid_for(n), kBlock, 0, s>>>(key, n, flag); }
 }
 
-void launch_fine_keys(const DevTree &t, bool split, const void *pos, const int32_t *leaf, int64_t n, int dmax,
-                      uint32_t *key, cudaStream_t s) {
-  if (n <= 0) return;
-  COUNT(1);
-  if (split)
-    k_fine_key32<<<grid_for(n), kBlock, 0, s>>>(t, leaf, (const float *)pos, n, dmax, key);
-  else
-    k_fine_key64<<<grid_for(n), kBlock, 0, s>>>(t, (const double *)pos, n, dmax, key);
-}
-
-void launch_adapt_bits(const uint32_t *key, int64_t n, int nch, int dmin, int dmax, int64_t ppc, int32_t *count,
-                       const int64_t *cnt_off, uint32_t *bits, const int64_t *bit_off, cudaStream_t s) {
+void launch_adapt_bits(const DevTree &t, bool split, const void *pos, const int32_t *leaf, int64_t n, int dmin, int dmax,
+                       int64_t ppc, int32_t *count, const int64_t *cnt_off, uint32_t *bits, const int64_t *bit_off,
+                       cudaStream_t s) {
   if (dmax <= dmin) return;
+  const int m0 = dmax - 1;
   int64_t ncells = 1;
-  for (int m = 0; m < dmax - 1; ++m) ncells *= nch;
-  int32_t *fine = count + cnt_off[dmax - 1];
+  for (int m = 0; m < m0; ++m) ncells *= t.nch;
+  int32_t *fine = count + cnt_off[m0];
   cudaMemsetAsync(fine, 0, sizeof(int32_t) * ncells, s);
-  if (n > 0) { COUNT(1); k_level_count<<<grid_for(n), kBlock, 0, s>>>(key, n, (uint32_t)nch, fine); }
-  for (int m = dmax - 1; m >= dmin; --m) {
-    if (m < dmax - 1) {
+  if (n > 0) {
+    COUNT(1);
+    const unsigned g = grid_for(n);
+    if (split) {
+      if (t.d == 3) k_level_count32<3><<<g, kBlock, 0, s>>>(t, leaf, (const float *)pos, n, m0, fine);
+      else k_level_count32<2><<<g, kBlock, 0, s>>>(t, leaf, (const float *)pos, n, m0, fine);
+    } else if (t.d == 3) {
+      k_level_count64<3><<<g, kBlock, 0, s>>>((const double *)pos, n, m0, fine);
+    } else {
+      k_level_count64<2><<<g, kBlock, 0, s>>>((const double *)pos, n, m0, fine);
+    }
+  }
+  for (int m = m0; m >= dmin; --m) {
+    if (m < m0) {
       COUNT(1);
-      k_count_parent<<<grid_for(ncells), kBlock, 0, s>>>(count + cnt_off[m + 1], ncells, nch, count + cnt_off[m]);
+      k_count_parent<<<grid_for(ncells), kBlock, 0, s>>>(count + cnt_off[m + 1], ncells, t.nch, count + cnt_off[m], false);
     }
     COUNT(1);
     k_threshold_bits<<<grid_for((ncells + 31) / 32), kBlock, 0, s>>>(count + cnt_off[m], ncells, ppc,
                                                                     bits + bit_off[m]);
-    ncells /= nch;
+    ncells /= t.nch;
   }
 }
 
-void launch_adapt_check(const DevTree &t, const int32_t *count, const int64_t *coff, int dmin, int dmax, int64_t ppc,
-                        int32_t *changed, cudaStream_t s) {
+void launch_adapt_check(const DevTree &t, const int32_t *start, int32_t *count, const int64_t *coff, int dmin, int dmax,
+                        int64_t ppc, int32_t *changed, cudaStream_t s) {
   AdaptCheck ac{};
   ac.count = count;
   for (int m = 0; m <= dmax && m < 11; ++m) ac.coff[m] = coff[m];
   ac.dmin = dmin;
   ac.dmax = dmax;
   ac.ppc = ppc;
-  if (t.n_leaves > 0) { COUNT(1); k_adapt_check<<<grid_for(t.n_leaves), kBlock, 0, s>>>(t, ac, changed); }
+  if (t.n_leaves <= 0) return;
+  const unsigned g = grid_for(t.n_leaves);
+  const int top = std::min(t.depth, dmax - 1);
+  if (top >= dmin) {
+    int64_t ncells = 1;
+    for (int m = 0; m < top; ++m) ncells *= t.nch;
+    cudaMemsetAsync(count + coff[dmin], 0, sizeof(int32_t) * (coff[top] + ncells - coff[dmin]), s);
+    COUNT(1);
+    if (t.d == 3) k_bucket_count<3><<<g, kBlock, 0, s>>>(t, start, ac, top);
+    else k_bucket_count<2><<<g, kBlock, 0, s>>>(t, start, ac, top);
+    for (int m = top - 1; m >= dmin; --m) {
+      ncells /= t.nch;
+      COUNT(1);
+      k_count_parent<<<grid_for(ncells), kBlock, 0, s>>>(count + coff[m + 1], ncells, t.nch, count + coff[m], true);
+    }
+  }
+  COUNT(1);
+  k_adapt_check<<<g, kBlock, 0, s>>>(t, ac, changed);
 }
 
 void launch_relocate32(const DevTree &from, const DevTree &to, const int32_t *leaf, const float *o, const float *v,
@@ -732,56 +705,6 @@ void launch_relocate32(const DevTree &from, const DevTree &to, const int32_t *le
   if (n <= 0) return;
   COUNT(1);
   k_relocate32<<<grid_for(n), kBlock, 0, s>>>(from, to, leaf, o, v, n, leaf2, o2, v2);
-}
-
-// Per-instance FP64 sums of the vertex charges, one block per instance (fixed order).
-template <typename T>
-__global__ void k_inst_sum(DevTree t, const T *Q, double *out) {
-  const InstInfo &I = t.inst[blockIdx.x];
-  double v = 0.0;
-  for (int64_t i = threadIdx.x; i < I.n_vert; i += blockDim.x) v += (double)Q[I.vert_off + i];
-  __shared__ double sh[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  if (w == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) out[blockIdx.x] = v;
-  }
-}
-
-void launch_vertex_charge(const DevTree &t, bool split, const void *part, void *Q, double *block_sum,
-                          double *total, cudaStream_t s) {
-  if (split) {
-    { COUNT(1); k_vertex_charge<float><<<grid_for(t.n_vert, bsz(t.block_vert)), bsz(t.block_vert), 0, s>>>(t, (const float *)part, (float *)Q, block_sum); }
-  } else {
-    { COUNT(1); k_vertex_charge<double><<<grid_for(t.n_vert, bsz(t.block_vert)), bsz(t.block_vert), 0, s>>>(t, (const double *)part, (double *)Q, block_sum); }
-  }
-  if (t.n_inst > 1) {
-    COUNT(2);
-    if (split)
-      k_inst_sum<float><<<t.n_inst, 256, 0, s>>>(t, (const float *)Q, total + 1);
-    else
-      k_inst_sum<double><<<t.n_inst, 256, 0, s>>>(t, (const double *)Q, total + 1);
-    k_sum_blocks<<<1, 1024, 0, s>>>(total + 1, t.n_inst, total);
-  } else {
-    COUNT(1);
-    k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, grid_for(t.n_vert, bsz(t.block_vert)), total);
-  }
-}
-
-void launch_deposit(const DevTree &t, bool split, const int32_t *start, const void *pos, int64_t n, void *part,
-                    void *Q, double *block_sum, double *total, cudaStream_t s) {
-  if (split) {
-    { COUNT(1); if (t.d == 3) k_leaf_partials<true, 3><<<grid_for(t.n_leaves, bsz(t.block_leaf)), bsz(t.block_leaf), 0, s>>>(t, start, pos, n, part);
-      else k_leaf_partials<true, 2><<<grid_for(t.n_leaves, bsz(t.block_leaf)), bsz(t.block_leaf), 0, s>>>(t, start, pos, n, part); }
-  } else {
-    { COUNT(1); if (t.d == 3) k_leaf_partials<false, 3><<<grid_for(t.n_leaves, bsz(t.block_leaf)), bsz(t.block_leaf), 0, s>>>(t, start, pos, n, part);
-      else k_leaf_partials<false, 2><<<grid_for(t.n_leaves, bsz(t.block_leaf)), bsz(t.block_leaf), 0, s>>>(t, start, pos, n, part); }
-  }
-  launch_vertex_charge(t, split, part, Q, block_sum, total, s);
 }
 
 // Sweeps on a uniform tree between V and Vtmp, then the residual's block sums;
@@ -857,42 +780,56 @@ void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *p
   else efield<double>(t, (const double *)V, (double *)E, (double *)part, s);
 }
 
-// Field at every leaf corner, expanded once per field instead of once per
-// particle: kStride values (D of them used) per leaf corner.
-template <typename T, int D, int kStride>
+// Field at every leaf corner ([leaf][corner][axis]), expanded once per field
+// instead of once per particle.
+template <typename T, int D>
 __global__ void k_corner_field(DevTree t, const T *__restrict__ E, T *__restrict__ Ec) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= t.n_leaves * t.nc) return;
   const T *w = corner_weights(t, (T)0);
-  T q[kStride];
+  T q[D];
 #pragma unroll
-  for (int k = 0; k < kStride; ++k) q[k] = (T)0;
+  for (int k = 0; k < D; ++k) q[k] = (T)0;
   for (int32_t j = t.cexp_ptr[i]; j < t.cexp_ptr[i + 1]; ++j) {
     const T wj = w[j];
     const T *e = E + t.cexp_vid[j];
 #pragma unroll
     for (int k = 0; k < D; ++k) q[k] = q[k] + wj * e[k * t.n_vert];
   }
-  T *out = Ec + i * kStride;
 #pragma unroll
-  for (int k = 0; k < kStride; ++k) out[k] = q[k];
+  for (int k = 0; k < D; ++k) Ec[i * D + k] = q[k];
 }
 
 size_t corner_field_bytes(const DevTree &t, bool split) {
-  return (size_t)t.n_leaves * t.nc * (split ? 16 : t.d == 3 ? 32 : 16);
+  return (size_t)t.n_leaves * t.nc * t.d * (split ? sizeof(float) : sizeof(double));
 }
 
 void launch_corner_field(const DevTree &t, bool split, const void *E, void *Ec, cudaStream_t s) {
   const unsigned g = grid_for(t.n_leaves * t.nc);
   COUNT(1);
   if (split) {
-    if (t.d == 3) k_corner_field<float, 3, 4><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
-    else k_corner_field<float, 2, 4><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
+    if (t.d == 3) k_corner_field<float, 3><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
+    else k_corner_field<float, 2><<<g, kBlock, 0, s>>>(t, (const float *)E, (float *)Ec);
   } else if (t.d == 3) {
-    k_corner_field<double, 3, 4><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
+    k_corner_field<double, 3><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
   } else {
-    k_corner_field<double, 2, 2><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
+    k_corner_field<double, 2><<<g, kBlock, 0, s>>>(t, (const double *)E, (double *)Ec);
   }
+}
+
+// Coordinates and level of every leaf in one 16-byte record.
+__global__ void k_leaf_records(DevTree t, int4 *rec) {
+  const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (L >= t.n_leaves) return;
+  int lev;
+  int32_t c[3] = {0, 0, 0};
+  leaf_info(t, (int32_t)L, &lev, c);
+  rec[L] = make_int4(c[0], c[1], c[2], lev);
+}
+
+void launch_leaf_records(const DevTree &t, int4 *rec, cudaStream_t s) {
+  COUNT(1);
+  k_leaf_records<<<grid_for(t.n_leaves), kBlock, 0, s>>>(t, rec);
 }
 
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s) {
@@ -925,6 +862,42 @@ void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s) {
   for (int a = 0; a < t.d; ++a) n *= t.jump_cells;
   if (t.d == 3) k_jump_table<3><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
   else k_jump_table<2><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
+}
+
+// Records of a fresh 3D state in rows: the gather then reads one 32- or 64-byte
+// record per particle instead of seven or eight scattered values.
+template <typename V, typename T>
+__global__ void k_make_records(int64_t n, const T *x, const T *v, const int32_t *leaf, const int32_t *key, V *rec);
+template <>
+__global__ void k_make_records(int64_t n, const float *x, const float *v, const int32_t *leaf, const int32_t *key,
+                               float4 *rec) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  rec[2 * p] = make_float4(x[p], x[n + p], x[2 * n + p], v[p]);
+  rec[2 * p + 1] = make_float4(v[n + p], v[2 * n + p], __int_as_float(leaf[p]), __int_as_float(key[p]));
+}
+template <>
+__global__ void k_make_records(int64_t n, const double *x, const double *v, const int32_t *leaf, const int32_t *key,
+                               double2 *rec) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  rec[4 * p] = make_double2(x[p], x[n + p]);
+  rec[4 * p + 1] = make_double2(x[2 * n + p], v[p]);
+  rec[4 * p + 2] = make_double2(v[n + p], v[2 * n + p]);
+  rec[4 * p + 3] = make_double2(
+      __longlong_as_double((long long)(((uint64_t)(uint32_t)key[p] << 32) | (uint32_t)leaf[p])), 0.0);
+}
+
+void launch_make_records(bool split, int64_t n, const void *x, const void *v, const int32_t *leaf, const int32_t *key,
+                         void *rec, cudaStream_t s) {
+  if (n <= 0) return;
+  COUNT(1);
+  if (split)
+    k_make_records<float4, float><<<grid_for(n), kBlock, 0, s>>>(n, (const float *)x, (const float *)v, leaf, key,
+                                                                 (float4 *)rec);
+  else
+    k_make_records<double2, double><<<grid_for(n), kBlock, 0, s>>>(n, (const double *)x, (const double *)v, leaf, key,
+                                                                   (double2 *)rec);
 }
 
 void launch_absolute_split(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, double *x,

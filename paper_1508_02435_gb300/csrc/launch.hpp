@@ -18,7 +18,7 @@ struct Push64Args {
   double *tx, *tv;              // the pushed state in rows [d][n] and tleaf
   int32_t *tleaf, *keyn;        // keyn: new key per particle (PIT: the leaf)
   const double *E;              // [d][n_vert]; NULL: no field (the particle-handling move, no kick)
-  const double *Ec;             // adaptive trees: field at every leaf corner, 4 (3D) or 2 doubles each
+  const double *Ec;             // adaptive trees: field at every leaf corner [leaf][corner][axis]
   double qmdt, dt;
   int32_t *count;               // movers per key, zeroed before the launch
   uint32_t *words;              // one ballot word of movers per 32 particles
@@ -36,7 +36,7 @@ struct Push32Args {
   float *to, *tv;               // the pushed state in rows [d][n] and tleaf
   int32_t *tleaf, *keyn;        // keyn: new key per particle (PIT: the leaf)
   const float *E;               // NULL (and Ec NULL): no field (the particle-handling move, no kick)
-  const float4 *Ec;             // field at every leaf corner [leaf][corner] (adaptive trees), or NULL
+  const float *Ec;              // adaptive trees: field at every leaf corner [leaf][corner][axis]
   float qmdt;
   double dt;
   float sl[19];                 // RN32(dt * 3^level) per level
@@ -170,20 +170,21 @@ void launch_rekey32(const DevTree &t, const int32_t *leaf, const float *o, int64
                     cudaStream_t s);
 void launch_check_sorted(const int32_t *key, int64_t n, int32_t *flag, cudaStream_t s);
 void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *words, int32_t *rank, cudaStream_t s);
-// Re-refinement: depth-first cell index on level dmax per particle; cells of
-// level m (index key / div) holding more than ppc particles as a bitmap.
-void launch_fine_keys(const DevTree &t, bool split, const void *pos, const int32_t *leaf, int64_t n, int dmax,
-                      uint32_t *key, cudaStream_t s);
-// *changed = 1 unless every leaf of t passes the particles-per-cell criterion
-// on the counts of levels dmin .. dmax-1 (level m at count + coff[m]), i.e.
-// unless the criterion gives back the installed tree.
-void launch_adapt_check(const DevTree &t, const int32_t *count, const int64_t *coff, int dmin, int dmax, int64_t ppc,
-                        int32_t *changed, cudaStream_t s);
-// Threshold bits (count > ppc) of every cell on levels dmin .. dmax-1 from
-// the level-dmax cell keys: counts on level dmax-1 summed up child by child;
-// level m's counts at count + cnt_off[m], its bits at bits + bit_off[m].
-void launch_adapt_bits(const uint32_t *key, int64_t n, int nch, int dmin, int dmax, int64_t ppc, int32_t *count,
-                       const int64_t *cnt_off, uint32_t *bits, const int64_t *bit_off, cudaStream_t s);
+// *changed = 1 unless every leaf of t passes the particles-per-cell criterion,
+// i.e. unless the criterion gives back the installed tree.  The counts of its
+// cells on levels dmin .. dmax-1 (level m at count + coff[m]) come from the
+// buckets (start); no particle is read.
+void launch_adapt_check(const DevTree &t, const int32_t *start, int32_t *count, const int64_t *coff, int dmin, int dmax,
+                        int64_t ppc, int32_t *changed, cudaStream_t s);
+// Threshold bits (count > ppc) of every cell on levels dmin .. dmax-1: particles
+// counted per cell of level dmax-1, summed up child by child; level m's counts
+// at count + cnt_off[m], its bits at bits + bit_off[m].
+void launch_adapt_bits(const DevTree &t, bool split, const void *pos, const int32_t *leaf, int64_t n, int dmin, int dmax,
+                       int64_t ppc, int32_t *count, const int64_t *cnt_off, uint32_t *bits, const int64_t *bit_off,
+                       cudaStream_t s);
+// One record per particle from the rows of a fresh 3D state.
+void launch_make_records(bool split, int64_t n, const void *x, const void *v, const int32_t *leaf, const int32_t *key,
+                         void *rec, cudaStream_t s);
 void launch_relocate32(const DevTree &from, const DevTree &to, const int32_t *leaf, const float *o, const float *v,
                        int64_t n, int32_t *leaf2, float *o2, float *v2, cudaStream_t s);
 
@@ -201,10 +202,12 @@ void launch_solve(const DevTree &t, bool split, const void *Q, const double *tot
 void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s);
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s);
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s);
-// Field at every leaf corner of an adaptive tree, the corner expansion applied
-// once per field: four floats, or four (3D) or two (2D) doubles per corner.
+// Field at every leaf corner of an adaptive tree, [leaf][corner][axis], the
+// corner expansion applied once per field.
 size_t corner_field_bytes(const DevTree &t, bool split);
 void launch_corner_field(const DevTree &t, bool split, const void *E, void *Ec, cudaStream_t s);
+// Coordinates (x, y, z) and level (w) of every leaf.
+void launch_leaf_records(const DevTree &t, int4 *rec, cudaStream_t s);
 // The jump table of t (jump_level and jump_cells set) into `jump`.
 void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s);
 void launch_exclusive_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *tile_sums, int32_t *total,

@@ -449,6 +449,10 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
     }
     dt.jump_cells = (int32_t)pow3(dt.jump_level);
     TabEntry *jump = nullptr;
+    int4 *rec = nullptr;
+    if ((rc = galloc(h, tb, &rec, nl))) return rc;
+    launch_leaf_records(dt, rec, h->stream);
+    dt.leaf_rec = rec;
     if (dt.jump_level > 0) {
       if ((rc = galloc(h, tb, &jump, cells))) return rc;
       launch_jump_table(dt, jump, h->stream);
@@ -883,7 +887,7 @@ int brick_push_and_rebin(pic_t h, double dt) {
 }
 
 // Stable re-bin of the pushed state into the current state [0]: from the
-// records of the generic push (records) or from the rows [1] (fresh state).
+// records (records; 3D) or from the rows [1].
 // old_start == NULL: fresh particles, every one counted as a mover.
 int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
   cudaStream_t s = h->stream;
@@ -940,7 +944,10 @@ int bin_fresh(pic_t h) {
   int32_t unsorted = 1;
   CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (unsorted) return rebin_and_gather(h, nullptr);
+  if (unsorted) {
+    if (h->prec) launch_make_records(h->split, h->n, h->pos[1], h->vel[1], h->leaf[1], h->key[1], h->prec, s);
+    return rebin_and_gather(h, nullptr, h->prec != nullptr);
+  }
   launch_exclusive_scan(h->count, h->dt.n_keys, h->start_new, h->tile_sums, h->scalars + 0, s);
   std::swap(h->pos[0], h->pos[1]);
   std::swap(h->vel[0], h->vel[1]);
@@ -1017,7 +1024,7 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
     a.tleaf = h->leaf[1];
     a.keyn = h->key[1];
     a.E = mk.field ? (const float *)h->E : nullptr;
-    if (mk.field) a.Ec = (const float4 *)h->ecorner;
+    if (mk.field) a.Ec = (const float *)h->ecorner;
     a.reflect = mk.reflect;
     a.flops = mk.flops;
     a.qmdt = (float)(h->cfg.qm * dt);
@@ -2082,16 +2089,13 @@ int pic_adapt(pic_t h, int64_t ppc, int32_t dmin, int32_t dmax) {
       h->adapt_cells = cells;
       h->adapt_words = words;
     }
-    uint32_t *key = (uint32_t *)h->perm;  // scratch until the next re-bin
-    launch_fine_keys(h->dt, h->split, h->pos[0], h->leaf[0], n, dmax, key, s);
-    launch_adapt_bits(key, n, nch, dmin, dmax, ppc, h->adapt_count, coff.data(), h->adapt_bits, boff.data(), s);
   }
-  // the criterion on the installed tree's leaves first: when it keeps the
-  // tree, no flags are built
+  // the criterion on the installed tree's leaves first, from the buckets: when
+  // it keeps the tree, no particle is counted and no flags are built
   {
     int32_t *changed = h->scalars + 7;  // free between re-bins
     CK(cudaMemsetAsync(changed, 0, sizeof(int32_t), s));
-    launch_adapt_check(h->dt, h->adapt_count, coff.data(), dmin, dmax, ppc, changed, s);
+    launch_adapt_check(h->dt, h->start_cur, h->adapt_count, coff.data(), dmin, dmax, ppc, changed, s);
     int32_t ch = 1;
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(&ch, changed, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
@@ -2099,6 +2103,8 @@ int pic_adapt(pic_t h, int64_t ppc, int32_t dmin, int32_t dmax) {
     if (!ch) return reset_grid_state(h);
   }
   if (dmax > dmin) {
+    launch_adapt_bits(h->dt, h->split, h->pos[0], h->leaf[0], n, dmin, dmax, ppc, h->adapt_count, coff.data(),
+                      h->adapt_bits, boff.data(), s);
     CK(cudaMemcpyAsync(bits.data(), h->adapt_bits, sizeof(uint32_t) * words, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
   }

@@ -40,6 +40,41 @@ __device__ __forceinline__ double fold64(double y, bool *flip) {
   return m;
 }
 
+// 32 bytes in one load (eight floats, four doubles), from a 32-byte boundary.
+__device__ __forceinline__ void load32(const float *p, float *v) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+__device__ __forceinline__ void load32(const double *p, double *v) {
+  asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+
+// The field at the corners of leaf L of an adaptive tree: [corner][axis], whole
+// 32-byte units.  PIDT particles of a warp lie in some eighteen leaves, and the
+// L1 looks up every leaf's line again for each load.
+template <typename T, int D>
+__device__ __forceinline__ void corner_row(const T *Ec, int32_t L, T *q) {
+  constexpr int N = D << D, W = 32 / (int)sizeof(T);
+#pragma unroll
+  for (int i = 0; i < N; i += W) load32(Ec + (int64_t)L * N + i, q + i);
+}
+
+// Level and coordinates of leaf L.
+template <int D, bool kUni>
+__device__ __forceinline__ int push_leaf(const DevTree &t, const InstInfo &I, int32_t L, int32_t *c) {
+  if (kUni) {
+#pragma unroll
+    for (int k = 0; k < D; ++k) c[k] = t.leaf_coords[(int64_t)L * D + k];
+    return I.depth;
+  }
+  const int4 r = t.leaf_rec[L];
+  c[0] = r.x;
+  c[1] = r.y;
+  if (D == 3) c[D - 1] = r.z;
+  return r.w;
+}
+
 // Sort key of a particle in leaf L through corner a.  Uniform trees: C is the
 // leaf's cell; adaptive ones read the owner-vertex table.
 template <int D, bool kUni>
@@ -116,10 +151,8 @@ __global__ void __launch_bounds__(512, 3) k_push32(DevTree t, Push32Args a) {
     for (int k = 0; k < D; ++k) v[k] = a.v[k * n + p];
     const int32_t kold = t.scheme == 0 ? L : a.key[p];
     const InstInfo &Ins = kUni ? inst_of_leaf(t, L) : t.inst[0];
-    const int lev = kUni ? Ins.depth : t.leaf_level[L];
     int32_t c[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) c[k] = t.leaf_coords[(int64_t)L * D + k];
+    const int lev = push_leaf<D, kUni>(t, Ins, L, c);
     const bool field = a.E || a.Ec;
     if (field) {
       float E[D];
@@ -135,14 +168,13 @@ __global__ void __launch_bounds__(512, 3) k_push32(DevTree t, Push32Args a) {
           for (int k = 0; k < D; ++k) E[k] = E[k] + w * a.E[k * t.n_vert + vid[e]];
         }
       } else {  // the corner values, expanded once per field
-        const float4 *ec = a.Ec + (int64_t)L * NC;
+        float q[NC * D];
+        corner_row<float, D>(a.Ec, L, q);
 #pragma unroll
         for (int e = 0; e < NC; ++e) {
           const float w = shape<float>(o, e, D);
-          const float4 q = ec[e];
-          const float qv[3] = {q.x, q.y, q.z};
 #pragma unroll
-          for (int k = 0; k < D; ++k) E[k] = E[k] + w * qv[k];
+          for (int k = 0; k < D; ++k) E[k] = E[k] + w * q[e * D + k];
         }
       }
 #pragma unroll
@@ -231,10 +263,8 @@ __global__ void k_push64(DevTree t, Push64Args a) {
     for (int k = 0; k < D; ++k) v[k] = a.v[k * n + p];
     const int32_t kold = t.scheme == 0 ? L : a.key[p];
     const InstInfo &Ins = kUni ? inst_of_leaf(t, L) : t.inst[0];
-    const int lev = kUni ? Ins.depth : t.leaf_level[L];
     int32_t c[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) c[k] = t.leaf_coords[(int64_t)L * D + k];
+    const int lev = push_leaf<D, kUni>(t, Ins, L, c);
     double t0 = 0.0;
     if (a.E) {
       const double s = c_pow3_64[lev];
@@ -246,13 +276,15 @@ __global__ void k_push64(DevTree t, Push64Args a) {
       }
       t0 = tl[0];
       int32_t vid[8];
+      double q[NC * D];
       if (kUni) corner_vertices(Ins, c, D, vid);
+      else corner_row<double, D>(a.Ec, L, q);
 #pragma unroll
       for (int e = 0; e < NC; ++e) {
         const double w = shape<double>(tl, e, D);
 #pragma unroll
         for (int k = 0; k < D; ++k)
-          E[k] = fma(w, kUni ? a.E[k * t.n_vert + vid[e]] : a.Ec[((int64_t)L * NC + e) * (D == 3 ? 4 : 2) + k], E[k]);
+          E[k] = fma(w, kUni ? a.E[k * t.n_vert + vid[e]] : q[e * D + k], E[k]);
       }
 #pragma unroll
       for (int k = 0; k < D; ++k) v[k] = fma(a.qmdt, E[k], v[k]);

@@ -68,8 +68,9 @@ __device__ __forceinline__ int32_t step_weight(const int32_t *sp, int32_t M, int
   return w < 0 ? -w : w;
 }
 
-__device__ __forceinline__ void order_swap(float &a, float &b, bool c) {
-  const float x = a, y = b;
+template <typename T>
+__device__ __forceinline__ void order_swap(T &a, T &b, bool c) {
+  const T x = a, y = b;
   a = c ? y : x;
   b = c ? x : y;
 }
@@ -78,8 +79,8 @@ __device__ __forceinline__ void order_swap(float &a, float &b, bool c) {
 // ascending leaf order; w[a], flip[a]: step weight and j == 0 per axis.  kLow:
 // axes 1.. are at no multiple of 3, so their weights are 3 (and 9) and only
 // axis 0 can come out of order: outermost.
-template <int D, bool kLow>
-__device__ __forceinline__ float ordered_sum(float *u, const int32_t *w, const bool *flip) {
+template <int D, bool kLow, typename T>
+__device__ __forceinline__ T ordered_sum(T *u, const int32_t *w, const bool *flip) {
   constexpr int NC = 1 << D;
   bool any = false;
 #pragma unroll
@@ -95,7 +96,7 @@ __device__ __forceinline__ float ordered_sum(float *u, const int32_t *w, const b
     order_swap(u[1], u[2], w[0] > (kLow ? 3 : w[1]));
   } else if (kLow) {
     const bool c = w[0] > 9;
-    const float v[8] = {u[0], u[1], u[2], u[3], u[4], u[5], u[6], u[7]};
+    const T v[8] = {u[0], u[1], u[2], u[3], u[4], u[5], u[6], u[7]};
     u[1] = c ? v[2] : v[1];
     u[2] = c ? v[4] : v[2];
     u[3] = c ? v[6] : v[3];
@@ -112,7 +113,7 @@ __device__ __forceinline__ float ordered_sum(float *u, const int32_t *w, const b
     order_swap(u[1], u[2], lo > w[2]);
     order_swap(u[5], u[6], lo > w[2]);
   }
-  float y = 0.0f;
+  T y = (T)0;
 #pragma unroll
   for (int i = 0; i < NC; ++i) y = y + u[i];
   return y;
