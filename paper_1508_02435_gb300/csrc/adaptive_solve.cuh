@@ -29,11 +29,15 @@ __global__ void __launch_bounds__(256) k_corner_pass(DevTree t, const T *V, T *_
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = i < t.n_leaves * NC;
   const int e = (int)threadIdx.x & (NC - 1);
-  int32_t j0 = 0, j1 = 0;
-  T c[NC];
+  // the tables do not change: read, first entry included, while the pass before runs
+  const T *w = corner_weights(t, (T)0);
+  int32_t j0 = 0, j1 = 0, vid0 = 0;
+  T c[NC], w0 = (T)0;
   if (act) {
     j0 = t.cexp_ptr[i];
     j1 = t.cexp_ptr[i + 1];
+    vid0 = t.cexp_vid[j0];
+    w0 = w[j0];
     if (kApply) {
       const T hs = D == 2 ? (T)1 : cell_width(t.leaf_level[i / NC], (T)0);
       const T k0 = kref_val(0, 0, (T)0) * hs, k1 = kref_val(0, 1, (T)0) * hs, k2 = kref_val(0, 3, (T)0) * hs;
@@ -47,9 +51,8 @@ __global__ void __launch_bounds__(256) k_corner_pass(DevTree t, const T *V, T *_
   }
   pdl_wait();
   pdl_release();
-  const T *w = corner_weights(t, (T)0);
-  T s = (T)0;
-  for (int32_t j = j0; j < j1; ++j) s = mul_add(w[j], V[t.cexp_vid[j]], s);
+  T s = act ? mul_add(w0, V[vid0], (T)0) : (T)0;
+  for (int32_t j = j0 + 1; j < j1; ++j) s = mul_add(w[j], V[t.cexp_vid[j]], s);
   if (!kApply) {
     if (act) out[i] = s;
     return;
@@ -80,10 +83,24 @@ __global__ void __launch_bounds__(256) k_vertex_pass(DevTree t, const T *b, cons
   const T *w = inc_weights(t, (T)0);
   const T diag = act && sizeof(T) == 4 ? diag_val(t, v, (T)0) : (T)1;
   double rr = 0.0;
+  constexpr int kPre = 4;  // incidences known before the pass before ends
+  int32_t lc[kPre];
+  T wl[kPre];
+#pragma unroll
+  for (int k = 0; k < kPre; ++k) {
+    const bool ok = j0 + k < j1;
+    lc[k] = ok ? t.inc_lc[j0 + k] : -1;
+    wl[k] = ok ? w[j0 + k] : (T)0;
+  }
   pdl_wait();
   pdl_release();
-  T y = (T)0;
-  for (int32_t j = j0; j < j1; ++j) y = mul_add(w[j], part[t.inc_lc[j]], y);
+  T y = (T)0, pv[kPre];
+#pragma unroll
+  for (int k = 0; k < kPre; ++k) pv[k] = lc[k] >= 0 ? part[lc[k]] : (T)0;
+#pragma unroll
+  for (int k = 0; k < kPre; ++k)
+    if (lc[k] >= 0) y = mul_add(wl[k], pv[k], y);
+  for (int32_t j = j0 + kPre; j < j1; ++j) y = mul_add(w[j], part[t.inc_lc[j]], y);
   if (act) {
     const T r = b[v] - y;
     if (kRes) rr = (double)r * (double)r;

@@ -42,6 +42,7 @@ struct DevTree {
   // is coarser), row-major; NULL where that level is the root
   const TabEntry *jump;
   int32_t jump_level, jump_cells;  // cells per axis: 3^jump_level
+  int32_t resident;                // the solve runs as one cluster
   const int4 *leaf_rec;            // adaptive trees: leaf coordinates and level
   // uniform trees: spread[a * M + c] = base-3 digits of c interleaved on axis a,
   // so the depth-first leaf id of cell c is the sum over the axes

@@ -193,6 +193,7 @@ __global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega,
 
 #include "uniform_solve.cuh"
 #include "adaptive_solve.cuh"
+#include "resident_solve.cuh"
 #include "relocate.cuh"
 
 namespace pic {
@@ -738,6 +739,10 @@ static int64_t sweep_adaptive(const DevTree &t, const T *b, T *V, T *part, const
 template <typename T>
 static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V, T *Vtmp, T *part, T *scale, int sweeps,
                   T omega, double *block_sum, double *resid2, cudaStream_t s) {
+  if (t.resident) {
+    resident_solve<T>(false, t, Q, total, V, sweeps, omega, resid2, s);
+    return;
+  }
   { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale); }
   int64_t nb;
   if (t.uniform)
@@ -747,6 +752,12 @@ static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V,
     nb = t.d == 3 ? sweep_adaptive<T, 3>(t, b, V, part, scale, sweeps, omega, block_sum, s)
                   : sweep_adaptive<T, 2>(t, b, V, part, scale, sweeps, omega, block_sum, s);
   { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
+}
+
+bool resident_solve_fits(const DevTree &t, bool split) {
+  if (!t.uniform || t.n_inst > 1) return false;
+  return split ? resident_solve<float>(true, t, nullptr, nullptr, nullptr, 0, 0.0f, nullptr, nullptr)
+               : resident_solve<double>(true, t, nullptr, nullptr, nullptr, 0, 0.0, nullptr, nullptr);
 }
 
 void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,

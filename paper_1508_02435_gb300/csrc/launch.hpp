@@ -195,6 +195,8 @@ void launch_vertex_charge(const DevTree &t, bool split, const void *part, void *
 // total[0] is the FP64 sum over all vertices, total[1 + i] per instance.
 void launch_deposit(const DevTree &t, bool split, const int32_t *start, const void *pos, int64_t n, void *part,
                     void *Q, double *block_sum, double *total, cudaStream_t s);
+// Whether the solve of t runs as one cluster (small uniform trees).
+bool resident_solve_fits(const DevTree &t, bool split);
 // part: scratch of one value per leaf corner (adaptive trees), free after the
 // vertex charges are summed.
 void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,

@@ -546,6 +546,7 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
   h->inst = inst;
   h->hts = std::move(hts);
   h->dt = dt;
+  h->dt.resident = resident_solve_fits(dt, h->split != 0);
   h->grid_dev = device_tables;
   if (!device_tables) h->gdev = DeviceGrid{};
   h->tree_gen++;

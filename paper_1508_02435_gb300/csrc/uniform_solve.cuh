@@ -19,9 +19,9 @@
 // FP64 sums the stencil by neighbour class: fewer operations (the FP64 pipe
 // bounds these kernels), hence fewer roundings.
 //
-// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 103 us (172 MB of
+// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 82 us (172 MB of
 // V, b and V' take 25 us; bound by latency and issue, 138 warp instructions per
-// 32 vertices), 81^3 FP32 149 -> 6.9 us and FP64 277 -> 26 us, 27^3 FP32
+// 32 vertices), 81^3 FP32 149 -> 5.9 us and FP64 277 -> 23.5 us, 27^3 FP32
 // 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us (both the rate of dependent launches).
 #pragma once
 
@@ -552,7 +552,7 @@ constexpr unsigned kJacobiThreads = 128;
 // Planes per thread of k_jacobi_strip3 (M a multiple of 27): a long march
 // reads fewer planes twice, but a small grid needs its threads.  Measured, 3 /
 // 9 / 27 planes: 243^3 FP32 121 / 103 / 109 us, 81^3 FP32 6.9 / 8.4 / 17.5 us,
-// 81^3 FP64 26.1 / 28.7 / 47.3 us.
+// 81^3 FP64 26.1 / 28.7 / 47.3 us (an earlier form of the kernel).
 inline int march_length(int64_t M, size_t width) {
   const int64_t cols = M * M / 3, want = width == 8 ? 40000 : 200000;
   int len = 27;
@@ -592,8 +592,11 @@ int64_t launch_jacobi_uniform(const DevTree &t, const T *b, const T *Vin, T *Vou
     return g.x;
   }
   const int len = march_length(M, sizeof(T));
-  const dim3 g(grid_for(M * (M / 3), kJacobiThreads), (unsigned)(M / len));
-  launch_pdl(k_jacobi_strip3<T, kRes>, g, dim3(kJacobiThreads), s, t, b, Vin, Vout, omega, r2, len);
+  // FP64: one warp a block spreads the work evenly over the SMs' FP64 pipes (81^3:
+  // 486 blocks of 128 threads leave the pipes idle for half the time, 29.7 -> 23.5 us)
+  const unsigned threads = sizeof(T) == 8 ? 32 : kJacobiThreads;
+  const dim3 g(grid_for(M * (M / 3), threads), (unsigned)(M / len));
+  launch_pdl(k_jacobi_strip3<T, kRes>, g, dim3(threads), s, t, b, Vin, Vout, omega, r2, len);
   return (int64_t)g.x * g.y;
 }
 
