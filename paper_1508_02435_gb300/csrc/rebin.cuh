@@ -388,45 +388,53 @@ __global__ void k_gather_state(SlotOrder so, int64_t n, const T *__restrict__ x,
   if (ids) ids2[p] = id;
 }
 
-// The same from the pushed-state records of the 3D step (two or four 16-byte
+// 32 bytes in one load (eight floats, four doubles), from a 32-byte boundary.
+__device__ __forceinline__ void load32(const float *p, float *v) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+__device__ __forceinline__ void load32(const double *p, double *v) {
+  asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+
+// The same from the pushed-state records of the 3D step (one or two 32-byte
 // loads per particle instead of one scattered 4- or 8-byte load per array).
-__global__ void k_gather_rec32(SlotOrder so, int64_t n, const float4 *__restrict__ rec, float *__restrict__ x2,
+__global__ void k_gather_rec32(SlotOrder so, int64_t n, const float *__restrict__ rec, float *__restrict__ x2,
                                float *__restrict__ v2, int32_t *__restrict__ leaf2, int32_t *__restrict__ key2,
                                const int32_t *__restrict__ ids, int32_t *__restrict__ ids2) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const int32_t i = so.perm[s];
-  const float4 r0 = rec[2 * (int64_t)i], r1 = rec[2 * (int64_t)i + 1];
+  float r[8];
+  load32(rec + 8 * (int64_t)i, r);
   const int32_t id = ids ? ids[i] : 0;
-  const int64_t p = so.place((int32_t)s, i, __float_as_int(r1.w));
-  x2[p] = r0.x;
-  x2[n + p] = r0.y;
-  x2[2 * n + p] = r0.z;
-  v2[p] = r0.w;
-  v2[n + p] = r1.x;
-  v2[2 * n + p] = r1.y;
-  leaf2[p] = __float_as_int(r1.z);
-  if (key2) key2[p] = __float_as_int(r1.w);
+  const int64_t p = so.place((int32_t)s, i, __float_as_int(r[7]));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) x2[k * n + p] = r[k];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v2[k * n + p] = r[3 + k];
+  leaf2[p] = __float_as_int(r[6]);
+  if (key2) key2[p] = __float_as_int(r[7]);
   if (ids) ids2[p] = id;
 }
 
-__global__ void k_gather_rec64(SlotOrder so, int64_t n, const double2 *__restrict__ rec, double *__restrict__ x2,
+__global__ void k_gather_rec64(SlotOrder so, int64_t n, const double *__restrict__ rec, double *__restrict__ x2,
                                double *__restrict__ v2, int32_t *__restrict__ leaf2, int32_t *__restrict__ key2,
                                const int32_t *__restrict__ ids, int32_t *__restrict__ ids2) {
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n) return;
   const int32_t i = so.perm[s];
-  const double2 *r = rec + 4 * (int64_t)i;
-  const double2 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
-  const uint64_t lk = (uint64_t)__double_as_longlong(r3.x);
+  double r[8];
+  load32(rec + 8 * (int64_t)i, r);
+  load32(rec + 8 * (int64_t)i + 4, r + 4);
+  const uint64_t lk = (uint64_t)__double_as_longlong(r[6]);
   const int32_t id = ids ? ids[i] : 0, k = (int32_t)(uint32_t)(lk >> 32);
   const int64_t p = so.place((int32_t)s, i, k);
-  x2[p] = r0.x;
-  x2[n + p] = r0.y;
-  x2[2 * n + p] = r1.x;
-  v2[p] = r1.y;
-  v2[n + p] = r2.x;
-  v2[2 * n + p] = r2.y;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) x2[a * n + p] = r[a];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) v2[a * n + p] = r[3 + a];
   leaf2[p] = (int32_t)(uint32_t)lk;
   if (key2) key2[p] = k;
   if (ids) ids2[p] = id;
@@ -512,10 +520,10 @@ void launch_gather_records(bool split, const RebinArgs &r, const void *rec, void
   COUNT(1);
   const SlotOrder so{r.perm, r.old_start ? r.base : r.new_start, r.new_start};
   if (split)
-    k_gather_rec32<<<grid_for(r.n), kBlock, 0, s>>>(so, r.n, (const float4 *)rec, (float *)x2, (float *)v2, leaf2, key2,
+    k_gather_rec32<<<grid_for(r.n), kBlock, 0, s>>>(so, r.n, (const float *)rec, (float *)x2, (float *)v2, leaf2, key2,
                                                     ids, ids2);
   else
-    k_gather_rec64<<<grid_for(r.n), kBlock, 0, s>>>(so, r.n, (const double2 *)rec, (double *)x2, (double *)v2, leaf2,
+    k_gather_rec64<<<grid_for(r.n), kBlock, 0, s>>>(so, r.n, (const double *)rec, (double *)x2, (double *)v2, leaf2,
                                                     key2, ids, ids2);
 }
 
