@@ -179,13 +179,14 @@ __device__ __forceinline__ void local_coords(const double *x, int64_t n, int64_t
 // a8 solve (auxiliary): b = Q - (sum Q) integral(phi); damped Jacobi
 // ---------------------------------------------------------------------------
 
-// With scale, also omega / diag per vertex.
+// With scale, also omega / diag per vertex; with `scaled`, b times that.
 template <typename T>
-__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale) {
+__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale, bool scaled) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= t.n_vert) return;
   T tot = (T)(t.n_inst > 1 ? total[1 + t.inst_of_vert[v]] : *total);
-  b[v] = Q[v] - tot * ion_load(t, v, (T)0);
+  const T r = Q[v] - tot * ion_load(t, v, (T)0);
+  b[v] = scaled ? r * (omega / diag_val(t, v, (T)0)) : r;
   if (scale) scale[v] = omega / diag_val(t, v, (T)0);
 }
 
@@ -194,6 +195,7 @@ __global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega,
 #include "uniform_solve.cuh"
 #include "adaptive_solve.cuh"
 #include "resident_solve.cuh"
+#include "row_solve.cuh"
 #include "relocate.cuh"
 
 namespace pic {
@@ -737,14 +739,23 @@ static int64_t sweep_adaptive(const DevTree &t, const T *b, T *V, T *part, const
 }
 
 template <typename T>
-static void solve(const DevTree &t, const T *Q, const double *total, T *b, T *V, T *Vtmp, T *part, T *scale, int sweeps,
-                  T omega, double *block_sum, double *resid2, cudaStream_t s) {
+static void solve(const DevTree &t, const RowMatrix &A, const T *Q, const double *total, T *b, T *V, T *Vtmp, T *part,
+                  int sweeps, T omega, double *block_sum, double *resid2, cudaStream_t s) {
   if (t.resident) {
     resident_solve<T>(false, t, Q, total, V, sweeps, omega, resid2, s);
     return;
   }
-  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale); }
+  // the FP64 two-pass solve of an adaptive tree leaves Vtmp free: it holds omega / diag
+  T *scale = sizeof(T) == 8 && !t.uniform && !A.val ? Vtmp : nullptr;
+  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale, A.val != nullptr); }
   int64_t nb;
+  if constexpr (sizeof(T) == 8) {
+    if (A.val) {
+      nb = sweep_rows(t, A, b, V, Vtmp, sweeps, omega, block_sum, s);
+      { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
+      return;
+    }
+  }
   if (t.uniform)
     nb = t.d == 3 ? sweep_uniform<T, 3>(t, b, V, Vtmp, sweeps, omega, block_sum, s)
                   : sweep_uniform<T, 2>(t, b, V, Vtmp, sweeps, omega, block_sum, s);
@@ -760,14 +771,14 @@ bool resident_solve_fits(const DevTree &t, bool split) {
                : resident_solve<double>(true, t, nullptr, nullptr, nullptr, 0, 0.0, nullptr, nullptr);
 }
 
-void launch_solve(const DevTree &t, bool split, const void *Q, const double *total, void *b, void *V, void *Vtmp,
-                  void *part, int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s) {
+void launch_solve(const DevTree &t, const RowMatrix &A, bool split, const void *Q, const double *total, void *b, void *V,
+                  void *Vtmp, void *part, int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s) {
   if (split)
-    solve<float>(t, (const float *)Q, total, (float *)b, (float *)V, (float *)Vtmp, (float *)part, nullptr, sweeps,
+    solve<float>(t, A, (const float *)Q, total, (float *)b, (float *)V, (float *)Vtmp, (float *)part, sweeps,
                  (float)omega, block_sum, resid2, s);
-  else  // an adaptive solve leaves Vtmp free: it holds omega / diag
-    solve<double>(t, (const double *)Q, total, (double *)b, (double *)V, (double *)Vtmp, (double *)part,
-                  t.uniform ? nullptr : (double *)Vtmp, sweeps, omega, block_sum, resid2, s);
+  else
+    solve<double>(t, A, (const double *)Q, total, (double *)b, (double *)V, (double *)Vtmp, (double *)part, sweeps,
+                  omega, block_sum, resid2, s);
 }
 
 template <typename T>

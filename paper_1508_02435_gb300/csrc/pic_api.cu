@@ -86,6 +86,7 @@ struct pic_s {
   void *part = nullptr, *Q = nullptr, *b = nullptr, *V = nullptr, *Vtmp = nullptr, *E = nullptr;
   double *block_sum = nullptr, *total = nullptr, *resid2 = nullptr;
   void *Ep = nullptr;  // d * n scratch (gather at the particles, FP64 staging)
+  RowMatrix rows{};           // FP64, adaptive: assembled rows of the solve
   char *ecorner = nullptr;    // adaptive: field at every leaf corner
   bool ecorner_valid = false; // ecorner holds the corners of the current E
   float *ebrick = nullptr;    // brick path: the field brick by brick (float4 / float2 per vertex)
@@ -638,6 +639,34 @@ int alloc_particles(pic_t h) {
   return PIC_OK;
 }
 
+// Assembles the rows of the FP64 solve of an adaptive tree, where the solve
+// sweeps often enough to repay it (assembly: about ten sweeps of the two passes)
+// and the rows take a few hundred megabytes at most.  Rows that do not fit leave
+// the two passes.
+int build_rows(pic_t h) {
+  h->rows = RowMatrix{};
+  if (h->split || h->dt.uniform || h->cfg.sweeps < 16 || h->dt.n_vert > 2000000) return PIC_OK;
+  cudaStream_t s = h->stream;
+  auto &gb = h->grid_bufs;
+  const int64_t ns = row_slices(h->dt);
+  int32_t *ptr, *len, *col, got[2] = {0, 0};
+  double *val;
+  int rc;
+  if ((rc = galloc(h, gb, &ptr, ns + 1)) || (rc = galloc(h, gb, &len, ns))) return rc;
+  CK(cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s));
+  launch_row_count(h->dt, len, h->scalars + 4, s);
+  launch_exclusive_scan(len, ns, ptr, h->tile_sums, h->scalars + 3, s);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (got[1]) return PIC_OK;
+  if ((rc = galloc(h, gb, &col, got[0])) || (rc = galloc(h, gb, &val, got[0]))) return rc;
+  launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, s);
+  CK(cudaGetLastError());
+  h->rows = RowMatrix{ptr, col, val};
+  return PIC_OK;
+}
+
 // Buffers sized from the installed tree (bucket offsets and counts, leaf
 // partials, vertex fields, the FP64 staging area); the solver's warm start
 // and the field start from zero.
@@ -677,6 +706,7 @@ int alloc_grid(pic_t h) {
   h->ecorner = nullptr;
   h->ecorner_valid = false;
   h->ebrick_valid = false;
+  if ((rc = build_rows(h))) return rc;
   if (!h->dt.uniform && (rc = galloc(h, sb, &h->ecorner, corner_field_bytes(h->dt, h->split)))) return rc;
   return reset_grid_state(h);
 }
@@ -993,7 +1023,7 @@ int field(pic_t h, pic_solve_fn hook, void *user) {
     if (r != 0) return fail(h, PIC_EHOOK, "field-solve hook returned " + std::to_string(r));
     return PIC_OK;
   }
-  launch_solve(h->dt, h->split, h->Q, h->total, h->b, h->V, h->Vtmp, h->part, h->cfg.sweeps, h->cfg.omega, h->block_sum,
+  launch_solve(h->dt, h->rows, h->split, h->Q, h->total, h->b, h->V, h->Vtmp, h->part, h->cfg.sweeps, h->cfg.omega, h->block_sum,
                h->resid2, s);
   launch_efield(h->dt, h->split, h->V, h->E, h->part, s);
   CK(cudaGetLastError());
