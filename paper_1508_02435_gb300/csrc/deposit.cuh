@@ -80,7 +80,7 @@ __host__ __device__ constexpr int shape_slice() {
 
 __device__ __forceinline__ void local_coord(float x, float, int32_t, float *t) { *t = x; }
 __device__ __forceinline__ void local_coord(double x, double s, int32_t c, double *t) {
-  *t = unit_clamp(fma(x, s, -(double)c));
+  *t = unit_clamp(x * s - (double)c);  // rounded as everywhere else
 }
 
 template <typename T, int D>
@@ -340,7 +340,7 @@ static void vertex_charge(const DevTree &t, const T *part, T *Q, double *block_s
   k_vertex_charge<T><<<g, b, 0, s>>>(t, part, Q, t.n_inst > 1 ? nullptr : block_sum, per);
   COUNT(t.n_inst > 1 ? 2 : 1);
   if (t.n_inst > 1) {
-    k_inst_sum<T><<<t.n_inst, 256, 0, s>>>(t, Q, total + 1);
+    k_inst_sum<T><<<t.n_inst, 1024, 0, s>>>(t, Q, total + 1);
     k_sum_blocks<<<1, 1024, 0, s>>>(total + 1, t.n_inst, total);
   } else {
     k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, g, total);

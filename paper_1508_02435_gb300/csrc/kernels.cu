@@ -298,8 +298,9 @@ __global__ void k_rekey32(DevTree t, const int32_t *leaf, const float *o, int64_
 // a6 stable counting sort
 // ---------------------------------------------------------------------------
 
-constexpr int kMedSeg = 2048;        // longest segment one warp sorts in shared memory
+constexpr int kMedSeg = 1024;        // longest segment one warp sorts in shared memory
 constexpr int kMedThreads = 256;
+constexpr unsigned kMedBlocks = 7 * 152;  // as many as fit the SMs' shared memory
 constexpr int kLargeSeg = 16384;     // chunk of a long segment sorted in shared memory
 constexpr int kLargeThreads = 1024;
 

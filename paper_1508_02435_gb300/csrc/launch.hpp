@@ -65,7 +65,7 @@ struct RebinArgs {
 };
 // Mover segments of up to this many are put in order by the gather; longer
 // ones (at most n / (kRankSegment + 1)) are listed and sorted.
-constexpr int64_t kRankSegment = 64;
+constexpr int64_t kRankSegment = 128;
 
 // Elements per tile of launch_exclusive_scan: a scan of n elements writes
 // scan_tiles_needed(n) = ceil(n / kScanTileElems) tile sums.

@@ -276,7 +276,7 @@ __global__ void k_push64(DevTree t, Push64Args a) {
       double tl[D], E[D];
 #pragma unroll
       for (int k = 0; k < D; ++k) {
-        tl[k] = unit_clamp(fma(x[k], s, -(double)c[k]));
+        tl[k] = unit_clamp(x[k] * s - (double)c[k]);
         E[k] = 0.0;
       }
       t0 = tl[0];

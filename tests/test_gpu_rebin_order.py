@@ -18,7 +18,9 @@ if not torch.cuda.is_available():  # pragma: no cover - CPU hosts
 
 
 @pytest.mark.parametrize("d,depth,n,m", [(2, 2, 3000, 0), (2, 2, 3000, 1), (2, 2, 3000, 63), (2, 2, 3000, 64),
-                                         (2, 2, 3000, 65), (2, 3, 9000, 2047), (2, 3, 9000, 2048), (2, 3, 9000, 2049),
+                                         (2, 2, 3000, 65), (2, 2, 3000, 127), (2, 2, 3000, 128),
+                                         (2, 2, 3000, 129), (2, 3, 9000, 1023), (2, 3, 9000, 1024), (2, 3, 9000, 1025),
+                                         (3, 2, 5000, 129), (2, 3, 9000, 2047), (2, 3, 9000, 2048), (2, 3, 9000, 2049),
                                          (2, 5, 70_001, 40_000), (3, 1, 1000, 64), (3, 2, 5000, 65),
                                          (3, 4, 60_001, 3000), (2, 2, 31, 31), (2, 2, 64, 40), (2, 6, 900_000, 300)])
 @pytest.mark.parametrize("scheme,precision", [(pic.PIT, pic.FP32_SPLIT), (pic.PIDT, pic.FP32_SPLIT), (pic.PIT, pic.FP64),
