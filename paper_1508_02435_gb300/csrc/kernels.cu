@@ -280,20 +280,6 @@ __global__ void k_init32(DevTree t, const double *x, const double *v, int64_t n,
   key[p] = key_of(t, L, pidt_corner_o(oo, t.d));
 }
 
-// Keys of a given split state (leaf + offsets); flags offsets outside [0,1).
-__global__ void k_rekey32(DevTree t, const int32_t *leaf, const float *o, int64_t n, int32_t *key, int32_t *err) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  int32_t L = leaf[p];
-  if (L < 0 || L >= t.n_leaves) { atomicOr(err, 2); L = 0; }
-  float oo[3] = {0.f, 0.f, 0.f};
-  for (int a = 0; a < t.d; ++a) {
-    oo[a] = o[a * n + p];
-    if (!(oo[a] >= 0.0f && oo[a] < 1.0f)) atomicOr(err, 2);
-  }
-  key[p] = key_of(t, L, pidt_corner_o(oo, t.d));
-}
-
 // ---------------------------------------------------------------------------
 // a6 stable counting sort
 // ---------------------------------------------------------------------------
@@ -533,6 +519,25 @@ __global__ void k_adapt_check(DevTree t, AdaptCheck ac, int32_t *changed) {
   if (bad) *changed = 1;
 }
 
+// The same on a uniform tree of one instance, PIT: the leaves below any cell are
+// contiguous, so its count is a difference of bucket offsets.
+__global__ void k_adapt_check_uniform(DevTree t, const int32_t *__restrict__ start, AdaptCheck ac, int32_t *changed) {
+  const int64_t L = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (L >= t.n_leaves) return;
+  const int l = t.depth;
+  bool bad = l < ac.dmin || l > ac.dmax;
+  int64_t width = 1;
+  for (int m = l; !bad && m >= ac.dmin; --m) {
+    if (m < ac.dmax) {
+      const int64_t b = L / width * width;
+      const int32_t cnt = start[b + width] - start[b];
+      bad = m < l ? cnt <= ac.ppc : cnt > ac.ppc;
+    }
+    width *= t.nch;
+  }
+  if (bad) *changed = 1;
+}
+
 // Split particles of tree `from` re-located in tree `to` (same positions):
 // the resolver of the split push with zero displacement.
 __global__ void k_relocate32(DevTree from, DevTree to, const int32_t *leaf, const float *o, const float *v,
@@ -627,11 +632,6 @@ void launch_init32(const DevTree &t, const double *x, const double *v, int64_t n
   if (n > 0) { COUNT(1); k_init32<<<grid_for(n), kBlock, 0, s>>>(t, x, v, n, leaf, o, vf, key, err); }
 }
 
-void launch_rekey32(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, int32_t *key, int32_t *err,
-                    cudaStream_t s) {
-  if (n > 0) { COUNT(1); k_rekey32<<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, n, key, err); }
-}
-
 // Flag = 1 if keys are not in ascending order.
 __global__ void k_check_sorted(const int32_t *key, int64_t n, int32_t *flag) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -686,6 +686,11 @@ void launch_adapt_check(const DevTree &t, const int32_t *start, int32_t *count, 
   ac.ppc = ppc;
   if (t.n_leaves <= 0) return;
   const unsigned g = grid_for(t.n_leaves);
+  if (t.uniform && t.scheme == 0) {
+    COUNT(1);
+    k_adapt_check_uniform<<<g, kBlock, 0, s>>>(t, start, ac, changed);
+    return;
+  }
   const int top = std::min(t.depth, dmax - 1);
   if (top >= dmin) {
     int64_t ncells = 1;
@@ -885,6 +890,60 @@ void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s) {
   for (int a = 0; a < t.d; ++a) n *= t.jump_cells;
   if (t.d == 3) k_jump_table<3><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
   else k_jump_table<2><<<grid_for(n), kBlock, 0, s>>>(t.tab, t.jump_level, t.jump_cells, jump);
+}
+
+// A given split state (leaf + offsets) as fresh particles, one pass: keys, ranks,
+// whether the keys ascend, and in 3D the records the gather reads.  Flags leaves
+// outside the tree and offsets outside [0,1).
+template <int D>
+__global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restrict__ o, const float *__restrict__ v,
+                          int64_t n, int32_t *key /* may be leaf */, float4 *__restrict__ rec,
+                          int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool act = p < n;
+  auto key_at = [&](int64_t q, float *oo, int32_t *L, bool *bad) {
+    *L = leaf[q];
+    if (*L < 0 || *L >= t.n_leaves) { *bad = true; *L = 0; }
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+      oo[a] = o[a * n + q];
+      if (!(oo[a] >= 0.0f && oo[a] < 1.0f)) *bad = true;
+    }
+    return key_of(t, *L, pidt_corner_o(oo, D));
+  };
+  int32_t k = 0, L = 0;
+  bool bad = false;
+  float oo[D];
+  if (act) {
+    k = key_at(p, oo, &L, &bad);
+    key[p] = k;
+    if (bad) atomicOr(err, 2);
+    if (D == 3) {
+      rec[2 * p] = make_float4(oo[0], oo[1], oo[D - 1], v[p]);
+      rec[2 * p + 1] = make_float4(v[n + p], v[(D - 1) * n + p], __int_as_float(L), __int_as_float(k));
+    }
+  }
+  int32_t prev = __shfl_up_sync(0xffffffffu, k, 1);
+  if ((threadIdx.x & 31) == 0 && act && p > 0) {
+    float po[D];
+    int32_t pl;
+    bool pb = false;
+    prev = key_at(p - 1, po, &pl, &pb);
+  }
+  const bool down = act && p > 0 && prev > k;
+  if (__syncthreads_or(down) && threadIdx.x == 0) atomicOr(unsorted, 1);
+  rank_movers<false>(p, act, k, count, words, rank);
+}
+
+void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const float *v, int64_t n, int32_t *key,
+                    void *rec, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err,
+                    cudaStream_t s) {
+  if (n <= 0) return;
+  COUNT(1);
+  if (t.d == 3)
+    k_fresh32<3><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, count, words, rank, unsorted, err);
+  else
+    k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, count, words, rank, unsorted, err);
 }
 
 // Records of a fresh 3D state in rows: the gather then reads one 32- or 64-byte

@@ -166,7 +166,10 @@ void launch_init64(const DevTree &t, double *x, int64_t n, int32_t *leaf, int32_
                    cudaStream_t s);
 void launch_init32(const DevTree &t, const double *x, const double *v, int64_t n, int32_t *leaf, float *o,
                    float *vf, int32_t *key, int32_t *err, cudaStream_t s);
-void launch_rekey32(const DevTree &t, const int32_t *leaf, const float *o, int64_t n, int32_t *key, int32_t *err,
+// A given split state as fresh particles: keys, ranks, *unsorted = 1 unless the
+// keys ascend, records in 3D; *err |= 2 where a leaf or an offset is out of range.
+void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const float *v, int64_t n, int32_t *key,
+                    void *rec, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err,
                     cudaStream_t s);
 void launch_check_sorted(const int32_t *key, int64_t n, int32_t *flag, cudaStream_t s);
 void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *words, int32_t *rank, cudaStream_t s);

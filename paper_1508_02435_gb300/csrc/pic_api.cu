@@ -927,9 +927,13 @@ int brick_push_and_rebin(pic_t h, double dt) {
 }
 
 // Stable re-bin of the pushed state into the current state [0]: from the
-// records (records; 3D) or from the rows [1].
+// records (records; 3D) or from rows ([1] unless given).
 // old_start == NULL: fresh particles, every one counted as a mover.
-int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
+struct Rows {  // positions (offsets), velocities, leaves of a pushed or fresh state
+  const void *pos, *vel;
+  const int32_t *leaf;
+};
+int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false, const Rows *rows = nullptr) {
   cudaStream_t s = h->stream;
   const int64_t n = h->n;
   RebinArgs r{};
@@ -960,10 +964,30 @@ int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
     launch_gather_records(h->split, r, h->prec, h->pos[0], h->vel[0], h->leaf[0], pidt ? h->key[0] : nullptr,
                           ids ? h->ids[0] : nullptr, ids ? h->ids[1] : nullptr, s);
   else
-    launch_gather_state(h->split, r, h->d, h->pos[1], h->pos[0], h->vel[1], h->vel[0], h->leaf[1], h->leaf[0],
+    launch_gather_state(h->split, r, h->d, rows ? rows->pos : h->pos[1], h->pos[0], rows ? rows->vel : h->vel[1],
+                        h->vel[0], rows ? rows->leaf : h->leaf[1], h->leaf[0],
                         pidt ? h->key[1] : nullptr, pidt ? h->key[0] : nullptr, ids ? h->ids[0] : nullptr,
                         ids ? h->ids[1] : nullptr, s);
   if (ids) std::swap(h->ids[0], h->ids[1]);
+  std::swap(h->start_cur, h->start_new);
+  h->leaf_stale = false;
+  CK(cudaGetLastError());
+  return PIC_OK;
+}
+
+// Fresh state in [1] whose keys ascend: it is in bucket order already, only the
+// bucket offsets are computed.
+int take_sorted(pic_t h) {
+  cudaStream_t s = h->stream;
+  launch_exclusive_scan(h->count, h->dt.n_keys, h->start_new, h->tile_sums, h->scalars + 0, s);
+  std::swap(h->pos[0], h->pos[1]);
+  std::swap(h->vel[0], h->vel[1]);
+  std::swap(h->leaf[0], h->leaf[1]);
+  if (h->key[0] != h->leaf[1]) std::swap(h->key[0], h->key[1]);  // PIT keys alias the leaves
+  else {
+    h->key[0] = h->leaf[0];
+    h->key[1] = h->leaf[1];
+  }
   std::swap(h->start_cur, h->start_new);
   h->leaf_stale = false;
   CK(cudaGetLastError());
@@ -988,19 +1012,32 @@ int bin_fresh(pic_t h) {
     if (h->prec) launch_make_records(h->split, h->n, h->pos[1], h->vel[1], h->leaf[1], h->key[1], h->prec, s);
     return rebin_and_gather(h, nullptr, h->prec != nullptr);
   }
-  launch_exclusive_scan(h->count, h->dt.n_keys, h->start_new, h->tile_sums, h->scalars + 0, s);
-  std::swap(h->pos[0], h->pos[1]);
-  std::swap(h->vel[0], h->vel[1]);
-  std::swap(h->leaf[0], h->leaf[1]);
-  if (h->key[0] != h->leaf[1]) std::swap(h->key[0], h->key[1]);  // PIT keys alias the leaves
-  else {
-    h->key[0] = h->leaf[0];
-    h->key[1] = h->leaf[1];
-  }
-  std::swap(h->start_cur, h->start_new);
-  h->leaf_stale = false;
+  return take_sorted(h);
+}
+
+// A split state handed over (host: copied to [1] first; device: read where it
+// is) as fresh particles.
+int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v, bool copied) {
+  h->q_valid = false;
+  cudaStream_t s = h->stream;
+  const int64_t n = h->n, m = n * h->d;
+  CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
+  CK(cudaMemsetAsync(h->scalars + 5, 0, sizeof(int32_t) * 3, s));  // segment lists and the order flag
+  launch_fresh32(h->dt, leaf, o, v, n, h->key[1], h->prec, h->count, h->words, h->rank, h->scalars + 6, h->err, s);
+  int32_t unsorted = 1;
   CK(cudaGetLastError());
-  return PIC_OK;
+  CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (unsorted) {
+    const Rows rows{o, v, h->scheme == PIC_PIT ? h->leaf[1] : leaf};  // PIT: the keys just written
+    return rebin_and_gather(h, nullptr, h->prec != nullptr, &rows);
+  }
+  if (!copied) {
+    CK(cudaMemcpyAsync(h->pos[1], o, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(h->vel[1], v, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
+    if (h->scheme != PIC_PIT) CK(cudaMemcpyAsync(h->leaf[1], leaf, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+  }
+  return take_sorted(h);
 }
 
 int deposit(pic_t h) {
@@ -1855,13 +1892,13 @@ int pic_set_state(pic_t h, const int32_t *leaf, const void *x_or_o, const void *
   const size_t fs = h->split ? sizeof(float) : sizeof(double);
   const size_t m = (size_t)h->n * h->d;
   int rc;
+  if (h->split && where == PIC_DEVICE)
+    return bin_split_state(h, leaf, (const float *)x_or_o, (const float *)v, false);
   if ((rc = copy_in(h, h->pos[1], x_or_o, fs * m, where))) return rc;
   if ((rc = copy_in(h, h->vel[1], v, fs * m, where))) return rc;
   if (h->split) {
     if ((rc = copy_in(h, h->leaf[1], leaf, sizeof(int32_t) * h->n, where))) return rc;
-    launch_rekey32(h->dt, h->leaf[1], (const float *)h->pos[1], h->n, h->key[1], h->err, h->stream);
-    CK(cudaGetLastError());
-    return bin_fresh(h);
+    return bin_split_state(h, h->leaf[1], (const float *)h->pos[1], (const float *)h->vel[1], true);
   }
   launch_init64(h->dt, (double *)h->pos[1], h->n, h->leaf[1], h->key[1], h->err, h->stream);
   CK(cudaGetLastError());
@@ -2077,14 +2114,16 @@ int pic_retree(pic_t h, const pic_tree_desc *tree) {
   if (h->split) {
     launch_relocate32(old_dt, h->dt, h->leaf[0], (const float *)h->pos[0], (const float *)h->vel[0], n,
                       h->leaf[1], (float *)h->pos[1], (float *)h->vel[1], s);
-    launch_rekey32(h->dt, h->leaf[1], (const float *)h->pos[1], n, h->key[1], h->err, s);
+    CK(cudaGetLastError());
+    rc = bin_split_state(h, h->leaf[1], (const float *)h->pos[1], (const float *)h->vel[1], true);
   } else {
     std::swap(h->pos[0], h->pos[1]);  // FP64 positions do not change
     std::swap(h->vel[0], h->vel[1]);
     launch_init64(h->dt, (double *)h->pos[1], n, h->leaf[1], h->key[1], h->err, s);
+    CK(cudaGetLastError());
+    rc = bin_fresh(h);
   }
-  CK(cudaGetLastError());
-  if ((rc = bin_fresh(h))) {
+  if (rc) {
     free_bufs(h, old_tree);
     return rc;
   }
