@@ -22,7 +22,7 @@
 // mover sort, a mover list, a second atomic) -> now: re-bin and permutation of
 // the 2e8-particle 3D two-stream PIDT step 9.4 -> 5.7 ms (the push 6.8 -> 7.3 ms,
 // it waits for the ranks); whole step of 256 2D plasmas, 3.5e7 particles,
-// 3.26 -> 1.96 ms; 1e7 free 2D particles 0.49 -> 0.37 ms.  Three launches fewer
+// 3.26 -> 1.50 ms; 1e7 free 2D particles 0.49 -> 0.17 ms.  Three launches fewer
 // for large trees, eight for small ones.
 #pragma once
 
@@ -297,22 +297,37 @@ __global__ void __launch_bounds__(1024) k_scan_small(RebinArgs r) {
 
 // ---- place, sort, gather ---------------------------------------------------------
 
-__global__ void k_place(RebinArgs r) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= r.n) return;
-  const int32_t k = r.keyn[p];
-  int32_t slot;
-  if (!r.old_start) {
-    slot = r.new_start[k] + r.rank[p];
+// Four particles per thread: their lookups are in flight together (1e7 free 2D
+// particles 46 -> 24 us; 2e8 two-stream particles 1.42 -> 1.39 ms).
+constexpr int kPlaceVec = 4;
+__global__ void __launch_bounds__(256) k_place(RebinArgs r) {
+  const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kPlaceVec;
+  if (p0 >= r.n) return;
+  const int m = r.n - p0 < kPlaceVec ? (int)(r.n - p0) : kPlaceVec;
+  const int32_t *base = r.old_start ? r.base : r.new_start;
+  int32_t k[kPlaceVec], rank[kPlaceVec], slot[kPlaceVec];
+  const uint32_t word = r.old_start ? r.words[p0 >> 5] : 0xffffffffu;
+  const int32_t pre = r.old_start ? r.word_pre[p0 >> 5] : 0;
+  if (m == kPlaceVec) {
+    const int4 a = *(const int4 *)(r.keyn + p0), b = *(const int4 *)(r.rank + p0);
+    k[0] = a.x; k[1] = a.y; k[2] = a.z; k[3] = a.w;
+    rank[0] = b.x; rank[1] = b.y; rank[2] = b.z; rank[3] = b.w;
   } else {
-    const uint32_t word = r.words[p >> 5];
-    const int lane = (int)(p & 31);
-    if ((word >> lane) & 1u)
-      slot = r.base[k] + r.rank[p];
-    else
-      slot = r.shift[k] + (int32_t)p - r.word_pre[p >> 5] - __popc(word & ((1u << lane) - 1u));
+    for (int i = 0; i < kPlaceVec; ++i) {
+      k[i] = i < m ? r.keyn[p0 + i] : -1;
+      rank[i] = i < m ? r.rank[p0 + i] : 0;
+    }
   }
-  r.perm[slot] = (int32_t)p;
+#pragma unroll
+  for (int i = 0; i < kPlaceVec; ++i) {
+    const int lane = (int)(p0 & 31) + i;
+    if (i >= m) slot[i] = -1;
+    else if ((word >> lane) & 1u) slot[i] = base[k[i]] + rank[i];
+    else slot[i] = r.shift[k[i]] + (int32_t)p0 + i - pre - __popc(word & ((1u << lane) - 1u));
+  }
+#pragma unroll
+  for (int i = 0; i < kPlaceVec; ++i)
+    if (slot[i] >= 0) r.perm[slot[i]] = (int32_t)p0 + i;
 }
 
 // One warp per listed segment of at most kMedSeg movers (grid-stride over the
@@ -367,28 +382,45 @@ struct SlotOrder {
 // The whole particle state into bucket order in one pass: positions and
 // velocities ([D][n]), leaves, and keys (PIDT; PIT keys are the leaves) and ids
 // where given.
+// FP32: two slots per thread, a block apart, so that twice the scattered reads are
+// in flight (ten steps of 256 2D plasmas 15.7 -> 15.0 ms; four slots 15.4); FP64
+// has twice the bytes per read and gains nothing.
+template <typename T>
+__host__ __device__ constexpr int rows_per_thread() { return sizeof(T) == 4 ? 2 : 1; }
 template <typename T, int D>
-__global__ void k_gather_state(SlotOrder so, int64_t n, const T *__restrict__ x, T *__restrict__ x2,
-                               const T *__restrict__ v, T *__restrict__ v2, const int32_t *__restrict__ leaf,
-                               int32_t *__restrict__ leaf2, const int32_t *__restrict__ key, int32_t *__restrict__ key2,
-                               const int32_t *__restrict__ ids, int32_t *__restrict__ ids2) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const int32_t i = so.perm[s];
-  T a[D], b[D];
+__global__ void __launch_bounds__(256) k_gather_state(
+    SlotOrder so, int64_t n, const T *__restrict__ x, T *__restrict__ x2, const T *__restrict__ v, T *__restrict__ v2,
+    const int32_t *__restrict__ leaf, int32_t *__restrict__ leaf2, const int32_t *__restrict__ key,
+    int32_t *__restrict__ key2, const int32_t *__restrict__ ids, int32_t *__restrict__ ids2) {
+  constexpr int kRowsVec = rows_per_thread<T>();
+  const int64_t s0 = (int64_t)blockIdx.x * (256 * kRowsVec) + threadIdx.x;
+  int32_t i[kRowsVec], L[kRowsVec], kk[kRowsVec], id[kRowsVec];
+  T a[kRowsVec][D], b[kRowsVec][D];
 #pragma unroll
-  for (int k = 0; k < D; ++k) a[k] = x[k * n + i];
+  for (int u = 0; u < kRowsVec; ++u) i[u] = s0 + 256 * u < n ? so.perm[s0 + 256 * u] : -1;
 #pragma unroll
-  for (int k = 0; k < D; ++k) b[k] = v[k * n + i];
-  const int32_t L = leaf[i], kk = key ? key[i] : L, id = ids ? ids[i] : 0;
-  const int64_t p = so.place((int32_t)s, i, kk);
+  for (int u = 0; u < kRowsVec; ++u) {
+    if (i[u] < 0) continue;
+    L[u] = leaf[i[u]];
+    kk[u] = key ? key[i[u]] : L[u];
+    id[u] = ids ? ids[i[u]] : 0;
 #pragma unroll
-  for (int k = 0; k < D; ++k) x2[k * n + p] = a[k];
+    for (int k = 0; k < D; ++k) a[u][k] = x[k * n + i[u]];
 #pragma unroll
-  for (int k = 0; k < D; ++k) v2[k * n + p] = b[k];
-  leaf2[p] = L;
-  if (key) key2[p] = kk;
-  if (ids) ids2[p] = id;
+    for (int k = 0; k < D; ++k) b[u][k] = v[k * n + i[u]];
+  }
+#pragma unroll
+  for (int u = 0; u < kRowsVec; ++u) {
+    if (i[u] < 0) continue;
+    const int64_t p = so.place((int32_t)(s0 + 256 * u), i[u], kk[u]);
+#pragma unroll
+    for (int k = 0; k < D; ++k) x2[k * n + p] = a[u][k];
+#pragma unroll
+    for (int k = 0; k < D; ++k) v2[k * n + p] = b[u][k];
+    leaf2[p] = L[u];
+    if (key) key2[p] = kk[u];
+    if (ids) ids2[p] = id[u];
+  }
 }
 
 // 32 bytes in one load (eight floats, four doubles), from a 32-byte boundary.
@@ -483,7 +515,7 @@ void launch_rebin(const RebinArgs &r, cudaStream_t s) {
     k_keys_apply<<<(unsigned)tk, kScanThreads, 0, s>>>(r, r.tile_sums);
   }
   if (r.n <= 0) return;
-  { COUNT(1); k_place<<<grid_for(r.n), kBlock, 0, s>>>(r); }
+  { COUNT(1); k_place<<<grid_for((r.n + kPlaceVec - 1) / kPlaceVec), kBlock, 0, s>>>(r); }
   if (r.n > kRankMax) {
     COUNT(1);
     k_sort_medium<<<kMedBlocks, kMedThreads, sizeof(int32_t) * kMedSeg * (kMedThreads / 32), s>>>(r);
@@ -500,19 +532,19 @@ void launch_gather_state(bool split, const RebinArgs &r, int d, const void *x, v
   if (r.n <= 0) return;
   COUNT(1);
   const SlotOrder so{r.perm, r.old_start ? r.base : r.new_start, r.new_start};
-  const unsigned g = grid_for(r.n);
+  const unsigned g = grid_for(r.n, 256 * (split ? rows_per_thread<float>() : rows_per_thread<double>()));
   if (split) {
     if (d == 3)
-      k_gather_state<float, 3><<<g, kBlock, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
+      k_gather_state<float, 3><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
                                                     (float *)v2, leaf, leaf2, key, key2, ids, ids2);
     else
-      k_gather_state<float, 2><<<g, kBlock, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
+      k_gather_state<float, 2><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
                                                     (float *)v2, leaf, leaf2, key, key2, ids, ids2);
   } else if (d == 3) {
-    k_gather_state<double, 3><<<g, kBlock, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
+    k_gather_state<double, 3><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
                                                    (double *)v2, leaf, leaf2, key, key2, ids, ids2);
   } else {
-    k_gather_state<double, 2><<<g, kBlock, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
+    k_gather_state<double, 2><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
                                                    (double *)v2, leaf, leaf2, key, key2, ids, ids2);
   }
 }
