@@ -23,7 +23,8 @@ struct InstInfo {
   int32_t leaf_off, vert_off, key_off, spread_off, tab_root, n_vert;
   int64_t poff;                // first particle of the instance in input order
   double q, ion, ion_load, diag;
-  double h, rdiag;             // uniform trees: leaf width 3^-depth, 1 / diag
+  double h;                    // uniform trees: leaf width 3^-depth
+  double jac[3];               // FP64 sweep: 1 - omega, -omega / diag times the face and edge / corner entries
   float q32, ion32, ion_load32, diag32, h32;
   float rdiag32, rdiag_lo32;   // 1 / diag32 in two floats
 };

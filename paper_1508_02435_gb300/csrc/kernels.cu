@@ -753,7 +753,8 @@ static void solve(const DevTree &t, const RowMatrix &A, const T *Q, const double
   }
   // the FP64 two-pass solve of an adaptive tree leaves Vtmp free: it holds omega / diag
   T *scale = sizeof(T) == 8 && !t.uniform && !A.val ? Vtmp : nullptr;
-  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale, A.val != nullptr); }
+  const bool scaled = sizeof(T) == 8 && !scale;  // the other FP64 sweeps take b times omega / diag
+  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale, scaled); }
   int64_t nb;
   if constexpr (sizeof(T) == 8) {
     if (A.val) {

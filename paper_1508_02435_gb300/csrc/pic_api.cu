@@ -367,7 +367,15 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
     I.ion_load = ht.uniform ? ht.ion_load[0] : 0.0;
     I.diag = ht.uniform ? ht.diag[0] : 0.0;
     I.h = 1.0 / (double)ht.M;
-    I.rdiag = ht.uniform ? 1.0 / I.diag : 0.0;
+    if (ht.uniform) {
+      // FP64 sweep V' = jac0 V + b omega / diag + jac1 (face neighbours) + jac2 (2 edge + corner
+      // neighbours): matrix entries 8/3 h^(d-2) on the diagonal, in 2D -1/3 (faces) and -1/3
+      // (corners), in 3D -1/12 h per shared leaf
+      const double w = h->cfg.omega / I.diag, hs = d == 3 ? I.h : 1.0;
+      I.jac[0] = 1.0 - h->cfg.omega;
+      I.jac[1] = w * (1.0 / 3.0);
+      I.jac[2] = d == 3 ? w * (hs / 12.0) : w * (1.0 / 3.0);
+    }
     I.h32 = (float)I.h;
     I.q32 = (float)I.q;
     I.ion32 = (float)I.ion;
@@ -683,7 +691,7 @@ int alloc_grid(pic_t h) {
   if ((rc = galloc(h, sb, &h->count, nk))) return rc;
   if ((rc = galloc(h, sb, &h->base, nk))) return rc;
   if ((rc = galloc(h, sb, &h->shift, nk))) return rc;
-  if ((rc = galloc(h, sb, &h->tile_sums, scan_tiles_needed(nk) + 1))) return rc;
+  if ((rc = galloc(h, sb, &h->tile_sums, scan_tiles_needed(nk) + 512))) return rc;  // 489 quarter tiles below 1e6 keys
   char *p;
   if ((rc = galloc(h, sb, &p, fs * nl * h->dt.nc))) return rc;
   h->part = p;

@@ -53,7 +53,7 @@ __device__ __forceinline__ void peer_store(uint32_t a, int v) {
 // nine columns (3D) or three (2D) around it, row: its slab row (2D).
 template <int M>
 __device__ __forceinline__ float resident_row3(const float *s, const int *col, int i, float v, const StencilC<float> &c,
-                                               const int32_t *w, const bool *flip, bool bad) {
+                                               const int32_t *w, const bool *flip, bool bad, float) {
   constexpr int PL = M * M;
   float p[27];
 #pragma unroll
@@ -72,19 +72,19 @@ __device__ __forceinline__ float resident_row3(const float *s, const int *col, i
 
 template <int M>
 __device__ __forceinline__ double resident_row3(const double *s, const int *col, int i, double v,
-                                                const StencilC<double> &c, const int32_t *, const bool *, bool bad) {
+                                                const StencilC<double> &c, const int32_t *, const bool *, bool bad, double b) {
   constexpr int PL = M * M;
   auto at = [&](int k, int dz) { return s[(i + 1 + dz) * PL + col[k]]; };
   auto diag = [&](int dz) { return (at(0, dz) + at(2, dz)) + (at(6, dz) + at(8, dz)); };
   auto cross = [&](int dz) { return (at(3, dz) + at(5, dz)) + (at(1, dz) + at(7, dz)); };
-  double y = stencil_row3(v, diag(0) + (cross(-1) + cross(1)), diag(-1) + diag(1), c);
+  double y = sweep3(v, diag(0) + (cross(-1) + cross(1)), diag(-1) + diag(1), c, b);
   if (bad) y = y + (0.0 * at(1, 0) + 0.0 * at(7, 0)) + (0.0 * at(3, 0) + 0.0 * at(5, 0)) + (0.0 * at(4, -1) + 0.0 * at(4, 1));
   return y;
 }
 
 template <int M>
 __device__ __forceinline__ float resident_row2(const float *s, const int *col, int row, float v, const StencilC<float> &c,
-                                               const int32_t *w, const bool *flip) {
+                                               const int32_t *w, const bool *flip, float) {
   float p[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -97,10 +97,10 @@ __device__ __forceinline__ float resident_row2(const float *s, const int *col, i
 
 template <int M>
 __device__ __forceinline__ double resident_row2(const double *s, const int *col, int row, double v,
-                                                const StencilC<double> &c, const int32_t *, const bool *) {
+                                                const StencilC<double> &c, const int32_t *, const bool *, double b) {
   auto at = [&](int k, int dy) { return s[(row + 1 + dy) * M + col[k]]; };
-  return stencil_row2(v, (at(0, 0) + at(2, 0)) + (at(1, -1) + at(1, 1)),
-                      (at(0, -1) + at(2, -1)) + (at(0, 1) + at(2, 1)), c);
+  return sweep2(v, (at(0, 0) + at(2, 0)) + (at(1, -1) + at(1, 1)), (at(0, -1) + at(2, -1)) + (at(0, 1) + at(2, 1)), c,
+                b);
 }
 
 __device__ __forceinline__ bool not_finite(float x) { return !(fabsf(x) < __int_as_float(0x7f800000)); }
@@ -115,7 +115,8 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
   __shared__ T buf[2][R::kBuf];
   __shared__ int bad;  // some V is not finite: the zero terms of the 3D face neighbours count
   const InstInfo &I = t.inst[0];
-  const StencilC<T> c = stencil_consts<T, D>(I, omega);
+  StencilC<T> c;
+  stencil_consts<D>(I, omega, true, &c);
   const int rank = (int)cluster_rank(), z0 = rank * R::kSlab, tid = threadIdx.x;
   const bool act = tid < R::kWork;
   const int row = D == 3 ? 0 : tid / M;
@@ -142,6 +143,10 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
   const uint32_t lo_buf = peer_addr(&buf[0][0], lo_peer), hi_buf = peer_addr(&buf[0][0], hi_peer);
   const T tot = (T)*total;
   T v[N], b[N];
+  auto stored = [&](T u) {  // what shared memory holds of a value
+    if constexpr (R::kScaled) return c.c2 * u;
+    else return u;
+  };
   if (tid == 0) bad = 0;
   __syncthreads();
   bool odd = false;
@@ -149,19 +154,20 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
     const int z = (z0 + k / PL - 1 + M) % M;
     const T u = V[z * PL + k % PL];
     odd |= not_finite(u);
-    buf[0][k] = R::kScaled ? c.c2 * u : u;
+    buf[0][k] = stored(u);
   }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     const int at = act ? (z0 + (D == 3 ? i : row)) * PL + own : 0;
     v[i] = V[at];
     b[i] = Q[at] - tot * ion_load(t, 0, (T)0);
+    if constexpr (sizeof(T) == 8) b[i] = b[i] * (omega / I.diag);
   }
   auto apply = [&](const T *s, int i, bool any) {
     if (sizeof(T) == 4) w[D - 1] = wl[i];
     flip[D - 1] = z0 + (D == 3 ? i : row) == 0;
-    if constexpr (D == 3) return resident_row3<M>(s, col, i, v[i], c, w, flip, any);
-    else return resident_row2<M>(s, col, row, v[i], c, w, flip);
+    if constexpr (D == 3) return resident_row3<M>(s, col, i, v[i], c, w, flip, any, b[i]);
+    else return resident_row2<M>(s, col, row, v[i], c, w, flip, b[i]);
   };
   auto report = [&](bool found) {  // to every CTA, seen after the next meeting
     if (D == 3 && found)
@@ -186,7 +192,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
       for (int i = 0; i < N; ++i) {
         v[i] = out[i];
         odd |= not_finite(out[i]);
-        const T u = R::kScaled ? c.c2 * out[i] : out[i];
+        const T u = stored(out[i]);
         const int r = D == 3 ? i : row;
         buf[nb][(r + 1) * PL + own] = u;
         // the outer rows also to the neighbours' halos
@@ -203,7 +209,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const T yv = apply(buf[sweeps & 1], i, any);
-      rr = rr + residual2<1>(&yv, &b[i]);
+      rr = rr + residual2<1>(&yv, &b[i], &v[i], c);
       V[(z0 + (D == 3 ? i : row)) * PL + own] = v[i];
     }
   }

@@ -37,29 +37,36 @@ __host__ __device__ constexpr int pop3(int x) { return (x & 1) + ((x >> 1) & 1) 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Constants of one uniform instance: c0, c1, c2 = kref(0, 1, 2 axes differ) h^(d-2).
+// Constants of one uniform instance.  FP32: c0, c1, c2 = kref(0, 1, 2 axes differ)
+// h^(d-2), the diagonal, and 1 / diagonal in two floats.  FP64: the sweep's weights.
 template <typename T>
-struct StencilC {
-  T c0, c1, c2, omega, diag, rhi, rlo;  // FP64: rhi = omega / A_vv; FP32: 1 / diag in two parts
+struct StencilC;
+template <>
+struct StencilC<float> {
+  float c0, c1, c2, omega, diag, rhi, rlo;
+};
+template <>
+struct StencilC<double> {
+  double k0, k1, k2, inv;  // inv = diag / omega (residual only)
 };
 
-__device__ __forceinline__ double inst_h(const InstInfo &I, double) { return I.h; }
-__device__ __forceinline__ float inst_h(const InstInfo &I, float) { return I.h32; }
-__device__ __forceinline__ double inst_diag(const InstInfo &I, double) { return I.diag; }
-__device__ __forceinline__ float inst_diag(const InstInfo &I, float) { return I.diag32; }
-
-template <typename T, int D>
-__device__ __forceinline__ StencilC<T> stencil_consts(const InstInfo &I, T omega) {
-  StencilC<T> s;
-  const T hs = D == 2 ? (T)1 : inst_h(I, (T)0);
-  s.c0 = kref_val(0, 0, (T)0) * hs;
-  s.c1 = kref_val(0, 1, (T)0) * hs;
-  s.c2 = kref_val(0, 3, (T)0) * hs;
-  s.omega = omega;
-  s.diag = inst_diag(I, (T)0);
-  s.rhi = sizeof(T) == 8 ? (T)(omega * I.rdiag) : (T)I.rdiag32;
-  s.rlo = (T)I.rdiag_lo32;
-  return s;
+template <int D>
+__device__ __forceinline__ void stencil_consts(const InstInfo &I, float omega, bool, StencilC<float> *s) {
+  const float hs = D == 2 ? 1.0f : I.h32;
+  s->c0 = c_kref32[0][0] * hs;
+  s->c1 = c_kref32[0][1] * hs;
+  s->c2 = c_kref32[0][3] * hs;
+  s->omega = omega;
+  s->diag = I.diag32;
+  s->rhi = I.rdiag32;
+  s->rlo = I.rdiag_lo32;
+}
+template <int D>
+__device__ __forceinline__ void stencil_consts(const InstInfo &I, double omega, bool res, StencilC<double> *s) {
+  s->k0 = I.jac[0];
+  s->k1 = I.jac[1];
+  s->k2 = I.jac[2];
+  s->inv = res ? I.diag / omega : 0.0;
 }
 
 // |spread(j) - spread(j - 1)| on one axis (0 on a one-cell axis).
@@ -157,13 +164,14 @@ __device__ __forceinline__ float face_terms(Q q) {
 
 __device__ __forceinline__ uint32_t high_word(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// FP64 (A V): an edge neighbour shares two leaves with the vertex, a corner
-// neighbour one, the centre eight (2D: a face neighbour two, the centre four).
-__device__ __forceinline__ double stencil_row3(double c, double edges, double corners, const StencilC<double> &s) {
-  return fma(s.c2, fma(2.0, edges, corners), (8.0 * s.c0) * c);
+// FP64, one sweep at a vertex with b times omega / diag: an edge neighbour shares
+// two leaves with the vertex, a corner neighbour one (2D: a face neighbour two, of
+// half the entry).  Three fused operations beside the neighbour sums.
+__device__ __forceinline__ double sweep3(double c, double edges, double corners, const StencilC<double> &s, double b) {
+  return fma(s.k2, fma(2.0, edges, corners), fma(s.k0, c, b));
 }
-__device__ __forceinline__ double stencil_row2(double c, double faces, double corners, const StencilC<double> &s) {
-  return fma(s.c2, corners, fma(2.0 * s.c1, faces, (4.0 * s.c0) * c));
+__device__ __forceinline__ double sweep2(double c, double faces, double corners, const StencilC<double> &s, double b) {
+  return fma(s.k2, corners, fma(s.k1, faces, fma(s.k0, c, b)));
 }
 
 // V + omega r / diag.  The FP32 quotient by the instance's constant diagonal
@@ -193,20 +201,32 @@ __device__ __forceinline__ void jacobi_update(const float *y, const float *b, co
   }
 }
 
+// FP64 rows give the new value itself.
 template <int N>
-__device__ __forceinline__ void jacobi_update(const double *y, const double *b, const double *vc,
-                                              const StencilC<double> &s, double *out) {
+__device__ __forceinline__ void jacobi_update(const double *y, const double *, const double *, const StencilC<double> &,
+                                              double *out) {
 #pragma unroll
-  for (int j = 0; j < N; ++j) out[j] = fma(s.rhi, b[j] - y[j], vc[j]);
+  for (int j = 0; j < N; ++j) out[j] = y[j];
 }
 
 // Squared residuals of N vertices, in order.
-template <int N, typename T>
-__device__ __forceinline__ double residual2(const T *y, const T *b) {
+template <int N>
+__device__ __forceinline__ double residual2(const float *y, const float *b, const float *, const StencilC<float> &) {
   double rr = 0.0;
 #pragma unroll
   for (int j = 0; j < N; ++j) {
     const double r = (double)(b[j] - y[j]);
+    rr = rr + r * r;
+  }
+  return rr;
+}
+template <int N>
+__device__ __forceinline__ double residual2(const double *y, const double *, const double *vc,
+                                            const StencilC<double> &s) {
+  double rr = 0.0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const double r = (y[j] - vc[j]) * s.inv;  // omega / diag times the residual is the step
     rr = rr + r * r;
   }
   return rr;
@@ -217,7 +237,7 @@ __device__ __forceinline__ double residual2(const T *y, const T *b) {
 // A V at vertex j of an instance (base: its first vertex), and V there.
 template <int D>
 __device__ __forceinline__ float apply_at(const float *base, int32_t M, const int32_t *j,
-                                          const int32_t *sp, const StencilC<float> &s, float *vc) {
+                                          const int32_t *sp, const StencilC<float> &s, float, float *vc) {
   int32_t o[3][3], w[3] = {0, 0, 0}, stride = 1;
   bool flip[3];
 #pragma unroll
@@ -248,7 +268,7 @@ __device__ __forceinline__ float apply_at(const float *base, int32_t M, const in
 
 template <int D>
 __device__ __forceinline__ double apply_at(const double *base, int32_t M, const int32_t *j,
-                                           const int32_t *, const StencilC<double> &s, double *vc) {
+                                           const int32_t *, const StencilC<double> &s, double b, double *vc) {
   int32_t o[3][3], stride = 1;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
@@ -262,12 +282,12 @@ __device__ __forceinline__ double apply_at(const double *base, int32_t M, const 
   };
   *vc = at(0, 0, 0);
   if (D == 2)
-    return stencil_row2(*vc, (at(-1, 0, 0) + at(1, 0, 0)) + (at(0, -1, 0) + at(0, 1, 0)),
-                        (at(-1, -1, 0) + at(1, -1, 0)) + (at(-1, 1, 0) + at(1, 1, 0)), s);
+    return sweep2(*vc, (at(-1, 0, 0) + at(1, 0, 0)) + (at(0, -1, 0) + at(0, 1, 0)),
+                  (at(-1, -1, 0) + at(1, -1, 0)) + (at(-1, 1, 0) + at(1, 1, 0)), s, b);
   auto diag = [&](int dz) { return (at(-1, -1, dz) + at(1, -1, dz)) + (at(-1, 1, dz) + at(1, 1, dz)); };
   const double f[6] = {at(-1, 0, 0), at(1, 0, 0), at(0, -1, 0), at(0, 1, 0), at(0, 0, -1), at(0, 0, 1)};
   auto cross = [&](int dz) { return (at(-1, 0, dz) + at(1, 0, dz)) + (at(0, -1, dz) + at(0, 1, dz)); };
-  double y = stencil_row3(*vc, diag(0) + (cross(-1) + cross(1)), diag(-1) + diag(1), s);
+  double y = sweep3(*vc, diag(0) + (cross(-1) + cross(1)), diag(-1) + diag(1), s, b);
   uint32_t top = 0u;
 #pragma unroll
   for (int k = 0; k < 6; ++k) top = max(top, high_word(f[k]));
@@ -300,7 +320,8 @@ __global__ void __launch_bounds__(128) k_jacobi_vertex(DevTree t, const T *b, co
   double rr = 0.0;
   const InstInfo &I = inst_of_vertex(t, act ? v : 0);
   const int32_t M = I.M;
-  const StencilC<T> s = stencil_consts<T, D>(I, omega);
+  StencilC<T> s;
+  stencil_consts<D>(I, omega, kRes, &s);
   int32_t j[3] = {0, 0, 0}, r = act ? (int32_t)(v - I.vert_off) : 0;
 #pragma unroll
   for (int a = 0; a < D; ++a) {
@@ -313,8 +334,8 @@ __global__ void __launch_bounds__(128) k_jacobi_vertex(DevTree t, const T *b, co
   if (act) {
     const T bv = b[v];
     T vc;
-    const T y = apply_at<D>(Vin + I.vert_off, M, j, t.spread + I.spread_off, s, &vc);
-    if (kRes) rr = residual2<1>(&y, &bv);
+    const T y = apply_at<D>(Vin + I.vert_off, M, j, t.spread + I.spread_off, s, bv, &vc);
+    if (kRes) rr = residual2<1>(&y, &bv, &vc, s);
     else jacobi_update<1>(&y, &bv, &vc, s, Vout + v);
   }
   if (kRes) block_sum_store_at(rr, r2 + blockIdx.x);
@@ -364,7 +385,8 @@ struct Slab3<double> {
 // (A V) of the three rows at the middle plane.  kLow: z is no multiple of 3.
 template <bool kLow>
 __device__ __forceinline__ void strip_rows(const Slab3<float> &lo, const Slab3<float> &mid, const Slab3<float> &hi,
-                                           const StencilC<float> &s, const int32_t *w, const bool *flip, float *y) {
+                                           const StencilC<float> &s, const int32_t *w, const bool *flip, const float *,
+                                           float *y) {
   auto at = [&](int j, int dx, int dy, int dz) {
     return (dz < 0 ? lo : dz > 0 ? hi : mid).q[(j + 1 + dy) * 3 + dx + 1];
   };
@@ -396,10 +418,11 @@ __device__ __forceinline__ void strip_rows(const Slab3<float> &lo, const Slab3<f
 
 template <bool kLow>
 __device__ __forceinline__ void strip_rows(const Slab3<double> &lo, const Slab3<double> &mid, const Slab3<double> &hi,
-                                           const StencilC<double> &s, const int32_t *, const bool *, double *y) {
+                                           const StencilC<double> &s, const int32_t *, const bool *, const double *b,
+                                           double *y) {
 #pragma unroll
   for (int j = 0; j < 3; ++j)
-    y[j] = stencil_row3(mid.c[j], mid.diag[j] + (lo.cross[j] + hi.cross[j]), lo.diag[j] + hi.diag[j], s);
+    y[j] = sweep3(mid.c[j], mid.diag[j] + (lo.cross[j] + hi.cross[j]), lo.diag[j] + hi.diag[j], s, b[j]);
   if (max(mid.top, max(lo.top, hi.top)) >= 0x7ff00000u) {
 #pragma unroll
     for (int j = 0; j < 3; ++j) y[j] = y[j] + (0.0 * mid.cross[j] + 0.0 * (lo.c[j] + hi.c[j]));
@@ -420,7 +443,8 @@ __global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, co
                                                        T *__restrict__ Vout, T omega, double *r2, int len) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M, plane = M * M;
-  const StencilC<T> s = stencil_consts<T, 3>(I, omega);
+  StencilC<T> s;
+  stencil_consts<3>(I, omega, kRes, &s);
   const int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x), k = i / M, x = i - k * M;
   const bool act = 3 * k < M;
   const int32_t y0 = act ? 3 * k : 0;
@@ -455,12 +479,12 @@ __global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, co
       if (!low) {
         flip[2] = z == 0;
         if (sizeof(T) == 4) w[2] = step_weight(t.spread + 2 * M, M, z);
-        strip_rows<false>(lo, mid, hi, s, w, flip, y);
+        strip_rows<false>(lo, mid, hi, s, w, flip, bv, y);
       } else {
-        strip_rows<true>(lo, mid, hi, s, w, flip, y);
+        strip_rows<true>(lo, mid, hi, s, w, flip, bv, y);
       }
       if (kRes) {
-        rr = rr + residual2<3>(y, bv);
+        rr = rr + residual2<3>(y, bv, mid.c, s);
       } else {
         T out[3];
         jacobi_update<3>(y, bv, mid.c, s, out);
@@ -480,7 +504,7 @@ __global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, co
 }
 
 __device__ __forceinline__ void strip_rows2(const float *v, const StencilC<float> &s, const int32_t *w,
-                                            const bool *flip, float *y) {
+                                            const bool *flip, const float *, float *y) {
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
     auto q = [&](int dx, int dy, int) {
@@ -492,13 +516,13 @@ __device__ __forceinline__ void strip_rows2(const float *v, const StencilC<float
 }
 
 __device__ __forceinline__ void strip_rows2(const double *v, const StencilC<double> &s, const int32_t *, const bool *,
-                                            double *y) {
+                                            const double *b, double *y) {
   double a[5];
 #pragma unroll
   for (int r = 0; r < 5; ++r) a[r] = v[r * 3] + v[r * 3 + 2];
 #pragma unroll
   for (int j = 0; j < 3; ++j)
-    y[j] = stencil_row2(v[(j + 1) * 3 + 1], a[j + 1] + (v[j * 3 + 1] + v[(j + 2) * 3 + 1]), a[j] + a[j + 2], s);
+    y[j] = sweep2(v[(j + 1) * 3 + 1], a[j + 1] + (v[j * 3 + 1] + v[(j + 2) * 3 + 1]), a[j] + a[j + 2], s, b[j]);
 }
 
 template <typename T, bool kRes>
@@ -506,7 +530,8 @@ __global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, co
                                                        T *__restrict__ Vout, T omega, double *r2) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M;
-  const StencilC<T> s = stencil_consts<T, 2>(I, omega);
+  StencilC<T> s;
+  stencil_consts<2>(I, omega, kRes, &s);
   const int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x), k = i / M, x = i - k * M;
   const bool act = 3 * k < M;
   const int32_t y0 = act ? 3 * k : 0;
@@ -527,11 +552,11 @@ __global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, co
 #pragma unroll
     for (int j = 0; j < 3; ++j) bv[j] = b[row[j + 1] + x];
     strip_load(Vin, row, col, v);
-    strip_rows2(v, s, w, flip, y);
+    strip_rows2(v, s, w, flip, bv, y);
+    const T vc[3] = {v[4], v[7], v[10]};
     if (kRes) {
-      rr = residual2<3>(y, bv);
+      rr = residual2<3>(y, bv, vc, s);
     } else {
-      const T vc[3] = {v[4], v[7], v[10]};
       T out[3];
       jacobi_update<3>(y, bv, vc, s, out);
 #pragma unroll
