@@ -7,8 +7,8 @@
 // neighbours' halos as it updates them, and meets the others at a cluster
 // barrier after every sweep.  The sums are those of uniform_solve.cuh.
 //
-// 100 sweeps of 27^2 cells, FP64: 188 us as launches, 88 us here; 81^2 FP32 190 ->
-// R81 us.
+// 100 sweeps of 27^2 cells, FP64: 188 us as launches, 88 us here; 81^2 FP32 188 ->
+// 75 us.
 #pragma once
 
 namespace pic {

@@ -19,10 +19,10 @@
 // FP64 sums the stencil by neighbour class: fewer operations (the FP64 pipe
 // bounds these kernels), hence fewer roundings.
 //
-// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 82 us (172 MB of
-// V, b and V' take 25 us; bound by latency and issue, 138 warp instructions per
-// 32 vertices), 81^3 FP32 149 -> 5.9 us and FP64 277 -> 23.5 us, 27^3 FP32
-// 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us (both the rate of dependent launches).
+// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 70 us (172 MB of
+// V, b and V' take 25 us; bound by latency and issue), 81^3 FP32 149 -> 5.6 us
+// and FP64 277 -> 20.8 us, 27^3 FP32 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us
+// (both the rate of dependent launches).
 #pragma once
 
 namespace pic {
@@ -385,8 +385,7 @@ struct Slab3<double> {
 // (A V) of the three rows at the middle plane.  kLow: z is no multiple of 3.
 template <bool kLow>
 __device__ __forceinline__ void strip_rows(const Slab3<float> &lo, const Slab3<float> &mid, const Slab3<float> &hi,
-                                           const StencilC<float> &s, const int32_t *w, const bool *flip, const float *,
-                                           float *y) {
+                                           const StencilC<float> &s, const int32_t *w, const bool *flip, float *y) {
   auto at = [&](int j, int dx, int dy, int dz) {
     return (dz < 0 ? lo : dz > 0 ? hi : mid).q[(j + 1 + dy) * 3 + dx + 1];
   };
@@ -416,10 +415,8 @@ __device__ __forceinline__ void strip_rows(const Slab3<float> &lo, const Slab3<f
   }
 }
 
-template <bool kLow>
 __device__ __forceinline__ void strip_rows(const Slab3<double> &lo, const Slab3<double> &mid, const Slab3<double> &hi,
-                                           const StencilC<double> &s, const int32_t *, const bool *, const double *b,
-                                           double *y) {
+                                           const StencilC<double> &s, const double *b, double *y) {
 #pragma unroll
   for (int j = 0; j < 3; ++j)
     y[j] = sweep3(mid.c[j], mid.diag[j] + (lo.cross[j] + hi.cross[j]), lo.diag[j] + hi.diag[j], s, b[j]);
@@ -438,12 +435,14 @@ __device__ __forceinline__ void strip_load(const T *p, const int32_t *row, const
     for (int i = 0; i < 3; ++i) v[r * 3 + i] = p[row[r] + col[i]];
 }
 
-template <typename T, bool kRes>
-__global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, const T *Vin,
-                                                       T *__restrict__ Vout, T omega, double *r2, int len) {
+// FP64, straight from global memory: the FP64 pipe is the bound, and warps that
+// need no barrier keep it busy.
+template <bool kRes>
+__global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const double *b, const double *Vin,
+                                                       double *__restrict__ Vout, double omega, double *r2, int len) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M, plane = M * M;
-  StencilC<T> s;
+  StencilC<double> s;
   stencil_consts<3>(I, omega, kRes, &s);
   const int32_t i = (int32_t)(blockIdx.x * blockDim.x + threadIdx.x), k = i / M, x = i - k * M;
   const bool act = 3 * k < M;
@@ -451,54 +450,160 @@ __global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const T *b, co
   const int32_t col[3] = {x == 0 ? M - 1 : x - 1, x, x + 1 == M ? 0 : x + 1};
   const int32_t row[5] = {(y0 == 0 ? M - 1 : y0 - 1) * M, y0 * M, (y0 + 1) * M, (y0 + 2) * M,
                           (y0 + 3 == M ? 0 : y0 + 3) * M};
-  int32_t w[3] = {0, 0, 0};
-  bool flip[3] = {x == 0, y0 == 0, false};
-  if (sizeof(T) == 4) {
-    w[0] = step_weight(t.spread, M, x);
-    w[1] = step_weight(t.spread + M, M, y0);
-  }
   double rr = 0.0;
   pdl_wait();
   pdl_release();
   if (act) {
     const int32_t z0 = (int32_t)blockIdx.y * len;
-    Slab3<T> p0, p1, p2;
-    auto load = [&](int32_t z, Slab3<T> &p) {
-      T v[15];
+    Slab3<double> p0, p1, p2;
+    auto load = [&](int32_t z, Slab3<double> &p) {
+      double v[15];
       strip_load(Vin + (int64_t)z * plane, row, col, v);
       p.set(v, s);
     };
-    auto put = [&](int32_t z, bool low, const Slab3<T> &lo, const Slab3<T> &mid, Slab3<T> &hi) {
-      T bv[3], y[3];
+    auto put = [&](int32_t z, const Slab3<double> &lo, const Slab3<double> &mid, Slab3<double> &hi) {
+      double bv[3], y[3];
       const int64_t at = (int64_t)z * plane + x;
 #pragma unroll
       for (int j = 0; j < 3; ++j) bv[j] = b[at + row[j + 1]];
       load(z + 1 == M ? 0 : z + 1, hi);
-      flip[2] = false;
-      w[2] = 9;
-      if (!low) {
-        flip[2] = z == 0;
-        if (sizeof(T) == 4) w[2] = step_weight(t.spread + 2 * M, M, z);
-        strip_rows<false>(lo, mid, hi, s, w, flip, bv, y);
-      } else {
-        strip_rows<true>(lo, mid, hi, s, w, flip, bv, y);
-      }
+      strip_rows(lo, mid, hi, s, bv, y);
       if (kRes) {
         rr = rr + residual2<3>(y, bv, mid.c, s);
       } else {
-        T out[3];
-        jacobi_update<3>(y, bv, mid.c, s, out);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) Vout[at + row[j + 1]] = out[j];
+        for (int j = 0; j < 3; ++j) Vout[at + row[j + 1]] = y[j];
       }
     };
     load(z0 == 0 ? M - 1 : z0 - 1, p0);
     load(z0, p1);
     for (int32_t z = z0; z < z0 + len; z += 3) {  // the three slabs take turns
-      put(z, false, p0, p1, p2);
-      put(z + 1, true, p1, p2, p0);
-      put(z + 2, true, p2, p0, p1);
+      put(z, p0, p1, p2);
+      put(z + 1, p1, p2, p0);
+      put(z + 2, p2, p0, p1);
     }
+  }
+  if (kRes) block_sum_store_at(rr, r2 + (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// FP32: the planes are staged in shared memory by asynchronous copies, three at a
+// time and three ahead, by blocks of 32 columns x 27 rows (nine strips); a thread
+// reads its neighbourhood at fixed distances from one address.  One barrier for
+// three planes, and a thread's nine b of them loaded ahead of it: with a barrier a
+// plane the wait for the slowest warp took what the staging gave (243^3 80 us).
+// Strips from global memory 82 us, this 70 (81^3: 5.9, 5.6).  Three blocks an SM
+// leave too few registers (75 us, 81^3 8.2); 9 planes a block are the best march at
+// 243^3 (27: 77 us, 81: 99), 3 at 81^3, whose 243 blocks are little more than one an
+// SM.  Paired FP32 additions (two rows in one instruction) gave nothing: 71 us.
+constexpr int kTileX = 32, kTileY = 27, kTileStrips = kTileY / 3;
+constexpr int kTileRow = kTileX + 2, kTilePlane = kTileRow * (kTileY + 2);
+constexpr int kTileThreads = kTileX * kTileStrips;
+constexpr int kTileCopies = (kTilePlane + kTileThreads - 1) / kTileThreads;
+template <bool kRes>
+__global__ void __launch_bounds__(kTileThreads, 2) k_jacobi_tile3(DevTree t, const float *b, const float *Vin,
+                                                                    float *__restrict__ Vout, float omega, double *r2,
+                                                                    int len) {
+  __shared__ float ring[2][3][kTilePlane];
+  const InstInfo &I = t.inst[0];
+  const int32_t M = I.M, plane = M * M;
+  StencilC<float> s;
+  stencil_consts<3>(I, omega, kRes, &s);
+  const int tid = threadIdx.x, lane = tid & 31, strip = tid >> 5;
+  const int32_t tiles = (M + kTileX - 1) / kTileX;
+  const int32_t x0 = (int32_t)(blockIdx.x % tiles) * kTileX, yb = (int32_t)(blockIdx.x / tiles) * kTileY;
+  const int32_t x = x0 + lane, y0 = yb + 3 * strip, z0 = (int32_t)blockIdx.y * len;
+  const bool act = x < M;  // M is a multiple of 27: every row is a row of the grid
+  int32_t src[kTileCopies];  // this thread's share of a plane's copies
+#pragma unroll
+  for (int k = 0; k < kTileCopies; ++k) {
+    const int i = tid + k * kTileThreads, r = i / kTileRow, c = i - r * kTileRow;
+    int32_t yy = yb + r - 1, xx = x0 + c - 1;
+    yy = yy < 0 ? M - 1 : yy >= M ? 0 : yy;
+    xx = xx < 0 ? M - 1 : xx >= M ? xx - M : xx;  // columns past the grid: any value
+    src[k] = yy * M + xx;
+  }
+  const int32_t xc = act ? x : 0;
+  int32_t w[3] = {step_weight(t.spread, M, xc), step_weight(t.spread + M, M, y0), 0};
+  bool flip[3] = {xc == 0, y0 == 0, false};
+  const int32_t at0 = y0 * M + xc;
+  int32_t w2 = step_weight(t.spread + 2 * M, M, z0);
+  double rr = 0.0;
+  pdl_wait();
+  pdl_release();
+  auto fetch = [&](int32_t z, float *stage) {  // plane z (periodic)
+    const float *p = Vin + (int64_t)(z < 0 ? z + M : z >= M ? z - M : z) * plane;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage + tid);
+#pragma unroll
+    for (int k = 0; k < kTileCopies; ++k)
+      if (k + 1 < kTileCopies || tid + k * kTileThreads < kTilePlane)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + k * kTileThreads * 4), "l"(p + src[k])
+                     : "memory");
+  };
+  auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
+  Slab3<float> p0, p1, p2;
+  auto take = [&](const float *stage, Slab3<float> &p) {
+    const float *q = stage + 3 * strip * kTileRow + lane;
+    float v[15];
+#pragma unroll
+    for (int r = 0; r < 5; ++r)
+#pragma unroll
+      for (int i = 0; i < 3; ++i) v[r * 3 + i] = q[r * kTileRow + i];
+    p.set(v, s);
+  };
+  auto put = [&](int32_t z, bool low, const float *stage, const Slab3<float> &lo, const Slab3<float> &mid,
+                 Slab3<float> &hi, const float *bv) {
+    float y[3];
+    take(stage, hi);
+    flip[2] = false;
+    w[2] = 9;
+    if (!low) {
+      flip[2] = z == 0;
+      w[2] = w2;
+      w2 = step_weight(t.spread + 2 * M, M, z + 3 < M ? z + 3 : 0);  // for the next such plane
+      strip_rows<false>(lo, mid, hi, s, w, flip, y);
+    } else {
+      strip_rows<true>(lo, mid, hi, s, w, flip, y);
+    }
+    if (kRes) {
+      if (act) rr = rr + residual2<3>(y, bv, mid.c, s);
+    } else {
+      float out[3];
+      jacobi_update<3>(y, bv, mid.c, s, out);
+      if (act) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) Vout[(int64_t)z * plane + at0 + j * M] = out[j];
+      }
+    }
+  };
+  // planes z0 - 1, z0 by way of the second half of the ring
+  fetch(z0 - 1, ring[1][0]);
+  fetch(z0, ring[1][1]);
+  commit();
+#pragma unroll
+  for (int k = 0; k < 3; ++k) fetch(z0 + 1 + k, ring[0][k]);
+  commit();
+  asm volatile("cp.async.wait_group 1;" ::: "memory");
+  __syncthreads();
+  take(ring[1][0], p0);
+  take(ring[1][1], p1);
+  int half = 0;
+  for (int32_t z = z0; z < z0 + len; z += 3) {  // the three slabs take turns
+    float bv[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) bv[k][j] = b[(int64_t)(z + k) * plane + at0 + j * M];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // planes z + 1 .. z + 3 are there, and the other half has been read
+    if (z + 3 < z0 + len) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fetch(z + 4 + k, ring[half ^ 1][k]);
+      commit();
+    }
+    put(z, false, ring[half][0], p0, p1, p2, bv[0]);
+    put(z + 1, true, ring[half][1], p1, p2, p0, bv[1]);
+    put(z + 2, true, ring[half][2], p2, p0, p1, bv[2]);
+    half ^= 1;
   }
   if (kRes) block_sum_store_at(rr, r2 + (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
 }
@@ -570,18 +675,17 @@ __global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, co
 
 // Grids of this many vertices fill the chip with three vertices a thread; the
 // sizes next to the line are 3^10 = 59,049 and 3^12 = 531,441 (81^3 FP32: 8.2 us a
-// sweep with a thread per vertex, 6.9 us with strips).
+// sweep with a thread per vertex, 5.6 us in tiles).
 constexpr int64_t kStripVertices = 200000;
 constexpr unsigned kJacobiThreads = 128;
 
-// Planes per thread of k_jacobi_strip3 (M a multiple of 27): a long march
-// reads fewer planes twice, but a small grid needs its threads.  Measured, 3 /
-// 9 / 27 planes: 243^3 FP32 121 / 103 / 109 us, 81^3 FP32 6.9 / 8.4 / 17.5 us,
-// 81^3 FP64 26.1 / 28.7 / 47.3 us (an earlier form of the kernel).
-inline int march_length(int64_t M, size_t width) {
-  const int64_t cols = M * M / 3, want = width == 8 ? 40000 : 200000;
+// Planes per thread of k_jacobi_strip3 (M a multiple of 27): a long march reads
+// fewer planes twice, but a small grid needs its threads.  Measured at 81^3,
+// 3 / 9 / 27 planes: 26.1 / 28.7 / 47.3 us (an earlier form of the kernel).
+inline int march_length(int64_t M) {
+  const int64_t cols = M * M / 3;
   int len = 27;
-  while (len > 3 && cols * (M / len) < want) len /= 3;
+  while (len > 3 && cols * (M / len) < 40000) len /= 3;
   return len;
 }
 
@@ -611,18 +715,24 @@ int64_t launch_jacobi_uniform(const DevTree &t, const T *b, const T *Vin, T *Vou
     return g.x;
   }
   const int64_t M = t.M;
-  if (D == 2) {
+  if constexpr (D == 2) {
     const dim3 g(grid_for(M * (M / 3), kJacobiThreads));
     launch_pdl(k_jacobi_strip2<T, kRes>, g, dim3(kJacobiThreads), s, t, b, Vin, Vout, omega, r2);
     return g.x;
   }
-  const int len = march_length(M, sizeof(T));
-  // FP64: one warp a block spreads the work evenly over the SMs' FP64 pipes (81^3:
-  // 486 blocks of 128 threads leave the pipes idle for half the time, 29.7 -> 23.5 us)
-  const unsigned threads = sizeof(T) == 8 ? 32 : kJacobiThreads;
-  const dim3 g(grid_for(M * (M / 3), threads), (unsigned)(M / len));
-  launch_pdl(k_jacobi_strip3<T, kRes>, g, dim3(threads), s, t, b, Vin, Vout, omega, r2, len);
-  return (int64_t)g.x * g.y;
+  if constexpr (D == 3 && sizeof(T) == 4) {
+    const int len = M >= 243 ? 9 : 3;
+    const dim3 g((unsigned)((M + kTileX - 1) / kTileX * (M / kTileY)), (unsigned)(M / len));
+    launch_pdl(k_jacobi_tile3<kRes>, g, dim3(kTileThreads), s, t, b, Vin, Vout, omega, r2, len);
+    return (int64_t)g.x * g.y;
+  } else if constexpr (D == 3) {
+    // one warp a block spreads the work evenly over the SMs' FP64 pipes (81^3: 486
+    // blocks of 128 threads leave the pipes idle for half the time, 29.7 -> 23.5 us)
+    const int len = march_length(M);
+    const dim3 g(grid_for(M * (M / 3), 32), (unsigned)(M / len));
+    launch_pdl(k_jacobi_strip3<kRes>, g, dim3(32), s, t, b, Vin, Vout, omega, r2, len);
+    return (int64_t)g.x * g.y;
+  }
 }
 
 // ---- vertex field -----------------------------------------------------------------

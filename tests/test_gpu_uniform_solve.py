@@ -80,3 +80,21 @@ def test_batch_solve_matches_single_plasmas(d, precision):
         else:
             assert np.max(np.abs(a - c)) <= TOL64 * max(1e-300, np.max(np.abs(c)))
             assert np.max(np.abs(ea - ec)) <= TOL64 * max(1e-300, np.max(np.abs(c))) * 3 ** depths[i]
+
+
+@pytest.mark.parametrize("sweeps", [1, 4])
+def test_long_march_matches_fp64(sweeps):
+    """243^3: blocks that march over several groups of planes, against the FP64
+    solve of the same particles.  A sweep rounds the at most 64 terms of a vertex
+    by 2^-24 each, and its iteration matrix does not amplify (norm 1)."""
+    x, v = W.random_particles(3, 200001, 17, vmax=0.2)
+    kw = dict(q=-1.0 / len(x), qm=-1.0, ion=0.3, sweeps=sweeps, omega=0.8, scheme=pic.PIT)
+    V = []
+    for precision in (pic.FP32_SPLIT, pic.FP64):
+        g = pic.Pic(3, W.uniform_tree_flags(3, 5), x, v, precision=precision, **kw)
+        g.step(0.05)
+        g.sync()
+        V.append(g.potential())
+        del g
+    assert np.max(np.abs(V[1])) > 0
+    assert np.max(np.abs(V[0] - V[1])) <= sweeps * 64 * 2.0 ** -24 * np.max(np.abs(V[1]))
