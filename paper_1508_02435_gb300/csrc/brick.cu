@@ -322,25 +322,44 @@ size_t push_st_smem() {
          sizeof(uint8_t) * kHalfCap + sizeof(int32_t) * (kHThreads / 32) * kUnitSlots;
 }
 
-// Writes one arrival into slot `slot` of brick dest's staging area, or into
+// The staged state of arrival `at`: 16 bytes, and in 3D eight more in a second
+// array.  Consecutive arrivals store whole sectors; one record of 24 bytes a lane
+// is three stores over the same six lines (1.15e8 particles on 243^3 cells: K1
+// 1.86 -> 1.77 ms, K2 1.45 -> 1.37 with its whole-sector partials).  Doubling K1's
+// phases one by one showed the stores to cost a quarter of it, and the gather
+// nothing.  Writing 24-byte records in order across the lanes: 1.98 ms.
+__device__ __forceinline__ float4 *stage_head(const BrickStage &st) { return reinterpret_cast<float4 *>(st.rec); }
+__device__ __forceinline__ float2 *stage_tail(const BrickStage &st) {
+  return reinterpret_cast<float2 *>(st.rec + 4 * st.row);
+}
+
+// Index of slot `slot` of unit dest in the staging arrays.
+__device__ __forceinline__ uint32_t stage_index(const BrickStage &st, int32_t dest, int32_t slot) {
+  return (uint32_t)dest * (uint32_t)st.cap + (uint32_t)slot;  // < 2^31 (checked at set-up)
+}
+
+template <int D>
+__device__ __forceinline__ void stage_write(const BrickStage &st, uint32_t at, const float *on, const float *vn,
+                                            uint16_t code, uint32_t key, int32_t id, bool with_id) {
+  if constexpr (D == 3) {
+    stage_head(st)[at] = make_float4(on[0], on[1], on[2], vn[0]);
+    stage_tail(st)[at] = make_float2(vn[1], vn[2]);
+  } else {
+    stage_head(st)[at] = make_float4(on[0], on[1], vn[0], vn[1]);
+  }
+  st.code[at] = code;
+  st.key[at] = key;
+  if (with_id) st.id[at] = id;
+}
+
+// Writes one arrival into slot `slot` of unit dest's staging area, or into
 // the overflow list when the area is full.
 template <int D>
 __device__ __forceinline__ void stage_put(const BrickStage &st, int32_t dest, int32_t slot, const float *on,
                                           const float *vn, uint16_t code, uint32_t key, int32_t id, bool with_id,
                                           int32_t *err) {
   if (slot < st.cap) {
-    const uint32_t at = (uint32_t)dest * (uint32_t)st.cap + (uint32_t)slot;  // < 2^31 (checked at set-up)
-    float *r = st.rec + (size_t)at * (2 * D);  // 8-byte aligned (3D) / 16-byte aligned (2D)
-    if constexpr (D == 3) {
-      reinterpret_cast<float2 *>(r)[0] = make_float2(on[0], on[1]);
-      reinterpret_cast<float2 *>(r)[1] = make_float2(on[2], vn[0]);
-      reinterpret_cast<float2 *>(r)[2] = make_float2(vn[1], vn[2]);
-    } else {
-      *reinterpret_cast<float4 *>(r) = make_float4(on[0], on[1], vn[0], vn[1]);
-    }
-    st.code[at] = code;
-    st.key[at] = key;
-    if (with_id) st.id[at] = id;
+    stage_write<D>(st, stage_index(st, dest, slot), on, vn, code, key, id, with_id);
   } else {
     const int32_t k = atomicAdd(st.ovf_n, 1);
     if (k >= st.ovf_cap) {
@@ -535,15 +554,19 @@ __device__ __forceinline__ void push_half_warp(const DevTree &t, const BrickGeom
     __syncwarp();  // the counts are read by other lanes in the next chunk
   }
   // the warp reserves its runs in the destination units' staging areas (one
-  // atomic per unit it sends to; the count becomes the run's first slot)
+  // atomic per unit it sends to); the count becomes the index of the run's first
+  // slot in the staging arrays, or that slot and kRunOver if the run leaves the
+  // unit's area
+  constexpr uint32_t kRunOver = 0x80000000u;
   {  // both of a lane's atomics in flight at once
     const int us1 = lane + 32;
     const int32_t c0 = wc[lane], c1 = us1 < 54 ? wc[us1] : 0;
+    const int32_t u0 = 2 * hv.nbr[lane >> 1] + (lane & 1), u1 = us1 < 54 ? 2 * hv.nbr[us1 >> 1] + (us1 & 1) : 0;
     int32_t r0 = 0, r1 = 0;
-    if (c0 > 0) r0 = atomicAdd(&a.st.fill[2 * hv.nbr[lane >> 1] + (lane & 1)], c0);
-    if (c1 > 0) r1 = atomicAdd(&a.st.fill[2 * hv.nbr[us1 >> 1] + (us1 & 1)], c1);
-    if (c0 > 0) wc[lane] = r0;
-    if (c1 > 0) wc[us1] = r1;
+    if (c0 > 0) r0 = atomicAdd(&a.st.fill[u0], c0);
+    if (c1 > 0) r1 = atomicAdd(&a.st.fill[u1], c1);
+    if (c0 > 0) wc[lane] = (int32_t)(r0 + c0 <= a.st.cap ? stage_index(a.st, u0, r0) : kRunOver | (uint32_t)r0);
+    if (c1 > 0) wc[us1] = (int32_t)(r1 + c1 <= a.st.cap ? stage_index(a.st, u1, r1) : kRunOver | (uint32_t)r1);
   }
   __syncwarp();
   // pass B, the warp's own chunks: every arrival to its reserved slot
@@ -556,18 +579,22 @@ __device__ __forceinline__ void push_half_warp(const DevTree &t, const BrickGeom
     const int dir = (cd >> 10) & 31;
     if (dir == kFarSlot) continue;
     const int hh = (cd & 0x3ff) >= K::LH;
-    const int us = 2 * dir + hh;
-    const int32_t slot = wc[us] + hv.lslot[q];
+    const uint32_t run = (uint32_t)wc[2 * dir + hh], rank = hv.lslot[q];
+    const uint16_t code = (uint16_t)(cd & (kStayBit | 0x3ff));
+    const uint32_t key = ((cd & kStayBit) != 0 ? 0u : 0x80000000u) | (uint32_t)(hs + q);
+    const int32_t id = a.ids ? a.ids[hs + q] : 0;
     float on[D], vn[D];
 #pragma unroll
     for (int ax = 0; ax < D; ++ax) {
       on[ax] = O(ax, q);
       vn[ax] = V(ax, q);
     }
-    const bool stay = (cd & kStayBit) != 0;
-    stage_put<D>(a.st, 2 * hv.nbr[dir] + hh, slot, on, vn, (uint16_t)(cd & (kStayBit | 0x3ff)),
-                 (stay ? 0u : 0x80000000u) | (uint32_t)(hs + q), a.ids ? a.ids[hs + q] : 0, a.ids != nullptr,
-                 a.err);
+    if (run < kRunOver) {
+      stage_write<D>(a.st, run + rank, on, vn, code, key, id, a.ids != nullptr);
+    } else {
+      stage_put<D>(a.st, 2 * hv.nbr[dir] + hh, (int32_t)((run & ~kRunOver) + rank), on, vn, code, key, id,
+                   a.ids != nullptr, a.err);
+    }
   }
   __syncwarp();
   for (int us = lane; us < kUnitSlots; us += 32) wc[us] = 0;  // ready for the warp's next half brick
@@ -914,8 +941,9 @@ template <int D>
 __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, BrickGeom g, BrickPullArgs a) {
   using K = BK<D>;
   extern __shared__ __align__(128) float smf[];
-  float *srec = smf;                                 // kStCap records of 2 D floats (arrival order)
-  uint32_t *key = (uint32_t *)(srec + 2 * D * kStCap);  // canonical keys
+  float4 *head = (float4 *)smf;                      // staged state (arrival order)
+  float2 *tail = (float2 *)(head + kStCap);          // 3D: its last two floats
+  uint32_t *key = (uint32_t *)(smf + 2 * D * kStCap);  // canonical keys
   uint16_t *code = (uint16_t *)(key + kStCap);       // local leaf | stayer bit; later the final position
   uint16_t *map = code + kStCap;                     // bucket position -> arrival
   __shared__ int32_t cnt[K::LH + 1];
@@ -948,9 +976,10 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
       mbar_expect_tx(&s_bar, rb + cb);
       bulk_g2s(key, st.key + at, rb, &s_bar);
       bulk_g2s(code, st.code + at, cb, &s_bar);
-      const uint32_t sb = (uint32_t)((nin * 8 * D + 15) & ~15);
-      mbar_expect_tx(&s_bar2, sb);
-      bulk_g2s(srec, st.rec + at * (2 * D), sb, &s_bar2);
+      const uint32_t hb = (uint32_t)(nin * 16), tb = D == 3 ? (uint32_t)((nin * 8 + 15) & ~15) : 0u;
+      mbar_expect_tx(&s_bar2, hb + tb);
+      bulk_g2s(head, stage_head(st) + at, hb, &s_bar2);
+      if (D == 3) bulk_g2s(tail, stage_tail(st) + at, tb, &s_bar2);
     }
   }
   for (int i = tid; i <= nlf; i += blockDim.x) cnt[i] = 0;
@@ -1071,15 +1100,14 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
       gV[ax] = a.v + ax * n + bstart;
     }
     for (int32_t j = tid; j < nin; j += blockDim.x) {
-      const float *r = srec + 2 * D * map[j];
+      const int i = map[j];
+      const float4 r0 = head[i];
+      gO[0][j] = r0.x; gO[1][j] = r0.y;
       if constexpr (D == 3) {
-        const float2 r0 = reinterpret_cast<const float2 *>(r)[0], r1 = reinterpret_cast<const float2 *>(r)[1],
-                     r2 = reinterpret_cast<const float2 *>(r)[2];
-        gO[0][j] = r0.x; gO[1][j] = r0.y; gO[2][j] = r1.x;
-        gV[0][j] = r1.y; gV[1][j] = r2.x; gV[2][j] = r2.y;
+        const float2 r1 = tail[i];
+        gO[2][j] = r0.z;
+        gV[0][j] = r0.w; gV[1][j] = r1.x; gV[2][j] = r1.y;
       } else {
-        const float4 r0 = *reinterpret_cast<const float4 *>(r);
-        gO[0][j] = r0.x; gO[1][j] = r0.y;
         gV[0][j] = r0.z; gV[1][j] = r0.w;
       }
     }
@@ -1094,24 +1122,16 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
 #pragma unroll
       for (int e = 0; e < K::NC; ++e) acc[e] = 0.0f;
       const int32_t lo = cnt[l], hi = cnt[l + 1];
-      float on[D];
-      if (lo < hi) {
-        const float *r = srec + 2 * D * map[lo];
-#pragma unroll
-        for (int ax = 0; ax < D; ++ax) on[ax] = r[ax];
-      }
+      float4 next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (lo < hi) next = head[map[lo]];
       for (int32_t j = lo; j < hi; ++j) {
         float o[D], om[D];
+        o[0] = next.x;
+        o[1] = next.y;
+        if (D == 3) o[D - 1] = next.z;
 #pragma unroll
-        for (int ax = 0; ax < D; ++ax) {
-          o[ax] = on[ax];
-          om[ax] = 1.0f - o[ax];
-        }
-        if (j + 1 < hi) {
-          const float *r = srec + 2 * D * map[j + 1];
-#pragma unroll
-          for (int ax = 0; ax < D; ++ax) on[ax] = r[ax];
-        }
+        for (int ax = 0; ax < D; ++ax) om[ax] = 1.0f - o[ax];
+        if (j + 1 < hi) next = head[map[j + 1]];
         // corner weights (f0 * f1) [* f2] as in the push, two corners per
         // paired multiply, then summed per corner in bucket order
         const float2 f0 = make_float2(om[0], o[0]);
@@ -1128,9 +1148,10 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
           acc[0] = acc[0] + a01.x; acc[1] = acc[1] + a01.y; acc[2] = acc[2] + a23.x; acc[3] = acc[3] + a23.y;
         }
       }
+      // whole sectors: eight stores of four bytes each would be eight writes of every one
       float *gp = a.part + (int64_t)(L0 + l) * K::NC;
-#pragma unroll
-      for (int e = 0; e < K::NC; ++e) gp[e] = acc[e];
+      if constexpr (D == 3) store32(gp, acc);
+      else *reinterpret_cast<float4 *>(gp) = make_float4(acc[0], acc[1], acc[2], acc[3]);
     }
   }
 }
@@ -1238,11 +1259,18 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
     const int32_t r = a.fb_idx[bstart + j];
     const int32_t dst = bstart + j;
     if (r < nf) {
-      const float *rr = st.rec + (at + r) * (2 * D);
-#pragma unroll
-      for (int ax = 0; ax < D; ++ax) {
-        a.o[ax * n + dst] = rr[ax];
-        a.v[ax * n + dst] = rr[D + ax];
+      const float4 r0 = stage_head(st)[at + r];
+      a.o[dst] = r0.x;
+      a.o[n + dst] = r0.y;
+      if constexpr (D == 3) {
+        const float2 r1 = stage_tail(st)[at + r];
+        a.o[2 * n + dst] = r0.z;
+        a.v[dst] = r0.w;
+        a.v[n + dst] = r1.x;
+        a.v[2 * n + dst] = r1.y;
+      } else {
+        a.v[dst] = r0.z;
+        a.v[n + dst] = r0.w;
       }
       if (a.ids) a.ids[dst] = st.id[at + r];
     } else {

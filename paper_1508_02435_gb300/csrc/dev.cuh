@@ -60,6 +60,18 @@ struct DevTree {
   float ion_u32, diag_u32;
 };
 
+// 32 bytes in one store (eight floats, four doubles), to a 32-byte boundary: a
+// whole sector, which two stores would write in two parts.
+__device__ __forceinline__ void store32(float *p, const float *v) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+__device__ __forceinline__ void store32(double *p, const double *v) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+               : "memory");
+}
+
 // ---- quantisation ---------------------------------------------------------
 
 __device__ __forceinline__ double wrap01(double x) {

@@ -89,7 +89,7 @@ struct BrickGeom {
 struct BrickStage {
   int32_t cap;                   // slots per destination unit (a multiple of 8)
   int64_t row;                   // slots in all (2 n_bricks cap, padded)
-  float *rec;                    // [row][2 D] one record per slot: the D offsets, then the D velocities
+  float *rec;                    // [row][4] o0 o1 v0 v1; 3D: o0 o1 o2 v0, then [row][2] v1 v2
   uint16_t *code;                // destination local leaf | stayer bit
   uint32_t *key;                 // moved << 31 | storage index before the step (canonical order)
   int32_t *id;                   // particle ids (tracked ids only)
