@@ -192,8 +192,8 @@ __global__ void k_leaf_walk(int64_t n_leaves, const int32_t *__restrict__ start,
 #pragma unroll
     for (int e = 0; e < NC; ++e) acc[e] = acc[e] + shape<float>(tl, e, D);
   }
-#pragma unroll
-  for (int e = 0; e < NC; ++e) part[L * NC + e] = acc[e];
+  if (D == 3) store32(part + L * NC, acc);
+  else *(float4 *)(part + L * NC) = make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
 
 // ---- per vertex ------------------------------------------------------------------

@@ -920,8 +920,9 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
     key[p] = k;
     if (bad) atomicOr(err, 2);
     if (D == 3) {
-      rec[2 * p] = make_float4(oo[0], oo[1], oo[D - 1], v[p]);
-      rec[2 * p + 1] = make_float4(v[n + p], v[(D - 1) * n + p], __int_as_float(L), __int_as_float(k));
+      const float r[8] = {oo[0],    oo[1],    oo[D - 1], v[p], v[n + p], v[(D - 1) * n + p], __int_as_float(L),
+                          __int_as_float(k)};
+      store32((float *)(rec + 2 * p), r);
     }
   }
   int32_t prev = __shfl_up_sync(0xffffffffu, k, 1);
@@ -956,19 +957,21 @@ __global__ void k_make_records(int64_t n, const float *x, const float *v, const 
                                float4 *rec) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  rec[2 * p] = make_float4(x[p], x[n + p], x[2 * n + p], v[p]);
-  rec[2 * p + 1] = make_float4(v[n + p], v[2 * n + p], __int_as_float(leaf[p]), __int_as_float(key[p]));
+  const float r[8] = {x[p],     x[n + p],     x[2 * n + p],           v[p],
+                      v[n + p], v[2 * n + p], __int_as_float(leaf[p]), __int_as_float(key[p])};
+  store32((float *)(rec + 2 * p), r);
 }
 template <>
 __global__ void k_make_records(int64_t n, const double *x, const double *v, const int32_t *leaf, const int32_t *key,
                                double2 *rec) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
-  rec[4 * p] = make_double2(x[p], x[n + p]);
-  rec[4 * p + 1] = make_double2(x[2 * n + p], v[p]);
-  rec[4 * p + 2] = make_double2(v[n + p], v[2 * n + p]);
-  rec[4 * p + 3] = make_double2(
-      __longlong_as_double((long long)(((uint64_t)(uint32_t)key[p] << 32) | (uint32_t)leaf[p])), 0.0);
+  const double r[8] = {x[p],     x[n + p],     x[2 * n + p], v[p],
+                       v[n + p], v[2 * n + p], __longlong_as_double((long long)(((uint64_t)(uint32_t)key[p] << 32) |
+                                                                                (uint32_t)leaf[p])),
+                       0.0};
+  store32((double *)(rec + 4 * p), r);
+  store32((double *)(rec + 4 * p + 2), r + 4);
 }
 
 void launch_make_records(bool split, int64_t n, const void *x, const void *v, const int32_t *leaf, const int32_t *key,

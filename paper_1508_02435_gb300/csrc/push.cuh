@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(512, 4) k_push32(DevTree t, Push32Args a) {
     knew = push_key<D, kUni>(t, Ins, L2, I, pidt_corner_o(o2, D));
     moved = knew != kold;
     if (D == 3) {
-      a.rec[2 * p] = make_float4(o2[0], o2[1], o2[D - 1], v[0]);
-      a.rec[2 * p + 1] = make_float4(v[1], v[D - 1], __int_as_float(L2), __int_as_float(knew));
+      const float r[8] = {o2[0], o2[1], o2[D - 1], v[0], v[1], v[D - 1], __int_as_float(L2), __int_as_float(knew)};
+      store32((float *)(a.rec + 2 * p), r);
     } else {
 #pragma unroll
       for (int k = 0; k < D; ++k) a.tv[k * n + p] = v[k];
@@ -341,11 +341,10 @@ __global__ void k_push64(DevTree t, Push64Args a) {
     knew = push_key<D, kUni>(t, Ins, L2, C, corner);
     moved = knew != kold;
     if (D == 3) {  // one 64-byte record per particle: the re-bin gathers it whole
-      double2 *r = a.rec + 4 * p;
-      r[0] = make_double2(x[0], x[1]);
-      r[1] = make_double2(x[D - 1], v[0]);
-      r[2] = make_double2(v[1], v[D - 1]);
-      r[3] = make_double2(__longlong_as_double((long long)(((uint64_t)(uint32_t)knew << 32) | (uint32_t)L2)), 0.0);
+      const double r[8] = {x[0], x[1], x[D - 1], v[0], v[1], v[D - 1],
+                           __longlong_as_double((long long)(((uint64_t)(uint32_t)knew << 32) | (uint32_t)L2)), 0.0};
+      store32((double *)(a.rec + 4 * p), r);
+      store32((double *)(a.rec + 4 * p + 2), r + 4);
     } else {
 #pragma unroll
       for (int k = 0; k < D; ++k) a.tv[k * n + p] = v[k];
