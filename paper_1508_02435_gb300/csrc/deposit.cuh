@@ -257,14 +257,11 @@ __global__ void k_vertex_charge(DevTree t, const T *__restrict__ part, T *__rest
   if (block_sum) block_sum_store(mine, block_sum);
 }
 
-// The same on the grid of one uniform 3D instance: blocks of 32 x 8 columns
+// The same on the grid of one uniform 3D instance, FP64: blocks of 32 x 8 columns
 // march `len` planes, so that a leaf's row of eight partials, which eight
-// vertices read, comes from the L2 about once (row-major blocks fetch it four
-// times: 243^3 cells 184 -> 162 us; the block sums over one vertex a thread
-// took 214 us).
-template <typename T>
-__global__ void __launch_bounds__(256) k_vertex_charge_grid(DevTree t, const T *__restrict__ part, T *__restrict__ Q,
-                                                            double *block_sum, int len) {
+// vertices read, comes from the L2 about once.
+__global__ void __launch_bounds__(256) k_vertex_charge_grid(DevTree t, const double *__restrict__ part,
+                                                            double *__restrict__ Q, double *block_sum, int len) {
   const InstInfo &I = t.inst[0];
   const int32_t M = I.M, tiles = (M + 31) / 32;
   const int32_t x = (int32_t)(blockIdx.x % tiles) * 32 + (threadIdx.x & 31);
@@ -272,7 +269,7 @@ __global__ void __launch_bounds__(256) k_vertex_charge_grid(DevTree t, const T *
   double mine = 0.0;
   if (x < M && y < M) {
     const int32_t *sp = t.spread;
-    const T q = inst_q(I, (T)0), ion = inst_ion(I, (T)0) * ion_load(t, 0, (T)0);
+    const double q = inst_q(I, 0.0), ion = inst_ion(I, 0.0) * ion_load(t, 0, 0.0);
     int32_t w[3], s2[4];
     bool flip[3] = {x == 0, y == 0, false};
     const int32_t x1 = __ldg(sp + x), x0 = __ldg(sp + (flip[0] ? M - 1 : x - 1));
@@ -290,13 +287,83 @@ __global__ void __launch_bounds__(256) k_vertex_charge_grid(DevTree t, const T *
       const int32_t hi = __ldg(sp + z);
       w[2] = abs(hi - lo);
       flip[2] = z == 0;
-      T u[8];
+      double u[8];
 #pragma unroll
       for (int f = 0; f < 8; ++f) u[7 - f] = part[(int64_t)(s2[f & 3] + (f >> 2 ? lo : hi)) * 8 + f];
       lo = hi;
-      const T val = q * ordered_sum<3, false>(u, w, flip) + ion;
+      const double val = q * ordered_sum<3, false>(u, w, flip) + ion;
       Q[((int64_t)z * M + y) * M + x] = val;
       mine = mine + (double)val;
+    }
+  }
+  block_sum_store_at(mine, block_sum + (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
+}
+
+// FP32: a leaf's row of eight partials goes to eight vertices, so a thread loads it
+// whole and hands the values out through shared memory; the upper four wait in
+// registers for the next plane.  Loads of single partials, each over the sectors
+// of 32 rows, are bound by the L1: 243^3 cells 160 us that way, 117 here (516 MB:
+// 76 us).  FP64 rows take twice the registers and shared memory, and lose by it
+// (243^3 1.63 -> 1.81 ms with the leaf sums).
+constexpr int kChargeX = 32, kChargeY = 8, kChargeRow = kChargeX + 1, kChargeCells = kChargeRow * (kChargeY + 1);
+__global__ void __launch_bounds__(256) k_vertex_charge_tile(DevTree t, const float *__restrict__ part,
+                                                            float *__restrict__ Q, double *block_sum, int len) {
+  __shared__ float plane[2][8][kChargeCells + 7];
+  const InstInfo &I = t.inst[0];
+  const int32_t M = I.M, tiles = (M + kChargeX - 1) / kChargeX, *sp = t.spread;
+  const int32_t bx = (int32_t)(blockIdx.x % tiles) * kChargeX, by = (int32_t)(blockIdx.x / tiles) * kChargeY;
+  const int32_t x = bx + (threadIdx.x & 31), y = by + (threadIdx.x >> 5), z0 = (int32_t)blockIdx.y * len;
+  const bool act = x < M && y < M;
+  // this thread's leaves of a plane, and the cells x - 1, y - 1 of its vertex
+  int32_t leaf[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int i = (int)threadIdx.x + h * 256, r = i / kChargeRow;
+    const int32_t cx = bx + (i - r * kChargeRow) - 1, cy = by + r - 1;
+    leaf[h] = -1;
+    if (i < kChargeCells && cx < M && cy < M)
+      leaf[h] = __ldg(sp + (cx < 0 ? M - 1 : cx)) + __ldg(sp + M + (cy < 0 ? M - 1 : cy));
+  }
+  const int at = (int)(threadIdx.x >> 5) * kChargeRow + (int)(threadIdx.x & 31);
+  const float q = inst_q(I, 0.0f), ion = inst_ion(I, 0.0f) * ion_load(t, 0, 0.0f);
+  int32_t w[3] = {act ? step_weight(sp, M, x) : 0, act ? step_weight(sp + M, M, y) : 0, 0};
+  bool flip[3] = {x == 0, y == 0, false};
+  sp += 2 * M;
+  float row[2][8], below[4];
+  auto fetch = [&](int32_t z) {
+    const int32_t sz = __ldg(sp + (z < 0 ? M - 1 : z));
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (leaf[h] >= 0) load32(part + (int64_t)(leaf[h] + sz) * 8, row[h]);
+  };
+  double mine = 0.0;
+  fetch(z0 - 1);
+  for (int32_t z = z0 - 1; z < z0 + len; ++z) {
+    float(*s)[kChargeCells + 7] = plane[(z - z0) & 1];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (leaf[h] >= 0) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e][threadIdx.x + h * 256] = row[h][e];
+      }
+    __syncthreads();
+    if (z + 1 < z0 + len) fetch(z + 1);
+    if (act) {
+      float u[8];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int c = at + (f & 1 ? 0 : 1) + (f >> 1 ? 0 : kChargeRow);
+        u[7 - f] = s[f][c];
+        u[3 - f] = below[f];
+        below[f] = s[4 + f][c];
+      }
+      if (z >= z0) {
+        w[2] = step_weight(sp, M, z);
+        flip[2] = z == 0;
+        const float val = q * ordered_sum<3, false>(u, w, flip) + ion;
+        Q[((int64_t)z * M + y) * M + x] = val;
+        mine = mine + (double)val;
+      }
     }
   }
   block_sum_store_at(mine, block_sum + (int64_t)blockIdx.y * gridDim.x + blockIdx.x);
@@ -325,10 +392,13 @@ __global__ void k_inst_sum(DevTree t, const T *Q, double *out) {
 template <typename T>
 static void vertex_charge(const DevTree &t, const T *part, T *Q, double *block_sum, double *total, cudaStream_t s) {
   if (t.uniform && t.n_inst == 1 && t.d == 3 && t.M >= 81) {
-    const int len = 9;
-    const dim3 g((unsigned)((t.M + 31) / 32 * ((t.M + 7) / 8)), (unsigned)(t.M / len));
+    // FP32 at 243^3, 9 / 27 planes a block: 128 / 117 us; smaller grids need the blocks
+    const int len = sizeof(T) == 4 && t.M >= 243 ? 27 : 9;
+    const dim3 g((unsigned)((t.M + kChargeX - 1) / kChargeX * ((t.M + kChargeY - 1) / kChargeY)),
+                 (unsigned)(t.M / len));
     COUNT(2);
-    k_vertex_charge_grid<T><<<g, 256, 0, s>>>(t, part, Q, block_sum, len);
+    if constexpr (sizeof(T) == 4) k_vertex_charge_tile<<<g, 256, 0, s>>>(t, part, Q, block_sum, len);
+    else k_vertex_charge_grid<<<g, 256, 0, s>>>(t, part, Q, block_sum, len);
     k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, (int64_t)g.x * g.y, total);
     return;
   }
