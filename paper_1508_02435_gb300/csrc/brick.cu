@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
   uint16_t *code = (uint16_t *)(key + kStCap);       // local leaf | stayer bit; later the final position
   uint16_t *map = code + kStCap;                     // bucket position -> arrival
   __shared__ int32_t cnt[K::LH + 1];
-  __shared__ int32_t cur[K::LH];
+  __shared__ uint16_t list[K::LH];
   __shared__ int32_t wsum[kStThreads / 32];
   __shared__ int32_t s_max, s_ccount[4];
   __shared__ uint64_t s_bar, s_bar2;  // keys and codes; offsets and velocities
@@ -995,30 +995,30 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
       return;
     }
   }
-  // leaf counts: four consecutive arrivals per thread (one 8-byte load of
-  // their codes), one shared atomic per run
+  // leaf counts, and every arrival's rank in its leaf (in any order): four
+  // consecutive arrivals per thread (one 8-byte load of their codes), one shared
+  // atomic per run of one leaf
   bool badc = false;
-  for (int32_t r0 = 4 * tid; r0 < nin; r0 += 4 * kStThreads) {
-    int leaf = -1, run = 0;
-    const uint2 c4 = *reinterpret_cast<const uint2 *>(code + r0);
-    const uint32_t cw[2] = {c4.x, c4.y};
+  constexpr int kGroups = (kStCap + 4 * kStThreads - 1) / (4 * kStThreads);
+  int32_t lf4[kGroups][4], rank4[kGroups][4];  // local leaf (-1: none), rank
+#pragma unroll
+  for (int h = 0; h < kGroups; ++h) {
+    const int32_t r0 = 4 * (tid + h * kStThreads);
+    const uint2 c4 = r0 < nin ? *reinterpret_cast<const uint2 *>(code + r0) : make_uint2(0u, 0u);
+    int run[4];
+#pragma unroll
+    for (int k = 3; k >= 0; --k) {
+      int lf = (int)(((k < 2 ? c4.x : c4.y) >> (16 * (k & 1))) & 0x3ffu) - lf0;
+      if (r0 + k >= nin) lf = -1;
+      else if (lf < 0 || lf >= nlf) badc = true;
+      lf4[h][k] = lf;
+      run[k] = k < 3 && lf == lf4[h][k < 3 ? k + 1 : 3] ? run[k < 3 ? k + 1 : 3] + 1 : 1;
+    }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      if (r0 + k >= nin) break;
-      const int lf = (int)((cw[k >> 1] >> (16 * (k & 1))) & 0x3ffu) - lf0;
-      if (lf < 0 || lf >= nlf) {
-        badc = true;
-        continue;
-      }
-      if (lf == leaf) {
-        ++run;
-      } else {
-        if (run) atomicAdd(&cnt[leaf], run);
-        leaf = lf;
-        run = 1;
-      }
+      if (k > 0 && lf4[h][k] == lf4[h][k > 0 ? k - 1 : 0]) rank4[h][k] = rank4[h][k > 0 ? k - 1 : 0] + 1;
+      else rank4[h][k] = lf4[h][k] >= 0 && lf4[h][k] < nlf ? atomicAdd(&cnt[lf4[h][k]], run[k]) : 0;
     }
-    if (run) atomicAdd(&cnt[leaf], run);
   }
   if (__syncthreads_or(badc)) {  // a staged code names no leaf of the unit
     if (nin > 0) mbar_wait(&s_bar2, 0, kWaitCycles);  // let the state copy land before leaving
@@ -1033,7 +1033,6 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
     const int32_t off = block_excl_scan(c, wsum);
     if (tid < nlf) {
       cnt[tid] = off;
-      cur[tid] = off;
     }
     const int32_t wmax = __reduce_max_sync(0xffffffffu, c);
     if (lane == 0 && wmax > 0) atomicMax(&s_max, wmax);
@@ -1046,12 +1045,14 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
     crank = __shfl_sync(0xffffffffu, base, leader) + __popc(peers & ((1u << lane) - 1u));
   }
   __syncthreads();
-  // bucket positions in any order
-  for (int32_t i = tid; i < nin; i += blockDim.x) map[atomicAdd(&cur[(code[i] & 0x3ff) - lf0], 1)] = (uint16_t)i;
-  __syncthreads();
-  // leaves to sort, grouped by size class (the cursors are free now), so that
-  // the threads of a warp run the same network
-  uint16_t *list = (uint16_t *)cur;
+  // bucket positions, any order within a leaf
+#pragma unroll
+  for (int h = 0; h < kGroups; ++h)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (lf4[h][k] >= 0) map[cnt[lf4[h][k]] + rank4[h][k]] = (uint16_t)(4 * (tid + h * kStThreads) + k);
+  // leaves to sort, grouped by size class, so that the threads of a warp run
+  // the same network
   const int32_t nA = s_ccount[0], nB = s_ccount[1], nC = s_ccount[2], nD = s_ccount[3];
   if (cls >= 0) list[(cls > 0 ? nA : 0) + (cls > 1 ? nB : 0) + (cls > 2 ? nC : 0) + crank] = (uint16_t)tid;
   __syncthreads();
