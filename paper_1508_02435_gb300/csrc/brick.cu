@@ -86,6 +86,10 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
                "l"(src), "r"(bytes), "r"(smem_addr(bar))
                : "memory");
 }
+// Brings `bytes` (a multiple of 16, from a 16-byte boundary) to the L2.
+__device__ __forceinline__ void bulk_prefetch(const void *src, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
+}
 // Bounded wait for phase `parity` of the mbarrier: false if it did not
 // complete within about `cycles` SM clocks.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, long long cycles) {
@@ -752,6 +756,21 @@ __global__ void __launch_bounds__(kHThreads, 2) k_brick_push_st(DevTree t, Brick
         return;
       }
       parity ^= 1u;
+      // the next half brick's bytes on their way to the L2 meanwhile (its copies go
+      // out when the shared memory is free, and land sooner: 1.77 -> 1.73 ms)
+      if (lane == 0 && w < 2 * D + 1 && hn < nh) {
+        const int32_t nn = pe_next - ps_next, hh = hn & 1;
+        const int32_t c0 = half_start(nn, hh), c1 = hh ? nn : half_start(nn, 1);
+        if (nn <= 2 * kHalfCap && c1 > c0) {
+          if (w < 2 * D) {
+            const float *p = (w < D ? a.o + w * n : a.v + (w - D) * n) + ps_next + c0;
+            const uintptr_t a0 = (uintptr_t)p & ~(uintptr_t)15;
+            bulk_prefetch((const void *)a0, (uint32_t)(((uintptr_t)(p + (c1 - c0)) - a0 + 15u) & ~(uintptr_t)15));
+          } else {
+            bulk_prefetch((const EV *)a.Ebrick + (int64_t)(hn >> 1) * K::NVB, K::NVB * sizeof(EV));
+          }
+        }
+      }
       for (int l = tid; l < K::LB; l += blockDim.x) {
         const int32_t lo = max(ls[l] - hs, 0), hi = min(ls[l + 1] - hs, nb);
         for (int32_t q = lo; q < hi; ++q) pos[q] = (uint16_t)l;
@@ -872,7 +891,10 @@ __global__ void k_brick_totals(int64_t n_units, int32_t cap, const int32_t *fill
 // K2: one CTA per destination unit (half brick), two CTAs per SM
 // ---------------------------------------------------------------------------
 
-constexpr int kStThreads = 512;
+// 1.15e8 particles on 243^3 cells, 365 leaves a unit: 384 threads 1.27 ms, 512
+// threads (a quarter of them idle in the per-leaf phases) 1.31.
+constexpr int kStThreads = 384;
+static_assert(BK<3>::LH <= kStThreads && BK<2>::LH <= kStThreads, "a thread per leaf");
 constexpr int kStCap = 3456;  // arrivals per unit held in shared memory (the largest staging capacity)
 
 template <int D>
@@ -913,10 +935,9 @@ __device__ __forceinline__ void sort_leaf_net(uint16_t *mp, int m, const uint32_
     if (t < m) mp[t] = (uint16_t)v[t];
 }
 
-// Size class of a leaf's sort: -1 nothing to sort, 0..2 networks of 4, 8
-// and 16, 3 a warp.
+// Size class of a leaf: sorted by a network of 4, 8 or 16, or by a warp.
 __device__ __forceinline__ int leaf_class(int32_t m) {
-  return m <= 1 ? -1 : (m <= 4 ? 0 : (m <= 8 ? 1 : (m <= 16 ? 2 : 3)));
+  return m <= 4 ? 0 : (m <= 8 ? 1 : (m <= 16 ? 2 : 3));
 }
 
 // Exclusive scan of c over the first nl <= blockDim.x threads of the block
@@ -1037,7 +1058,7 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
     const int32_t wmax = __reduce_max_sync(0xffffffffu, c);
     if (lane == 0 && wmax > 0) atomicMax(&s_max, wmax);
     if (tid == 0) cnt[nlf] = nin;
-    cls = leaf_class(c);
+    cls = tid < nlf ? leaf_class(c) : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, cls);
     const int leader = __ffs(peers) - 1;
     int32_t base = 0;
@@ -1051,8 +1072,8 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       if (lf4[h][k] >= 0) map[cnt[lf4[h][k]] + rank4[h][k]] = (uint16_t)(4 * (tid + h * kStThreads) + k);
-  // leaves to sort, grouped by size class, so that the threads of a warp run
-  // the same network
+  // leaves grouped by size class, so that the threads of a warp run the same
+  // network and have about as many arrivals to sum
   const int32_t nA = s_ccount[0], nB = s_ccount[1], nC = s_ccount[2], nD = s_ccount[3];
   if (cls >= 0) list[(cls > 0 ? nA : 0) + (cls > 1 ? nB : 0) + (cls > 2 ? nC : 0) + crank] = (uint16_t)tid;
   __syncthreads();
@@ -1092,67 +1113,74 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
       return;
     }
   }
-  // coalesced writes in destination order
-  {
-    float *gO[D], *gV[D];
+  // Half of the warps write the state out first and half sum the partials first,
+  // so that the stores spread over both (1.27 -> 1.22 ms).
+#pragma unroll 1
+  for (int ph = 0; ph < 2; ++ph) {
+    const int turn = ph ^ (w & 1);
+    // coalesced writes in destination order
+    if (turn == 0) {
+      float *gO[D], *gV[D];
 #pragma unroll
-    for (int ax = 0; ax < D; ++ax) {
-      gO[ax] = a.o + ax * n + bstart;
-      gV[ax] = a.v + ax * n + bstart;
-    }
-    for (int32_t j = tid; j < nin; j += blockDim.x) {
-      const int i = map[j];
-      const float4 r0 = head[i];
-      gO[0][j] = r0.x; gO[1][j] = r0.y;
-      if constexpr (D == 3) {
-        const float2 r1 = tail[i];
-        gO[2][j] = r0.z;
-        gV[0][j] = r0.w; gV[1][j] = r1.x; gV[2][j] = r1.y;
-      } else {
-        gV[0][j] = r0.z; gV[1][j] = r0.w;
+      for (int ax = 0; ax < D; ++ax) {
+        gO[ax] = a.o + ax * n + bstart;
+        gV[ax] = a.v + ax * n + bstart;
       }
-    }
-    if (a.ids)
-      for (int32_t j = tid; j < nin; j += blockDim.x) a.ids[bstart + j] = st.id[at + map[j]];
-  }
-  // deposit partials of the new positions, per leaf in bucket order; the
-  // next particle's offsets are fetched while the current one is summed
-  if (a.part) {
-    for (int l = tid; l < nlf; l += blockDim.x) {
-      float acc[K::NC];
-#pragma unroll
-      for (int e = 0; e < K::NC; ++e) acc[e] = 0.0f;
-      const int32_t lo = cnt[l], hi = cnt[l + 1];
-      float4 next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-      if (lo < hi) next = head[map[lo]];
-      for (int32_t j = lo; j < hi; ++j) {
-        float o[D], om[D];
-        o[0] = next.x;
-        o[1] = next.y;
-        if (D == 3) o[D - 1] = next.z;
-#pragma unroll
-        for (int ax = 0; ax < D; ++ax) om[ax] = 1.0f - o[ax];
-        if (j + 1 < hi) next = head[map[j + 1]];
-        // corner weights (f0 * f1) [* f2] as in the push, two corners per
-        // paired multiply, then summed per corner in bucket order
-        const float2 f0 = make_float2(om[0], o[0]);
-        const float2 a01 = mul2_rn(f0, make_float2(om[1], om[1]));
-        const float2 a23 = mul2_rn(f0, make_float2(o[1], o[1]));
+      for (int32_t j = tid; j < nin; j += blockDim.x) {
+        const int i = map[j];
+        const float4 r0 = head[i];
+        gO[0][j] = r0.x; gO[1][j] = r0.y;
         if constexpr (D == 3) {
-          const float2 w01 = mul2_rn(a01, make_float2(om[2], om[2]));
-          const float2 w23 = mul2_rn(a23, make_float2(om[2], om[2]));
-          const float2 w45 = mul2_rn(a01, make_float2(o[2], o[2]));
-          const float2 w67 = mul2_rn(a23, make_float2(o[2], o[2]));
-          acc[0] = acc[0] + w01.x; acc[1] = acc[1] + w01.y; acc[2] = acc[2] + w23.x; acc[3] = acc[3] + w23.y;
-          acc[4] = acc[4] + w45.x; acc[5] = acc[5] + w45.y; acc[6] = acc[6] + w67.x; acc[7] = acc[7] + w67.y;
+          const float2 r1 = tail[i];
+          gO[2][j] = r0.z;
+          gV[0][j] = r0.w; gV[1][j] = r1.x; gV[2][j] = r1.y;
         } else {
-          acc[0] = acc[0] + a01.x; acc[1] = acc[1] + a01.y; acc[2] = acc[2] + a23.x; acc[3] = acc[3] + a23.y;
+          gV[0][j] = r0.z; gV[1][j] = r0.w;
         }
       }
-      // whole sectors: eight stores of four bytes each would be eight writes of every one
-      float *gp = a.part + (int64_t)(L0 + l) * K::NC;
-      if constexpr (D == 3) store32(gp, acc);
-      else *reinterpret_cast<float4 *>(gp) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      if (a.ids)
+        for (int32_t j = tid; j < nin; j += blockDim.x) a.ids[bstart + j] = st.id[at + map[j]];
+    }
+    // deposit partials of the new positions, per leaf in bucket order; the
+    // next particle's offsets are fetched while the current one is summed
+    if (turn == 1 && a.part) {
+      for (int t = tid; t < nlf; t += blockDim.x) {
+        const int l = list[t];
+        float acc[K::NC];
+#pragma unroll
+        for (int e = 0; e < K::NC; ++e) acc[e] = 0.0f;
+        const int32_t lo = cnt[l], hi = cnt[l + 1];
+        float4 next = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (lo < hi) next = head[map[lo]];
+        for (int32_t j = lo; j < hi; ++j) {
+          float o[D], om[D];
+          o[0] = next.x;
+          o[1] = next.y;
+          if (D == 3) o[D - 1] = next.z;
+#pragma unroll
+          for (int ax = 0; ax < D; ++ax) om[ax] = 1.0f - o[ax];
+          if (j + 1 < hi) next = head[map[j + 1]];
+          // corner weights (f0 * f1) [* f2] as in the push, two corners per
+          // paired multiply, then summed per corner in bucket order
+          const float2 f0 = make_float2(om[0], o[0]);
+          const float2 a01 = mul2_rn(f0, make_float2(om[1], om[1]));
+          const float2 a23 = mul2_rn(f0, make_float2(o[1], o[1]));
+          if constexpr (D == 3) {
+            const float2 w01 = mul2_rn(a01, make_float2(om[2], om[2]));
+            const float2 w23 = mul2_rn(a23, make_float2(om[2], om[2]));
+            const float2 w45 = mul2_rn(a01, make_float2(o[2], o[2]));
+            const float2 w67 = mul2_rn(a23, make_float2(o[2], o[2]));
+            acc[0] = acc[0] + w01.x; acc[1] = acc[1] + w01.y; acc[2] = acc[2] + w23.x; acc[3] = acc[3] + w23.y;
+            acc[4] = acc[4] + w45.x; acc[5] = acc[5] + w45.y; acc[6] = acc[6] + w67.x; acc[7] = acc[7] + w67.y;
+          } else {
+            acc[0] = acc[0] + a01.x; acc[1] = acc[1] + a01.y; acc[2] = acc[2] + a23.x; acc[3] = acc[3] + a23.y;
+          }
+        }
+        // whole sectors: eight stores of four bytes each would be eight writes of every one
+        float *gp = a.part + (int64_t)(L0 + l) * K::NC;
+        if constexpr (D == 3) store32(gp, acc);
+        else *reinterpret_cast<float4 *>(gp) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      }
     }
   }
 }
