@@ -20,9 +20,9 @@
 //                       order -- before the coalesced writes of the new bucket
 //                       order and the leaf-corner deposit partials.
 //
-// Bricks over the shared-memory capacity (K1) and units over their staging
-// capacity (K2) take global-memory kernels with the same arithmetic.  The
-// result is bit-identical to the generic path.
+// Bricks over the shared-memory capacity are pushed in more parts; units over
+// their staging capacity take a global-memory form of K2 with the same
+// arithmetic.  The result is bit-identical to the generic path.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -39,8 +39,7 @@ constexpr int kFarSlot = 27;
 constexpr int kSelfDir = 13;         // (0, 0, 0)
 constexpr uint16_t kStayBit = 0x8000;
 constexpr uint16_t kMoverCode = 0;   // leaf code flags of an arrival from another leaf
-constexpr int kPushThreads = 512;
-constexpr unsigned kFallbackBlocks = 608;  // blocks of the global-memory fallback kernels (4 per SM)
+constexpr unsigned kFallbackBlocks = 608;  // blocks of the global-memory pull (4 per SM)
 constexpr unsigned kPersistBlocks = 304;   // CTAs of K1's shared-memory kernel (2 per SM, each taking half bricks in turn)
 constexpr int kPullThreads = 256;
 
@@ -126,101 +125,6 @@ __device__ __forceinline__ int32_t brick_of_coords(const DevTree &t, const int32
 // K1
 // ---------------------------------------------------------------------------
 
-// Gather + kick + drift + re-location of one particle -- the arithmetic of
-// the generic split push, field values from the staged brick field.  o and v
-// are the particle's offset and velocity; returns the destination direction
-// slot and writes the new offset, velocity and leaf.
-template <int D>
-__device__ __forceinline__ int push_core(const DevTree &t, const BrickGeom &g, const BrickPushArgs &a,
-                                         const float *o, const float *vin, const int32_t *lc,
-                                         const int32_t *origin, const int32_t *bc, const float *Eb, float *on,
-                                         float *vn, int32_t &L2, bool &bad) {
-  using K = BK<D>;
-  float om[D];
-#pragma unroll
-  for (int ax = 0; ax < D; ++ax) om[ax] = 1.0f - o[ax];
-  float E[D];
-#pragma unroll
-  for (int ax = 0; ax < D; ++ax) E[ax] = 0.0f;
-  const int base = lc[0] + K::V1 * (lc[1] + (D == 3 ? K::V1 * lc[2] : 0));
-#pragma unroll
-  for (int e = 0; e < K::NC; ++e) {
-    float w = 1.0f;
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax) w = w * (((e >> ax) & 1) ? o[ax] : om[ax]);
-    const int lv = base + (e & 1) + ((e >> 1) & 1) * K::V1 + ((e >> 2) & 1) * K::V1 * K::V1;
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax) E[ax] = E[ax] + w * Eb[ax * K::NVB + lv];
-  }
-  int32_t I[3] = {0, 0, 0};
-  const int32_t per = t.M;
-  int dir = 0, mul = 1;
-  bool far = false;
-#pragma unroll
-  for (int ax = 0; ax < D; ++ax) {
-    float v = vin[ax] + a.qmdt * E[ax];
-    float tt = o[ax] + v * a.sl;
-    if (!isfinite(v) || !isfinite(tt)) { bad = true; tt = 0.0f; }
-    float fl = floorf(tt);
-    float f = tt - fl;
-    int32_t c = origin[ax] + lc[ax], cc;
-    if (fabsf(fl) < 1.0e9f) {
-      cc = c + (int32_t)fl;
-      if (cc < 0 || cc >= per) {
-        cc %= per;
-        if (cc < 0) cc += per;
-      }
-    } else {
-      int64_t c64 = ((int64_t)c + (int64_t)fminf(fmaxf(fl, -1.0e15f), 1.0e15f)) % per;
-      cc = (int32_t)(c64 < 0 ? c64 + per : c64);
-    }
-    I[ax] = cc;
-    vn[ax] = v;
-    on[ax] = clamp_off(f);
-    int32_t db = cc / K::B - bc[ax];
-    if (db < 0) db += g.nbx;
-    int dl = db == 0 ? 0 : (db == 1 ? 1 : (db == g.nbx - 1 ? -1 : 2));
-    far |= dl == 2;
-    dir += (dl + 1) * mul;
-    mul *= 3;
-  }
-  if (D == 2) dir += 9;
-  L2 = uniform_leaf_of_cell(t.spread, t.M, I, D);
-  return far ? kFarSlot : dir;
-}
-
-template <int D>
-__device__ __forceinline__ int brick_push_one(const DevTree &t, const BrickGeom &g, const BrickPushArgs &a,
-                                              int32_t p, const int32_t *lc, const int32_t *origin,
-                                              const int32_t *bc, const float *Eb, float *on, float *vn,
-                                              int32_t &L2, bool &bad) {
-  const int64_t n = a.n;
-  float o[D], v[D];
-#pragma unroll
-  for (int ax = 0; ax < D; ++ax) {
-    o[ax] = a.o[ax * n + p];
-    v[ax] = a.v[ax * n + p];
-  }
-  return push_core<D>(t, g, a, o, v, lc, origin, bc, Eb, on, vn, L2, bad);
-}
-
-// Stage the brick's vertex field: (B+1)^D vertices, periodic.
-template <int D>
-__device__ __forceinline__ void stage_field(const DevTree &t, const BrickPushArgs &a, const int32_t *origin,
-                                            float *Eb) {
-  using K = BK<D>;
-  for (int i = threadIdx.x; i < K::NVB; i += blockDim.x) {
-    int lx = i % K::V1, ly = (i / K::V1) % K::V1, lz = D == 3 ? i / (K::V1 * K::V1) : 0;
-    int32_t gx = origin[0] + lx, gy = origin[1] + ly, gz = D == 3 ? origin[2] + lz : 0;
-    if (gx >= t.M) gx -= t.M;
-    if (gy >= t.M) gy -= t.M;
-    if (gz >= t.M) gz -= t.M;
-    int64_t vid = gx + (int64_t)t.M * (gy + (int64_t)t.M * gz);
-#pragma unroll
-    for (int ax = 0; ax < D; ++ax) Eb[ax * K::NVB + i] = a.E[ax * t.n_vert + vid];
-  }
-}
-
 // ---------------------------------------------------------------------------
 // K1, shared-memory form
 // ---------------------------------------------------------------------------
@@ -300,14 +204,21 @@ __device__ __noinline__ SlowOut relocate_slow(const DevTree &t, const BrickGeom 
 }
 
 // K1 runs two CTAs per SM, each on one half of a brick's particles (storage
-// order); bricks with more than 2 kHalfCap particles take k_brick_push.
+// order).
 constexpr int kHThreads = 512;
 constexpr int kUnitSlots = 56;       // destination units by direction: 27 neighbour bricks x 2 halves (+ pad)
 constexpr int kHalfCap = 3200;       // particles of one half held in shared memory (two CTAs still fit an SM)
 constexpr int kHS = kHalfCap + 8;    // shared row stride (room for a 16-byte aligned head)
 
-// First storage offset (within the brick) of half h of a brick holding nb particles.
-__host__ __device__ __forceinline__ int32_t half_start(int32_t nb, int h) { return h == 0 ? 0 : (nb + 1) / 2; }
+// A brick's particles in storage order are cut into an even share for each of two
+// parts, or of as many as it takes to hold one in shared memory; a "half" h takes
+// the parts h, h + 2, ...
+__device__ __forceinline__ int32_t brick_parts(int32_t nb) {
+  return nb <= 2 * kHalfCap ? 2 : (nb + kHalfCap - 1) / kHalfCap;
+}
+__device__ __forceinline__ int32_t part_share(int32_t nb, int32_t parts) {
+  return parts == 2 ? (nb + 1) / 2 : (nb + parts - 1) / parts;
+}
 
 // Shared-memory offsets of K1's bulk-copy targets must be multiples of 16 bytes.
 template <int D>
@@ -380,30 +291,6 @@ __device__ __forceinline__ void stage_put(const BrickStage &st, int32_t dest, in
     st.ovf_key[k] = key;
     if (with_id) st.ovf_id[k] = id;
   }
-}
-
-// Appends the pushed particles of one warp to the staging areas of their
-// destination units (the global-memory K1): one global atomic per distinct
-// destination of the warp, lanes in lane order; arrivals beyond the area's
-// capacity go to the overflow list.  Inactive lanes pass dest < 0.
-template <int D>
-__device__ __forceinline__ void stage_append(const BrickStage &st, int32_t dest, const float *on, const float *vn,
-                                             uint16_t code, uint32_t key, int32_t id, bool with_id,
-                                             int32_t *err) {
-  const int lane = threadIdx.x & 31;
-  unsigned todo = __ballot_sync(0xffffffffu, dest >= 0);
-  int32_t slot = -1;
-  while (todo) {
-    const int leader = __ffs(todo) - 1;
-    const int32_t dd = __shfl_sync(0xffffffffu, dest, leader);
-    const unsigned m = __ballot_sync(0xffffffffu, dest == dd);
-    int32_t base = 0;
-    if (lane == leader) base = atomicAdd(&st.fill[dd], __popc(m));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (dest == dd) slot = base + __popc(m & ((1u << lane) - 1u));
-    todo &= ~m;
-  }
-  if (dest >= 0) stage_put<D>(st, dest, slot, on, vn, code, key, id, with_id, err);
 }
 
 // A half brick in shared memory, as one warp of K1 sees it.
@@ -675,22 +562,22 @@ __global__ void __launch_bounds__(kHThreads, 2) k_brick_push_st(DevTree t, Brick
     pe = a.start[(hb >> 1) * K::LB + K::LB];
   }
   __syncthreads();  // tables written, barrier initialised
-  for (; hb < nh; hb += gridDim.x) {
-    const int32_t b = hb >> 1, h = hb & 1, L0 = b * K::LB;
-    const int32_t nbr_n = pe - ps;
-    const int32_t q0 = half_start(nbr_n, h), q1 = h ? nbr_n : half_start(nbr_n, 1), nb = q1 - q0;
-    const int32_t hs = ps + q0;  // storage index of this half's first particle
-    // the next half brick's offsets, read now and used after this one
-    const int32_t hn = hb + (int32_t)gridDim.x;
+  int32_t part = hb & 1;
+  while (hb < nh) {
+    const int32_t b = hb >> 1, L0 = b * K::LB;
+    const int32_t nbr_n = pe - ps, parts = brick_parts(nbr_n), share = part_share(nbr_n, parts);
+    const int32_t q0 = min(part * share, nbr_n), nb = min(share, nbr_n - q0);
+    const int32_t hs = ps + q0;  // storage index of the part's first particle
+    // the next part, mostly that of another half brick, whose offsets are read
+    // now and used after this one
+    const bool last = part + 2 >= parts;
+    const int32_t hn = last ? hb + (int32_t)gridDim.x : hb, part_next = last ? hn & 1 : part + 2;
     int32_t ps_next = 0, pe_next = 0;
     if (hn < nh) {
       ps_next = a.start[(hn >> 1) * K::LB];
       pe_next = a.start[(hn >> 1) * K::LB + K::LB];
     }
-    // bricks over 2 kHalfCap particles: listed for the global-memory kernel;
-    // empty halves: nothing to push
-    if (nbr_n > 2 * kHalfCap && h == 0 && tid == 0) a.st.over_bricks[atomicAdd(&a.st.over[0], 1)] = b;
-    if (nbr_n <= 2 * kHalfCap && nb > 0) {
+    if (nb > 0) {  // else nothing to push
       HalfView<D> hv;
       hv.so = so;
       hv.sv = sv;
@@ -759,9 +646,9 @@ __global__ void __launch_bounds__(kHThreads, 2) k_brick_push_st(DevTree t, Brick
       // the next half brick's bytes on their way to the L2 meanwhile (its copies go
       // out when the shared memory is free, and land sooner: 1.77 -> 1.73 ms)
       if (lane == 0 && w < 2 * D + 1 && hn < nh) {
-        const int32_t nn = pe_next - ps_next, hh = hn & 1;
-        const int32_t c0 = half_start(nn, hh), c1 = hh ? nn : half_start(nn, 1);
-        if (nn <= 2 * kHalfCap && c1 > c0) {
+        const int32_t nn = pe_next - ps_next, sn = part_share(nn, brick_parts(nn));
+        const int32_t c0 = min(part_next * sn, nn), c1 = min(c0 + sn, nn);
+        if (c1 > c0) {
           if (w < 2 * D) {
             const float *p = (w < D ? a.o + w * n : a.v + (w - D) * n) + ps_next + c0;
             const uintptr_t a0 = (uintptr_t)p & ~(uintptr_t)15;
@@ -779,6 +666,8 @@ __global__ void __launch_bounds__(kHThreads, 2) k_brick_push_st(DevTree t, Brick
       push_half_warp<D, kAligned>(t, g, a, hv, w, kW, wc + w * kUnitSlots, bad, movers);
       __syncthreads();  // the shared memory is free for the next half brick's copies
     }
+    hb = hn;
+    part = part_next;
     ps = ps_next;
     pe = pe_next;
   }
@@ -789,94 +678,36 @@ __global__ void __launch_bounds__(kHThreads, 2) k_brick_push_st(DevTree t, Brick
   if (tid == 0 && s_movers) atomicAdd(a.n_movers, s_movers);
 }
 
-// K1 for bricks over 2 kHalfCap particles: the same arithmetic (push_core),
-// particles and field read from global memory, one thread per particle.
-template <int D>
-__device__ __forceinline__ void brick_push_fallback(const DevTree &t, const BrickGeom &g, const BrickPushArgs &a,
-                                                    const int32_t b) {
-  using K = BK<D>;
-  __shared__ int32_t ls[K::LB + 1];
-  __shared__ uint32_t dec[K::LB];
-  __shared__ float Eb[D * K::NVB];
-  __shared__ int32_t s_movers;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int32_t L0 = b * K::LB;
-  const int32_t ps = a.start[L0], pe = a.start[L0 + K::LB], nb = pe - ps;
-  if (nb <= 2 * kHalfCap) return;  // the shared-memory kernel took this brick
-  int32_t origin[3] = {0, 0, 0}, bc[3] = {0, 0, 0};
-  for (int ax = 0; ax < D; ++ax) {
-    origin[ax] = t.leaf_coords[(int64_t)L0 * D + ax];
-    bc[ax] = origin[ax] / K::B;
-  }
-  for (int i = tid; i <= K::LB; i += blockDim.x) ls[i] = a.start[L0 + i] - ps;
-  for (int i = tid; i < K::LB; i += blockDim.x) dec[i] = g.decodeL[i];
-  stage_field<D>(t, a, origin, Eb);
-  if (tid == 0) s_movers = 0;
-  __syncthreads();
-  bool bad = false;
-  int movers = 0;
-  for (int32_t base = 0; base < nb; base += blockDim.x) {
-    const int32_t q = base + tid;
-    const bool act = q < nb;
-    int32_t dest = -1;
-    float on[D], vn[D];
-    uint16_t code = 0;
-    uint32_t key = 0;
-    if (act) {
-      int lo = 0, hi = K::LB - 1;  // leaf of storage position q: last l with ls[l] <= q
-      while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (ls[mid] <= q) lo = mid;
-        else hi = mid - 1;
-      }
-      const int l = lo;
-      const uint32_t pk = dec[l];
-      const int32_t lc[3] = {(int32_t)(pk & 1023u), (int32_t)((pk >> 10) & 1023u), (int32_t)(pk >> 20)};
-      int32_t L2;
-      const int dir = brick_push_one<D>(t, g, a, ps + q, lc, origin, bc, Eb, on, vn, L2, bad);
-      (void)dir;
-      const bool stay = L2 == L0 + l;
-      movers += !stay;
-      dest = unit_of<D>(L2 / K::LB, L2 % K::LB);
-      code = (uint16_t)((L2 % K::LB) | (stay ? kStayBit : 0));
-      key = (stay ? 0u : 0x80000000u) | (uint32_t)(ps + q);
-    }
-    stage_append<D>(a.st, dest, on, vn, code, key, (a.ids && act) ? a.ids[ps + q] : 0, a.ids != nullptr, a.err);
-  }
-  if (bad) atomicOr(a.err, 1);
-  for (int o = 16; o > 0; o >>= 1) movers += __shfl_down_sync(0xffffffffu, movers, o);
-  if (lane == 0) atomicAdd(&s_movers, movers);
-  __syncthreads();
-  if (tid == 0 && s_movers) atomicAdd(a.n_movers, s_movers);
-}
-
-// Bricks too large for the shared-memory kernel (listed by it), from global
-// memory; the blocks take the listed bricks in turn.
-template <int D>
-__global__ void __launch_bounds__(kPushThreads) k_brick_push(DevTree t, BrickGeom g, BrickPushArgs a) {
-  const int32_t m = min(*a.st.over, (int32_t)g.n_bricks);
-  for (int32_t i = blockIdx.x; i < m; i += gridDim.x) {
-    brick_push_fallback<D>(t, g, a, a.st.over_bricks[i]);
-    __syncthreads();
-  }
-}
-
 // ---------------------------------------------------------------------------
 // between K1 and K2: overflow arrivals grouped by destination, brick totals
 // ---------------------------------------------------------------------------
 
-__global__ void k_ovf_count(const int32_t *ovf_n, int32_t ovf_cap, const int32_t *ovf_dest, int32_t *fcount) {
-  const int32_t nf = min(*ovf_n, ovf_cap);
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += gridDim.x * blockDim.x)
-    atomicAdd(&fcount[ovf_dest[i]], 1);
+// Overflowing arrivals come from few units, so a warp adds one unit's together.
+__device__ __forceinline__ int32_t ovf_add(int32_t *cell, int32_t dest) {  // this lane's old value; dest < 0: none
+  const int lane = threadIdx.x & 31;
+  const unsigned peers = __match_any_sync(0xffffffffu, dest);
+  const int leader = __ffs(peers) - 1;
+  int32_t base = 0;
+  if (dest >= 0 && lane == leader) base = atomicAdd(cell + dest, __popc(peers));
+  return __shfl_sync(0xffffffffu, base, leader) + __popc(peers & ((1u << lane) - 1u));
 }
 
-__global__ void k_ovf_scatter(const int32_t *ovf_n, int32_t ovf_cap, const int32_t *ovf_dest, const int32_t *fstart,
-                              int32_t *fcursor, int32_t *sorted) {
+__global__ void __launch_bounds__(256) k_ovf_count(const int32_t *ovf_n, int32_t ovf_cap, const int32_t *ovf_dest,
+                                                   int32_t *fcount) {
   const int32_t nf = min(*ovf_n, ovf_cap);
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += gridDim.x * blockDim.x) {
-    const int32_t db = ovf_dest[i];
-    sorted[fstart[db] + atomicAdd(&fcursor[db], 1)] = i;
+  for (int32_t i0 = blockIdx.x * 256; i0 < nf; i0 += gridDim.x * 256) {
+    const int32_t i = i0 + (int32_t)threadIdx.x;
+    ovf_add(fcount, i < nf ? ovf_dest[i] : -1);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_ovf_scatter(const int32_t *ovf_n, int32_t ovf_cap, const int32_t *ovf_dest,
+                                                     const int32_t *fstart, int32_t *fcursor, int32_t *sorted) {
+  const int32_t nf = min(*ovf_n, ovf_cap);
+  for (int32_t i0 = blockIdx.x * 256; i0 < nf; i0 += gridDim.x * 256) {
+    const int32_t i = i0 + (int32_t)threadIdx.x, db = i < nf ? ovf_dest[i] : -1;
+    const int32_t k = ovf_add(fcursor, db);
+    if (db >= 0) sorted[fstart[db] + k] = i;
   }
 }
 
@@ -980,7 +811,7 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
   const int64_t n = a.n;
   const int32_t nin = st.fill[u];
   if (nin > st.cap) {  // listed for the global-memory kernel
-    if (tid == 0) st.over_units[atomicAdd(&st.over[1], 1)] = u;
+    if (tid == 0) st.over_units[atomicAdd(st.over, 1)] = u;
     return;
   }
   const int64_t at = (int64_t)u * st.cap;
@@ -1345,7 +1176,7 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
 // units in turn.
 template <int D>
 __global__ void __launch_bounds__(kPullThreads) k_brick_pull(DevTree t, BrickGeom g, BrickPullArgs a) {
-  const int32_t m = min(a.st.over[1], (int32_t)(2 * g.n_bricks));
+  const int32_t m = min(*a.st.over, (int32_t)(2 * g.n_bricks));
   for (int32_t i = blockIdx.x; i < m; i += gridDim.x) {
     brick_pull_fallback<D>(t, g, a, a.st.over_units[i]);
     __syncthreads();
@@ -1383,7 +1214,7 @@ __global__ void __launch_bounds__(256) k_expand_leaves(const int32_t *__restrict
 void launch_brick_push(const DevTree &t, const BrickGeom &g, const BrickPushArgs &pa, cudaStream_t s) {
   cudaMemsetAsync(pa.st.fill, 0, sizeof(int32_t) * 2 * g.n_bricks, s);
   cudaMemsetAsync(pa.st.ovf_n, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(pa.st.over, 0, 2 * sizeof(int32_t), s);
+  cudaMemsetAsync(pa.st.over, 0, sizeof(int32_t), s);
   const unsigned nb = (unsigned)g.n_bricks;
   const bool al = pa.n % 4 == 0;
   const unsigned np = std::min(2 * nb, kPersistBlocks);
@@ -1394,10 +1225,7 @@ void launch_brick_push(const DevTree &t, const BrickGeom &g, const BrickPushArgs
     if (al) k_brick_push_st<2, true><<<np, kHThreads, push_st_smem<2>(), s>>>(t, g, pa);
     else k_brick_push_st<2, false><<<np, kHThreads, push_st_smem<2>(), s>>>(t, g, pa);
   }
-  const unsigned nf = std::min(nb, kFallbackBlocks);  // the fallback visits every brick with fewer blocks
-  if (g.d == 3) k_brick_push<3><<<nf, kPushThreads, 0, s>>>(t, g, pa);
-  else k_brick_push<2><<<nf, kPushThreads, 0, s>>>(t, g, pa);
-  count_launches(2);
+  count_launches(1);
 }
 
 void launch_brick_pull(const DevTree &t, const BrickGeom &g, const BrickPullArgs &qa, int32_t *fcount,
@@ -1405,9 +1233,9 @@ void launch_brick_pull(const DevTree &t, const BrickGeom &g, const BrickPullArgs
   const int64_t nu = 2 * g.n_bricks;  // destination units
   cudaMemsetAsync(fcount, 0, sizeof(int32_t) * nu, s);
   cudaMemsetAsync(fcursor, 0, sizeof(int32_t) * nu, s);
-  k_ovf_count<<<64, 256, 0, s>>>(qa.st.ovf_n, qa.st.ovf_cap, qa.st.ovf_dest, fcount);
+  k_ovf_count<<<kPersistBlocks, 256, 0, s>>>(qa.st.ovf_n, qa.st.ovf_cap, qa.st.ovf_dest, fcount);
   launch_exclusive_scan(fcount, nu, qa.fstart_w, tile_sums, scratch_total, s);
-  k_ovf_scatter<<<64, 256, 0, s>>>(qa.st.ovf_n, qa.st.ovf_cap, qa.st.ovf_dest, qa.fstart, fcursor, qa.ovf_sorted_w);
+  k_ovf_scatter<<<kPersistBlocks, 256, 0, s>>>(qa.st.ovf_n, qa.st.ovf_cap, qa.st.ovf_dest, qa.fstart, fcursor, qa.ovf_sorted_w);
   k_brick_totals<<<(unsigned)((nu + 255) / 256), 256, 0, s>>>(nu, qa.st.cap, qa.st.fill, qa.fstart, qa.tot_w);
   launch_exclusive_scan(qa.tot_w, nu, qa.bstart_w, tile_sums, scratch_total, s);
   if (g.d == 3) {

@@ -38,3 +38,28 @@ def test_steps_replays_and_deposits(d, n):
         assert np.array_equal(a.deposit(), b.deposit())
         assert np.array_equal(a.bins()[1], b.bins()[1])
         assert a.stats().movers == b.stats().movers and a.stats().max_bucket == b.stats().max_bucket
+
+
+# one brick among 9 (27) sparse ones: parts of up to 3,200 particles, their last one full or short, and units whose
+# arrivals overflow
+@pytest.mark.parametrize("d", [2, 3])
+@pytest.mark.parametrize("dense", [6400, 6401, 9599, 9600, 9601, 12801, 50_003])
+def test_uneven_bricks(d, dense):
+    rng = np.random.default_rng(dense)
+    flags = W.uniform_tree_flags(d, 3)
+    x, v = W.random_particles(d, dense + 1001, 4, vmax=0.3)
+    x[:, :dense] = (1 + rng.random((d, dense))) / 3
+    order = rng.permutation(x.shape[1])
+    x, v = x[:, order], v[:, order]
+    kw = dict(q=-1.0 / x.shape[1], ion=1.0, sweeps=5, scheme=pic.PIT, precision=pic.FP32_SPLIT)
+    a = pic.Pic(d, flags, x, v, track_ids=True, **kw)
+    assert a.info().brick == 1
+    b = pic.Pic(d, flags, x, v, path=pic.PATH_GENERIC, track_ids=True, **kw)
+    for _ in range(4):
+        a.step(0.05)
+        b.step(0.05)
+        for p, q in zip(a.get_state(), b.get_state()):
+            assert np.array_equal(p, q)
+        assert np.array_equal(a.bins()[1], b.bins()[1])
+        assert np.array_equal(a.deposit(), b.deposit())
+        assert a.stats().movers == b.stats().movers and a.stats().max_bucket == b.stats().max_bucket
