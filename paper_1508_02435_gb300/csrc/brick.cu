@@ -41,7 +41,7 @@ constexpr uint16_t kStayBit = 0x8000;
 constexpr uint16_t kMoverCode = 0;   // leaf code flags of an arrival from another leaf
 constexpr unsigned kFallbackBlocks = 608;  // blocks of the global-memory pull (4 per SM)
 constexpr unsigned kPersistBlocks = 304;   // CTAs of K1's shared-memory kernel (2 per SM, each taking half bricks in turn)
-constexpr int kPullThreads = 256;
+constexpr int kPullThreads = 512;
 
 // Compile-time brick shape: B = 9 leaves per axis (two levels).
 template <int D>
@@ -733,17 +733,10 @@ size_t pull_st_smem() {
   return (sizeof(float) * 2 * D + sizeof(uint32_t) + 2 * sizeof(uint16_t)) * kStCap;
 }
 
-// Sorts the m <= N arrival indices mp[0..m) of one leaf by their keys
-// (distinct) with Batcher's odd-even merge network (5, 19 and 63 comparators
-// for N = 4, 8, 16) over (key, index) pairs in registers.
-template <int N>
-__device__ __forceinline__ void sort_leaf_net(uint16_t *mp, int m, const uint32_t *key) {
-  uint32_t k[N], v[N];
-#pragma unroll
-  for (int t = 0; t < N; ++t) {
-    v[t] = t < m ? mp[t] : 0u;
-    k[t] = t < m ? key[v[t]] : 0xffffffffu;
-  }
+// Batcher's odd-even merge network over N (key, value) pairs in registers (5, 19
+// and 63 comparators for N = 4, 8, 16).
+template <int N, typename V>
+__device__ __forceinline__ void sort_net(uint32_t *k, V *v) {
 #pragma unroll
   for (int p = 1; p < N; p <<= 1)
 #pragma unroll
@@ -755,12 +748,25 @@ __device__ __forceinline__ void sort_leaf_net(uint16_t *mp, int m, const uint32_
           if (i < c && i < N - j - c && (i + j) / (2 * p) == (i + j + c) / (2 * p)) {
             const int x = i + j, y = i + j + c;
             const bool sw = k[x] > k[y];
-            const uint32_t tk = k[x], tv = v[x];
+            const uint32_t tk = k[x];
+            const V tv = v[x];
             k[x] = sw ? k[y] : tk;
             v[x] = sw ? v[y] : tv;
             k[y] = sw ? tk : k[y];
             v[y] = sw ? tv : v[y];
           }
+}
+
+// Sorts the m <= N arrival indices mp[0..m) of one leaf by their keys (distinct).
+template <int N>
+__device__ __forceinline__ void sort_leaf_net(uint16_t *mp, int m, const uint32_t *key) {
+  uint32_t k[N], v[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    v[t] = t < m ? mp[t] : 0u;
+    k[t] = t < m ? key[v[t]] : 0xffffffffu;
+  }
+  sort_net<N>(k, v);
 #pragma unroll
   for (int t = 0; t < N; ++t)
     if (t < m) mp[t] = (uint16_t)v[t];
@@ -1019,10 +1025,13 @@ __global__ void __launch_bounds__(kStThreads, 2) k_brick_pull_st(DevTree t, Bric
 // K2 for units over their staging capacity: the staging area (first cap
 // arrivals) and the unit's overflow arrivals; a counting sort by leaf in
 // global scratch (fb_key / fb_idx at the unit's output range), a per-leaf
-// sort by key (insertion by one thread up to kPullSmallLeaf arrivals, the
-// block's bitonic network above), then gathers in bucket order.  Arrival r < cap is
-// staging slot r, arrival cap + k the unit's k-th overflow entry.
-constexpr int kPullSmallLeaf = 32;  // leaves up to this many arrivals: one thread's insertion sort
+// sort by key (in one thread's registers up to 16 arrivals, a warp's up to
+// kPullSmallLeaf, the block's bitonic network above), then gathers in bucket
+// order.  Arrival r < cap is staging slot r, arrival cap + k the unit's k-th
+// overflow entry.  A unit is a chain of memory latencies: with a thread's
+// insertion sorts in memory, 256 threads and one load in flight each, 157 to 194 us
+// for the full units of an 81^3 plasma with density waves; this form 92 to 98.
+constexpr int kPullSmallLeaf = 32;
 constexpr int kPullChunk = 2048;    // (key, index) pairs of a crowded leaf sorted at once in shared memory
 
 template <int D>
@@ -1055,7 +1064,14 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
   for (int i = tid; i <= nlf; i += blockDim.x) cnt[i] = 0;
   if (tid == 0) s_max = 0;
   __syncthreads();
-  for (int32_t r = tid; r < nin; r += blockDim.x) atomicAdd(&cnt[leaf_of(r)], 1);
+  for (int32_t r0 = tid; r0 < nin; r0 += 4 * kPullThreads) {  // four codes in flight
+    int lf[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) lf[i] = r0 + i * kPullThreads < nin ? leaf_of(r0 + i * kPullThreads) : -1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (lf[i] >= 0) atomicAdd(&cnt[lf[i]], 1);
+  }
   __syncthreads();
   int32_t carry = 0;
   for (int base = 0; base < nlf; base += blockDim.x) {
@@ -1084,28 +1100,48 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
   if (tid == 0) cnt[nlf] = carry;
   __syncthreads();
   const int32_t bstart = a.bstart[u];
-  for (int32_t r = tid; r < nin; r += blockDim.x) {
-    const int32_t p = bstart + atomicAdd(&cur[leaf_of(r)], 1);
-    a.fb_key[p] = key_of(r);
-    a.fb_idx[p] = r;
+  for (int32_t r0 = tid; r0 < nin; r0 += 4 * kPullThreads) {
+    int lf[4];
+    uint32_t key[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int32_t r = r0 + i * kPullThreads;
+      lf[i] = r < nin ? leaf_of(r) : -1;
+      key[i] = r < nin ? key_of(r) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (lf[i] >= 0) {
+        const int32_t p = bstart + atomicAdd(&cur[lf[i]], 1);
+        a.fb_key[p] = key[i];
+        a.fb_idx[p] = r0 + i * kPullThreads;
+      }
   }
   __syncthreads();
   for (int l = tid; l < nlf; l += blockDim.x) {
     a.new_start[L0 + l] = bstart + cnt[l];
-    const int32_t lo = bstart + cnt[l], hi = bstart + cnt[l + 1];
-    if (hi - lo > kPullSmallLeaf) continue;  // crowded: sorted by the whole block below
-    for (int32_t i = lo + 1; i < hi; ++i) {
-      const uint32_t kx = a.fb_key[i];
-      const int32_t vx = a.fb_idx[i];
-      int32_t j = i - 1;
-      while (j >= lo && a.fb_key[j] > kx) {
-        a.fb_key[j + 1] = a.fb_key[j];
-        a.fb_idx[j + 1] = a.fb_idx[j];
-        --j;
-      }
-      a.fb_key[j + 1] = kx;
-      a.fb_idx[j + 1] = vx;
+    const int32_t lo = bstart + cnt[l], m = cnt[l + 1] - cnt[l];
+    if (m > 16) continue;
+    uint32_t k[16];
+    int32_t v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      k[i] = i < m ? a.fb_key[lo + i] : 0xffffffffu;
+      v[i] = i < m ? a.fb_idx[lo + i] : 0;
     }
+    sort_net<16>(k, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < m) a.fb_idx[lo + i] = v[i];  // the keys are not needed any more
+  }
+  for (int l = w; l < nlf; l += nw) {  // a warp per fuller leaf
+    const int32_t lo = bstart + cnt[l], m = cnt[l + 1] - cnt[l];
+    if (m <= 16 || m > kPullSmallLeaf) continue;
+    const uint32_t kx = lane < m ? a.fb_key[lo + lane] : 0xffffffffu;
+    const int32_t vx = lane < m ? a.fb_idx[lo + lane] : 0;
+    int32_t r = 0;
+    for (int i = 0; i < m; ++i) r += __shfl_sync(0xffffffffu, kx, i) < kx;
+    if (lane < m) a.fb_idx[lo + r] = vx;
   }
   __syncthreads();
   for (int l = 0; l < nlf; ++l) {  // crowded leaves, one at a time, by the whole block
@@ -1150,7 +1186,9 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
       float acc[K::NC];
 #pragma unroll
       for (int e = 0; e < K::NC; ++e) acc[e] = 0.0f;
-      for (int32_t p = bstart + cnt[l]; p < bstart + cnt[l + 1]; ++p) {
+      const int32_t hi = bstart + cnt[l + 1];
+#pragma unroll 4
+      for (int32_t p = bstart + cnt[l]; p < hi; ++p) {
         float o[D], om[D];
 #pragma unroll
         for (int ax = 0; ax < D; ++ax) {
@@ -1175,7 +1213,7 @@ __device__ __forceinline__ void brick_pull_fallback(const DevTree &t, const Bric
 // the shared-memory kernel), from global memory; the blocks take the listed
 // units in turn.
 template <int D>
-__global__ void __launch_bounds__(kPullThreads) k_brick_pull(DevTree t, BrickGeom g, BrickPullArgs a) {
+__global__ void __launch_bounds__(kPullThreads, 2) k_brick_pull(DevTree t, BrickGeom g, BrickPullArgs a) {
   const int32_t m = min(*a.st.over, (int32_t)(2 * g.n_bricks));
   for (int32_t i = blockIdx.x; i < m; i += gridDim.x) {
     brick_pull_fallback<D>(t, g, a, a.st.over_units[i]);
