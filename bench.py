@@ -47,9 +47,9 @@ _BRICK_SOURCES = ("paper_1508_02435_gb300/csrc/brick.cu", "paper_1508_02435_gb30
                   "paper_1508_02435_gb300/csrc/segsort.cuh", "paper_1508_02435_gb300/csrc/launch.hpp")
 # the sources each measured kernel is compiled from
 KERNEL_SOURCES = {"k_brick_push_st": _BRICK_SOURCES, "k_brick_pull_st": _BRICK_SOURCES,
-                  "k_vertex_charge": ("paper_1508_02435_gb300/csrc/kernels.cu", "paper_1508_02435_gb300/csrc/dev.cuh",
-                                      "paper_1508_02435_gb300/csrc/launch.hpp")}
-PHASE_KERNEL = {"push": "k_brick_push_st", "rebin": "k_brick_pull_st", "deposit": "k_vertex_charge"}
+                  "k_vertex_charge_tile": tuple("paper_1508_02435_gb300/csrc/" + f for f in (
+                      "kernels.cu", "deposit.cuh", "uniform_solve.cuh", "rebin.cuh", "dev.cuh", "launch.hpp"))}
+PHASE_KERNEL = {"push": "k_brick_push_st", "rebin": "k_brick_pull_st", "deposit": "k_vertex_charge_tile"}
 
 
 def kernel_digest(kernel: str) -> str:
@@ -773,7 +773,7 @@ def main():
     shares = step_shares(d, split, cfg["ppc"], bool(info.brick))
     names = {"push": "k_brick_push_st (gather + kick + drift + re-location + append to the destination's staging area)",
              "rebin": "k_brick_pull_st (+ overflow and unit-offset helpers): canonical re-bin + corner partials",
-             "deposit": "k_vertex_charge (vertex sums of the corner partials)"} if info.brick else {}
+             "deposit": "k_vertex_charge_tile (vertex sums of the corner partials)"} if info.brick else {}
     dom = max(("deposit", "push", "rebin", "permute"), key=lambda k: phases[k][0])
     dom_ms = phases[dom][0] / args.steps
     achieved = shares[dom] * n / (dom_ms / 1e3) / 1e9

@@ -8,8 +8,9 @@
 // vertex instead of 2^d).  The order of every FP32 sum is that of the
 // leaf-by-leaf assembly; FP64 uses fused multiply-adds.
 //
-// One sweep of the 1e6-particle bump (2D, 75,451 vertices, FP64): 64 -> 10.5 us,
-// two dependent launches.
+// One sweep of the 1e6-particle bump (2D, 75,451 vertices, FP64): 64 -> 9.9 us, two
+// dependent launches.  FP64 handles take assembled rows where row_solve.cuh has
+// built them (4.0 us); FP32 sums must keep this order, so FP32 stays here.
 #pragma once
 
 namespace pic {

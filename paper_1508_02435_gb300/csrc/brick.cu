@@ -1353,10 +1353,11 @@ int32_t brick_stage_cap(int64_t n, int64_t n_units) {
   return (int32_t)std::min<int64_t>(kStCap, (want + 7) & ~(int64_t)7);
 }
 
-// A half brick over kHalfCap goes through the global-memory kernels. When the
-// mean is over it nearly all do, and the generic passes are the faster way
-// (243 x 243 cells of 100 particles: 1.96 ms a step with the global-memory brick
-// kernels, 0.45 ms generic); below it the fallbacks take the few crowded ones.
+// When the mean is over kHalfCap per half brick, nearly every unit overflows its
+// staging area, and the generic passes are the faster way (243 x 243 cells of 100
+// particles: 2.1 ms a step with the brick kernels, 0.26 ms generic; 81^3 cells of
+// 10: 0.56, 0.28 ms); below it the parts and the global pull take the few crowded
+// ones.
 bool brick_crowded(int64_t n, int64_t n_units) { return n > n_units * kHalfCap; }
 
 cudaError_t brick_configure(const BrickGeom &g) {

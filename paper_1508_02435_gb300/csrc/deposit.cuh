@@ -14,7 +14,7 @@ namespace pic {
 // thread per leaf waits for each particle in turn.  One thread a leaf -> here:
 // 2e8 two-stream particles, 14 a leaf in 8 sub-buckets, 2.5 -> 1.7 ms; 256 2D
 // plasmas with up to 1,370 particles a leaf 304 -> 230 us; 81^3 cells of 8 FP64
-// 540 -> 289 us; the FP64 2D bump 177 -> 37 us.)
+// 540 -> 340 us; the FP64 2D bump 177 -> 37 us.)
 
 // What a particle's lane hands over, and the contribution lane e takes from it.
 template <typename T, int D>

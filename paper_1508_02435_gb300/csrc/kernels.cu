@@ -2,7 +2,7 @@
 //
 // Step structure (Section 3 PIC cycle + Section 5 re-binning):
 //   deposit   k_leaf_partials -> k_vertex_charge -> k_sum_blocks        (item 1)
-//   solve     k_rhs -> k_jacobi x sweeps (auxiliary)                    (item 2)
+//   solve     k_rhs -> sweeps of uniform_solve / adaptive_solve / row_solve / resident_solve (auxiliary, item 2)
 //   field     k_efield                                                  (item 3)
 //   push      k_push64 / k_push32: gather E_i = R^T(x_i) E, leapfrog kick
 //             and drift, wrap, re-location (descent / split resolve), new

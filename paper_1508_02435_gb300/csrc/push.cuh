@@ -8,10 +8,11 @@
 //
 // Measured against one kernel for all trees with divisions by 3^k, a descent
 // from the root and separate FP64 products and sums: FP64 push of 4.25e6
-// particles on 81^3 cells 0.98 -> 0.49 ms, FP64 push of the 1e6-particle 2D bump
+// particles on 81^3 cells 0.98 -> 0.52 ms, FP64 push of the 1e6-particle 2D bump
 // 0.19 -> 0.07 ms (adaptive FP64 trees now expand the field at the leaf corners
 // once per field, as FP32 did), 1e7 free 2D particles in a reflecting box 0.17 ->
-// 0.13 ms, 2e8 two-stream particles 7.3 -> 6.6 ms.
+// 0.11 ms, 2e8 two-stream particles 7.3 -> 5.03 ms (whole-sector corner rows and
+// records, four blocks per SM).
 #pragma once
 
 namespace pic {

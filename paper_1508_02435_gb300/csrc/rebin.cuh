@@ -20,10 +20,10 @@
 // No pass runs over one bucket per thread, and stayers take no atomic.
 // Measured per step, before (a thread per bucket for the stayers and for the
 // mover sort, a mover list, a second atomic) -> now: re-bin and permutation of
-// the 2e8-particle 3D two-stream PIDT step 9.4 -> 5.7 ms (the push 6.8 -> 7.3 ms,
-// it waits for the ranks); whole step of 256 2D plasmas, 3.5e7 particles,
-// 3.26 -> 1.50 ms; 1e7 free 2D particles 0.49 -> 0.17 ms.  Three launches fewer
-// for large trees, eight for small ones.
+// the 2e8-particle 3D two-stream PIDT step 9.4 -> 5.7 ms (the push waits for the
+// ranks, some 0.5 ms); whole step of 256 2D plasmas, 3.5e7 particles, 3.26 ->
+// 1.50 ms; 1e7 free 2D particles 0.49 -> 0.16 ms.  Three launches fewer for large
+// trees, eight for small ones.
 #pragma once
 
 namespace pic {
