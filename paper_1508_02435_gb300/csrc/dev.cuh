@@ -35,7 +35,6 @@ struct DevTree {
   int32_t block_push, block_leaf, block_vert;  // threads per block (autotuned; 0 = 256)
   const InstInfo *inst;
   const int32_t *inst_of_leaf, *inst_of_vert;
-  const int32_t *inst_of_block;  // batches: instance of particle 256 i
   int64_t n_leaves, n_vert, n_pv, n_keys;
   int32_t M;  // 3^depth
   const TabEntry *tab;

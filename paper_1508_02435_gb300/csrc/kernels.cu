@@ -865,11 +865,13 @@ void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s) {
   COUNT(1);
   const unsigned b = bsz(t.block_push), g = grid_for(a.n, b);
   if (t.d == 3) {
-    if (t.uniform) k_push32<3, true><<<g, b, 0, s>>>(t, a);
-    else k_push32<3, false><<<g, b, 0, s>>>(t, a);
+    if (t.n_inst > 1) k_push32<3, true, true><<<g, b, 0, s>>>(t, a);
+    else if (t.uniform) k_push32<3, true, false><<<g, b, 0, s>>>(t, a);
+    else k_push32<3, false, false><<<g, b, 0, s>>>(t, a);
   } else {
-    if (t.uniform) k_push32<2, true><<<g, b, 0, s>>>(t, a);
-    else k_push32<2, false><<<g, b, 0, s>>>(t, a);
+    if (t.n_inst > 1) k_push32<2, true, true><<<g, b, 0, s>>>(t, a);
+    else if (t.uniform) k_push32<2, true, false><<<g, b, 0, s>>>(t, a);
+    else k_push32<2, false, false><<<g, b, 0, s>>>(t, a);
   }
 }
 
@@ -877,11 +879,13 @@ void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s) {
   COUNT(1);
   const unsigned b = bsz(t.block_push), g = grid_for(a.n, b);
   if (t.d == 3) {
-    if (t.uniform) k_push64<3, true><<<g, b, 0, s>>>(t, a);
-    else k_push64<3, false><<<g, b, 0, s>>>(t, a);
+    if (t.n_inst > 1) k_push64<3, true, true><<<g, b, 0, s>>>(t, a);
+    else if (t.uniform) k_push64<3, true, false><<<g, b, 0, s>>>(t, a);
+    else k_push64<3, false, false><<<g, b, 0, s>>>(t, a);
   } else {
-    if (t.uniform) k_push64<2, true><<<g, b, 0, s>>>(t, a);
-    else k_push64<2, false><<<g, b, 0, s>>>(t, a);
+    if (t.n_inst > 1) k_push64<2, true, true><<<g, b, 0, s>>>(t, a);
+    else if (t.uniform) k_push64<2, true, false><<<g, b, 0, s>>>(t, a);
+    else k_push64<2, false, false><<<g, b, 0, s>>>(t, a);
   }
 }
 

@@ -575,15 +575,6 @@ int install_tree(pic_t h, const pic_tree_desc *tree, std::vector<DevBuf> *old = 
 int set_particle_offsets(pic_t h, const std::vector<int64_t> &poff) {
   for (size_t i = 0; i < h->inst.size(); ++i) h->inst[i].poff = poff[i];
   CK(cudaMemcpy((void *)h->dt.inst, h->inst.data(), sizeof(InstInfo) * h->inst.size(), cudaMemcpyHostToDevice));
-  if (poff.size() > 1) {
-    std::vector<int32_t> blk((h->n >> 8) + 1);
-    size_t i = 0;
-    for (size_t b = 0; b < blk.size(); ++b) {
-      while (i + 1 < poff.size() && poff[i + 1] <= (int64_t)b << 8) ++i;
-      blk[b] = (int32_t)i;
-    }
-    return gupload(h, h->tree_bufs, &h->dt.inst_of_block, blk);
-  }
   return PIC_OK;
 }
 
