@@ -306,7 +306,9 @@ PIC_API int pic_get_particles(pic_t h, double *x, double *v, int32_t where);
  * handle's precision), for checkpoints and host round trips.
  * FP64: x[d][n], v[d][n] (double).  Split: leaf[n] (int32), o[d][n], v[d][n]
  * (float).  Unused pointers may be NULL.  pic_set_state replaces the particles
- * (same n) and re-bins them. */
+ * (same n) and re-bins them; it is done with the given arrays, device ones
+ * included, when it returns.  A split state of a batch may hold other numbers of
+ * particles per instance than before: a particle belongs to its leaf's instance. */
 PIC_API int pic_get_state(pic_t h, int32_t *leaf, void *x_or_o, void *v, int32_t where);
 PIC_API int pic_set_state(pic_t h, const int32_t *leaf, const void *x_or_o, const void *v,
                   int32_t where);

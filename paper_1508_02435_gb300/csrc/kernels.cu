@@ -898,11 +898,13 @@ void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s) {
 }
 
 // A given split state (leaf + offsets) as fresh particles, one pass: keys, ranks,
-// whether the keys ascend, and in 3D the records the gather reads.  Flags leaves
-// outside the tree and offsets outside [0,1).
+// whether the keys ascend, and what the gather reads -- in 3D the records, in 2D
+// the rows (r.o NULL: the state is in them already).  It is the only pass over the
+// given arrays, which may be the caller's.  Flags leaves outside the tree and
+// offsets outside [0,1).
 template <int D>
 __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restrict__ o, const float *__restrict__ v,
-                          int64_t n, int32_t *key /* may be leaf */, float4 *__restrict__ rec,
+                          int64_t n, int32_t *key /* may be leaf */, float4 *__restrict__ rec, StateRows r,
                           int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = p < n;
@@ -924,9 +926,16 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
     key[p] = k;
     if (bad) atomicOr(err, 2);
     if (D == 3) {
-      const float r[8] = {oo[0],    oo[1],    oo[D - 1], v[p], v[n + p], v[(D - 1) * n + p], __int_as_float(L),
+      const float q[8] = {oo[0],    oo[1],    oo[D - 1], v[p], v[n + p], v[(D - 1) * n + p], __int_as_float(L),
                           __int_as_float(k)};
-      store32((float *)(rec + 2 * p), r);
+      store32((float *)(rec + 2 * p), q);
+    } else if (r.o) {
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        r.o[a * n + p] = oo[a];
+        r.v[a * n + p] = v[a * n + p];
+      }
+      if (r.leaf != key) r.leaf[p] = L;  // PIT keys are the leaves
     }
   }
   int32_t prev = __shfl_up_sync(0xffffffffu, k, 1);
@@ -942,14 +951,31 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
 }
 
 void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const float *v, int64_t n, int32_t *key,
-                    void *rec, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err,
-                    cudaStream_t s) {
+                    void *rec, const StateRows &r, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted,
+                    int32_t *err, cudaStream_t s) {
   if (n <= 0) return;
   COUNT(1);
   if (t.d == 3)
-    k_fresh32<3><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, count, words, rank, unsorted, err);
+    k_fresh32<3><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, count, words, rank, unsorted, err);
   else
-    k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, count, words, rank, unsorted, err);
+    k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, count, words, rank, unsorted, err);
+}
+
+// The rows of a state in records (3D, split).
+__global__ void k_record_rows(int64_t n, const float *__restrict__ rec, StateRows r) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  float q[8];
+  load32(rec + 8 * p, q);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r.o[k * n + p] = q[k];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r.v[k * n + p] = q[3 + k];
+  r.leaf[p] = __float_as_int(q[6]);
+}
+
+void launch_record_rows(int64_t n, const void *rec, const StateRows &r, cudaStream_t s) {
+  if (n > 0) { COUNT(1); k_record_rows<<<grid_for(n), kBlock, 0, s>>>(n, (const float *)rec, r); }
 }
 
 // Records of a fresh 3D state in rows: the gather then reads one 32- or 64-byte

@@ -925,13 +925,9 @@ int brick_push_and_rebin(pic_t h, double dt) {
 }
 
 // Stable re-bin of the pushed state into the current state [0]: from the
-// records (records; 3D) or from rows ([1] unless given).
+// records (records; 3D) or from the rows [1].
 // old_start == NULL: fresh particles, every one counted as a mover.
-struct Rows {  // positions (offsets), velocities, leaves of a pushed or fresh state
-  const void *pos, *vel;
-  const int32_t *leaf;
-};
-int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false, const Rows *rows = nullptr) {
+int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
   cudaStream_t s = h->stream;
   const int64_t n = h->n;
   RebinArgs r{};
@@ -962,8 +958,7 @@ int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false, co
     launch_gather_records(h->split, r, h->prec, h->pos[0], h->vel[0], h->leaf[0], pidt ? h->key[0] : nullptr,
                           ids ? h->ids[0] : nullptr, ids ? h->ids[1] : nullptr, s);
   else
-    launch_gather_state(h->split, r, h->d, rows ? rows->pos : h->pos[1], h->pos[0], rows ? rows->vel : h->vel[1],
-                        h->vel[0], rows ? rows->leaf : h->leaf[1], h->leaf[0],
+    launch_gather_state(h->split, r, h->d, h->pos[1], h->pos[0], h->vel[1], h->vel[0], h->leaf[1], h->leaf[0],
                         pidt ? h->key[1] : nullptr, pidt ? h->key[0] : nullptr, ids ? h->ids[0] : nullptr,
                         ids ? h->ids[1] : nullptr, s);
   if (ids) std::swap(h->ids[0], h->ids[1]);
@@ -1014,27 +1009,25 @@ int bin_fresh(pic_t h) {
 }
 
 // A split state handed over (host: copied to [1] first; device: read where it
-// is) as fresh particles.
+// is) as fresh particles.  The caller may overwrite or free its arrays when the
+// call returns, on any stream: one pass reads them, and it is over when the order
+// flag is here.  (2D, 2e7 particles in no order: NN ms; copies first as for host
+// arrays MM ms.)
 int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v, bool copied) {
   h->q_valid = false;
   cudaStream_t s = h->stream;
-  const int64_t n = h->n, m = n * h->d;
+  const int64_t n = h->n;
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
   CK(cudaMemsetAsync(h->scalars + 5, 0, sizeof(int32_t) * 3, s));  // segment lists and the order flag
-  launch_fresh32(h->dt, leaf, o, v, n, h->key[1], h->prec, h->count, h->words, h->rank, h->scalars + 6, h->err, s);
+  const StateRows rows{(float *)h->pos[1], (float *)h->vel[1], h->leaf[1]};
+  launch_fresh32(h->dt, leaf, o, v, n, h->key[1], h->prec, copied ? StateRows{} : rows, h->count, h->words, h->rank,
+                 h->scalars + 6, h->err, s);
   int32_t unsorted = 1;
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (unsorted) {
-    const Rows rows{o, v, h->scheme == PIC_PIT ? h->leaf[1] : leaf};  // PIT: the keys just written
-    return rebin_and_gather(h, nullptr, h->prec != nullptr, &rows);
-  }
-  if (!copied) {
-    CK(cudaMemcpyAsync(h->pos[1], o, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
-    CK(cudaMemcpyAsync(h->vel[1], v, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
-    if (h->scheme != PIC_PIT) CK(cudaMemcpyAsync(h->leaf[1], leaf, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-  }
+  if (unsorted) return rebin_and_gather(h, nullptr, h->prec != nullptr);
+  if (!copied && h->prec) launch_record_rows(n, h->prec, rows, s);
   return take_sorted(h);
 }
 
