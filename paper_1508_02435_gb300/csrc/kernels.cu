@@ -961,6 +961,17 @@ void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const
     k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, count, words, rank, unsorted, err);
 }
 
+// Two offsets and two velocities of a 2D particle side by side.
+__global__ void k_pack_rows(int64_t n, const float *__restrict__ o, const float *__restrict__ v,
+                            float4 *__restrict__ quad) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p < n) quad[p] = make_float4(o[p], o[n + p], v[p], v[n + p]);
+}
+
+void launch_pack_rows(int64_t n, const float *o, const float *v, void *quad, cudaStream_t s) {
+  if (n > 0) { COUNT(1); k_pack_rows<<<grid_for(n), kBlock, 0, s>>>(n, o, v, (float4 *)quad); }
+}
+
 // The rows of a state in records (3D, split).
 __global__ void k_record_rows(int64_t n, const float *__restrict__ rec, StateRows r) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

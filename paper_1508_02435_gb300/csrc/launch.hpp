@@ -238,7 +238,9 @@ void launch_exclusive_scan(const int32_t *in, int64_t n, int32_t *out, int32_t *
 void launch_rebin(const RebinArgs &r, cudaStream_t s);
 // The pushed state into bucket order after launch_rebin, in one kernel: from the
 // rows (positions, velocities [d][n], leaves and, where not NULL, keys and ids;
-// split: float, else double) or from the records of the 3D step.  key NULL: PIT.
+// split: float, else double; 2D, split, v NULL: x holds a float4 per particle,
+// launch_pack_rows) or from the records of the 3D step.  key NULL: PIT.
+void launch_pack_rows(int64_t n, const float *o, const float *v, void *quad, cudaStream_t s);
 void launch_gather_state(bool split, const RebinArgs &r, int d, const void *x, void *x2, const void *v, void *v2,
                          const int32_t *leaf, int32_t *leaf2, const int32_t *key, int32_t *key2, const int32_t *ids,
                          int32_t *ids2, cudaStream_t s);

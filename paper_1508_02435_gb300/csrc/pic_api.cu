@@ -925,9 +925,9 @@ int brick_push_and_rebin(pic_t h, double dt) {
 }
 
 // Stable re-bin of the pushed state into the current state [0]: from the
-// records (records; 3D) or from the rows [1].
-// old_start == NULL: fresh particles, every one counted as a mover.
-int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
+// records (records; 3D), from the rows [1], or from the rows' packed form (quad;
+// 2D, split).  old_start == NULL: fresh particles, every one counted as a mover.
+int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false, const void *quad = nullptr) {
   cudaStream_t s = h->stream;
   const int64_t n = h->n;
   RebinArgs r{};
@@ -958,9 +958,9 @@ int rebin_and_gather(pic_t h, const int32_t *old_start, bool records = false) {
     launch_gather_records(h->split, r, h->prec, h->pos[0], h->vel[0], h->leaf[0], pidt ? h->key[0] : nullptr,
                           ids ? h->ids[0] : nullptr, ids ? h->ids[1] : nullptr, s);
   else
-    launch_gather_state(h->split, r, h->d, h->pos[1], h->pos[0], h->vel[1], h->vel[0], h->leaf[1], h->leaf[0],
-                        pidt ? h->key[1] : nullptr, pidt ? h->key[0] : nullptr, ids ? h->ids[0] : nullptr,
-                        ids ? h->ids[1] : nullptr, s);
+    launch_gather_state(h->split, r, h->d, quad ? quad : h->pos[1], h->pos[0], quad ? nullptr : h->vel[1], h->vel[0],
+                        h->leaf[1], h->leaf[0], pidt ? h->key[1] : nullptr, pidt ? h->key[0] : nullptr,
+                        ids ? h->ids[0] : nullptr, ids ? h->ids[1] : nullptr, s);
   if (ids) std::swap(h->ids[0], h->ids[1]);
   std::swap(h->start_cur, h->start_new);
   h->leaf_stale = false;
@@ -1011,8 +1011,12 @@ int bin_fresh(pic_t h) {
 // A split state handed over (host: copied to [1] first; device: read where it
 // is) as fresh particles.  The caller may overwrite or free its arrays when the
 // call returns, on any stream: one pass reads them, and it is over when the order
-// flag is here.  (2D, 2e7 particles in no order: NN ms; copies first as for host
-// arrays MM ms.)
+// flag is here.  Large 2D states in no order are packed, so that the gather reads
+// one sector of a particle's offsets and velocities instead of four, whose rows
+// together are more than the L2 holds (2e7 particles, PIT / PIDT: rows 2.27 / 2.94
+// ms, packed 1.57 / 2.17; 5e6: 0.45 / 0.61, 0.39 / 0.51; 1e6: 0.145 / 0.173, 0.150 /
+// 0.167, where the line lies).
+constexpr int64_t kPackRows = 1 << 20;
 int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v, bool copied) {
   h->q_valid = false;
   cudaStream_t s = h->stream;
@@ -1026,7 +1030,11 @@ int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
-  if (unsorted) return rebin_and_gather(h, nullptr, h->prec != nullptr);
+  if (unsorted) {
+    void *quad = h->d == 2 && !copied && n >= kPackRows ? h->Ep : nullptr;  // 16 n of its bytes
+    if (quad) launch_pack_rows(n, rows.o, rows.v, quad, s);
+    return rebin_and_gather(h, nullptr, h->prec != nullptr, quad);
+  }
   if (!copied && h->prec) launch_record_rows(n, h->prec, rows, s);
   return take_sorted(h);
 }

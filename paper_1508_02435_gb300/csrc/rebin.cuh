@@ -387,7 +387,8 @@ struct SlotOrder {
 // has twice the bytes per read and gains nothing.
 template <typename T>
 __host__ __device__ constexpr int rows_per_thread() { return sizeof(T) == 4 ? 2 : 1; }
-template <typename T, int D>
+// kQuad: x is one float4 per particle (two offsets, two velocities).
+template <typename T, int D, bool kQuad>
 __global__ void __launch_bounds__(256) k_gather_state(
     SlotOrder so, int64_t n, const T *__restrict__ x, T *__restrict__ x2, const T *__restrict__ v, T *__restrict__ v2,
     const int32_t *__restrict__ leaf, int32_t *__restrict__ leaf2, const int32_t *__restrict__ key,
@@ -404,10 +405,18 @@ __global__ void __launch_bounds__(256) k_gather_state(
     L[u] = leaf[i[u]];
     kk[u] = key ? key[i[u]] : L[u];
     id[u] = ids ? ids[i[u]] : 0;
+    if constexpr (kQuad) {
+      const float4 q = __ldg((const float4 *)x + i[u]);
+      a[u][0] = q.x;
+      a[u][1] = q.y;
+      b[u][0] = q.z;
+      b[u][1] = q.w;
+    } else {
 #pragma unroll
-    for (int k = 0; k < D; ++k) a[u][k] = x[k * n + i[u]];
+      for (int k = 0; k < D; ++k) a[u][k] = x[k * n + i[u]];
 #pragma unroll
-    for (int k = 0; k < D; ++k) b[u][k] = v[k * n + i[u]];
+      for (int k = 0; k < D; ++k) b[u][k] = v[k * n + i[u]];
+    }
   }
 #pragma unroll
   for (int u = 0; u < kRowsVec; ++u) {
@@ -539,17 +548,20 @@ void launch_gather_state(bool split, const RebinArgs &r, int d, const void *x, v
   const unsigned g = grid_for(r.n, 256 * (split ? rows_per_thread<float>() : rows_per_thread<double>()));
   if (split) {
     if (d == 3)
-      k_gather_state<float, 3><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
-                                                    (float *)v2, leaf, leaf2, key, key2, ids, ids2);
+      k_gather_state<float, 3, false><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
+                                                           (float *)v2, leaf, leaf2, key, key2, ids, ids2);
+    else if (v)
+      k_gather_state<float, 2, false><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
+                                                           (float *)v2, leaf, leaf2, key, key2, ids, ids2);
     else
-      k_gather_state<float, 2><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, (const float *)v,
-                                                    (float *)v2, leaf, leaf2, key, key2, ids, ids2);
+      k_gather_state<float, 2, true><<<g, 256, 0, s>>>(so, r.n, (const float *)x, (float *)x2, nullptr, (float *)v2,
+                                                          leaf, leaf2, key, key2, ids, ids2);
   } else if (d == 3) {
-    k_gather_state<double, 3><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
-                                                   (double *)v2, leaf, leaf2, key, key2, ids, ids2);
+    k_gather_state<double, 3, false><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
+                                                          (double *)v2, leaf, leaf2, key, key2, ids, ids2);
   } else {
-    k_gather_state<double, 2><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
-                                                   (double *)v2, leaf, leaf2, key, key2, ids, ids2);
+    k_gather_state<double, 2, false><<<g, 256, 0, s>>>(so, r.n, (const double *)x, (double *)x2, (const double *)v,
+                                                          (double *)v2, leaf, leaf2, key, key2, ids, ids2);
   }
 }
 
