@@ -899,13 +899,13 @@ void launch_jump_table(const DevTree &t, TabEntry *jump, cudaStream_t s) {
 
 // A given split state (leaf + offsets) as fresh particles, one pass: keys, ranks,
 // whether the keys ascend, and what the gather reads -- in 3D the records, in 2D
-// the rows (r.o NULL: the state is in them already).  It is the only pass over the
+// the rows (`given`: the state is in them already).  It is the only pass over the
 // given arrays, which may be the caller's.  Flags leaves outside the tree and
-// offsets outside [0,1).
+// offsets outside [0,1), and stores them as 0: later passes index by both.
 template <int D>
-__global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restrict__ o, const float *__restrict__ v,
+__global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *o, const float *__restrict__ v,
                           int64_t n, int32_t *key /* may be leaf */, float4 *__restrict__ rec, StateRows r,
-                          int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err) {
+                          bool given, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted, int32_t *err) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = p < n;
   auto key_at = [&](int64_t q, float *oo, int32_t *L, bool *bad) {
@@ -914,7 +914,7 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
 #pragma unroll
     for (int a = 0; a < D; ++a) {
       oo[a] = o[a * n + q];
-      if (!(oo[a] >= 0.0f && oo[a] < 1.0f)) *bad = true;
+      if (!(oo[a] >= 0.0f && oo[a] < 1.0f)) { *bad = true; oo[a] = 0.0f; }
     }
     return key_of(t, *L, pidt_corner_o(oo, D));
   };
@@ -929,13 +929,15 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
       const float q[8] = {oo[0],    oo[1],    oo[D - 1], v[p], v[n + p], v[(D - 1) * n + p], __int_as_float(L),
                           __int_as_float(k)};
       store32((float *)(rec + 2 * p), q);
-    } else if (r.o) {
+    }
+    if ((D == 2 && !given) || bad) {
 #pragma unroll
-      for (int a = 0; a < D; ++a) {
-        r.o[a * n + p] = oo[a];
-        r.v[a * n + p] = v[a * n + p];
-      }
+      for (int a = 0; a < D; ++a) r.o[a * n + p] = oo[a];
       if (r.leaf != key) r.leaf[p] = L;  // PIT keys are the leaves
+    }
+    if (D == 2 && !given) {
+#pragma unroll
+      for (int a = 0; a < D; ++a) r.v[a * n + p] = v[a * n + p];
     }
   }
   int32_t prev = __shfl_up_sync(0xffffffffu, k, 1);
@@ -951,14 +953,16 @@ __global__ void k_fresh32(DevTree t, const int32_t *leaf, const float *__restric
 }
 
 void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const float *v, int64_t n, int32_t *key,
-                    void *rec, const StateRows &r, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted,
-                    int32_t *err, cudaStream_t s) {
+                    void *rec, const StateRows &r, bool given, int32_t *count, uint32_t *words, int32_t *rank,
+                    int32_t *unsorted, int32_t *err, cudaStream_t s) {
   if (n <= 0) return;
   COUNT(1);
   if (t.d == 3)
-    k_fresh32<3><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, count, words, rank, unsorted, err);
+    k_fresh32<3><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, given, count, words, rank,
+                                                  unsorted, err);
   else
-    k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, count, words, rank, unsorted, err);
+    k_fresh32<2><<<grid_for(n), kBlock, 0, s>>>(t, leaf, o, v, n, key, (float4 *)rec, r, given, count, words, rank,
+                                                  unsorted, err);
 }
 
 // Two offsets and two velocities of a 2D particle side by side.

@@ -171,11 +171,12 @@ struct StateRows {
   int32_t *leaf;
 };
 // A given split state as fresh particles: keys, ranks, *unsorted = 1 unless the
-// keys ascend; the state itself into the records (3D) or, unless r.o is NULL, the
-// rows r (2D).  *err |= 2 where a leaf or an offset is out of range.
+// keys ascend; the state itself into the records (3D) or, unless it is `given`
+// there, the rows r (2D).  *err |= 2 where a leaf or an offset is out of range;
+// such a value is stored as 0, in the rows too.
 void launch_fresh32(const DevTree &t, const int32_t *leaf, const float *o, const float *v, int64_t n, int32_t *key,
-                    void *rec, const StateRows &r, int32_t *count, uint32_t *words, int32_t *rank, int32_t *unsorted,
-                    int32_t *err, cudaStream_t s);
+                    void *rec, const StateRows &r, bool given, int32_t *count, uint32_t *words, int32_t *rank,
+                    int32_t *unsorted, int32_t *err, cudaStream_t s);
 void launch_record_rows(int64_t n, const void *rec, const StateRows &r, cudaStream_t s);
 void launch_check_sorted(const int32_t *key, int64_t n, int32_t *flag, cudaStream_t s);
 void launch_count_all(const int32_t *key, int64_t n, int32_t *count, uint32_t *words, int32_t *rank, cudaStream_t s);

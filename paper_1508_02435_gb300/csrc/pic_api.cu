@@ -1024,7 +1024,7 @@ int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
   CK(cudaMemsetAsync(h->scalars + 5, 0, sizeof(int32_t) * 3, s));  // segment lists and the order flag
   const StateRows rows{(float *)h->pos[1], (float *)h->vel[1], h->leaf[1]};
-  launch_fresh32(h->dt, leaf, o, v, n, h->key[1], h->prec, copied ? StateRows{} : rows, h->count, h->words, h->rank,
+  launch_fresh32(h->dt, leaf, o, v, n, h->key[1], h->prec, rows, copied, h->count, h->words, h->rank,
                  h->scalars + 6, h->err, s);
   int32_t unsorted = 1;
   CK(cudaGetLastError());
