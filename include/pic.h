@@ -188,7 +188,8 @@ PIC_API int pic_create_batch(pic_t *out, int32_t n_inst, const pic_tree_desc *tr
 
 /* Per-instance offsets (no counterpart in the paper) into the concatenated
  * particle storage, vertex arrays and bucket list; each array has n_instances + 1 entries (host memory, any
- * may be NULL).  Particle ranges are fixed: no particle leaves its instance. */
+ * may be NULL).  No particle leaves its instance in a step, so particle ranges
+ * change only where pic_set_state hands over other numbers of particles. */
 PIC_API int pic_instances(pic_t h, int64_t *particle_start, int64_t *vertex_start, int64_t *bucket_start);
 
 /* Leapfrog start: v_{-1/2} = v_0 - (q/m) E(x_0) dt/2 (deposit, solve, gather):

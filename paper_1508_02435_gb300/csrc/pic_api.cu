@@ -113,6 +113,7 @@ struct pic_s {
   bool brick_crowded = false;  // too many particles per brick: its steps run the generic passes (same bits)
   bool leaf_stale = false;  // leaf[0] not yet expanded from the offsets
   bool q_valid = false;     // Q holds the charges of the current positions
+  bool ranges_stale = false;  // batch: a split state was handed over, whose instances may hold other counts
 
   // CUDA graphs of one fixed-field step: [0] from the current buffer
   // assignment, [1] from the swapped one (the step alternates ping-pong offsets)
@@ -1030,6 +1031,7 @@ int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(&unsorted, h->scalars + 6, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
+  h->ranges_stale = h->dt.n_inst > 1;
   if (unsorted) {
     void *quad = h->d == 2 && !copied && n >= kPackRows ? h->Ep : nullptr;  // 16 n of its bytes
     if (quad) launch_pack_rows(n, rows.o, rows.v, quad, s);
@@ -1344,8 +1346,23 @@ int pic_create_batch(pic_t *out, int32_t n_inst, const pic_tree_desc *trees, con
   return create_forest(out, n_inst, trees, parts, q, cfg);
 }
 
+// Particle ranges of the instances from the bucket offsets, where a state that
+// was handed over may have changed them.
+static int instance_ranges(pic_t h) {
+  if (!h->ranges_stale) return PIC_OK;
+  std::vector<int32_t> first(h->inst.size());
+  for (size_t i = 0; i < first.size(); ++i)
+    CK(cudaMemcpyAsync(&first[i], h->start_cur + h->inst[i].key_off, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  const int rc = set_particle_offsets(h, std::vector<int64_t>(first.begin(), first.end()));
+  if (!rc) h->ranges_stale = false;
+  return rc;
+}
+
 int pic_instances(pic_t h, int64_t *particle_start, int64_t *vertex_start, int64_t *bucket_start) {
   if (check_handle(h)) return PIC_EINVAL;
+  const int rc = instance_ranges(h);
+  if (rc) return rc;
   const int32_t ni = h->dt.n_inst;
   const int stride = h->scheme == PIC_PIT ? 1 : h->dt.nc;
   for (int32_t i = 0; i <= ni; ++i) {
@@ -2279,6 +2296,7 @@ int pic_save(pic_t h, const char *path) {
   int32_t err = 0;
   if ((rc = read_err(h, &err))) return rc;
   if (err) return fail(h, PIC_ESTATE, "the handle holds a sticky device error; nothing was saved");
+  if ((rc = instance_ranges(h))) return rc;
   SnapshotMeta m;
   m.d = h->d;
   m.scheme = h->scheme;
@@ -2407,6 +2425,7 @@ int pic_load(pic_t *out, const char *path, void *stream) {
     return bail(rc, "");
   if (n > 0 && (rc = pic_set_state(h, split ? a.leaf.data() : nullptr, a.pos.data(), a.vel.data(), PIC_HOST)))
     return bail(rc, "");
+  h->ranges_stale = false;  // the leaves were checked against the saved ranges
   if ((rc = copy_in(h, h->V, a.V.data(), a.V.size(), PIC_HOST)) ||
       (rc = copy_in(h, h->E, a.E.data(), a.E.size(), PIC_HOST)))
     return bail(rc, "");

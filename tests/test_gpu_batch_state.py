@@ -65,3 +65,23 @@ def test_steps_match_single_plasmas(d, scheme, new, device):
         l1, p1, v1 = s.get_state()
         assert np.array_equal(leaf[r], l1 + off[i]) and np.array_equal(pos[:, r], p1) and np.array_equal(vel[:, r], v1)
         assert np.array_equal(Q[vs[i]:vs[i + 1]], s.deposit())
+
+
+@pytest.mark.parametrize("scheme", [pic.PIT, pic.PIDT])
+@pytest.mark.parametrize("new", [[2000, 300, 900], [0, 1, 3199], [3200, 0, 0]])
+def test_ranges_and_checkpoint_follow(scheme, new, tmp_path):
+    b, _, off = setup(2, scheme, [700, 2100, 400], new, True)
+    want = np.concatenate([[0], np.cumsum(new)])
+    assert np.array_equal(b.instances()[0], want)
+    b.step(0.05)
+    assert np.array_equal(b.instances()[0], want)
+    b.save(tmp_path / "batch.pic")
+    c = pic.Pic.load(tmp_path / "batch.pic")
+    assert np.array_equal(c.instances()[0], want)
+    for h in (b, c):
+        h.step(0.05)
+        h.sync()
+    for u, w in zip(b.get_state(), c.get_state()):
+        assert np.array_equal(u, w)
+    leaf = b.get_state()[0]
+    assert np.array_equal(np.searchsorted(leaf, off[:-1]), want[:-1]) or scheme == pic.PIDT
