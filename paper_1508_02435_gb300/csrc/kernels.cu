@@ -179,14 +179,16 @@ __device__ __forceinline__ void local_coords(const double *x, int64_t n, int64_t
 // a8 solve (auxiliary): b = Q - (sum Q) integral(phi); damped Jacobi
 // ---------------------------------------------------------------------------
 
-// With scale, also omega / diag per vertex; with `scaled`, b times that.
+// With scale, also omega / diag per vertex; with raw, b itself there and b times
+// omega / diag in b.
 template <typename T>
-__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale, bool scaled) {
+__global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale, T *raw) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= t.n_vert) return;
   T tot = (T)(t.n_inst > 1 ? total[1 + t.inst_of_vert[v]] : *total);
   const T r = Q[v] - tot * ion_load(t, v, (T)0);
-  b[v] = scaled ? r * (omega / diag_val(t, v, (T)0)) : r;
+  b[v] = raw ? r * (omega / diag_val(t, v, (T)0)) : r;
+  if (raw) raw[v] = r;
   if (scale) scale[v] = omega / diag_val(t, v, (T)0);
 }
 
@@ -716,10 +718,10 @@ void launch_relocate32(const DevTree &from, const DevTree &to, const int32_t *le
   k_relocate32<<<grid_for(n), kBlock, 0, s>>>(from, to, leaf, o, v, n, leaf2, o2, v2);
 }
 
-// Sweeps on a uniform tree between V and Vtmp, then the residual's block sums;
-// returns their number.
+// Sweeps on a uniform tree between V and Vtmp, then the residual's block sums from
+// `raw` (FP64; FP32: b again); returns their number.
 template <typename T, int D>
-static int64_t sweep_uniform(const DevTree &t, const T *b, T *V, T *Vtmp, int sweeps, T omega, double *r2,
+static int64_t sweep_uniform(const DevTree &t, const T *b, const T *raw, T *V, T *Vtmp, int sweeps, T omega, double *r2,
                              cudaStream_t s) {
   T *in = V, *out = Vtmp;
   for (int it = 0; it < sweeps; ++it) {
@@ -727,7 +729,7 @@ static int64_t sweep_uniform(const DevTree &t, const T *b, T *V, T *Vtmp, int sw
     std::swap(in, out);
   }
   if (in != V) cudaMemcpyAsync(V, in, sizeof(T) * t.n_vert, cudaMemcpyDeviceToDevice, s);
-  return launch_jacobi_uniform<T, D, true>(t, b, V, nullptr, omega, r2, s);
+  return launch_jacobi_uniform<T, D, true>(t, raw, V, nullptr, omega, r2, s);
 }
 
 // The same on an adaptive tree, V in place; part: one value per leaf corner.
@@ -753,19 +755,20 @@ static void solve(const DevTree &t, const RowMatrix &A, const T *Q, const double
   }
   // the FP64 two-pass solve of an adaptive tree leaves Vtmp free: it holds omega / diag
   T *scale = sizeof(T) == 8 && !t.uniform && !A.val ? Vtmp : nullptr;
-  const bool scaled = sizeof(T) == 8 && !scale;  // the other FP64 sweeps take b times omega / diag
-  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale, scaled); }
+  // FP64 sweeps of a uniform tree take b times omega / diag; the leaf corners' scratch keeps b for the residual
+  T *raw = sizeof(T) == 8 && t.uniform ? part : nullptr;
+  { COUNT(1); k_rhs<T><<<grid_for(t.n_vert), kBlock, 0, s>>>(t, Q, total, b, omega, scale, raw); }
   int64_t nb;
   if constexpr (sizeof(T) == 8) {
     if (A.val) {
-      nb = sweep_rows(t, A, b, V, Vtmp, sweeps, omega, block_sum, s);
+      nb = sweep_rows(t, A, b, V, Vtmp, sweeps, block_sum, s);
       { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
       return;
     }
   }
   if (t.uniform)
-    nb = t.d == 3 ? sweep_uniform<T, 3>(t, b, V, Vtmp, sweeps, omega, block_sum, s)
-                  : sweep_uniform<T, 2>(t, b, V, Vtmp, sweeps, omega, block_sum, s);
+    nb = t.d == 3 ? sweep_uniform<T, 3>(t, b, raw ? raw : b, V, Vtmp, sweeps, omega, block_sum, s)
+                  : sweep_uniform<T, 2>(t, b, raw ? raw : b, V, Vtmp, sweeps, omega, block_sum, s);
   else
     nb = t.d == 3 ? sweep_adaptive<T, 3>(t, b, V, part, scale, sweeps, omega, block_sum, s)
                   : sweep_adaptive<T, 2>(t, b, V, part, scale, sweeps, omega, block_sum, s);

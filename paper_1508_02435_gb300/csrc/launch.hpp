@@ -205,24 +205,26 @@ void launch_vertex_charge(const DevTree &t, bool split, const void *part, void *
 // total[0] is the FP64 sum over all vertices, total[1 + i] per instance.
 void launch_deposit(const DevTree &t, bool split, const int32_t *start, const void *pos, int64_t n, void *part,
                     void *Q, double *block_sum, double *total, cudaStream_t s);
-// Assembled rows of the FP64 solve on an adaptive tree, in slices of 32 rows and
-// scaled by omega / diag; val NULL: not assembled.
+// Assembled rows of the FP64 solve on an adaptive tree, in slices of 32 rows; val
+// NULL: not assembled.
 struct RowMatrix {
   const int32_t *ptr;           // first entry of every slice
   const int32_t *col;
   const double *val;
+  const double *scale;          // omega / diag per vertex
 };
 // Whether the solve of t runs as one cluster (small uniform trees).
 bool resident_solve_fits(const DevTree &t, bool split);
-// part: scratch of one value per leaf corner (adaptive trees), free after the
-// vertex charges are summed.
+// part: scratch of one value per leaf corner, free after the vertex charges are
+// summed.
 void launch_solve(const DevTree &t, const RowMatrix &A, bool split, const void *Q, const double *total, void *b, void *V,
                   void *Vtmp, void *part, int sweeps, double omega, double *block_sum, double *resid2, cudaStream_t s);
 // Assembly of the rows: entries per slice (row_slices of them), their scan is
 // RowMatrix::ptr, then columns and values.
 int64_t row_slices(const DevTree &t);
 void launch_row_count(const DevTree &t, int32_t *slice, int32_t *too_long, cudaStream_t s);
-void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, cudaStream_t s);
+void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, double *scale,
+                     cudaStream_t s);
 void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s);
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s);
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s);

@@ -650,7 +650,7 @@ int build_rows(pic_t h) {
   auto &gb = h->grid_bufs;
   const int64_t ns = row_slices(h->dt);
   int32_t *ptr, *len, *col, got[2] = {0, 0};
-  double *val;
+  double *val, *scale;
   int rc;
   if ((rc = galloc(h, gb, &ptr, ns + 1)) || (rc = galloc(h, gb, &len, ns))) return rc;
   CK(cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s));
@@ -660,10 +660,12 @@ int build_rows(pic_t h) {
   CK(cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   if (got[1]) return PIC_OK;
-  if ((rc = galloc(h, gb, &col, got[0])) || (rc = galloc(h, gb, &val, got[0]))) return rc;
-  launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, s);
+  if ((rc = galloc(h, gb, &col, got[0])) || (rc = galloc(h, gb, &val, got[0])) ||
+      (rc = galloc(h, gb, &scale, h->dt.n_vert)))
+    return rc;
+  launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, scale, s);
   CK(cudaGetLastError());
-  h->rows = RowMatrix{ptr, col, val};
+  h->rows = RowMatrix{ptr, col, val, scale};
   return PIC_OK;
 }
 

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
   __shared__ int bad;  // some V is not finite: the zero terms of the 3D face neighbours count
   const InstInfo &I = t.inst[0];
   StencilC<T> c;
-  stencil_consts<D>(I, omega, true, &c);
+  stencil_consts<D>(I, omega, false, &c);
   const int rank = (int)cluster_rank(), z0 = rank * R::kSlab, tid = threadIdx.x;
   const bool act = tid < R::kWork;
   const int row = D == 3 ? 0 : tid / M;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
   const uint32_t lo_peer = (uint32_t)((rank + R::kCtas - 1) % R::kCtas), hi_peer = (uint32_t)((rank + 1) % R::kCtas);
   const uint32_t lo_buf = peer_addr(&buf[0][0], lo_peer), hi_buf = peer_addr(&buf[0][0], hi_peer);
   const T tot = (T)*total;
-  T v[N], b[N];
+  T v[N], b[N], raw[N];
   auto stored = [&](T u) {  // what shared memory holds of a value
     if constexpr (R::kScaled) return c.c2 * u;
     else return u;
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
   for (int i = 0; i < N; ++i) {
     const int at = act ? (z0 + (D == 3 ? i : row)) * PL + own : 0;
     v[i] = V[at];
-    b[i] = Q[at] - tot * ion_load(t, 0, (T)0);
+    b[i] = raw[i] = Q[at] - tot * ion_load(t, 0, (T)0);
     if constexpr (sizeof(T) == 8) b[i] = b[i] * (omega / I.diag);
   }
   auto apply = [&](const T *s, int i, bool any) {
@@ -204,12 +204,14 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
     cluster_meet();
   }
   double rr = 0.0;
+  stencil_consts<D>(I, omega, true, &c);
   if (act) {
     const bool any = D == 3 && bad != 0;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
+      b[i] = raw[i];
       const T yv = apply(buf[sweeps & 1], i, any);
-      rr = rr + residual2<1>(&yv, &b[i], &v[i], c);
+      rr = rr + residual2<1>(&yv, &b[i]);
       V[(z0 + (D == 3 ? i : row)) * PL + own] = v[i];
     }
   }

@@ -4,8 +4,8 @@
 // and one per incidence, some 30 a vertex in 2D, and two launches a sweep.  The
 // same operator assembled per vertex has 9 entries in most rows (27 in 3D): one
 // launch, 9 fused adds.  Rows are stored in slices of 32, entry k of the slice's
-// rows side by side, padded to the slice's longest row, and scaled by omega / diag
-// so that a sweep is V' = V + (b' - A' V).
+// rows side by side, padded to the slice's longest row; a sweep is V' = V + scale
+// (b - A V) with scale = omega / diag per vertex, tabulated beside them.
 //
 // One sweep of the 2D bump (75,451 vertices): 9.9 -> 4.0 us.
 #pragma once
@@ -57,31 +57,31 @@ __global__ void __launch_bounds__(128) k_row_count(DevTree t, int32_t *slice, in
 
 template <int D>
 __global__ void __launch_bounds__(128) k_row_fill(DevTree t, const int32_t *ptr, double omega, int32_t *cols,
-                                                  double *vals) {
+                                                  double *vals, double *scale) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if ((v & ~(int64_t)31) >= t.n_vert) return;
   int32_t col[kRowMax];
   double val[kRowMax];
   const int len = v < t.n_vert ? assemble_row<D>(t, v, col, val) : 0;
-  const double scale = v < t.n_vert ? omega / t.diag64[v] : 0.0;
+  if (v < t.n_vert) scale[v] = omega / t.diag64[v];
   const int32_t b = ptr[v >> 5], m = (ptr[(v >> 5) + 1] - b) >> 5;
   for (int k = 0; k < m; ++k) {
     const int64_t at = b + 32 * k + (v & 31);
     cols[at] = k < len ? col[k] : v < t.n_vert ? (int32_t)v : 0;
-    vals[at] = k < len ? scale * val[k] : 0.0;
+    vals[at] = k < len ? val[k] : 0.0;
   }
 }
 
-// b and V as in k_jacobi_vertex, b scaled by omega / diag; kRes: block sums of
-// the squared residual (unscaled).
+// b and V as in k_vertex_pass; kRes: block sums of the squared residual.
 template <bool kRes>
 __global__ void __launch_bounds__(128) k_row_sweep(DevTree t, RowMatrix A, const double *b, const double *Vin,
-                                                   double *__restrict__ Vout, double omega, double *r2) {
+                                                   double *__restrict__ Vout, double *r2) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool act = v < t.n_vert;
   constexpr int kPre = 9;  // entries read while the sweep before runs
   int32_t col[kPre], p = 0, end = 0;
   double val[kPre];
+  const double scale = !kRes && act ? A.scale[v] : 0.0;
   if (act) {
     p = A.ptr[v >> 5];
     end = A.ptr[(v >> 5) + 1];
@@ -105,12 +105,9 @@ __global__ void __launch_bounds__(128) k_row_sweep(DevTree t, RowMatrix A, const
     for (int k = 0; k < kPre; ++k)
       if (col[k] >= 0) y = fma(val[k], u[k], y);
     for (int32_t i = p + 32 * kPre; i < end; i += 32) y = fma(A.val[i], Vin[A.col[i]], y);
-    if (kRes) {
-      const double r = (bv - y) * (t.diag64[v] / omega);
-      rr = r * r;
-    } else {
-      Vout[v] = vc + (bv - y);
-    }
+    const double r = bv - y;
+    if (kRes) rr = r * r;
+    else Vout[v] = fma(scale, r, vc);
   }
   if (kRes) block_sum_store_at(rr, r2 + blockIdx.x);
 }
@@ -123,25 +120,26 @@ void launch_row_count(const DevTree &t, int32_t *slice, int32_t *too_long, cudaS
   else k_row_count<2><<<grid_for(t.n_vert, 128), 128, 0, s>>>(t, slice, too_long);
 }
 
-void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, cudaStream_t s) {
+void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, double *scale,
+                     cudaStream_t s) {
   COUNT(1);
-  if (t.d == 3) k_row_fill<3><<<grid_for(t.n_vert, 128), 128, 0, s>>>(t, ptr, omega, cols, vals);
-  else k_row_fill<2><<<grid_for(t.n_vert, 128), 128, 0, s>>>(t, ptr, omega, cols, vals);
+  if (t.d == 3) k_row_fill<3><<<grid_for(t.n_vert, 128), 128, 0, s>>>(t, ptr, omega, cols, vals, scale);
+  else k_row_fill<2><<<grid_for(t.n_vert, 128), 128, 0, s>>>(t, ptr, omega, cols, vals, scale);
 }
 
 // Sweeps between V and Vtmp, then the residual's block sums; returns their number.
 static int64_t sweep_rows(const DevTree &t, const RowMatrix &A, const double *b, double *V, double *Vtmp, int sweeps,
-                          double omega, double *r2, cudaStream_t s) {
+                          double *r2, cudaStream_t s) {
   const dim3 g(grid_for(t.n_vert, 128)), block(128);
   double *in = V, *out = Vtmp;
   for (int it = 0; it < sweeps; ++it) {
     COUNT(1);
-    launch_pdl(k_row_sweep<false>, g, block, s, t, A, b, in, out, omega, r2);
+    launch_pdl(k_row_sweep<false>, g, block, s, t, A, b, in, out, r2);
     std::swap(in, out);
   }
   if (in != V) cudaMemcpyAsync(V, in, sizeof(double) * t.n_vert, cudaMemcpyDeviceToDevice, s);
   COUNT(1);
-  launch_pdl(k_row_sweep<true>, g, block, s, t, A, b, V, nullptr, omega, r2);
+  launch_pdl(k_row_sweep<true>, g, block, s, t, A, b, V, nullptr, r2);
   return g.x;
 }
 

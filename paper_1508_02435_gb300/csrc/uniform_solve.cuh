@@ -38,7 +38,10 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Constants of one uniform instance.  FP32: c0, c1, c2 = kref(0, 1, 2 axes differ)
-// h^(d-2), the diagonal, and 1 / diagonal in two floats.  FP64: the sweep's weights.
+// h^(d-2), the diagonal, and 1 / diagonal in two floats.  FP64: the weights of the
+// value itself and of its neighbours that give the sweep's new value beside b omega /
+// diag, or (res) the residual b - A V beside b -- from the matrix, so that it does
+// not hang on omega, which may be zero.
 template <typename T>
 struct StencilC;
 template <>
@@ -47,7 +50,7 @@ struct StencilC<float> {
 };
 template <>
 struct StencilC<double> {
-  double k0, k1, k2, inv;  // inv = diag / omega (residual only)
+  double k0, k1, k2;
 };
 
 template <int D>
@@ -62,11 +65,10 @@ __device__ __forceinline__ void stencil_consts(const InstInfo &I, float omega, b
   s->rlo = I.rdiag_lo32;
 }
 template <int D>
-__device__ __forceinline__ void stencil_consts(const InstInfo &I, double omega, bool res, StencilC<double> *s) {
-  s->k0 = I.jac[0];
-  s->k1 = I.jac[1];
-  s->k2 = I.jac[2];
-  s->inv = res ? I.diag / omega : 0.0;
+__device__ __forceinline__ void stencil_consts(const InstInfo &I, double, bool res, StencilC<double> *s) {
+  s->k0 = res ? -I.diag : I.jac[0];
+  s->k1 = res ? 1.0 / 3.0 : I.jac[1];
+  s->k2 = res ? (D == 3 ? I.h * (1.0 / 12.0) : 1.0 / 3.0) : I.jac[2];
 }
 
 // |spread(j) - spread(j - 1)| on one axis (0 on a one-cell axis).
@@ -164,7 +166,7 @@ __device__ __forceinline__ float face_terms(Q q) {
 
 __device__ __forceinline__ uint32_t high_word(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// FP64, one sweep at a vertex with b times omega / diag: an edge neighbour shares
+// FP64, one sweep at a vertex with b times omega / diag, or the residual with b as it is: an edge neighbour shares
 // two leaves with the vertex, a corner neighbour one (2D: a face neighbour two, of
 // half the entry).  Three fused operations beside the neighbour sums.
 __device__ __forceinline__ double sweep3(double c, double edges, double corners, const StencilC<double> &s, double b) {
@@ -211,7 +213,7 @@ __device__ __forceinline__ void jacobi_update(const double *y, const double *, c
 
 // Squared residuals of N vertices, in order.
 template <int N>
-__device__ __forceinline__ double residual2(const float *y, const float *b, const float *, const StencilC<float> &) {
+__device__ __forceinline__ double residual2(const float *y, const float *b) {
   double rr = 0.0;
 #pragma unroll
   for (int j = 0; j < N; ++j) {
@@ -221,14 +223,10 @@ __device__ __forceinline__ double residual2(const float *y, const float *b, cons
   return rr;
 }
 template <int N>
-__device__ __forceinline__ double residual2(const double *y, const double *, const double *vc,
-                                            const StencilC<double> &s) {
+__device__ __forceinline__ double residual2(const double *y, const double *) {  // rows give the residual itself
   double rr = 0.0;
 #pragma unroll
-  for (int j = 0; j < N; ++j) {
-    const double r = (y[j] - vc[j]) * s.inv;  // omega / diag times the residual is the step
-    rr = rr + r * r;
-  }
+  for (int j = 0; j < N; ++j) rr = rr + y[j] * y[j];
   return rr;
 }
 
@@ -335,7 +333,7 @@ __global__ void __launch_bounds__(128) k_jacobi_vertex(DevTree t, const T *b, co
     const T bv = b[v];
     T vc;
     const T y = apply_at<D>(Vin + I.vert_off, M, j, t.spread + I.spread_off, s, bv, &vc);
-    if (kRes) rr = residual2<1>(&y, &bv, &vc, s);
+    if (kRes) rr = residual2<1>(&y, &bv);
     else jacobi_update<1>(&y, &bv, &vc, s, Vout + v);
   }
   if (kRes) block_sum_store_at(rr, r2 + blockIdx.x);
@@ -469,7 +467,7 @@ __global__ void __launch_bounds__(128) k_jacobi_strip3(DevTree t, const double *
       load(z + 1 == M ? 0 : z + 1, hi);
       strip_rows(lo, mid, hi, s, bv, y);
       if (kRes) {
-        rr = rr + residual2<3>(y, bv, mid.c, s);
+        rr = rr + residual2<3>(y, bv);
       } else {
 #pragma unroll
         for (int j = 0; j < 3; ++j) Vout[at + row[j + 1]] = y[j];
@@ -565,7 +563,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_jacobi_tile3(DevTree t, con
       strip_rows<true>(lo, mid, hi, s, w, flip, y);
     }
     if (kRes) {
-      if (act) rr = rr + residual2<3>(y, bv, mid.c, s);
+      if (act) rr = rr + residual2<3>(y, bv);
     } else {
       float out[3];
       jacobi_update<3>(y, bv, mid.c, s, out);
@@ -660,7 +658,7 @@ __global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, co
     strip_rows2(v, s, w, flip, bv, y);
     const T vc[3] = {v[4], v[7], v[10]};
     if (kRes) {
-      rr = residual2<3>(y, bv, vc, s);
+      rr = residual2<3>(y, bv);
     } else {
       T out[3];
       jacobi_update<3>(y, bv, vc, s, out);
@@ -704,7 +702,8 @@ inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A
 }
 
 // One sweep, or with kRes the residual's block sums: at most
-// (n_vert + 127) / 128 of them.  Returns the number of blocks.
+// (n_vert + 127) / 128 of them.  FP64 sweeps take b omega / diag, the residual
+// takes b.  Returns the number of blocks.
 template <typename T, int D, bool kRes>
 int64_t launch_jacobi_uniform(const DevTree &t, const T *b, const T *Vin, T *Vout, T omega, double *r2,
                               cudaStream_t s) {
