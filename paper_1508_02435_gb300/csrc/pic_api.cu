@@ -641,31 +641,42 @@ int alloc_particles(pic_t h) {
 
 // Assembles the rows of the FP64 solve of an adaptive tree, where the solve
 // sweeps often enough to repay it (assembly: about ten sweeps of the two passes)
-// and the rows take a few hundred megabytes at most.  Rows that do not fit leave
-// the two passes.
+// and the tree has at most two million vertices: 12 bytes an entry, 9 to 12 entries
+// a vertex in most 2D trees (0.25 GB), 27 and more in 3D (0.65 GB; 1.15 GB if every
+// slice has a row of kRowMax).  The solve needs none of it: where the memory is
+// refused, or a row is longer than kRowMax, the two passes stay.
 int build_rows(pic_t h) {
   h->rows = RowMatrix{};
   if (h->split || h->dt.uniform || h->cfg.sweeps < 16 || h->dt.n_vert > 2000000) return PIC_OK;
   cudaStream_t s = h->stream;
-  auto &gb = h->grid_bufs;
   const int64_t ns = row_slices(h->dt);
-  int32_t *ptr, *len, *col, got[2] = {0, 0};
+  int32_t *ptr, *len, *col, got[2] = {0, 1};
   double *val, *scale;
-  int rc;
-  if ((rc = galloc(h, gb, &ptr, ns + 1)) || (rc = galloc(h, gb, &len, ns))) return rc;
-  CK(cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s));
-  launch_row_count(h->dt, len, h->scalars + 4, s);
-  launch_exclusive_scan(len, ns, ptr, h->tile_sums, h->scalars + 3, s);
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
-  if (got[1]) return PIC_OK;
-  if ((rc = galloc(h, gb, &col, got[0])) || (rc = galloc(h, gb, &val, got[0])) ||
-      (rc = galloc(h, gb, &scale, h->dt.n_vert)))
-    return rc;
-  launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, scale, s);
-  CK(cudaGetLastError());
-  h->rows = RowMatrix{ptr, col, val, scale};
+  std::vector<DevBuf> mine;
+  const std::string message = h->last_error;
+  cudaError_t e = cudaSuccess;
+  if (!galloc(h, mine, &ptr, ns + 1) && !galloc(h, mine, &len, ns)) {
+    e = cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s);
+    launch_row_count(h->dt, len, h->scalars + 4, s);
+    launch_exclusive_scan(len, ns, ptr, h->tile_sums, h->scalars + 3, s);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
+  if (e == cudaSuccess && !got[1] && !galloc(h, mine, &col, got[0]) && !galloc(h, mine, &val, got[0]) &&
+      !galloc(h, mine, &scale, h->dt.n_vert)) {
+    launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, scale, s);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) {
+      h->rows = RowMatrix{ptr, col, val, scale};
+      h->grid_bufs.insert(h->grid_bufs.end(), mine.begin(), mine.end());
+      return PIC_OK;
+    }
+  }
+  free_bufs(h, mine);
+  if (e != cudaSuccess) return cuda_fail(h, e, "row assembly");
+  cudaGetLastError();  // a refused cudaMalloc is no error of this call
+  h->last_error = message;
   return PIC_OK;
 }
 
@@ -708,8 +719,8 @@ int alloc_grid(pic_t h) {
   h->ecorner = nullptr;
   h->ecorner_valid = false;
   h->ebrick_valid = false;
-  if ((rc = build_rows(h))) return rc;
   if (!h->dt.uniform && (rc = galloc(h, sb, &h->ecorner, corner_field_bytes(h->dt, h->split)))) return rc;
+  if ((rc = build_rows(h))) return rc;  // last: what every solve needs comes first
   return reset_grid_state(h);
 }
 
