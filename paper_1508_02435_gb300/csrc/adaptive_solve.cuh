@@ -41,8 +41,7 @@ __global__ void __launch_bounds__(256) k_corner_pass(DevTree t, const T *V, T *_
     w0 = w[j0];
     if (kApply) {
       const T hs = D == 2 ? (T)1 : cell_width(t.leaf_level[i / NC], (T)0);
-      const T k0 = kref_val(0, 0, (T)0) * hs, k1 = kref_val(0, 1, (T)0) * hs, k2 = kref_val(0, 3, (T)0) * hs;
-      const T k3 = kref_val(0, D == 3 ? 7 : 3, (T)0) * hs;
+      const T k0 = (T)kref<D>(0) * hs, k1 = (T)kref<D>(1) * hs, k2 = (T)kref<D>(2) * hs, k3 = (T)kref<D>(3) * hs;
 #pragma unroll
       for (int f = 0; f < NC; ++f) {
         const int df = __popc(e ^ f);

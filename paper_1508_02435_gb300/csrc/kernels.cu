@@ -26,8 +26,14 @@
 
 namespace pic {
 
-__constant__ double c_kref64[8][8];
-__constant__ float c_kref32[8][8];
+// Entry of the reference element's matrix for two corners that differ on k axes.
+// Of the dimension alone: handles of both dimensions may be alive together.
+template <int D>
+__host__ __device__ constexpr double kref(int k) {
+  return D == 2 ? (k == 0 ? 4.0 / 6.0 : k == 1 ? -1.0 / 6.0 : -2.0 / 6.0)
+                : (k == 0 ? 4.0 / 12.0 : k == 1 ? 0.0 : -1.0 / 12.0);
+}
+
 __constant__ double c_width64[19];  // 3^-level
 __constant__ float c_width32[19];
 
@@ -121,8 +127,6 @@ __device__ __forceinline__ float corner_value(const DevTree &t, int32_t L, const
 
 __device__ __forceinline__ const double *inc_weights(const DevTree &t, double) { return t.inc_w64; }
 __device__ __forceinline__ const float *inc_weights(const DevTree &t, float) { return t.inc_w32; }
-__device__ __forceinline__ double kref_val(int e, int f, double) { return c_kref64[e][f]; }
-__device__ __forceinline__ float kref_val(int e, int f, float) { return c_kref32[e][f]; }
 __device__ __forceinline__ double ion_load(const DevTree &t, int64_t v, double) {
   return t.uniform ? inst_of_vertex(t, v).ion_load : t.ion64[v];
 }
@@ -597,31 +601,6 @@ cudaError_t set_constants(cudaStream_t s) {
                            (int)(sizeof(int32_t) * kMedSeg * (kMedThreads / 32)));
   if (e != cudaSuccess) return e;
   return cudaMemcpyToSymbolAsync(c_pow3, p3, sizeof(p3), 0, cudaMemcpyHostToDevice, s);
-}
-
-cudaError_t set_kref(int d, cudaStream_t s) {
-  double k64[8][8];
-  float k32[8][8];
-  int nc = 1 << d;
-  for (int e = 0; e < 8; ++e)
-    for (int f = 0; f < 8; ++f) {
-      double v = 0.0;
-      if (e < nc && f < nc) {
-        int diff = __builtin_popcount((unsigned)(e ^ f));
-        if (d == 2) {
-          const double k2[3] = {4.0 / 6.0, -1.0 / 6.0, -2.0 / 6.0};
-          v = k2[diff];
-        } else {
-          const double k3[4] = {4.0 / 12.0, 0.0, -1.0 / 12.0, -1.0 / 12.0};
-          v = k3[diff];
-        }
-      }
-      k64[e][f] = v;
-      k32[e][f] = (float)v;
-    }
-  cudaError_t err = cudaMemcpyToSymbolAsync(c_kref64, k64, sizeof(k64), 0, cudaMemcpyHostToDevice, s);
-  if (err != cudaSuccess) return err;
-  return cudaMemcpyToSymbolAsync(c_kref32, k32, sizeof(k32), 0, cudaMemcpyHostToDevice, s);
 }
 
 void launch_init64(const DevTree &t, double *x, int64_t n, int32_t *leaf, int32_t *key, int32_t *err,

@@ -158,7 +158,6 @@ void launch_brick_field(const DevTree &t, const BrickGeom &g, const float *E, fl
 void launch_wait_selftest(long long cycles, int32_t *flag, cudaStream_t s);
 
 cudaError_t set_constants(cudaStream_t s);
-cudaError_t set_kref(int d, cudaStream_t s);
 int64_t scan_tiles_needed(int64_t n);
 
 void launch_init64(const DevTree &t, double *x, int64_t n, int32_t *leaf, int32_t *key, int32_t *err,

@@ -1332,8 +1332,6 @@ static int create_forest(pic_t *out, int32_t n_inst, const pic_tree_desc *trees,
     for (int32_t i = 0; i < n_inst; ++i) qs[i] = q[i];
   if ((rc = install_forest(h, trees, n_inst, qs))) { pic_destroy(h); return rc; }
   if ((rc = set_particle_offsets(h, poff))) { pic_destroy(h); return rc; }
-  e = set_kref(h->d, h->stream);
-  if (e != cudaSuccess) { rc = cuda_fail(h, e, "set_kref"); pic_destroy(h); return rc; }
   if ((rc = alloc_state(h))) { pic_destroy(h); return rc; }
   if ((rc = setup_brick(h))) { pic_destroy(h); return rc; }
   if (h->n > 0) {

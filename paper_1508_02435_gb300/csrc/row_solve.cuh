@@ -25,7 +25,7 @@ __device__ __forceinline__ int assemble_row(const DevTree &t, int64_t v, int32_t
     const int e = lc - L * NC;
     const double w = t.inc_w64[i] * (D == 2 ? 1.0 : c_width64[t.leaf_level[L]]);
     for (int f = 0; f < NC; ++f) {
-      const double k = w * c_kref64[e][f];
+      const double k = w * kref<D>(__popc(e ^ f));
       const int32_t c = L * NC + f;
       for (int32_t j = t.cexp_ptr[c]; j < t.cexp_ptr[c + 1]; ++j) {
         const int32_t u = t.cexp_vid[j];

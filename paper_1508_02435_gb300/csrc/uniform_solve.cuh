@@ -56,9 +56,9 @@ struct StencilC<double> {
 template <int D>
 __device__ __forceinline__ void stencil_consts(const InstInfo &I, float omega, bool, StencilC<float> *s) {
   const float hs = D == 2 ? 1.0f : I.h32;
-  s->c0 = c_kref32[0][0] * hs;
-  s->c1 = c_kref32[0][1] * hs;
-  s->c2 = c_kref32[0][3] * hs;
+  s->c0 = (float)kref<D>(0) * hs;
+  s->c1 = (float)kref<D>(1) * hs;
+  s->c2 = (float)kref<D>(2) * hs;
   s->omega = omega;
   s->diag = I.diag32;
   s->rhi = I.rdiag32;
