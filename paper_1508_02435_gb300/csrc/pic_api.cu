@@ -124,6 +124,7 @@ struct pic_s {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   HostView graph_pre[2]{}, graph_post[2]{};
   int64_t graph_kernels = 0;
+  bool graph_solves = false;  // the captured steps solve for the field
   BrickGeom bg{};
   std::vector<DevBuf> brick_bufs;
   BrickStage stage{};      // per-destination staging between the two brick kernels
@@ -871,6 +872,19 @@ int ensure_leaf(pic_t h) {
   return PIC_OK;
 }
 
+// The copies of the vertex field that the push reads, where E changed since they
+// were made: at the leaf corners of an adaptive tree, brick by brick.
+void refresh_corner_field(pic_t h) {
+  if (!h->ecorner || h->ecorner_valid) return;
+  launch_corner_field(h->dt, h->split, h->E, h->ecorner, h->stream);
+  h->ecorner_valid = true;
+}
+void refresh_brick_field(pic_t h) {
+  if (h->ebrick_valid) return;
+  launch_brick_field(h->dt, h->bg, (const float *)h->E, h->ebrick, h->stream);
+  h->ebrick_valid = true;
+}
+
 int brick_push_and_rebin(pic_t h, double dt) {
   cudaStream_t s = h->stream;
   BrickPushArgs pa{};
@@ -880,10 +894,7 @@ int brick_push_and_rebin(pic_t h, double dt) {
   pa.start = h->start_cur;
   pa.ids = h->cfg.track_ids ? h->ids[0] : nullptr;
   pa.E = (const float *)h->E;
-  if (!h->ebrick_valid) {
-    launch_brick_field(h->dt, h->bg, (const float *)h->E, h->ebrick, s);
-    h->ebrick_valid = true;
-  }
+  refresh_brick_field(h);
   pa.Ebrick = h->ebrick;
   pa.qmdt = (float)(h->cfg.qm * dt);
   pa.sl = (float)(dt * (double)pow3(h->ht0().depth));
@@ -1098,10 +1109,7 @@ int push_and_rebin(pic_t h, double dt, MoveKind mk = MoveKind{}) {
   CK(cudaMemsetAsync(h->count, 0, sizeof(int32_t) * h->dt.n_keys, s));
   CK(cudaMemsetAsync(h->scalars + 2, 0, sizeof(int32_t) * 6, s));  // largest bucket, segment lists
   PhaseScope *ps = new PhaseScope(h, PIC_PHASE_PUSH);
-  if (h->ecorner && mk.field && !h->ecorner_valid) {
-    launch_corner_field(h->dt, h->split, h->E, h->ecorner, s);
-    h->ecorner_valid = true;
-  }
+  if (mk.field) refresh_corner_field(h);
   if (h->split) {
     Push32Args a{};
     a.n = h->n;
@@ -1620,6 +1628,7 @@ static int graph_capture(pic_t h, double dt, bool with_solve) {
     }
   }
   set_host_view(h, start);
+  h->graph_solves = with_solve;
   h->graph_kernels = (launches() - k0) / 2;
   return PIC_OK;
 }
@@ -1631,6 +1640,11 @@ int pic_graph_capture_step(pic_t h, double dt) { return graph_capture(h, dt, tru
 int pic_graph_launch(pic_t h, int32_t steps) {
   if (check_handle(h) || steps < 0) return PIC_EINVAL;
   if (!h->graph[0]) return fail(h, PIC_ESTATE, "no captured step (pic_graph_capture)");
+  if (steps > 0 && !h->graph_solves) {  // the captured steps read the field's copies as they are
+    refresh_corner_field(h);
+    if (h->brick && !h->brick_crowded) refresh_brick_field(h);
+    CK(cudaGetLastError());
+  }
   for (int32_t i = 0; i < steps; ++i) {
     int rc;
     if (!h->graph_pre[0].leaf_stale && (rc = ensure_leaf(h))) return rc;
