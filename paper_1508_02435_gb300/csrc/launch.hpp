@@ -221,6 +221,7 @@ void launch_solve(const DevTree &t, const RowMatrix &A, bool split, const void *
 // Assembly of the rows: entries per slice (row_slices of them), their scan is
 // RowMatrix::ptr, then columns and values.
 int64_t row_slices(const DevTree &t);
+int64_t row_capacity(const DevTree &t);  // entries reserved for them
 void launch_row_count(const DevTree &t, int32_t *slice, int32_t *too_long, cudaStream_t s);
 void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, double *scale,
                      cudaStream_t s);

@@ -87,6 +87,10 @@ struct pic_s {
   double *block_sum = nullptr, *total = nullptr, *resid2 = nullptr;
   void *Ep = nullptr;  // d * n scratch (gather at the particles, FP64 staging)
   RowMatrix rows{};           // FP64, adaptive: assembled rows of the solve
+  struct RowMemory {          // memory for them, until the first solve on the tree
+    int32_t *ptr = nullptr, *len = nullptr, *col = nullptr;
+    double *val = nullptr, *scale = nullptr;
+  } row_mem;
   char *ecorner = nullptr;    // adaptive: field at every leaf corner
   bool ecorner_valid = false; // ecorner holds the corners of the current E
   float *ebrick = nullptr;    // brick path: the field brick by brick (float4 / float2 per vertex)
@@ -640,44 +644,59 @@ int alloc_particles(pic_t h) {
   return PIC_OK;
 }
 
-// Assembles the rows of the FP64 solve of an adaptive tree, where the solve
-// sweeps often enough to repay it (assembly: about ten sweeps of the two passes)
-// and the tree has at most two million vertices: 12 bytes an entry, 9 to 12 entries
-// a vertex in most 2D trees (0.25 GB), 27 and more in 3D (0.65 GB; 1.15 GB if every
-// slice has a row of kRowMax).  The solve needs none of it: where the memory is
-// refused, or a row is longer than kRowMax, the two passes stay.
-int build_rows(pic_t h) {
+// Memory for the assembled rows of the FP64 solve of an adaptive tree, where the
+// solve sweeps often enough to repay them (assembly: about ten sweeps of the two
+// passes) and the tree has at most two million vertices (12 bytes an entry: 0.77 GB
+// in 2D, 1.15 GB in 3D).  The solve needs none of it: where it is refused the two
+// passes stay.
+int reserve_rows(pic_t h) {
   h->rows = RowMatrix{};
+  h->row_mem = pic_s::RowMemory{};
   if (h->split || h->dt.uniform || h->cfg.sweeps < 16 || h->dt.n_vert > 2000000) return PIC_OK;
-  cudaStream_t s = h->stream;
-  const int64_t ns = row_slices(h->dt);
-  int32_t *ptr, *len, *col, got[2] = {0, 1};
-  double *val, *scale;
+  const int64_t ns = row_slices(h->dt), cap = row_capacity(h->dt);
+  pic_s::RowMemory m;
   std::vector<DevBuf> mine;
   const std::string message = h->last_error;
-  cudaError_t e = cudaSuccess;
-  if (!galloc(h, mine, &ptr, ns + 1) && !galloc(h, mine, &len, ns)) {
-    e = cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s);
-    launch_row_count(h->dt, len, h->scalars + 4, s);
-    launch_exclusive_scan(len, ns, ptr, h->tile_sums, h->scalars + 3, s);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (galloc(h, mine, &m.ptr, ns + 1) || galloc(h, mine, &m.len, ns) || galloc(h, mine, &m.col, cap) ||
+      galloc(h, mine, &m.val, cap) || galloc(h, mine, &m.scale, h->dt.n_vert)) {
+    free_bufs(h, mine);
+    cudaGetLastError();  // a refused cudaMalloc is no error of this call
+    h->last_error = message;
+    return PIC_OK;
   }
-  if (e == cudaSuccess && !got[1] && !galloc(h, mine, &col, got[0]) && !galloc(h, mine, &val, got[0]) &&
-      !galloc(h, mine, &scale, h->dt.n_vert)) {
-    launch_row_fill(h->dt, ptr, h->cfg.omega, col, val, scale, s);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) {
-      h->rows = RowMatrix{ptr, col, val, scale};
-      h->grid_bufs.insert(h->grid_bufs.end(), mine.begin(), mine.end());
-      return PIC_OK;
-    }
+  h->row_mem = m;
+  h->grid_bufs.insert(h->grid_bufs.end(), mine.begin(), mine.end());
+  return PIC_OK;
+}
+
+// Assembles the rows, by the first solve on a tree: handles that re-tree and never
+// solve do not pay for them.  (Re-trees of the 3D bump, 47,965 vertices: 1.34 ms
+// without rows, 5.8 with the rows assembled at each by a thread a row.)  Rows that do
+// not fit leave the two passes.  Under capture nothing can be read back: the rows
+// wait for a solve outside.
+int assemble_rows(pic_t h) {
+  pic_s::RowMemory &m = h->row_mem;
+  cudaStream_t s = h->stream;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    return PIC_OK;
   }
-  free_bufs(h, mine);
-  if (e != cudaSuccess) return cuda_fail(h, e, "row assembly");
-  cudaGetLastError();  // a refused cudaMalloc is no error of this call
-  h->last_error = message;
+  if (capture != cudaStreamCaptureStatusNone) return PIC_OK;
+  int32_t got[2] = {0, 0};
+  const int64_t ns = row_slices(h->dt);
+  CK(cudaMemsetAsync(h->scalars + 3, 0, sizeof(int32_t) * 2, s));
+  launch_row_count(h->dt, m.len, h->scalars + 4, s);
+  launch_exclusive_scan(m.len, ns, m.ptr, h->tile_sums, h->scalars + 3, s);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s));
+  CK(cudaStreamSynchronize(s));
+  if (!got[1] && got[0] <= row_capacity(h->dt)) {
+    launch_row_fill(h->dt, m.ptr, h->cfg.omega, m.col, m.val, m.scale, s);
+    CK(cudaGetLastError());
+    h->rows = RowMatrix{m.ptr, m.col, m.val, m.scale};
+  }
+  m = pic_s::RowMemory{};  // assembled, or no use on this tree
   return PIC_OK;
 }
 
@@ -721,7 +740,7 @@ int alloc_grid(pic_t h) {
   h->ecorner_valid = false;
   h->ebrick_valid = false;
   if (!h->dt.uniform && (rc = galloc(h, sb, &h->ecorner, corner_field_bytes(h->dt, h->split)))) return rc;
-  if ((rc = build_rows(h))) return rc;  // last: what every solve needs comes first
+  if ((rc = reserve_rows(h))) return rc;  // last: what every solve needs comes first
   return reset_grid_state(h);
 }
 
@@ -1085,6 +1104,8 @@ int field(pic_t h, pic_solve_fn hook, void *user) {
     if (r != 0) return fail(h, PIC_EHOOK, "field-solve hook returned " + std::to_string(r));
     return PIC_OK;
   }
+  int rc;
+  if (h->row_mem.ptr && (rc = assemble_rows(h))) return rc;
   launch_solve(h->dt, h->rows, h->split, h->Q, h->total, h->b, h->V, h->Vtmp, h->part, h->cfg.sweeps, h->cfg.omega, h->block_sum,
                h->resid2, s);
   launch_efield(h->dt, h->split, h->V, h->E, h->part, s);

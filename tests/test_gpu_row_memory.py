@@ -108,3 +108,31 @@ def test_refused_rows_leave_the_two_passes(d):
     # a block that every handle needs is still an error
     with pytest.raises(pic.PicError):
         handle(d, large, ROWS_FROM, refuse=0)
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_rows_wait_for_the_first_solve(d):
+    """Creations and re-trees leave the rows to the first solve outside a capture; the solves of a captured
+    step before it are by the two passes."""
+    small, large = trees(d)
+    n = 3001
+    x, v = W.random_particles(d, n, 8, vmax=0.1)
+    kw = dict(precision=pic.FP64, q=-1.0 / n, ion=0.3, sweeps=ROWS_FROM)
+    s = torch.cuda.Stream()
+    a = pic.Pic(d, small, x, v, stream=s, **kw)
+    b = pic.Pic(d, large, *a.particles(), **kw)
+    a.retree(large)
+    held = a.info().device_bytes
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s, capture_error_mode="thread_local"):
+        a.init_leapfrog(0.0)
+    graph.replay()
+    torch.cuda.synchronize()
+    b.init_leapfrog(0.0)  # rows, from the same charges and a potential of zero
+    b.sync()
+    assert close(a.potential(), b.potential()) and np.any(b.potential())
+    for h in (a, b):
+        h.step(0.05)
+        h.sync()
+    assert close(a.potential(), b.potential())
+    assert a.info().device_bytes == held  # a step takes no memory
