@@ -21,7 +21,7 @@
 //
 // One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 70 us (172 MB of
 // V, b and V' take 25 us; bound by latency and issue), 81^3 FP32 149 -> 5.6 us
-// and FP64 277 -> 20.8 us, 27^3 FP32 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us
+// and FP64 277 -> 20.6 us, 27^3 FP32 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us
 // (both the rate of dependent launches).
 #pragma once
 
@@ -677,15 +677,11 @@ __global__ void __launch_bounds__(128) k_jacobi_strip2(DevTree t, const T *b, co
 constexpr int64_t kStripVertices = 200000;
 constexpr unsigned kJacobiThreads = 128;
 
-// Planes per thread of k_jacobi_strip3 (M a multiple of 27): a long march reads
-// fewer planes twice, but a small grid needs its threads.  Measured at 81^3,
-// 3 / 9 / 27 planes: 26.1 / 28.7 / 47.3 us (an earlier form of the kernel).
-inline int march_length(int64_t M) {
-  const int64_t cols = M * M / 3;
-  int len = 27;
-  while (len > 3 && cols * (M / len) < 40000) len /= 3;
-  return len;
-}
+// Planes per thread of k_jacobi_strip3 (M is a multiple of 27): a long march reads
+// fewer planes twice, but leaves the FP64 pipes fewer warps.  3 / 9 / 27 / 81 planes:
+// 81^3 21.8 / 20.6 / 46.3 / 127.7 us a sweep with its share of the solve, 243^3 393 /
+// 344 / 349 / 413.
+constexpr int kMarch = 9;
 
 template <typename... P, typename... A>
 inline void launch_pdl(void (*k)(P...), dim3 grid, dim3 block, cudaStream_t s, A... args) {
@@ -727,9 +723,8 @@ int64_t launch_jacobi_uniform(const DevTree &t, const T *b, const T *Vin, T *Vou
   } else if constexpr (D == 3) {
     // one warp a block spreads the work evenly over the SMs' FP64 pipes (81^3: 486
     // blocks of 128 threads leave the pipes idle for half the time, 29.7 -> 23.5 us)
-    const int len = march_length(M);
-    const dim3 g(grid_for(M * (M / 3), 32), (unsigned)(M / len));
-    launch_pdl(k_jacobi_strip3<kRes>, g, dim3(32), s, t, b, Vin, Vout, omega, r2, len);
+    const dim3 g(grid_for(M * (M / 3), 32), (unsigned)(M / kMarch));
+    launch_pdl(k_jacobi_strip3<kRes>, g, dim3(32), s, t, b, Vin, Vout, omega, r2, kMarch);
     return (int64_t)g.x * g.y;
   }
 }
