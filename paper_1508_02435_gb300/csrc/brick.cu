@@ -125,10 +125,6 @@ __device__ __forceinline__ int32_t brick_of_coords(const DevTree &t, const int32
 // K1
 // ---------------------------------------------------------------------------
 
-// ---------------------------------------------------------------------------
-// K1, shared-memory form
-// ---------------------------------------------------------------------------
-
 // Two independent FP32 products in one instruction, each rounded to nearest.
 __device__ __forceinline__ float2 mul2_rn(float2 a, float2 b) {
   float2 r;
@@ -311,7 +307,7 @@ struct HalfView {
 // (chunk c = first, first + stride, ...), pass B appends them to the
 // destination units' staging areas after one reservation per unit.  wc holds
 // the warp's kUnitSlots counters (zero on entry).  Same arithmetic as
-// push_core (gather in corner order, kick, drift, split re-location), with
+// k_push32 (gather in corner order, kick, drift, split re-location), with
 // the destination found from the brick-local cell through a per-axis table.
 template <int D, bool kAligned>
 __device__ __forceinline__ void push_half_warp(const DevTree &t, const BrickGeom &g, const BrickPushArgs &a,

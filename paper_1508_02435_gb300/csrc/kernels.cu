@@ -3,7 +3,7 @@
 // Step structure (Section 3 PIC cycle + Section 5 re-binning):
 //   deposit   k_leaf_partials -> k_vertex_charge -> k_sum_blocks        (item 1)
 //   solve     k_rhs -> sweeps of uniform_solve / adaptive_solve / row_solve / resident_solve (auxiliary, item 2)
-//   field     k_efield                                                  (item 3)
+//   field     k_efield_uniform / k_efield_adaptive                      (item 3)
 //   push      k_push64 / k_push32: gather E_i = R^T(x_i) E, leapfrog kick
 //             and drift, wrap, re-location (descent / split resolve), new
 //             key, moved flag (warp ballot), mover ranks                 (items 3-4)
@@ -63,14 +63,6 @@ static inline unsigned grid_for(int64_t n, int block = kBlock) {
 __device__ __forceinline__ void leaf_info(const DevTree &t, int32_t L, int *lev, int32_t *c) {
   *lev = t.leaf_level[L];
   for (int a = 0; a < t.d; ++a) c[a] = t.leaf_coords[(int64_t)L * t.d + a];
-}
-
-// The same with the dimension known at compile time (the loop unrolls).
-template <int D>
-__device__ __forceinline__ void leaf_info_d(const DevTree &t, int32_t L, int *lev, int32_t *c) {
-  *lev = t.leaf_level[L];
-#pragma unroll
-  for (int a = 0; a < D; ++a) c[a] = t.leaf_coords[(int64_t)L * D + a];
 }
 
 __device__ __forceinline__ const InstInfo &inst_of_leaf(const DevTree &t, int32_t L) {

@@ -131,9 +131,12 @@ __device__ __forceinline__ int32_t reflected_cell(int32_t c, float fl, int32_t p
   return per - 1;
 }
 
-// Four blocks of 512 per SM (32 registers; 3D spills a few): the push waits for
-// memory, and more warps wait together.  Three blocks -> four: 1e7 free 2D
-// particles 0.131 -> 0.112 ms, 2e8 two-stream particles 5.35 -> 5.07 ms.
+// Four blocks of 512 per SM (32 registers): the push waits for memory, and more
+// warps wait together.  It costs 20 to 36 bytes of spills a thread (56 in 3D
+// batches).  Three blocks -> four: 1e7 free 2D particles 0.131 -> 0.112 ms, 2e8
+// two-stream particles 5.35 -> 5.07; uniform PIDT, 8e6 particles on 729^2 cells 0.143
+// -> 0.136, 8e6 on 81^3 0.170 -> 0.167, 3e7 on 243^3, which alone loses, 0.784 ->
+// 0.815.
 template <int D, bool kUni, bool kBatch>
 __global__ void __launch_bounds__(512, 4) k_push32(DevTree t, Push32Args a) {
   constexpr int NC = 1 << D;

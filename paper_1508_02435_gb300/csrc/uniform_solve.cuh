@@ -180,8 +180,8 @@ __device__ __forceinline__ double sweep2(double c, double faces, double corners,
 // is formed as fma(x, zh, x zl) with zh + zl = 1 / diag in two floats
 // (Brisebarre, Muller and Raina, IEEE Trans. Computers 53(8), 2004): correctly
 // rounded for every x at every diagonal a uniform tree can have (2D: 8/3; 3D:
-// 8/3 3^-depth, depth 0 to 7, all 2^23 significands tried), as long as nothing
-// underflows or overflows, which the range check sees to.
+// 8/3 3^-depth, depth 0 to 7; tests/test_quotient.py tries all 2^23 significands),
+// as long as nothing underflows or overflows, which the range check sees to.
 constexpr float kQuotLo = 0x1p-60f, kQuotHi = 0x1p60f;
 
 template <int N>
