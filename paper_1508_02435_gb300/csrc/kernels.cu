@@ -73,7 +73,8 @@ __device__ __forceinline__ const InstInfo &inst_of_vertex(const DevTree &t, int6
 }
 
 // Global vertex ids of the corners of uniform-grid cell c of instance I.
-__device__ __forceinline__ void corner_vertices(const InstInfo &I, const int32_t *c, int d, int32_t *vid) {
+template <typename Grid>
+__device__ __forceinline__ void corner_vertices(const Grid &I, const int32_t *c, int d, int32_t *vid) {
   uniform_corner_vertices(c, d, I.M, vid);
   for (int e = 0; e < (1 << d); ++e) vid[e] += I.vert_off;
 }

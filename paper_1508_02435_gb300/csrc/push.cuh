@@ -6,13 +6,15 @@
 // (kBatch, uniform trees).  A batch's particle belongs to the instance of its
 // leaf: a state that is handed over may change the numbers of particles per
 // instance.  Single plasmas do not wait for that lookup (243 x 243 cells of 100
-// particles, five steps: 1.20 ms with it, 1.18 without).  3D steps
+// particles, five steps: 1.20 ms with it, 1.18 without) and have their grid in the
+// kernel's parameters (1e7 free 2D particles: from the instance table 0.111 ms, from
+// the parameters 0.109).  3D steps
 // write the pushed state as one record per particle, which the re-bin gathers
 // whole; 2D steps write rows.
 //
 // Measured against one kernel for all trees with divisions by 3^k, a descent
 // from the root and separate FP64 products and sums: FP64 push of 4.25e6
-// particles on 81^3 cells 0.98 -> 0.52 ms, FP64 push of the 1e6-particle 2D bump
+// particles on 81^3 cells 0.98 -> 0.51 ms, FP64 push of the 1e6-particle 2D bump
 // 0.19 -> 0.07 ms (adaptive FP64 trees now expand the field at the leaf corners
 // once per field, as FP32 did), 1e7 free 2D particles in a reflecting box 0.17 ->
 // 0.11 ms, 2e8 two-stream particles 7.3 -> 5.03 ms (whole-sector corner rows and
@@ -55,9 +57,20 @@ __device__ __forceinline__ void corner_row(const T *Ec, int32_t L, T *q) {
   for (int i = 0; i < N; i += W) load32(Ec + (int64_t)L * N + i, q + i);
 }
 
+// The grid of leaf L's instance.  A single plasma's is in the kernel's parameters.
+struct PushGrid {
+  int32_t M, depth, leaf_off, vert_off, spread_off;
+};
+template <bool kBatch>
+__device__ __forceinline__ PushGrid push_grid(const DevTree &t, int32_t L) {
+  if (!kBatch) return PushGrid{t.M, t.depth, 0, 0, 0};
+  const InstInfo &I = t.inst[t.inst_of_leaf[L]];
+  return PushGrid{I.M, I.depth, I.leaf_off, I.vert_off, I.spread_off};
+}
+
 // Level and coordinates of leaf L.
 template <int D, bool kUni>
-__device__ __forceinline__ int push_leaf(const DevTree &t, const InstInfo &I, int32_t L, int32_t *c) {
+__device__ __forceinline__ int push_leaf(const DevTree &t, const PushGrid &I, int32_t L, int32_t *c) {
   if (kUni) {
 #pragma unroll
     for (int k = 0; k < D; ++k) c[k] = t.leaf_coords[(int64_t)L * D + k];
@@ -72,8 +85,8 @@ __device__ __forceinline__ int push_leaf(const DevTree &t, const InstInfo &I, in
 
 // Sort key of a particle in leaf L through corner a.  Uniform trees: C is the
 // leaf's cell; adaptive ones read the owner-vertex table.
-template <int D, bool kUni>
-__device__ __forceinline__ int32_t push_key(const DevTree &t, const InstInfo &I, int32_t L, const uint32_t *C, int a) {
+template <int D, bool kUni, typename Grid>
+__device__ __forceinline__ int32_t push_key(const DevTree &t, const Grid &I, int32_t L, const uint32_t *C, int a) {
   constexpr int NC = 1 << D;
   if (t.scheme == 0) return L;
   int32_t pv;
@@ -132,11 +145,10 @@ __device__ __forceinline__ int32_t reflected_cell(int32_t c, float fl, int32_t p
 }
 
 // Four blocks of 512 per SM (32 registers): the push waits for memory, and more
-// warps wait together.  It costs 20 to 36 bytes of spills a thread (56 in 3D
-// batches).  Three blocks -> four: 1e7 free 2D particles 0.131 -> 0.112 ms, 2e8
-// two-stream particles 5.35 -> 5.07; uniform PIDT, 8e6 particles on 729^2 cells 0.143
-// -> 0.136, 8e6 on 81^3 0.170 -> 0.167, 3e7 on 243^3, which alone loses, 0.784 ->
-// 0.815.
+// warps wait together.  It costs 16 to 36 bytes of spills a thread (56 in 3D
+// batches).  Three blocks -> four: 1e7 free 2D particles 0.122 -> 0.109 ms, 2e8
+// two-stream particles 5.35 -> 5.07; uniform PIDT, 8e6 particles on 729^2 cells 0.139
+// -> 0.133, 8e6 on 81^3 0.171 -> 0.164, 3e7 on 243^3 0.796 -> 0.793.
 template <int D, bool kUni, bool kBatch>
 __global__ void __launch_bounds__(512, 4) k_push32(DevTree t, Push32Args a) {
   constexpr int NC = 1 << D;
@@ -151,7 +163,7 @@ __global__ void __launch_bounds__(512, 4) k_push32(DevTree t, Push32Args a) {
 #pragma unroll
     for (int k = 0; k < D; ++k) v[k] = a.v[k * n + p];
     const int32_t kold = t.scheme == 0 ? L : a.key[p];
-    const InstInfo &Ins = t.inst[kBatch ? t.inst_of_leaf[L] : 0];
+    const PushGrid Ins = push_grid<kBatch>(t, L);
     int32_t c[D];
     const int lev = push_leaf<D, kUni>(t, Ins, L, c);
     const bool field = a.E || a.Ec;
@@ -212,7 +224,7 @@ __global__ void __launch_bounds__(512, 4) k_push32(DevTree t, Push32Args a) {
 #pragma unroll
       for (int k = 0; k < D; ++k) o2[k] = clamp_off(f[k]);
     } else {
-      L2 = locate_split<D>(t, lev, I, f, o2, Ins.tab_root);
+      L2 = locate_split<D>(t, lev, I, f, o2, 0);
     }
     knew = push_key<D, kUni>(t, Ins, L2, I, pidt_corner_o(o2, D));
     moved = knew != kold;
@@ -263,7 +275,7 @@ __global__ void k_push64(DevTree t, Push64Args a) {
 #pragma unroll
     for (int k = 0; k < D; ++k) v[k] = a.v[k * n + p];
     const int32_t kold = t.scheme == 0 ? L : a.key[p];
-    const InstInfo &Ins = t.inst[kBatch ? t.inst_of_leaf[L] : 0];
+    const PushGrid Ins = push_grid<kBatch>(t, L);
     int32_t c[D];
     const int lev = push_leaf<D, kUni>(t, Ins, L, c);
     double t0 = 0.0;
@@ -325,7 +337,7 @@ __global__ void k_push64(DevTree t, Push64Args a) {
       const int32_t cc[3] = {(int32_t)C[0], (int32_t)C[1], D == 3 ? (int32_t)C[D - 1] : 0};
       L2 = Ins.leaf_off + uniform_leaf_of_cell(t.spread + Ins.spread_off, Ins.M, cc, D);
     } else if (!inside) {  // still inside its leaf: the covering leaf is the old one, no descent
-      L2 = locate_q<D>(t, Q, Ins.tab_root, &lev2, C);
+      L2 = locate_q<D>(t, Q, 0, &lev2, C);
     }
     int corner = 0;
     if (t.scheme != 0) {  // upper half of the leaf on each axis
