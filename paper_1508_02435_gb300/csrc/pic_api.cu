@@ -1057,9 +1057,9 @@ int bin_fresh(pic_t h) {
 // call returns, on any stream: one pass reads them, and it is over when the order
 // flag is here.  Large 2D states in no order are packed, so that the gather reads
 // one sector of a particle's offsets and velocities instead of four, whose rows
-// together are more than the L2 holds (2e7 particles, PIT / PIDT: rows 2.27 / 2.94
-// ms, packed 1.57 / 2.17; 5e6: 0.45 / 0.61, 0.39 / 0.51; 1e6: 0.145 / 0.173, 0.150 /
-// 0.167, where the line lies).
+// together are more than the L2 holds (with the state and the charges read back,
+// 2e7 particles, PIT / PIDT: rows 2.37 / 3.01 ms, packed 1.57 / 2.17; 5e6: 0.45 /
+// 0.61, 0.39 / 0.51; 1e6: 0.145 / 0.173, 0.150 / 0.167, where the line lies).
 constexpr int64_t kPackRows = 1 << 20;
 int bin_split_state(pic_t h, const int32_t *leaf, const float *o, const float *v, bool copied) {
   h->q_valid = false;

@@ -19,9 +19,9 @@
 // FP64 sums the stencil by neighbour class: fewer operations (the FP64 pipe
 // bounds these kernels), hence fewer roundings.
 //
-// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 70 us (172 MB of
-// V, b and V' take 25 us; bound by latency and issue), 81^3 FP32 149 -> 5.6 us
-// and FP64 277 -> 20.6 us, 27^3 FP32 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us
+// One sweep, leaf walk -> here (GB300): 243^3 FP32 3,770 -> 68 us (172 MB of
+// V, b and V' take 25 us; bound by latency and issue), 81^3 FP32 149 -> 5.4 us
+// and FP64 277 -> 19.1 us, 27^3 FP32 22 -> 2.1 us and 27^2 FP64 11 -> 1.6 us
 // (both the rate of dependent launches).
 #pragma once
 
