@@ -689,8 +689,13 @@ int assemble_rows(pic_t h) {
   launch_row_count(h->dt, m.len, h->scalars + 4, s);
   launch_exclusive_scan(m.len, ns, m.ptr, h->tile_sums, h->scalars + 3, s);
   CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s));
-  CK(cudaStreamSynchronize(s));
+  // the read-back must not end a capture that another thread holds, as no other call of a step would
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  CK(cudaThreadExchangeStreamCaptureMode(&mode));
+  cudaError_t e = cudaMemcpyAsync(got, h->scalars + 3, sizeof(got), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  CK(e);
   if (!got[1] && got[0] <= row_capacity(h->dt)) {
     launch_row_fill(h->dt, m.ptr, h->cfg.omega, m.col, m.val, m.scale, s);
     CK(cudaGetLastError());

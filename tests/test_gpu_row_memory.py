@@ -3,6 +3,8 @@ of their blocks is refused, at creation or at a re-tree, the handle solves by th
 two passes and gives the other blocks back."""
 from __future__ import annotations
 
+import threading
+
 import numpy as np
 import pytest
 
@@ -136,3 +138,33 @@ def test_rows_wait_for_the_first_solve(d):
         h.sync()
     assert close(a.potential(), b.potential())
     assert a.info().device_bytes == held  # a step takes no memory
+
+
+def test_first_solve_leaves_another_threads_capture_alone():
+    flags = trees(2)[1]
+    n = 3001
+    x, v = W.random_particles(2, n, 8, vmax=0.1)
+    kw = dict(precision=pic.FP64, q=-1.0 / n, ion=0.3, sweeps=ROWS_FROM)
+    want = stepped(pic.Pic(2, flags, x, v, **kw))
+    h = pic.Pic(2, flags, x, v, stream=torch.cuda.Stream(), **kw)
+    a = torch.zeros(1000, device="cuda")
+    graph, failed = torch.cuda.CUDAGraph(), []
+
+    def step():
+        try:
+            h.step(0.05)
+        except pic.PicError as e:
+            failed.append(e)
+
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream(), capture_error_mode="global"):
+        a += 1
+        other = threading.Thread(target=step)
+        other.start()
+        other.join()
+        a += 1
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not failed and torch.all(a == 2)
+    h.sync()
+    assert np.array_equal(h.potential(), want)
