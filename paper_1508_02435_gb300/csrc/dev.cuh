@@ -25,6 +25,7 @@ struct InstInfo {
   double q, ion, ion_load, diag;
   double h;                    // uniform trees: leaf width 3^-depth
   double jac[3];               // FP64 sweep: 1 - omega, -omega / diag times the face and edge / corner entries
+  double rhs, rhs_lo;          // omega / diag in two doubles
   float q32, ion32, ion_load32, diag32, h32;
   float rdiag32, rdiag_lo32;   // 1 / diag32 in two floats
 };

@@ -176,15 +176,22 @@ __device__ __forceinline__ void local_coords(const double *x, int64_t n, int64_t
 // a8 solve (auxiliary): b = Q - (sum Q) integral(phi); damped Jacobi
 // ---------------------------------------------------------------------------
 
-// With scale, also omega / diag per vertex; with raw, b itself there and b times
-// omega / diag in b.
+// With scale, also omega / diag per vertex; with raw (FP64, uniform trees), b itself
+// there and b times omega / diag, rounded once, in b: a rounded factor would shift
+// the whole potential (field of 2D batches against plain 64-bit values, with the
+// leaf width's rounding in k_efield_uniform: 2.8e-16 relative, 2.1e-16 so).
 template <typename T>
 __global__ void k_rhs(DevTree t, const T *Q, const double *total, T *b, T omega, T *scale, T *raw) {
   int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= t.n_vert) return;
   T tot = (T)(t.n_inst > 1 ? total[1 + t.inst_of_vert[v]] : *total);
   const T r = Q[v] - tot * ion_load(t, v, (T)0);
-  b[v] = raw ? r * (omega / diag_val(t, v, (T)0)) : r;
+  if (raw) {
+    const InstInfo &I = inst_of_vertex(t, v);
+    b[v] = (T)fma((double)r, I.rhs, (double)r * I.rhs_lo);
+  } else {
+    b[v] = r;
+  }
   if (raw) raw[v] = r;
   if (scale) scale[v] = omega / diag_val(t, v, (T)0);
 }

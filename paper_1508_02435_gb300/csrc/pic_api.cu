@@ -378,6 +378,8 @@ int install_forest(pic_t h, const pic_tree_desc *trees, int32_t n_inst, const st
       // neighbours): matrix entries 8/3 h^(d-2) on the diagonal, in 2D -1/3 (faces) and -1/3
       // (corners), in 3D -1/12 h per shared leaf
       const double w = h->cfg.omega / I.diag, hs = d == 3 ? I.h : 1.0;
+      I.rhs = w;
+      I.rhs_lo = std::fma(-w, I.diag, h->cfg.omega) / I.diag;
       I.jac[0] = 1.0 - h->cfg.omega;
       I.jac[1] = w * (1.0 / 3.0);
       I.jac[2] = d == 3 ? w * (hs / 12.0) : w * (1.0 / 3.0);

@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(Resident<T, D, M>::kThreads) k_solve_resident(
     const int at = act ? (z0 + (D == 3 ? i : row)) * PL + own : 0;
     v[i] = V[at];
     b[i] = raw[i] = Q[at] - tot * ion_load(t, 0, (T)0);
-    if constexpr (sizeof(T) == 8) b[i] = b[i] * (omega / I.diag);
+    if constexpr (sizeof(T) == 8) b[i] = fma(b[i], I.rhs, b[i] * I.rhs_lo);
   }
   auto apply = [&](const T *s, int i, bool any) {
     if (sizeof(T) == 4) w[D - 1] = wl[i];

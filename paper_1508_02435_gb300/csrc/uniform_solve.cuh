@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(256) k_efield_uniform(DevTree t, const double 
   const double *F = V + I.vert_off;
   int32_t r = (int32_t)(v - I.vert_off), stride = 1;
   const int32_t at = r;
-  const double f = 0.5 * (double)M;  // 1 / (2 h)
+  const double f = 0.5 / I.h;  // the rounded leaf width, as in the edge differences (not M / 2 at 243)
 #pragma unroll
   for (int a = 0; a < D; ++a) {
     const int32_t q = r / M, j = r - q * M;
