@@ -10,7 +10,7 @@
 //
 // One sweep of the 1e6-particle bump (2D, 75,451 vertices, FP64): 64 -> 9.9 us, two
 // dependent launches.  FP64 handles take assembled rows where row_solve.cuh has
-// built them (3.7 us); FP32 sums must keep this order, so FP32 stays here.
+// built them (3.8 us); FP32 sums must keep this order, so FP32 stays here.
 #pragma once
 
 namespace pic {

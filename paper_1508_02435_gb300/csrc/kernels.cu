@@ -740,7 +740,8 @@ static void solve(const DevTree &t, const RowMatrix &A, const T *Q, const double
   int64_t nb;
   if constexpr (sizeof(T) == 8) {
     if (A.val) {
-      nb = sweep_rows(t, A, b, V, Vtmp, sweeps, block_sum, s);
+      nb = t.d == 3 ? sweep_rows<3>(t, A, b, V, Vtmp, sweeps, block_sum, s)
+                    : sweep_rows<2>(t, A, b, V, Vtmp, sweeps, block_sum, s);
       { COUNT(1); k_sum_blocks<<<1, 1024, 0, s>>>(block_sum, nb, resid2); }
       return;
     }

@@ -211,6 +211,7 @@ struct RowMatrix {
   const int32_t *col;
   const double *val;
   const double *scale;          // omega / diag per vertex
+  const double *rest;           // 2D: minus the sum of the row's entries, zero but for their rounding
 };
 // Whether the solve of t runs as one cluster (small uniform trees).
 bool resident_solve_fits(const DevTree &t, bool split);
@@ -224,7 +225,7 @@ int64_t row_slices(const DevTree &t);
 int64_t row_capacity(const DevTree &t);  // entries reserved for them
 void launch_row_count(const DevTree &t, int32_t *slice, int32_t *too_long, cudaStream_t s);
 void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, double *scale,
-                     cudaStream_t s);
+                     double *rest, cudaStream_t s);
 void launch_efield(const DevTree &t, bool split, const void *V, void *E, void *part, cudaStream_t s);
 void launch_push64(const DevTree &t, const Push64Args &a, cudaStream_t s);
 void launch_push32(const DevTree &t, const Push32Args &a, cudaStream_t s);

@@ -89,7 +89,7 @@ struct pic_s {
   RowMatrix rows{};           // FP64, adaptive: assembled rows of the solve
   struct RowMemory {          // memory for them, until the first solve on the tree
     int32_t *ptr = nullptr, *len = nullptr, *col = nullptr;
-    double *val = nullptr, *scale = nullptr;
+    double *val = nullptr, *scale = nullptr, *rest = nullptr;
   } row_mem;
   char *ecorner = nullptr;    // adaptive: field at every leaf corner
   bool ecorner_valid = false; // ecorner holds the corners of the current E
@@ -660,7 +660,7 @@ int reserve_rows(pic_t h) {
   std::vector<DevBuf> mine;
   const std::string message = h->last_error;
   if (galloc(h, mine, &m.ptr, ns + 1) || galloc(h, mine, &m.len, ns) || galloc(h, mine, &m.col, cap) ||
-      galloc(h, mine, &m.val, cap) || galloc(h, mine, &m.scale, h->dt.n_vert)) {
+      galloc(h, mine, &m.val, cap) || galloc(h, mine, &m.scale, h->dt.n_vert) || galloc(h, mine, &m.rest, h->dt.n_vert)) {
     free_bufs(h, mine);
     cudaGetLastError();  // a refused cudaMalloc is no error of this call
     h->last_error = message;
@@ -699,9 +699,9 @@ int assemble_rows(pic_t h) {
   cudaThreadExchangeStreamCaptureMode(&mode);
   CK(e);
   if (!got[1] && got[0] <= row_capacity(h->dt)) {
-    launch_row_fill(h->dt, m.ptr, h->cfg.omega, m.col, m.val, m.scale, s);
+    launch_row_fill(h->dt, m.ptr, h->cfg.omega, m.col, m.val, m.scale, m.rest, s);
     CK(cudaGetLastError());
-    h->rows = RowMatrix{m.ptr, m.col, m.val, m.scale};
+    h->rows = RowMatrix{m.ptr, m.col, m.val, m.scale, m.rest};
   }
   m = pic_s::RowMemory{};  // assembled, or no use on this tree
   return PIC_OK;

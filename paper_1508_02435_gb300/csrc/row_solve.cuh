@@ -7,7 +7,17 @@
 // rows side by side, padded to the slice's longest row; a sweep is V' = V + scale
 // (b - A V) with scale = omega / diag per vertex, tabulated beside them.
 //
-// One sweep of the 2D bump (75,451 vertices): 9.9 -> 3.7 us.
+// A row of the exact matrix sums to zero; of the rounded entries it does not, and that
+// acts on the potential like a term of its own in every sweep.  In 2D the missing part
+// (rest, exact to a rounding of itself) is a tenth term of the sum.  3D rows, whose 27
+// terms also round more, take differences to the vertex's own value, which cost a
+// subtraction an entry on the FP64 pipe (in 2D 4.8 us a sweep of the bump below).
+// Against sweeps in extended precision, 100 sweeps of 24,017 vertices in 2D: the
+// potential is off by 1.7e-16, the field by 9.0e-16, without the rest 2.7e-15 and
+// 2.4e-15, leaf by leaf 3.9e-16 and 8.6e-16; 833 vertices in 3D: 1.1e-16 and 2.4e-16, as
+// plain sums 3.0e-16 and 4.0e-16, leaf by leaf 1.1e-16 and 2.2e-16.
+//
+// One sweep of the 2D bump (75,451 vertices): 9.9 -> 3.8 us.
 #pragma once
 
 namespace pic {
@@ -116,9 +126,16 @@ __global__ void __launch_bounds__(row_threads<D>()) k_row_count(DevTree t, int32
   if (threadIdx.x == 0) slice[blockIdx.x] = 32 * most;
 }
 
+// Adds x to hi + lo (Knuth's two-sum).
+__device__ __forceinline__ void two_sum(double &hi, double &lo, double x) {
+  const double s = hi + x, z = s - hi;
+  lo += (hi - (s - z)) + (x - z);
+  hi = s;
+}
+
 template <int D>
 __global__ void __launch_bounds__(row_threads<D>()) k_row_fill(DevTree t, const int32_t *ptr, double omega, int32_t *cols,
-                                                               double *vals, double *scale) {
+                                                               double *vals, double *scale, double *rest) {
   const int32_t b = ptr[blockIdx.x], m = (ptr[blockIdx.x + 1] - b) >> 5;
   auto put = [&](int64_t v, int k, int len, int32_t col, double val) {  // entry k of the row, padded to m
     const int64_t at = b + 32 * k + (v & 31);
@@ -141,13 +158,18 @@ __global__ void __launch_bounds__(row_threads<D>()) k_row_fill(DevTree t, const 
     int32_t col[kRowMax];
     double val[kRowMax];
     const int len = v < t.n_vert ? assemble_row<D>(t, v, col, val) : 0;
-    if (v < t.n_vert) scale[v] = omega / t.diag64[v];
+    double hi = 0.0, lo = 0.0;
+    for (int k = 0; k < len; ++k) two_sum(hi, lo, val[k]);
+    if (v < t.n_vert) {
+      scale[v] = omega / t.diag64[v];
+      rest[v] = -(hi + lo);
+    }
     for (int k = 0; k < m; ++k) put(v, k, len, col[k], val[k]);
   }
 }
 
 // b and V as in k_vertex_pass; kRes: block sums of the squared residual.
-template <bool kRes>
+template <int D, bool kRes>
 __global__ void __launch_bounds__(128) k_row_sweep(DevTree t, RowMatrix A, const double *b, const double *Vin,
                                                    double *__restrict__ Vout, double *r2) {
   const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -155,7 +177,7 @@ __global__ void __launch_bounds__(128) k_row_sweep(DevTree t, RowMatrix A, const
   constexpr int kPre = 9;  // entries read while the sweep before runs
   int32_t col[kPre], p = 0, end = 0;
   double val[kPre];
-  const double scale = !kRes && act ? A.scale[v] : 0.0;
+  const double scale = !kRes && act ? A.scale[v] : 0.0, rest = D == 2 && act ? A.rest[v] : 0.0;
   if (act) {
     p = A.ptr[v >> 5];
     end = A.ptr[(v >> 5) + 1];
@@ -175,10 +197,11 @@ __global__ void __launch_bounds__(128) k_row_sweep(DevTree t, RowMatrix A, const
 #pragma unroll
     for (int k = 0; k < kPre; ++k) u[k] = col[k] >= 0 ? Vin[col[k]] : 0.0;
     const double bv = b[v], vc = Vin[v];
+    if (D == 2) y = rest * vc;
 #pragma unroll
     for (int k = 0; k < kPre; ++k)
-      if (col[k] >= 0) y = fma(val[k], u[k], y);
-    for (int32_t i = p + 32 * kPre; i < end; i += 32) y = fma(A.val[i], Vin[A.col[i]], y);
+      if (col[k] >= 0) y = fma(val[k], D == 3 ? u[k] - vc : u[k], y);
+    for (int32_t i = p + 32 * kPre; i < end; i += 32) y = fma(A.val[i], D == 3 ? Vin[A.col[i]] - vc : Vin[A.col[i]], y);
     const double r = bv - y;
     if (kRes) rr = r * r;
     else Vout[v] = fma(scale, r, vc);
@@ -202,26 +225,27 @@ void launch_row_count(const DevTree &t, int32_t *slice, int32_t *too_long, cudaS
 }
 
 void launch_row_fill(const DevTree &t, const int32_t *ptr, double omega, int32_t *cols, double *vals, double *scale,
-                     cudaStream_t s) {
+                     double *rest, cudaStream_t s) {
   COUNT(1);
   const unsigned g = (unsigned)row_slices(t);
-  if (t.d == 3) k_row_fill<3><<<g, row_threads<3>(), 0, s>>>(t, ptr, omega, cols, vals, scale);
-  else k_row_fill<2><<<g, row_threads<2>(), 0, s>>>(t, ptr, omega, cols, vals, scale);
+  if (t.d == 3) k_row_fill<3><<<g, row_threads<3>(), 0, s>>>(t, ptr, omega, cols, vals, scale, rest);
+  else k_row_fill<2><<<g, row_threads<2>(), 0, s>>>(t, ptr, omega, cols, vals, scale, rest);
 }
 
 // Sweeps between V and Vtmp, then the residual's block sums; returns their number.
+template <int D>
 static int64_t sweep_rows(const DevTree &t, const RowMatrix &A, const double *b, double *V, double *Vtmp, int sweeps,
                           double *r2, cudaStream_t s) {
   const dim3 g(grid_for(t.n_vert, 128)), block(128);
   double *in = V, *out = Vtmp;
   for (int it = 0; it < sweeps; ++it) {
     COUNT(1);
-    launch_pdl(k_row_sweep<false>, g, block, s, t, A, b, in, out, r2);
+    launch_pdl(k_row_sweep<D, false>, g, block, s, t, A, b, in, out, r2);
     std::swap(in, out);
   }
   if (in != V) cudaMemcpyAsync(V, in, sizeof(double) * t.n_vert, cudaMemcpyDeviceToDevice, s);
   COUNT(1);
-  launch_pdl(k_row_sweep<true>, g, block, s, t, A, b, V, nullptr, r2);
+  launch_pdl(k_row_sweep<D, true>, g, block, s, t, A, b, V, nullptr, r2);
   return g.x;
 }
 
